@@ -191,9 +191,9 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     const size_t ntaps = pl->taps_host.size();
     std::vector<float> t32(ntaps);
     for (size_t i = 0; i < ntaps; ++i) t32[i] = (float)pl->taps_host[i];
-    size_t part_elems = 0, max_smem = 0, gs_max = 0, fs_max = 0, ls_max = 0, es_max = 0;
+    size_t part_elems = 0, max_smem = 0, fs_max = 0, ls_max = 0, es_max = 0;
     uint32_t maxB = 0, max_groups = 0;
-    size_t sum_groups = 0, sum_B = 0;  // general: hashing groups and bins over all rounds
+    size_t sum_B = 0;  // general: bins over all rounds
     // exact mode: every round's partial folds live at once (the one-launch path gathers all rounds
     // before their finishers), round t at part_off[t] of a request's region
     std::vector<size_t> part_off;
@@ -223,15 +223,13 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     }
     for (const GeneralRound& r : pl->grounds) {
         pl->samples += (uint64_t)r.nhash * (2 * (uint64_t)r.T + 1);
-        const size_t e = (size_t)r.ngroups * r.ctas * 2 * r.B;
+        const size_t e = (size_t)r.ngroups * 2 * r.B;
         if (e > part_elems) part_elems = e;
         if ((size_t)r.nhash * r.B > pl->bins_stride) pl->bins_stride = (size_t)r.nhash * r.B;
         if ((size_t)r.npairs * r.B > pl->phase_stride) pl->phase_stride = (size_t)r.npairs * r.B;
         if (r.B > maxB) maxB = r.B;
         if (r.ngroups > max_groups) max_groups = r.ngroups;
-        sum_groups += r.ngroups;
         sum_B += r.B;
-        gs_max = r.smem_gather > gs_max ? r.smem_gather : gs_max;
         if (r.fin_global) {
             pl->gfin_stride = std::max(pl->gfin_stride, (r.smem_finish + 255) & ~size_t(255));
             pl->gfin_groups += r.ngroups;  // each such round has its own region
@@ -261,10 +259,8 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     SFFT_ALLOC(pl->d_taps64, ntaps * sizeof(double));
     SFFT_ALLOC(pl->d_wtab, pl->wtab_len * sizeof(double));
     SFFT_ALLOC(pl->d_part, pl->part_bytes);
-    // arrival counters: per (round, request) twice in exact mode; in general mode per (round, request,
-    // hashing group), each round in its own region because stream groups may run different rounds at
-    // once, then per request
-    const size_t ncounters = (size_t)max_batch * (general ? sum_groups + 1 : 2 * pl->rounds.size());
+    // arrival counters: per (round, request) twice in exact mode, per request in general mode
+    const size_t ncounters = (size_t)max_batch * (general ? 1 : 2 * pl->rounds.size());
     SFFT_ALLOC(pl->d_counter, ncounters * sizeof(uint32_t));
 
     SFFT_ALLOC(pl->d_zidx, (size_t)max_batch * p->z_cap * sizeof(uint32_t));
@@ -349,7 +345,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
             return fail(e, "create event");
     }
     if (!general && (e = set_exact_smem_limit(max_smem, fp64)) != cudaSuccess) return fail(e, "shared memory limit");
-    if (general && (e = general_set_smem(gs_max, fs_max, ls_max, es_max)) != cudaSuccess)
+    if (general && (e = general_set_smem(fs_max, ls_max, es_max)) != cudaSuccess)
         return fail(e, "shared memory limit");
     // The gather reads one 8- or 16-byte sample per 32-byte sector at random; ask L2 not to widen
     // its DRAM fetches beyond a sector (a per-context performance hint, ignored where unsupported).
@@ -430,13 +426,11 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
     SFFT_CUDA(cudaMemsetAsync(plan->d_zcount, 0, batch * sizeof(uint32_t), st), "clear zhat");
     SFFT_CUDA(cudaMemsetAsync(plan->d_zflag, 0, batch * sizeof(int32_t), st), "clear flags");
     const uint32_t R = (uint32_t)plan->grounds.size();
-    // stream groups may run different rounds at once, so every round has its own regions: gather
-    // counters from max_batch goff[r] (the estimate's counters at max_batch goff[R]), candidates,
+    // stream groups may run different rounds at once, so every round has its own regions: candidates,
     // estimates and magnitudes from max_batch boff[r], device-memory finish arrays from
     // max_batch foff[r] slices
-    std::vector<size_t> goff(R + 1, 0), boff(R + 1, 0), foff(R + 1, 0);
+    std::vector<size_t> boff(R + 1, 0), foff(R + 1, 0);
     for (uint32_t r = 0; r < R; ++r) {
-        goff[r + 1] = goff[r] + plan->grounds[r].ngroups;
         boff[r + 1] = boff[r] + plan->grounds[r].B;
         foff[r + 1] = foff[r] + (plan->grounds[r].fin_global ? plan->grounds[r].ngroups : 0);
     }
@@ -477,9 +471,8 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.B = gr.B;
             a.logB = gr.logB;
             a.T = gr.T;
-            a.chunks = gr.chunks;
-            a.cpb = gr.cpb;
-            a.ctas = gr.ctas;
+            a.rtaps = gr.rtaps;
+            a.batch = batch;
             a.dmax = gr.dmax;
             a.t = gr.t;
             a.logtp = gr.logtp;
@@ -501,8 +494,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.tw_shift = plan->tw_shift;
             a.part = reinterpret_cast<float2*>(plan->d_part);
             a.part_stride = plan->part_stride;
-            a.gcount = plan->d_counter + (size_t)plan->max_batch * goff[r];
-            a.ecount = plan->d_counter + (size_t)plan->max_batch * goff[R];
+            a.ecount = plan->d_counter;
             a.est_w = plan->d_estw + (size_t)plan->max_batch * boff[r];
             a.est_mag = reinterpret_cast<double*>(plan->d_estw + (size_t)plan->max_batch * boff[R]) +
                         (size_t)plan->max_batch * boff[r];

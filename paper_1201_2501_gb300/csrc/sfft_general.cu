@@ -7,9 +7,8 @@
 // So a round is four launches for the whole batch (five with the permuted copy):
 //   0. k_gen_permute  (rounds whose LocateInner pairs gather >= 2n samples) every request: x_{sigma m}
 //                     for all m under the round's sigma, so that the pairs read it in order;
-//   1. k_gen_gather   every (chunk range, hashing group, request): permuted gather, window,
-//                     modulation, fold mod B (HashToBins steps 1-2) into partial sums; the group's
-//                     last CTA to arrive sums them in chunk order;
+//   1. k_gen_gather   every (residue block, hashings, request): permuted gather, window, modulation,
+//                     fold mod B (HashToBins steps 1-2);
 //   2. k_gen_finish   every (hashing group, request): the fold's B-point FFT
 //                     (step 3), recovered coefficients subtracted in FP64 (step 4), bins stored;
 //                     for a LocateInner pair also c_j = phase(u_j / u'_j);
@@ -125,106 +124,136 @@ __global__ void __launch_bounds__(kThreads) k_gen_permute(const GenArgs a) {
 // ------------------------------------------------------------------------------------------------
 // 1. gather and fold
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads, 3) k_gen_gather(const GenArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t s = a.req_base + blockIdx.z, g = blockIdx.y, c = blockIdx.x, tid = threadIdx.x;
-    const ReqView rq = gen_req(a, s);
-    const HashDesc h = group_desc(a, rq.seed, rq.id, g);
-    float2* stage = reinterpret_cast<float2*>(smem);   // [2][kChunkTaps]
-    float2* red = stage + 2 * kChunkTaps;               // [H][max(B, kThreads)]
-    // a pair of a round with a permuted copy reads xperm[(t - a) mod n] = x_{sigma (t - a)} in order
-    const bool perm = a.xperm != nullptr && g < a.npairs;
-    const float2* __restrict__ x = perm ? a.xperm + (size_t)s * a.n : static_cast<const float2*>(rq.x);
-    const uint32_t xmul = perm ? 1u : h.sigma, xmask = perm ? a.nmask : rq.xmask;
-    const bool big = a.B > (uint32_t)kThreads;
-    if (big)
-        for (uint32_t i = tid; i < h.H * a.B; i += kThreads) red[i] = make_float2(0.f, 0.f);
-    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    const uint32_t sb = h.sigma * h.b;
-    const float inv_half_n = 2.0f / (float)a.n;
-    const uint32_t c0 = c * a.cpb, c1 = min(c0 + a.cpb, a.chunks);
-    int64_t t_first = -a.T + (int64_t)c0 * kChunkTaps;
-    for (uint32_t ch = c0; ch < c1; ++ch) {
-        const int64_t t_lo = -a.T + (int64_t)ch * kChunkTaps;
-        const uint32_t ntap = (uint32_t)(min(t_lo + (int64_t)kChunkTaps, a.T + 1) - t_lo);
-        // step 1a: x_{sigma (t - a_h)} for the chunk's taps of every hashing of the group, 16 loads in
-        // flight per thread (a pair's whole chunk in one batch)
-        const uint32_t total = h.H * ntap;
-        for (uint32_t f0 = tid; f0 < total; f0 += kThreads * 16) {
-            float2 v[16];
+// A CTA owns kThreads residues mod B of NH hashings that share (sigma, b) -- the two of each of NH / 2
+// LocateInner pairs, or one EstimateValues hashing -- and folds every tap of those residues, one
+// residue per thread: no partial fold leaves the CTA.  Samples go from L2 or HBM straight to the
+// thread that folds them (16 loads in flight each), and a tap's window product G_t w^{sigma b t} is
+// formed once for the NH hashings.
+// Measured against the form it replaces (four 2048-tap chunks per CTA staged in shared memory, partial
+// folds of every CTA summed by the last to arrive), whole calls: n = 2^22, k = 256, batch 8: 1323 us,
+// was 1552; n = 2^20, k = 500, batch 5: 1252 us, was 1797.  Bound by L2 (the pairs' in-order reads) or
+// by random 32-byte sectors of HBM (long signals).
+// Order of the sums: the window is cut into ranges of a.rtaps taps; a residue's taps of a range are
+// accumulated in order from zero (B < kThreads: by the kThreads / B threads of the residue, whose sums
+// are added in thread order), and the ranges' sums are added in range order.
+template <int NH>
+__device__ __forceinline__ void gather_residues(const GenArgs& a, const float2* __restrict__ x, uint32_t xmul,
+                                                uint32_t xmask, uint32_t sb, const uint32_t* ah, uint32_t nh,
+                                                float2* __restrict__ out, float2 (*red)[kThreads]) {
+    constexpr int TB = NH >= 8 ? 2 : (NH == 4 ? 4 : (NH == 2 ? 8 : 16));  // taps per batch of loads
+    const uint32_t tid = threadIdx.x, B = a.B;
+    const uint32_t step = B > (uint32_t)kThreads ? B : (uint32_t)kThreads;  // a thread's taps are step apart
+    const uint32_t k0 = blockIdx.x * kThreads + tid;
+    const uint32_t ntot = (uint32_t)(2 * a.T + 1);
+    const uint32_t t0 = (uint32_t)(int32_t)(-a.T) + k0;  // first tap, mod 2^32
+    const uint32_t nt = a.rtaps / step;                  // a thread's taps per range (a power of two if there are several)
+    const bool several = ntot > a.rtaps;
+    const uint32_t first = blockIdx.x * kThreads;
+    const uint32_t mend = first < ntot ? (ntot - first + step - 1) / step : 0;  // batches end here for every thread
+    float2 acc[NH], sum[NH];
+    uint32_t xi[NH];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const uint32_t f = f0 + (uint32_t)q * kThreads;
-                if (f < total) {
-                    const bool second = f >= ntap;
-                    const uint32_t i = second ? f - ntap : f;
-                    const int32_t base = (int32_t)(t_lo - (int64_t)(second ? h.a[1] : h.a[0]));
-                    v[q] = __ldcg(x + ((xmul * (uint32_t)(base + (int32_t)i)) & xmask));
+    for (int h = 0; h < NH; ++h) {
+        acc[h] = sum[h] = make_float2(0.f, 0.f);
+        xi[h] = xmul * (t0 - ah[h]);
+    }
+    const uint32_t xstep = xmul * step, estep = sb * step;
+    uint32_t e0 = sb * t0;
+    const float two_over_n = 2.0f / (float)a.n;
+    auto end_range = [&]() {
+        if (B >= (uint32_t)kThreads) {
+#pragma unroll
+            for (int h = 0; h < NH; ++h) sum[h] = cadd(sum[h], acc[h]);
+        } else {
+            // thread r < B owns residue (r - T) mod B: the threads r + i B folded its taps
+#pragma unroll
+            for (int h = 0; h < NH; ++h) red[h][tid] = acc[h];
+            __syncthreads();
+            if (tid < B)
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    float2 w = make_float2(0.f, 0.f);
+                    for (uint32_t i = tid; i < (uint32_t)kThreads; i += B) w = cadd(w, red[h][i]);
+                    sum[h] = cadd(sum[h], w);
                 }
-            }
+            __syncthreads();
+        }
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const uint32_t f = f0 + (uint32_t)q * kThreads;
-                if (f < total) stage[f < ntap ? f : kChunkTaps + (f - ntap)] = v[q];
-            }
-        }
-        __syncthreads();
-        // step 1b + 2: window, modulation w^{sigma b t}, fold mod B
-        for (uint32_t k = tid; k < ntap; k += kThreads) {
-            const int32_t t = (int32_t)t_lo + (int32_t)k;
-            const float gv = a.taps[t < 0 ? -t : t];
-            const uint32_t e = (sb * (uint32_t)t) & a.nmask;
-            const int32_t es = e > (a.nmask >> 1) ? (int32_t)((int64_t)e - (int64_t)a.n) : (int32_t)e;
-            float sn, cs;
-            sincospif((float)es * inv_half_n, &sn, &cs);
-            const float2 gt = make_float2(gv * cs, -gv * sn);
-            if (!big) {
-                for (uint32_t hh = 0; hh < h.H; ++hh) acc[hh] = cfma(gt, stage[hh * kChunkTaps + k], acc[hh]);
-            } else {
-                const uint32_t r = (uint32_t)t & (a.B - 1);
-                for (uint32_t hh = 0; hh < h.H; ++hh)
-                    red[hh * a.B + r] = cfma(gt, stage[hh * kChunkTaps + k], red[hh * a.B + r]);
-            }
-        }
-        __syncthreads();
-    }
-    float2* part = a.part + (size_t)s * a.part_stride + ((size_t)g * a.ctas + c) * 2 * a.B;
-    if (!big) {
-        // every chunk starts at a multiple of B away from the first, so thread tid always folds
-        // residue (t_first + tid) mod B; the threads of residue r are owner + m B
-        for (uint32_t hh = 0; hh < h.H; ++hh) red[hh * kThreads + tid] = acc[hh];
-        __syncthreads();
-        for (uint32_t r = tid; r < a.B; r += kThreads) {
-            const uint32_t owner = (r - (uint32_t)t_first) & (a.B - 1);
-            for (uint32_t hh = 0; hh < h.H; ++hh) {
-                float2 sum = make_float2(0.f, 0.f);
-                for (uint32_t m = owner; m < (uint32_t)kThreads; m += a.B) sum = cadd(sum, red[hh * kThreads + m]);
-                part[hh * a.B + r] = sum;
-            }
-        }
-    } else {
-        for (uint32_t i = tid; i < h.H * a.B; i += kThreads) part[i] = red[i];
-    }
-    // step 2 across CTAs: the last CTA of this (request, group) to arrive sums the partial folds in
-    // chunk order into slot 0, so the finish reads one fold per hashing
-    if (a.ctas == 1 || arrive(a.gcount + (size_t)s * a.ngroups + g, a.ctas) == 0) return;
-    float2* part0 = a.part + (size_t)s * a.part_stride + (size_t)g * a.ctas * 2 * a.B;
-    for (uint32_t i = tid; i < h.H * a.B; i += kThreads) {
-        const uint32_t hh = i / a.B, r = i - hh * a.B;
-        const float2* src = part0 + (size_t)hh * a.B + r;
-        float2 sum = make_float2(0.f, 0.f);
-        uint32_t c0 = 0;
-        for (; c0 + 8 <= a.ctas; c0 += 8) {  // 8 loads in flight, added in order
-            float2 v[8];
+        for (int h = 0; h < NH; ++h) acc[h] = make_float2(0.f, 0.f);
+    };
+    for (uint32_t m0 = 0; m0 < mend; m0 += TB) {
+        float2 v[TB][NH];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = __ldcg(src + (size_t)(c0 + q) * 2 * a.B);
+        for (int u = 0; u < TB; ++u) {
+            const bool in = k0 + (m0 + (uint32_t)u) * step < ntot;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) sum = cadd(sum, v[q]);
+            for (int h = 0; h < NH; ++h)
+                if (in) v[u][h] = __ldcg(x + ((xi[h] + (uint32_t)u * xstep) & xmask));
         }
-        for (; c0 < a.ctas; ++c0) sum = cadd(sum, __ldcg(src + (size_t)c0 * 2 * a.B));
-        part0[(size_t)hh * a.B + r] = sum;
+        float2 gt[TB];
+#pragma unroll
+        for (int u = 0; u < TB; ++u) {
+            if (k0 + (m0 + (uint32_t)u) * step < ntot) {
+                const int32_t t = (int32_t)(t0 + (m0 + (uint32_t)u) * step);
+                const float gv = a.taps[t < 0 ? -t : t];
+                const uint32_t e = (e0 + (uint32_t)u * estep) & a.nmask;
+                const int32_t es = e > (a.nmask >> 1) ? (int32_t)((int64_t)e - (int64_t)a.n) : (int32_t)e;
+                float sn, cs;
+                sincospif((float)es * two_over_n, &sn, &cs);
+                gt[u] = make_float2(gv * cs, -gv * sn);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < TB; ++u) {
+            if (u % 2 == 0 && several && m0 + (uint32_t)u != 0 && ((m0 + (uint32_t)u) & (nt - 1)) == 0 &&
+                m0 + (uint32_t)u < mend)  // nt >= 2
+                end_range();
+            if (k0 + (m0 + (uint32_t)u) * step < ntot) {
+#pragma unroll
+                for (int h = 0; h < NH; ++h) acc[h] = cfma(gt[u], v[u][h], acc[h]);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < NH; ++h) xi[h] += (uint32_t)TB * xstep;
+        e0 += (uint32_t)TB * estep;
     }
-    if (tid == 0) a.gcount[(size_t)s * a.ngroups + g] = 0;  // every CTA of the group has arrived
+    end_range();
+    if (B >= (uint32_t)kThreads || tid < B) {
+        const uint32_t r = t0 & (B - 1);
+#pragma unroll
+        for (int h = 0; h < NH; ++h)
+            if ((uint32_t)h < nh) out[(size_t)h * B + r] = sum[h];
+    }
+}
+
+// Grid (residue blocks, EstimateValues hashings then blocks of P pairs, requests).
+template <int P>
+__global__ void __launch_bounds__(kThreads, 2) k_gen_gather(const GenArgs a) {
+    __shared__ float2 red[2 * P][kThreads];
+    const uint32_t s = a.req_base + blockIdx.z;
+    const ReqView rq = gen_req(a, s);
+    float2* part = a.part + (size_t)s * a.part_stride;
+    if (blockIdx.y < a.R_est) {
+        const uint32_t g = a.npairs + blockIdx.y;
+        const HashDesc h = group_desc(a, rq.seed, rq.id, g);
+        gather_residues<1>(a, static_cast<const float2*>(rq.x), h.sigma, rq.xmask, h.sigma * h.b, h.a, 1,
+                           part + (size_t)g * 2 * a.B, red);
+        return;
+    }
+    const uint32_t g0 = (blockIdx.y - a.R_est) * P, np = min((uint32_t)P, a.npairs - g0);
+    // a round with a permuted copy reads xperm[(t - a) mod n] = x_{sigma (t - a)} in order
+    const bool perm = a.xperm != nullptr;
+    uint32_t sigma, b, ah[2 * P];
+    locate_sigma_b(rq.seed, rq.id, a.round, a.nmask, &sigma, &b);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const uint32_t g = g0 + min((uint32_t)p, np - 1), D = g / a.R_loc;  // past the last pair: it again, not stored
+        uint64_t beta;
+        inner_a_beta(rq.seed, rq.id, a.round, g, a.nmask, a.beta_lo[D], a.beta_hi[D], &ah[2 * p], &beta);
+        ah[2 * p + 1] = (uint32_t)((ah[2 * p] + beta) & a.nmask);
+    }
+    gather_residues<2 * P>(a, perm ? a.xperm + (size_t)s * a.n : static_cast<const float2*>(rq.x), perm ? 1u : sigma,
+                           perm ? a.nmask : rq.xmask, sigma * b, ah, 2 * np, part + (size_t)g0 * 2 * a.B, red);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -272,9 +301,8 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     uint32_t* bin_list = reinterpret_cast<uint32_t*>(fb + Ly.bin_list);
     uint32_t* scan = reinterpret_cast<uint32_t*>(fb + Ly.scan);
     const uint32_t logNp = (uint32_t)(63 - __clzll((long long)a.n)) - a.logB;
-    // step 3: the fold (summed over chunks by the gather's last CTA), bit-reversed, B-point FFT per
-    // hashing
-    const float2* part = a.part + (size_t)s * a.part_stride + (size_t)g * a.ctas * 2 * B;
+    // step 3: the fold, bit-reversed, B-point FFT per hashing
+    const float2* part = a.part + (size_t)s * a.part_stride + (size_t)g * 2 * B;
     const uint32_t shift_br = 32u - a.logB;
     for (uint32_t i = tid; i < h.H * B; i += kThreads) {
         const uint32_t hh = i / B, r = i - hh * B;
@@ -928,15 +956,11 @@ __global__ void __launch_bounds__(kThreads) k_estimate_from_bins(const EstArgs a
 // ------------------------------------------------------------------------------------------------
 // launchers
 // ------------------------------------------------------------------------------------------------
-cudaError_t general_set_smem(size_t gather, size_t finish, size_t locate, size_t estimate) {
+cudaError_t general_set_smem(size_t finish, size_t locate, size_t estimate) {
     static std::mutex mu;  // plans may be created from several threads
     std::lock_guard<std::mutex> lk(mu);
     static size_t lim[4] = {0, 0, 0, 0};
     cudaError_t e = cudaSuccess;
-    if (gather > lim[0] && (e = cudaFuncSetAttribute(k_gen_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)gather)) == cudaSuccess)
-        lim[0] = gather;
-    if (e != cudaSuccess) return e;
     if (finish > lim[1] && (e = cudaFuncSetAttribute(k_gen_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)finish)) == cudaSuccess)
         lim[1] = finish;
@@ -961,7 +985,18 @@ cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const General
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    k_gen_gather<<<dim3(r.ctas, r.ngroups, batch), kThreads, r.smem_gather, st>>>(a);
+    // pairs per gather CTA: as many as leave the chip (152 SMs, 2 CTAs each) two waves of CTAs over the
+    // whole call, so that a tap's window product serves more hashings
+    const uint32_t blocks = r.B > (uint32_t)kThreads ? r.B / kThreads : 1u;
+    const uint64_t pairs = (uint64_t)blocks * r.npairs * a.batch;
+    const uint32_t P = pairs >= 4 * 608 ? 4u : (pairs >= 2 * 608 ? 2u : 1u);
+    const dim3 grid(blocks, a.R_est + (r.npairs + P - 1) / P, batch);
+    if (P == 4)
+        k_gen_gather<4><<<grid, kThreads, 0, st>>>(a);
+    else if (P == 2)
+        k_gen_gather<2><<<grid, kThreads, 0, st>>>(a);
+    else
+        k_gen_gather<1><<<grid, kThreads, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_gen_finish<<<dim3(r.ngroups, batch), kThreads, r.fin_global ? 0 : r.smem_finish, st>>>(a);
@@ -980,7 +1015,7 @@ cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st) {
 
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st) {
     const size_t smem = est_layout(a.nL > 0 ? a.nL : 1, a.kprime > 0 ? a.kprime : 1, 1).total;
-    cudaError_t e = general_set_smem(0, 0, 0, smem);
+    cudaError_t e = general_set_smem(0, 0, smem);
     if (e != cudaSuccess) return e;
     k_estimate_from_bins<<<1, kThreads, smem, st>>>(a);
     return cudaGetLastError();

@@ -364,9 +364,7 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
         r.B = (uint32_t)B;
         r.logB = ceil_log2(B);
         r.T = window_halfwidth(r.B, p.alpha0, p.delta);
-        r.chunks = (uint32_t)((2 * (uint64_t)r.T + 1 + kChunkTaps - 1) / kChunkTaps);
-        r.cpb = r.chunks < 4 ? r.chunks : 4;  // chunks per gather CTA: 4 beat 2 and 8 at n = 2^22, k = 256
-        r.ctas = (r.chunks + r.cpb - 1) / r.cpb;
+        r.rtaps = 4 * kChunkTaps;
         r.t = t;
         r.logtp = logtp;
         const uint32_t lw = ceil_log2(p.n / B);
@@ -389,7 +387,6 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
         r.nhash = 2 * r.npairs + p.R_est;
         r.taps_off = taps_off;
         r.wtab_off = wtab_off;
-        r.smem_gather = (size_t)2 * kChunkTaps * 8 + (size_t)2 * (B > (uint64_t)kThreads ? B : kThreads) * 8;
         r.smem_finish = general_finish_smem(r.B, p.z_cap);
         r.smem_locate = general_locate_smem(r.B);
         r.smem_estimate = general_estimate_smem(r.B, r.kprime, p.z_cap);
@@ -397,7 +394,7 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
         // group), the estimate's per request (its launch then gives each request a single CTA)
         r.fin_global = r.smem_finish > kFinSmemMax;
         r.est_global = r.smem_estimate > kFinSmemMax;
-        if (r.smem_gather > 200 * 1024 || r.smem_locate > 200 * 1024) return SFFT_ERR_K_RANGE;
+        if (r.smem_locate > 200 * 1024) return SFFT_ERR_K_RANGE;
         const uint64_t Np = p.n / B;
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, p.alpha0, p.delta, r.T, pl->taps_host.data() + taps_off);

@@ -206,14 +206,12 @@ struct GeneralRound {
     uint32_t kr = 0, kprime = 0;   // k_r and k' = 3 k_r
     uint32_t B = 0, logB = 0;
     int64_t T = 0;
-    uint32_t chunks = 0;           // 2048-tap chunks of the window
-    uint32_t cpb = 0;              // chunks per CTA of the gather launch
-    uint32_t ctas = 0;             // CTAs per hashing group and request
+    uint32_t rtaps = 0;            // taps per range of the fold's summation order
     uint32_t dmax = 0, t = 0, logtp = 0;
     uint64_t beta_lo[kMaxLevels] = {}, beta_hi[kMaxLevels] = {};
     uint32_t npairs = 0, ngroups = 0, nhash = 0;
     size_t taps_off = 0, wtab_off = 0;
-    size_t smem_gather = 0, smem_finish = 0, smem_locate = 0, smem_estimate = 0;
+    size_t smem_finish = 0, smem_locate = 0, smem_estimate = 0;
     bool fin_global = false, est_global = false;  // arrays too large for shared memory: in d_gfin / d_gest
     bool perm = false;             // the pairs read the permuted copy x_{sigma m} (written first)
 };
@@ -230,7 +228,8 @@ struct GenArgs {
     const ReqDesc* reqs;   // optional per-request table (see ReqDesc)
     uint32_t B, logB;
     int64_t T;
-    uint32_t chunks, cpb, ctas;
+    uint32_t rtaps;        // taps per range of the fold's summation order (see k_gen_gather)
+    uint32_t batch;        // requests of the whole call (its stream groups together)
     uint32_t dmax, t, logtp, R_loc, R_est, npairs, ngroups, nhash, kprime;
     uint64_t beta_lo[kMaxLevels], beta_hi[kMaxLevels];
     double s, est_gmin;
@@ -238,9 +237,8 @@ struct GenArgs {
     const double* wtab;
     const double2* tw;     // FP64 twiddles w^e = tw[e mod 2^tw_shift] tw[2^tw_shift + (e >> tw_shift)]
     uint32_t tw_shift;
-    float2* part;          // [batch][ngroups][ctas][2][B]; after the gather, ctas slot 0 holds the sum
+    float2* part;          // [batch][ngroups][2][B]: the folds
     size_t part_stride;    // elements per request
-    uint32_t* gcount;      // [batch][ngroups] arrival counters of the gather CTAs (zero between launches)
     uint32_t* ecount;      // [batch] arrival counters of the estimate CTAs (zero between launches)
     double2* est_w;        // [batch][B] candidates' estimates shared by a request's estimate CTAs
     double* est_mag;       // [batch][B] their squared magnitudes
@@ -329,8 +327,7 @@ struct sfft_plan_s {
     void* d_part = nullptr;
     size_t part_bytes = 0;
     size_t part_stride = 0;  // elements of the partial-fold buffer owned by one request
-    // arrival counters, zero between launches: exact [2 R][max_batch]; general, per round r,
-    // [max_batch][ngroups_r] for the gather, then [max_batch] for the estimate
+    // arrival counters, zero between launches: exact [2 R][max_batch]; general [max_batch]
     uint32_t* d_counter = nullptr;
     std::vector<sfft::ExactArgs> rdesc;  // [R] round blocks of the one-launch exact path
     std::vector<size_t> chan_off;        // exact FP32: round t's partial folds in a channel slot's area
@@ -425,7 +422,7 @@ sfft_status build_general_schedule(sfft_plan_s* pl);
 size_t general_finish_smem(uint32_t B, uint32_t zcap);
 size_t general_locate_smem(uint32_t B);
 size_t general_estimate_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
-cudaError_t general_set_smem(size_t gather, size_t finish, size_t locate, size_t estimate);
+cudaError_t general_set_smem(size_t finish, size_t locate, size_t estimate);
 cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st);
 cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);
