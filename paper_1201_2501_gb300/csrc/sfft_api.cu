@@ -68,7 +68,6 @@ void free_plan(sfft_plan_s* pl) {
     }
     cudaFree(pl->d_fin);
     cudaFree(pl->d_gfin);
-    cudaFree(pl->d_gest);
     cudaFree(pl->d_stage);
     cudaFree(pl->d_out_idx);
     cudaFree(pl->d_out_val);
@@ -77,7 +76,6 @@ void free_plan(sfft_plan_s* pl) {
     cudaFree(pl->d_bins);
     cudaFree(pl->d_phase);
     cudaFree(pl->d_L);
-    cudaFree(pl->d_nL);
     cudaFree(pl->d_estw);
     cudaFree(pl->d_xperm);
     for (int i = 0; i < sfft_plan_s::kMaxStreams; ++i) {
@@ -191,7 +189,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     const size_t ntaps = pl->taps_host.size();
     std::vector<float> t32(ntaps);
     for (size_t i = 0; i < ntaps; ++i) t32[i] = (float)pl->taps_host[i];
-    size_t part_elems = 0, max_smem = 0, fs_max = 0, ls_max = 0, es_max = 0;
+    size_t part_elems = 0, max_smem = 0, fs_max = 0, ls_max = 0, ss_max = 0;
     uint32_t maxB = 0, max_groups = 0;
     size_t sum_B = 0;  // general: bins over all rounds
     // exact mode: every round's partial folds live at once (the one-launch path gathers all rounds
@@ -236,9 +234,8 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         } else {
             fs_max = r.smem_finish > fs_max ? r.smem_finish : fs_max;
         }
-        if (r.est_global) pl->gest_stride = std::max(pl->gest_stride, (r.smem_estimate + 255) & ~size_t(255));
         ls_max = r.smem_locate > ls_max ? r.smem_locate : ls_max;
-        if (!r.est_global) es_max = r.smem_estimate > es_max ? r.smem_estimate : es_max;
+        ss_max = r.smem_select > ss_max ? r.smem_select : ss_max;
     }
     pl->part_stride = part_elems;
     pl->max_B = maxB;
@@ -259,8 +256,8 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     SFFT_ALLOC(pl->d_taps64, ntaps * sizeof(double));
     SFFT_ALLOC(pl->d_wtab, pl->wtab_len * sizeof(double));
     SFFT_ALLOC(pl->d_part, pl->part_bytes);
-    // arrival counters: per (round, request) twice in exact mode, per request in general mode
-    const size_t ncounters = (size_t)max_batch * (general ? 1 : 2 * pl->rounds.size());
+    // exact mode's arrival counters: per (round, request), twice
+    const size_t ncounters = general ? 1 : (size_t)max_batch * 2 * pl->rounds.size();
     SFFT_ALLOC(pl->d_counter, ncounters * sizeof(uint32_t));
 
     SFFT_ALLOC(pl->d_zidx, (size_t)max_batch * p->z_cap * sizeof(uint32_t));
@@ -284,14 +281,12 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     // after another (round t + 1's waits for round t's arrival on the request's second counter)
     if (pl->fin_stride) SFFT_ALLOC(pl->d_fin, pl->fin_stride * max_batch);
     if (pl->gfin_stride) SFFT_ALLOC(pl->d_gfin, pl->gfin_stride * pl->gfin_groups * max_batch);
-    if (pl->gest_stride) SFFT_ALLOC(pl->d_gest, pl->gest_stride * max_batch);
     if (general) {
         SFFT_ALLOC(pl->d_bins, pl->bins_stride * max_batch * sizeof(double2));
-        SFFT_ALLOC(pl->d_phase, pl->phase_stride * max_batch * sizeof(double));
+        SFFT_ALLOC(pl->d_phase, pl->phase_stride * max_batch * sizeof(uint32_t));
         SFFT_ALLOC(pl->d_L, sum_B * max_batch * sizeof(uint32_t));
         pl->tw_shift = (ilog2_host(p->n) + 1) / 2;
         SFFT_ALLOC(pl->d_tw, ((size_t(1) << pl->tw_shift) + (p->n >> pl->tw_shift)) * sizeof(double2));
-        SFFT_ALLOC(pl->d_nL, (size_t)max_batch * sizeof(uint32_t));
         SFFT_ALLOC(pl->d_estw, (size_t)max_batch * sum_B * (sizeof(double2) + sizeof(double)));
         bool perm = false;
         for (const GeneralRound& r : pl->grounds) perm = perm || r.perm;
@@ -345,7 +340,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
             return fail(e, "create event");
     }
     if (!general && (e = set_exact_smem_limit(max_smem, fp64)) != cudaSuccess) return fail(e, "shared memory limit");
-    if (general && (e = general_set_smem(fs_max, ls_max, es_max)) != cudaSuccess)
+    if (general && (e = general_set_smem(fs_max, ls_max, ss_max, 0)) != cudaSuccess)
         return fail(e, "shared memory limit");
     // The gather reads one 8- or 16-byte sample per 32-byte sector at random; ask L2 not to widen
     // its DRAM fetches beyond a sector (a per-context performance hint, ignored where unsupported).
@@ -494,21 +489,17 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.tw_shift = plan->tw_shift;
             a.part = reinterpret_cast<float2*>(plan->d_part);
             a.part_stride = plan->part_stride;
-            a.ecount = plan->d_counter;
             a.est_w = plan->d_estw + (size_t)plan->max_batch * boff[r];
             a.est_mag = reinterpret_cast<double*>(plan->d_estw + (size_t)plan->max_batch * boff[R]) +
                         (size_t)plan->max_batch * boff[r];
             a.fin_scratch =
                 gr.fin_global ? plan->d_gfin + (size_t)plan->max_batch * foff[r] * plan->gfin_stride : nullptr;
             a.fin_stride = plan->gfin_stride;
-            a.est_scratch = gr.est_global ? plan->d_gest : nullptr;
-            a.est_stride = plan->gest_stride;
             a.bins = plan->d_bins;
             a.phase = plan->d_phase;
             a.bins_stride = plan->bins_stride;
             a.phase_stride = plan->phase_stride;
             a.L = plan->d_L + (size_t)plan->max_batch * boff[r];
-            a.nL = plan->d_nL;
             a.zidx = plan->d_zidx;
             a.zval = plan->d_zval;
             a.zcount = plan->d_zcount;

@@ -13,9 +13,9 @@
 //                     (step 3), recovered coefficients subtracted in FP64 (step 4), bins stored;
 //                     for a LocateInner pair also c_j = phase(u_j / u'_j);
 //   3. k_gen_locate   every (bin, request), t threads per bin (one per subregion): LocateSignal's
-//                     levels in order, votes, regions, the bin's candidate for the list L;
-//   4. k_gen_estimate every (candidate share, request): EstimateValues' medians; the request's last
-//                     CTA takes the top k' and zhat += w_J.
+//                     levels in order, votes, regions, the bin's candidate for the list L and
+//                     EstimateValues' medians of it;
+//   4. k_gen_select   every request: the distinct candidates' top k', zhat += w_J.
 // Reductions run in a fixed order; results are bit-reproducible.
 #include <cuda_runtime.h>
 
@@ -343,8 +343,13 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
         }
         for (uint32_t hh = 0; hh < h.H; ++hh) bins[(size_t)hash_index(a, g, hh) * B + j] = u[hh];
         // LocateInner's c_j: an FP32 arctangent of the FP64 product (the vote arcs are s pi wide and
-        // the FP32 bins carry ~1e-6 of phase noise; GB300 runs FP64 at 1/64 of the FP32 rate)
-        if (h.H == 2) a.phase[(size_t)s * a.phase_stride + (size_t)g * B + j] = phase01<float>(mul_conj_rn(u[0], u[1]));
+        // the FP32 bins carry ~1e-6 of phase noise; GB300 runs FP64 at 1/64 of the FP32 rate), kept in
+        // units of 2^-32 of a turn
+        if (h.H == 2) {
+            const double2 z = mul_conj_rn(u[0], u[1]);
+            a.phase[(size_t)s * a.phase_stride + (size_t)g * B + j] =
+                (uint32_t)__double2int_rn((double)atan2f((float)z.y, (float)z.x) * (4294967296.0 * 0.15915494309189533576888));
+        }
     }
 }
 
@@ -352,28 +357,19 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
 // 3. LocateSignal: votes over the levels
 // ------------------------------------------------------------------------------------------------
 // One LocateInner vote test (Algorithm 3: |beta theta_{j,q} - c_j| circular < s pi).  f = e / M with
-// e the exact fixed-point value of beta (m + sigma b) mod n and M = n 2^F.  The test is taken on
-// integers except for the (rare) e next to a boundary, where the double expression of the test
-// decides, evaluated exactly as written.
+// e the exact fixed-point value of beta (m + sigma b) mod n and M = n 2^F.  The caller-bins entry takes
+// the test on integers except for the (rare) e next to a boundary, where the double expression of the
+// test decides, evaluated exactly as written.
 struct VoteBounds {
     uint64_t ilo, len;    // e is inside iff (e - ilo) mod M <= len
     uint64_t amb0, amb1;  // integers within 0.25 of a boundary (or ~0 when none)
-    uint64_t g0, g1;      // starts of the guard windows around the two arc ends (glen = 0: none)
-    uint64_t glen;        // e with (e - g0) mod M <= glen or (e - g1) mod M <= glen is in a window
     double c;
 };
 constexpr int kVoteGuard = 16;  // extra fraction bits of the fixed-point boundaries
-// Guard band of an FP32 phase.  The pipeline's c comes from an FP32 arctangent of the FP64
-// product u_j conj(u'_j): rounding the product to float and atan2f's few-ulp error move it by less
-// than 2e-7 of a turn from the FP64 phase.  A vote whose e lies within 2^-20 of a turn (about 1e-6)
-// of an arc end of c is decided by the FP64 test on the FP64 phase instead; every other e is at
-// least 2^-20 - 2e-7 of a turn from the arc ends of either phase, so both give the same vote.
-constexpr int kPhaseGuardLog = 20;
 // Boundaries of the vote arc (c - s/2, c + s/2) in units of 1/M, as 64-bit fixed point with
 // kVoteGuard fraction bits: c M 2^G is one exact scaling of c (truncated to an integer, an error
-// below 2^-G units), so only one double operation is spent per (bin, round).  guard: half width of
-// the guard windows in units of 1/M (0 for an FP64 phase, which needs none).
-__device__ __forceinline__ VoteBounds vote_bounds(double c, int64_t hw_fix, uint32_t logM, uint64_t guard = 0) {
+// below 2^-G units), so only one double operation is spent per (bin, round).
+__device__ __forceinline__ VoteBounds vote_bounds(double c, int64_t hw_fix, uint32_t logM) {
     VoteBounds v;
     const int64_t one = int64_t(1) << kVoteGuard, frac_mask = one - 1;
     const int64_t xfix = (int64_t)(c * ldexp(1.0, (int)logM + kVoteGuard));
@@ -388,18 +384,11 @@ __device__ __forceinline__ VoteBounds vote_bounds(double c, int64_t hw_fix, uint
                           : (fl > 3 * (one / 4) ? ((uint64_t)((blf >> kVoteGuard) + 1) & mask) : ~0ull);
     v.amb1 = fh < one / 4 ? ((uint64_t)(bhf >> kVoteGuard) & mask)
                           : (fh > 3 * (one / 4) ? ((uint64_t)((bhf >> kVoteGuard) + 1) & mask) : ~0ull);
-    v.g0 = (uint64_t)((blf >> kVoteGuard) - (int64_t)guard) & mask;
-    v.g1 = (uint64_t)((bhf >> kVoteGuard) - (int64_t)guard) & mask;
-    v.glen = 2 * guard + 1;
-    if (guard == 0) v.glen = 0;
     v.c = c;
     return v;
 }
-__device__ __forceinline__ bool in_guard(const VoteBounds& v, uint64_t e, uint64_t mask) {
-    return v.glen != 0 && (((e - v.g0) & mask) <= v.glen || ((e - v.g1) & mask) <= v.glen);
-}
 // The vote test on a given phase c, as written in Algorithm 3 (circular distance below s pi), in
-// double precision: the decision of a guarded e.
+// double precision.
 __device__ __forceinline__ bool vote_hit_exact(double c, uint64_t e, uint64_t M, double s) {
     const double f = (double)e / (double)M;
     double dist = fabs(f - c);
@@ -475,206 +464,9 @@ __device__ void locate_bin(uint32_t t, uint32_t nrep, const uint64_t* beta, Phas
         locate_bin_t<32>(nrep, beta, phase, sb_fp, w_fp, logM, s, hw_fix, l_fp, valid, votes_out);
 }
 
-size_t general_locate_smem(uint32_t B) {
-    (void)B;
-    return 0;
-}
-
-// Ascending bitonic sort of the P keys of k[] (P a power of two), one CTA; ends with a barrier.
-__device__ void block_bitonic_sort_u32(uint32_t* k, uint32_t P) {
-    for (uint32_t size = 2; size <= P; size <<= 1) {
-        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-            for (uint32_t i = threadIdx.x; i < P; i += kThreads) {
-                const uint32_t j = i ^ stride;
-                if (j > i) {
-                    const uint32_t x = k[i], y = k[j];
-                    if ((i & size) == 0 ? x > y : x < y) {
-                        k[i] = y;
-                        k[j] = x;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// Sorts the m keys of key[0..m) ascending (key holds P >= m words, P a power of two; keys < 2^32 - 1)
-// and writes the distinct ones to out[0..returned count).  keep holds m words.  Up to kThreads keys
-// are ranked directly (one key per thread, ties by position); more are sorted by a bitonic network
-// over the smallest power of two >= m.
-__device__ uint32_t sort_unique_u32(uint32_t* key, uint32_t m, uint32_t P, uint32_t* out, uint32_t* keep,
-                                    uint32_t* scan) {
-    const uint32_t* sorted = key;
-    if (m <= (uint32_t)kThreads) {
-        if (threadIdx.x < m) {
-            const uint32_t c = threadIdx.x, k = key[c];
-            uint32_t r = 0;
-            for (uint32_t q = 0; q < m; ++q) r += (key[q] < k || (key[q] == k && q < c)) ? 1u : 0u;
-            out[r] = k;
-        }
-        __syncthreads();
-        sorted = out;
-    } else {
-        uint32_t Pm = 1;
-        while (Pm < m && Pm < P) Pm <<= 1;  // key holds P words and m <= P
-        for (uint32_t p = m + threadIdx.x; p < Pm; p += kThreads) key[p] = 0xFFFFFFFFu;  // sort last
-        __syncthreads();
-        block_bitonic_sort_u32(key, Pm);
-    }
-    for (uint32_t p = threadIdx.x; p < m; p += kThreads) keep[p] = (p == 0 || sorted[p - 1] != sorted[p]) ? 1u : 0u;
-    __syncthreads();
-    const uint32_t total = block_exclusive_scan(keep, m, scan);  // keep[p]: output slot of a kept key
-    // compaction: into out from key, or within out (then every kept key is read before any write)
-    if (sorted == out) {
-        uint32_t mine = 0, slot = 0;
-        bool kept = false;
-        if (threadIdx.x < m) {
-            const uint32_t p = threadIdx.x;
-            const uint32_t nxt = p + 1 < m ? keep[p + 1] : total;
-            kept = nxt != keep[p];
-            mine = out[p];
-            slot = keep[p];
-        }
-        __syncthreads();
-        if (kept) out[slot] = mine;
-    } else {
-        for (uint32_t p = threadIdx.x; p < m; p += kThreads) {
-            const uint32_t nxt = p + 1 < m ? keep[p + 1] : total;
-            if (nxt != keep[p]) out[keep[p]] = key[p];
-        }
-    }
-    __syncthreads();
-    return total;
-}
-
-// LocateSignal with t threads per bin, thread q owning subregion q: a CTA holds kThreads / t bins of
-// one request (the bins are independent until L is formed).  Per level, the vote arcs of the R_loc
-// rounds are formed once per bin (by threads q < R_loc, in shared memory), every thread counts the
-// votes of its subregion over the rounds, and the bin's t threads take the level's decision from the
-// t counts with warp shuffles (the decision of locate_bin_t, on the same integers).  The candidate of bin j
-// (pi^{-1} of the integer nearest the centre of its last region, or ~0 for bottom) goes to
-// L[s B + j]; EstimateValues sorts and de-duplicates them.
-constexpr int kLocBins = kThreads / 8;  // bins per CTA at the smallest t
-__global__ void __launch_bounds__(kThreads) k_gen_locate(const GenArgs a) {
-    __shared__ uint64_t s_beta[kMaxRloc];
-    __shared__ VoteBounds s_vb[kLocBins][kMaxRloc];
-    const uint32_t s = a.req_base + blockIdx.y, tid = threadIdx.x;
-    const uint32_t t = a.t;  // 8, 16 or 32 (the schedule checks it)
-    const uint32_t q = tid & (t - 1), lb = tid / t, nb = kThreads / t;
-    const uint32_t B = a.B;
-    const uint32_t j = blockIdx.x * nb + lb;
-    const ReqView rq = gen_req(a, s);
-    uint32_t sigma, b;
-    locate_sigma_b(rq.seed, rq.id, a.round, a.nmask, &sigma, &b);
-    const uint64_t n = a.n, Np = n >> a.logB;
-    const uint32_t logM = (uint32_t)(63 - __clzll((long long)n)) + kFracBits;
-    const uint64_t M = uint64_t(1) << logM, mask = M - 1;
-    const int64_t hw_fix = vote_halfwidth(a.s, logM);
-    const uint64_t guard = M >> kPhaseGuardLog;
-    const uint64_t sb_fp = ((uint64_t)((sigma * b) & a.nmask)) << kFracBits;
-    const double2* rbins = a.bins + (size_t)s * a.bins_stride;
-    // the bin's region (start l_fp, width w_D) and its bottom flag live in registers, the same in every
-    // lane of the bin's group: the t lanes of a bin share a warp (t divides 32), so the level's
-    // decision is taken with warp shuffles and ballots inside the group
-    uint64_t l_fp = ((((uint64_t)j * Np) + n - Np / 2) & (n - 1)) << kFracBits;  // centred on the bin
-    bool valid = j < B;
-    const uint32_t lane = tid & 31u, gbase = lane & ~(t - 1u);
-    const uint32_t gmask = t == 32u ? 0xFFFFFFFFu : ((1u << t) - 1u) << gbase;
-    const double* phase = a.phase + (size_t)s * a.phase_stride;
-    for (uint32_t D = 0; D < a.dmax; ++D) {
-        __syncthreads();  // the previous level's readers of s_beta and s_vb are done
-        if (tid < a.R_loc) {
-            uint32_t aa;
-            uint64_t be;
-            inner_a_beta(rq.seed, rq.id, a.round, D * a.R_loc + tid, a.nmask, a.beta_lo[D], a.beta_hi[D], &aa, &be);
-            s_beta[tid] = be;
-        }
-        const double* ph = phase + (size_t)D * a.R_loc * B;
-        if (valid)
-            for (uint32_t r = q; r < a.R_loc; r += t)
-                s_vb[lb][r] = vote_bounds(ph[(size_t)r * B + j], hw_fix, logM, guard);
-        __syncthreads();
-        const uint64_t w_fp = (Np << kFracBits) >> ((uint64_t)D * a.logtp);
-        const uint64_t half_step = w_fp / (2 * (uint64_t)t), step = w_fp / t;
-        uint32_t v = 0;
-        if (valid) {
-            for (uint32_t r = 0; r < a.R_loc; ++r) {
-                // e_q = beta (m_q + sigma b) mod M, m_q = l + (2q - 1) w / 2t
-                const uint64_t e0 = (s_beta[r] * ((l_fp + half_step + sb_fp) & mask)) & mask;
-                const uint64_t de = (s_beta[r] * step) & mask;
-                const uint64_t e = (e0 + (uint64_t)q * de) & mask;
-                const VoteBounds& vb = s_vb[lb][r];
-                bool hit;
-                if (in_guard(vb, e, mask)) {
-                    // near an arc end of the FP32 phase: the FP64 phase of the pair's stored bins
-                    const double2* pb = rbins + (size_t)2 * (D * a.R_loc + r) * B;
-                    hit = vote_hit_exact(phase01<double>(mul_conj_rn(pb[j], pb[B + j])), e, M, a.s);
-                } else {
-                    hit = vote_hit(vb, e, M, a.s);
-                }
-                if (hit) ++v;
-            }
-        }
-        // the level's decision (every lane of the warp takes part; a group's lanes share `valid`):
-        // Q* nonempty iff some subregion has more than R_loc / 2 votes; then the window of 4
-        // consecutive subregions with the most votes, the first on ties, gives the new region
-        const bool any = (__ballot_sync(0xFFFFFFFFu, 2u * v > a.R_loc) & gmask) != 0u;
-        uint32_t sum = v + __shfl_down_sync(0xFFFFFFFFu, v, 1, (int)t) + __shfl_down_sync(0xFFFFFFFFu, v, 2, (int)t) +
-                       __shfl_down_sync(0xFFFFFFFFu, v, 3, (int)t);
-        uint32_t key = q + 4u <= t ? (sum << 8) | (255u - q) : 0u;  // larger sum, then smaller q
-        for (uint32_t off = t >> 1; off > 0; off >>= 1) key = max(key, __shfl_xor_sync(0xFFFFFFFFu, key, (int)off, (int)t));
-        if (valid) {
-            if (!any)
-                valid = false;
-            else
-                l_fp = (l_fp + (uint64_t)(255u - (key & 255u)) * step) & mask;
-        }
-        if (q == 0 && j < B && a.dbg_lfp) {  // trace: the region and flag after this level
-            a.dbg_lfp[((size_t)s * a.dmax + D) * B + j] = l_fp;
-            a.dbg_valid[((size_t)s * a.dmax + D) * B + j] = (uint8_t)(valid ? 1 : 0);
-        }
-    }
-    if (q != 0 || j >= B) return;
-    uint32_t cand = 0xFFFFFFFFu;
-    if (valid) {
-        const uint64_t wlast = (Np << kFracBits) >> ((uint64_t)a.dmax * a.logtp);
-        const uint32_t tau = (uint32_t)(((l_fp + wlast / 2 + (1ull << (kFracBits - 1))) >> kFracBits) & (n - 1));
-        cand = ((inverse_odd(sigma) & a.nmask) * tau + b) & a.nmask;
-    }
-    a.L[(size_t)s * B + j] = cand;
-}
-
 // ------------------------------------------------------------------------------------------------
-// 4. EstimateValues, top k', zhat += w_J
+// EstimateValues on one candidate
 // ------------------------------------------------------------------------------------------------
-struct EstLayout {
-    size_t w, mag, perm, topi, topv, out_idx, out_val, keep, scan, draws, Lk, Lt, total;
-    uint32_t P;
-};
-__host__ __device__ inline EstLayout est_layout(uint32_t B, uint32_t kprime, uint32_t zcap) {
-    EstLayout L;
-    size_t off = 0;
-    uint32_t P = 1;
-    while (P < B) P <<= 1;
-    L.P = P;
-    L.w = gtake(&off, (size_t)B * 16);
-    L.mag = gtake(&off, (size_t)B * 8);
-    L.perm = gtake(&off, (size_t)P * 4);
-    L.topi = gtake(&off, (size_t)kprime * 4);
-    L.topv = gtake(&off, (size_t)kprime * 16);
-    L.out_idx = gtake(&off, (size_t)(zcap + kprime) * 4);
-    L.out_val = gtake(&off, (size_t)(zcap + kprime) * 16);
-    L.keep = gtake(&off, (size_t)(zcap + kprime > B ? zcap + kprime : B) * 4);
-    L.scan = gtake(&off, (size_t)(kThreads + 8) * 4);
-    L.draws = gtake(&off, (size_t)kMaxRest * 3 * 8);
-    L.Lk = gtake(&off, (size_t)B * 4);
-    L.Lt = gtake(&off, (size_t)B * 4);
-    L.total = off;
-    return L;
-}
-size_t general_estimate_smem(uint32_t B, uint32_t kprime, uint32_t zcap) { return est_layout(B, kprime, zcap).total; }
-
 // w_i = median_q Re e_q + i median_q Im e_q over the hashings q whose window gain at i is >= est_gmin,
 // e_q = u^{(q)}_{h_q(i)} w^{-a_q sigma_q i} / W(-o_q(i)); lower median; 0 when no hashing qualifies.
 // w^e = exp(-2 pi i e / n) for an exact exponent e in [0, n) from two tables of FP64 factors,
@@ -685,24 +477,32 @@ __device__ __forceinline__ double2 root_pow_tab(uint32_t e, const double2* tw, u
     return make_double2(hi.x * lo.x - hi.y * lo.y, hi.x * lo.y + hi.y * lo.x);
 }
 
-template <typename BinFn>
+// e_q of candidate i under one hashing (sigma, b, a) with bins u; false where the window gain is too small
+__device__ __forceinline__ bool estimate_term(uint32_t i, uint32_t sigma, uint32_t b, uint32_t a, const double2* u,
+                                              uint32_t n, uint32_t nmask, uint32_t logNp, const double* wtab, double gmin,
+                                              const double2* tw, uint32_t tw_shift, double2* e) {
+    uint32_t j;
+    const int32_t o = gen_offset((sigma * (i - b)) & nmask, n, nmask, logNp, &j);
+    const double gain = wtab[o < 0 ? -o : o];
+    const double2 w = root_pow_tab((a * sigma * i) & nmask, tw, tw_shift), uj = u[j];
+    if (!(gain >= gmin)) return false;
+    const double2 v = mul_conj_rn(uj, w);
+    *e = make_double2(__ddiv_rn(v.x, gain), __ddiv_rn(v.y, gain));
+    return true;
+}
+
+// w_i of the caller-bins entry: one thread per candidate, u = nrep x B bins
 __device__ double2 estimate_one(uint32_t i, uint32_t nrep, const uint64_t* sig, const uint64_t* bb, const uint64_t* aa,
-                                BinFn bin, uint32_t n, uint32_t nmask, uint32_t logNp, const double* wtab, double gmin,
-                                const double2* tw, uint32_t tw_shift) {
+                                const double2* u, uint32_t B, uint32_t n, uint32_t nmask, uint32_t logNp,
+                                const double* wtab, double gmin, const double2* tw, uint32_t tw_shift) {
     double re[kMaxRest], im[kMaxRest];
     uint32_t m = 0;
     for (uint32_t q = 0; q < nrep; ++q) {
-        const uint32_t sq = (uint32_t)sig[q];
-        const uint32_t p = (sq * (i - (uint32_t)bb[q])) & nmask;
-        uint32_t j;
-        const int32_t o = gen_offset(p, n, nmask, logNp, &j);
-        const double gain = wtab[o < 0 ? -o : o];
-        if (!(gain >= gmin)) continue;
-        const uint32_t e = ((uint32_t)aa[q] * sq * i) & nmask;
-        const double2 w = root_pow_tab(e, tw, tw_shift);
-        const double2 u = bin(q, j);
-        const double2 v = mul_conj_rn(u, w);
-        const double x = __ddiv_rn(v.x, gain), y = __ddiv_rn(v.y, gain);
+        double2 e;
+        if (!estimate_term(i, (uint32_t)sig[q], (uint32_t)bb[q], (uint32_t)aa[q], u + (size_t)q * B, n, nmask, logNp, wtab,
+                           gmin, tw, tw_shift, &e))
+            continue;
+        const double x = e.x, y = e.y;
         // insertion into the sorted prefixes
         uint32_t pr = m, pi = m;
         while (pr > 0 && re[pr - 1] > x) {
@@ -756,142 +556,465 @@ __device__ void sort_by_magnitude(const double* mag, const uint32_t* idx, uint32
     }
 }
 
-// Grid (E, batch): the E CTAs of a request each form L and estimate their share of its candidates;
-// with E > 1 the shares go through est_w / est_mag and the last CTA to arrive takes the top k' and
-// the merge.  E = 1 when the arrays live in est_scratch (one slice per request).
-__global__ void __launch_bounds__(kThreads) k_gen_estimate(const GenArgs a) {
+// ------------------------------------------------------------------------------------------------
+// 3. LocateSignal and EstimateValues per bin
+// ------------------------------------------------------------------------------------------------
+// LocateSignal with t threads per bin (in one warp), thread q owning subregion q: a CTA holds
+// kThreads / t bins of one request (the bins are independent until L is formed).  The phases and betas
+// of every level are brought to shared memory at once, so the levels follow one another without a
+// barrier: a level is R_loc vote tests per thread, one 64-bit product each, and a decision by ballots
+// and shuffles inside the bin's lanes (that of locate_bin_t, on the same integers).  The candidate of
+// bin j (pi^{-1} of the integer nearest the centre of its last region, kNoIndex for bottom) goes to
+// L[s B + j].  EstimateValues' R_est divisions per candidate then spread over the CTA (one
+// (candidate, hashing) per thread: GB300 issues FP64 at 1/64 of the FP32 rate, so the estimates of a
+// request run on as many SMs as its bins do), and two threads per candidate sort the quotients for
+// the medians.  Bound by latency: the level chain, then one chain of FP64 operations.
+//
+// A vote compares the position e / M of beta (m + sigma b) with the arc of half width s / 2 around c_j,
+// both as 32-bit fractions of a turn: with M = n 2^F scaled to 2^64 the product wraps by itself and its
+// upper word is the position.  The pipeline's c_j comes from an FP32 arctangent of the FP64 product
+// u_j conj(u'_j): rounding the product to float and atan2f's few-ulp error move it by less than 2e-7 of
+// a turn, and the 32-bit fractions by less than 1e-9.  A vote within 2^-20 of a turn (about 1e-6) of an
+// arc end is decided by the FP64 test on the FP64 phase of the pair's stored bins; every other one is
+// farther than that error from the arc ends of either phase, so both give the same vote.
+constexpr int kLocBins = kThreads / 8;               // bins per CTA at the smallest t
+constexpr uint32_t kPhaseGuard = (1u << 12) + 8u;    // 2^-20 of a turn, and the fractions' own rounding
+struct LocLayout {
+    size_t beta, vx, vy, c, ok, total;
+};
+__host__ __device__ inline LocLayout loc_layout(uint32_t npairs, uint32_t nb, uint32_t R_est) {
+    LocLayout L;
+    size_t off = 0;
+    L.beta = gtake(&off, (size_t)npairs * 8);
+    L.vx = gtake(&off, (size_t)nb * R_est * 8);
+    L.vy = gtake(&off, (size_t)nb * R_est * 8);
+    L.c = gtake(&off, (size_t)npairs * nb * 4);
+    L.ok = gtake(&off, (size_t)nb * R_est * 4);
+    L.total = off;
+    return L;
+}
+size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est) {
+    return loc_layout(npairs, kThreads / t, R_est).total;
+}
+
+__global__ void __launch_bounds__(kThreads) k_gen_locate(const GenArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t s = a.req_base + blockIdx.y, tid = threadIdx.x, B = a.B, E = gridDim.x;
-    const EstLayout Ly = est_layout(B, a.kprime, a.zcap);
-    // the arrays live in shared memory, or in this request's slice of est_scratch when large
-    unsigned char* eb = a.est_scratch ? a.est_scratch + (size_t)s * a.est_stride : smem;
-    double2* wv = reinterpret_cast<double2*>(eb + Ly.w);
-    double* mag = reinterpret_cast<double*>(eb + Ly.mag);
-    uint32_t* perm = reinterpret_cast<uint32_t*>(eb + Ly.perm);
-    uint32_t* topi = reinterpret_cast<uint32_t*>(eb + Ly.topi);
-    double2* topv = reinterpret_cast<double2*>(eb + Ly.topv);
-    uint32_t* out_idx = reinterpret_cast<uint32_t*>(eb + Ly.out_idx);
-    double2* out_val = reinterpret_cast<double2*>(eb + Ly.out_val);
-    uint32_t* keep = reinterpret_cast<uint32_t*>(eb + Ly.keep);
-    uint32_t* scan = reinterpret_cast<uint32_t*>(eb + Ly.scan);
-    uint64_t* dr = reinterpret_cast<uint64_t*>(eb + Ly.draws);  // sigma, b, a per hashing
+    __shared__ uint32_t s_cand[kLocBins], s_draw[3][kMaxRest];  // candidates; sigma, b, a of the estimation hashings
+    __shared__ double s_med[2][kLocBins];
+    const uint32_t s = a.req_base + blockIdx.y, tid = threadIdx.x;
+    const uint32_t t = a.t;  // 8, 16 or 32 (the schedule checks it)
+    const uint32_t q = tid & (t - 1), lb = tid / t, nb = kThreads / t;
+    const uint32_t B = a.B;
+    const uint32_t j0 = blockIdx.x * nb, j = j0 + lb;
+    const LocLayout Ly = loc_layout(a.npairs, nb, a.R_est);
+    uint64_t* s_beta = reinterpret_cast<uint64_t*>(smem + Ly.beta);
+    uint32_t* s_c = reinterpret_cast<uint32_t*>(smem + Ly.c);  // [npairs][nb]
     const ReqView rq = gen_req(a, s);
-    if (tid < a.R_est) {
-        const Words4 w = draw(rq.seed, rq.id, a.round, tid, kKindEstimate);
-        dr[tid] = (w.w[0] & a.nmask) | 1u;
-        dr[kMaxRest + tid] = w.w[1] & a.nmask;
-        dr[2 * kMaxRest + tid] = w.w[2] & a.nmask;
+    const uint32_t* phase = a.phase + (size_t)s * a.phase_stride;
+    for (uint32_t i = tid; i < a.npairs * nb; i += kThreads) {
+        const uint32_t g = i / nb, bin = j0 + (i & (nb - 1));
+        s_c[i] = bin < B ? phase[(size_t)g * B + bin] : 0u;
     }
-    __syncthreads();
-    // L: the candidates of the bins that LocateSignal did not reject, sorted and de-duplicated
-    uint32_t* Lk = reinterpret_cast<uint32_t*>(eb + Ly.Lk);
-    uint32_t* Lt = reinterpret_cast<uint32_t*>(eb + Ly.Lt);
-    __shared__ uint32_t s_m;
-    if (tid == 0) s_m = 0;
-    __syncthreads();
-    for (uint32_t j = tid; j < B; j += kThreads) {
-        const uint32_t c = a.L[(size_t)s * B + j];
-        if (c != 0xFFFFFFFFu) Lk[atomicAdd(&s_m, 1u)] = c;
+    for (uint32_t g = tid; g < a.npairs; g += kThreads) {
+        const uint32_t D = g / a.R_loc;
+        uint32_t aa;
+        uint64_t be;
+        inner_a_beta(rq.seed, rq.id, a.round, g, a.nmask, a.beta_lo[D], a.beta_hi[D], &aa, &be);
+        s_beta[g] = be;
     }
+    if (tid >= kThreads - 32 && tid - (kThreads - 32) < a.R_est) {
+        const uint32_t e = tid - (kThreads - 32);
+        const Words4 w = draw(rq.seed, rq.id, a.round, e, kKindEstimate);
+        s_draw[0][e] = (w.w[0] & a.nmask) | 1u;
+        s_draw[1][e] = w.w[1] & a.nmask;
+        s_draw[2][e] = w.w[2] & a.nmask;
+    }
+    uint32_t sigma, b;
+    locate_sigma_b(rq.seed, rq.id, a.round, a.nmask, &sigma, &b);
+    const uint64_t n = a.n, Np = n >> a.logB;
+    const uint32_t logM = (uint32_t)(63 - __clzll((long long)n)) + kFracBits;
+    const uint64_t M = uint64_t(1) << logM, mask = M - 1;
+    const uint32_t sh = 64u - logM;
+    const uint64_t sb_fp = ((uint64_t)((sigma * b) & a.nmask)) << kFracBits;
+    // half width of the vote arc, s / 2 of a turn (an arc of a whole turn or more takes every vote)
+    const uint32_t hw = a.s >= 1.0 ? 0xFFFFFFFFu - kPhaseGuard : (uint32_t)__double2uint_rn(a.s * 2147483648.0);
+    const double2* rbins = a.bins + (size_t)s * a.bins_stride;
+    // the bin's region (start l_fp, width w_D) and its bottom flag live in registers, the same in every
+    // lane of the bin's group (t divides 32)
+    uint64_t l_fp = ((((uint64_t)j * Np) + n - Np / 2) & (n - 1)) << kFracBits;  // centred on the bin
+    bool valid = j < B;
+    const uint32_t lane = tid & 31u, gbase = lane & ~(t - 1u);
+    const uint32_t gmask = t == 32u ? 0xFFFFFFFFu : ((1u << t) - 1u) << gbase;
     __syncthreads();
-    const uint32_t nL = sort_unique_u32(Lk, s_m, Ly.P, Lt, keep, scan);
-    const uint32_t* L = Lt;
-    if (tid == 0 && blockIdx.x == 0) a.nL[s] = nL;
-    const double2* bins = a.bins + (size_t)s * a.bins_stride + (size_t)2 * a.npairs * B;
-    const uint32_t logNp = (uint32_t)(63 - __clzll((long long)a.n)) - a.logB;
-    double2* gw = a.est_w + (size_t)s * B;
-    double* gmag = a.est_mag + (size_t)s * B;
-    for (uint32_t c = blockIdx.x * kThreads + tid; c < nL; c += E * kThreads) {
-        const double2 w = estimate_one(L[c], a.R_est, dr, dr + kMaxRest, dr + 2 * kMaxRest,
-                                       [&](uint32_t q, uint32_t j) { return bins[(size_t)q * B + j]; }, (uint32_t)a.n,
-                                       a.nmask, logNp, a.wtab, a.est_gmin, a.tw, a.tw_shift);
-        const double m2 = __dadd_rn(__dmul_rn(w.x, w.x), __dmul_rn(w.y, w.y));
-        if (E == 1) {
-            wv[c] = w;
-            mag[c] = m2;
-        } else {
-            gw[c] = w;
-            gmag[c] = m2;
+    for (uint32_t D = 0; D < a.dmax; ++D) {
+        const uint64_t w_fp = (Np << kFracBits) >> ((uint64_t)D * a.logtp);
+        const uint64_t half_step = w_fp / (2 * (uint64_t)t), step = w_fp / t;
+        uint32_t v = 0;
+        if (valid) {
+            // m_q = l + (2q - 1) w / 2t (q from 1): this thread's subregion centre, and sigma b
+            const uint64_t pos = (l_fp + half_step + sb_fp + (uint64_t)q * step) << sh;
+            const uint32_t* cl = s_c + D * a.R_loc * nb + lb;
+            const uint64_t* bl = s_beta + D * a.R_loc;
+            for (uint32_t r = 0; r < a.R_loc; ++r) {
+                const uint64_t e = bl[r] * pos;  // the position times 2^64 / M, mod 2^64
+                const int32_t d = (int32_t)((uint32_t)(e >> 32) - cl[r * nb]);
+                const uint32_t ad = (uint32_t)(d < 0 ? -(int64_t)d : (int64_t)d);
+                bool hit = ad < hw;
+                if (ad + kPhaseGuard - hw <= 2u * kPhaseGuard) {
+                    const double2* pb = rbins + (size_t)2 * (D * a.R_loc + r) * B;
+                    hit = vote_hit_exact(phase01<double>(mul_conj_rn(pb[j], pb[B + j])), e >> sh, M, a.s);
+                }
+                v += hit ? 1u : 0u;
+            }
+        }
+        // the level's decision (every lane of the warp takes part; a group's lanes share `valid`):
+        // Q* nonempty iff some subregion has more than R_loc / 2 votes; then the window of 4
+        // consecutive subregions with the most votes, the first on ties, gives the new region
+        const bool any = (__ballot_sync(0xFFFFFFFFu, 2u * v > a.R_loc) & gmask) != 0u;
+        uint32_t sum = v + __shfl_down_sync(0xFFFFFFFFu, v, 1, (int)t) + __shfl_down_sync(0xFFFFFFFFu, v, 2, (int)t) +
+                       __shfl_down_sync(0xFFFFFFFFu, v, 3, (int)t);
+        uint32_t key = q + 4u <= t ? (sum << 8) | (255u - q) : 0u;  // larger sum, then smaller q
+        for (uint32_t off = t >> 1; off > 0; off >>= 1) key = max(key, __shfl_xor_sync(0xFFFFFFFFu, key, (int)off, (int)t));
+        if (valid) {
+            if (!any)
+                valid = false;
+            else
+                l_fp = (l_fp + (uint64_t)(255u - (key & 255u)) * step) & mask;
+        }
+        if (q == 0 && j < B && a.dbg_lfp) {  // trace: the region and flag after this level
+            a.dbg_lfp[((size_t)s * a.dmax + D) * B + j] = l_fp;
+            a.dbg_valid[((size_t)s * a.dmax + D) * B + j] = (uint8_t)(valid ? 1 : 0);
         }
     }
-    if (E > 1) {
-        if (arrive(a.ecount + s, E) == 0) return;
-        for (uint32_t c = tid; c < nL; c += kThreads) {
-            wv[c] = __ldcg(gw + c);
-            mag[c] = __ldcg(gmag + c);
+    if (q == 0) {
+        uint32_t cand = kNoIndex;
+        if (valid) {
+            const uint64_t wlast = (Np << kFracBits) >> ((uint64_t)a.dmax * a.logtp);
+            const uint32_t tau = (uint32_t)(((l_fp + wlast / 2 + (1ull << (kFracBits - 1))) >> kFracBits) & (n - 1));
+            cand = ((inverse_odd(sigma) & a.nmask) * tau + b) & a.nmask;
         }
-        if (tid == 0) a.ecount[s] = 0;  // every CTA of the request has arrived
+        s_cand[lb] = cand;
+        if (j < B) a.L[(size_t)s * B + j] = cand;
     }
     __syncthreads();
-    sort_by_magnitude(mag, L, nL, Ly.P, perm);
-    const uint32_t nJ = nL < a.kprime ? nL : a.kprime;
-    // J sorted by index: the kept candidates are a subset of the ascending L, so keep L's order
-    for (uint32_t c = tid; c < nL; c += kThreads) keep[c] = 0;
-    __syncthreads();
-    for (uint32_t r = tid; r < nJ; r += kThreads) keep[perm[r]] = 1;
-    __syncthreads();
-    const uint32_t total = block_exclusive_scan(keep, nL, scan);
-    for (uint32_t c = tid; c < nL; c += kThreads) {
-        const uint32_t nxt = c + 1 < nL ? keep[c + 1] : total;
-        if (nxt != keep[c]) {
-            topi[keep[c]] = L[c];
-            topv[keep[c]] = wv[c];
-        }
+    // EstimateValues: e_q of every (candidate, hashing)
+    double* vx = reinterpret_cast<double*>(smem + Ly.vx);
+    double* vy = reinterpret_cast<double*>(smem + Ly.vy);
+    uint32_t* ok = reinterpret_cast<uint32_t*>(smem + Ly.ok);
+    const double2* ebins = rbins + (size_t)2 * a.npairs * B;
+    const uint32_t logNp = logM - kFracBits - a.logB;
+    for (uint32_t i = tid; i < nb * a.R_est; i += kThreads) {
+        const uint32_t bin = i & (nb - 1), h = i / nb, c = s_cand[bin];
+        double2 e = make_double2(0.0, 0.0);
+        bool good = false;
+        if (c != kNoIndex)
+            good = estimate_term(c, s_draw[0][h], s_draw[1][h], s_draw[2][h], ebins + (size_t)h * B, (uint32_t)n, a.nmask,
+                                 logNp, a.wtab, a.est_gmin, a.tw, a.tw_shift, &e);
+        vx[i] = e.x;
+        vy[i] = e.y;
+        ok[i] = good ? 1u : 0u;
     }
     __syncthreads();
-    // zhat <- zhat + w_J (zhat first on equal indices); nothing is dropped in the general case
-    const uint32_t nz = min(a.zcount[s], a.zcap);
+    // medians: thread (bin, component) sorts its quotients in place, in hashing order
+    if (tid < 2 * nb) {
+        const uint32_t bin = tid & (nb - 1);
+        double* v = tid < nb ? vx : vy;
+        uint32_t m = 0;
+        for (uint32_t h = 0; h < a.R_est; ++h) {
+            if (!ok[h * nb + bin]) continue;
+            const double x = v[h * nb + bin];
+            uint32_t p = m;
+            while (p > 0 && v[(p - 1) * nb + bin] > x) {
+                v[p * nb + bin] = v[(p - 1) * nb + bin];
+                --p;
+            }
+            v[p * nb + bin] = x;
+            ++m;
+        }
+        s_med[tid < nb ? 0 : 1][bin] = m == 0 ? 0.0 : v[((m - 1) / 2) * nb + bin];
+    }
+    __syncthreads();
+    if (tid < nb && j0 + tid < B && s_cand[tid] != kNoIndex) {
+        const double2 w = make_double2(s_med[0][tid], s_med[1][tid]);
+        a.est_w[(size_t)s * B + j0 + tid] = w;
+        a.est_mag[(size_t)s * B + j0 + tid] = __dadd_rn(__dmul_rn(w.x, w.x), __dmul_rn(w.y, w.y));
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// 4. top k' of the distinct candidates, zhat += w_J
+// ------------------------------------------------------------------------------------------------
+// One CTA per request.  Bins that decoded the same frequency are reduced to one (a hash table in shared
+// memory: copies carry the same estimate, so which one stays does not matter), the k' first in the
+// order (magnitude descending, index ascending) are found by a radix selection on the bits of
+// (mag2, ~index) -- mag2 >= 0, so its IEEE pattern orders like its value, on the integer units -- and
+// only those are sorted by index, for the merge with zhat.  Bound by latency: about 30 barriers.
+constexpr uint32_t kSelThreads = 1024;
+constexpr uint32_t kSelDigits = 1024;  // one digit value per thread
+struct SelLayout {
+    size_t table, js, zi, dup, total;
+    uint32_t H, P;
+};
+__host__ __device__ inline SelLayout sel_layout(uint32_t B, uint32_t kprime, uint32_t zcap) {
+    SelLayout L;
+    size_t off = 0;
+    L.H = 2;
+    while (L.H < 2 * B) L.H <<= 1;
+    const uint32_t nJ = kprime < B ? kprime : B;
+    L.P = 2;
+    while (L.P < nJ) L.P <<= 1;
+    L.table = gtake(&off, (size_t)L.H * 4);
+    L.js = gtake(&off, (size_t)L.P * 8);
+    L.zi = gtake(&off, (size_t)zcap * 4);
+    L.dup = gtake(&off, (size_t)L.P * 4);
+    L.total = off;
+    return L;
+}
+size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap) { return sel_layout(B, kprime, zcap).total; }
+
+// exclusive prefix sum over the CTA of one value per thread; tmp holds 33 words.  Starts and ends with
+// every thread done with tmp.
+__device__ __forceinline__ uint32_t sel_scan(uint32_t v, uint32_t* tmp, uint32_t* total) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (uint32_t off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    if (lane == 31) tmp[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t w = tmp[lane];
+        uint32_t wi = w;
+#pragma unroll
+        for (uint32_t off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, off);
+            if (lane >= off) wi += y;
+        }
+        tmp[lane] = wi - w;
+        if (lane == 31) tmp[32] = wi;
+    }
+    __syncthreads();
+    const uint32_t r = tmp[warp] + incl - v;
+    *total = tmp[32];
+    __syncthreads();
+    return r;
+}
+
+// Ascending sort of the nJ distinct keys js[0..nJ) (js holds P >= nJ words, P a power of two).
+__device__ __forceinline__ void sel_sort(unsigned long long* js, uint32_t nJ) {
+    const uint32_t tid = threadIdx.x;
+    uint32_t P = 2;
+    while (P < nJ) P <<= 1;
+    if (P <= kSelThreads) {  // one key per thread; partners less than 32 apart are exchanged by shuffles
+        unsigned long long k = tid < nJ ? js[tid] : ~0ull;
+        for (uint32_t size = 2; size <= P; size <<= 1) {
+            for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+                unsigned long long o;
+                if (stride < 32) {
+                    o = __shfl_xor_sync(0xffffffffu, k, (int)stride);
+                } else {
+                    __syncthreads();
+                    if (tid < P) js[tid] = k;
+                    __syncthreads();
+                    o = tid < P ? js[tid ^ stride] : k;
+                }
+                const bool up = (tid & size) == 0, lower = (tid & stride) == 0;
+                if ((lower == up) == (o < k)) k = o;
+            }
+        }
+        __syncthreads();
+        if (tid < nJ) js[tid] = k;
+        __syncthreads();
+        return;
+    }
+    for (uint32_t p = nJ + tid; p < P; p += kSelThreads) js[p] = ~0ull;
+    __syncthreads();
+    for (uint32_t size = 2; size <= P; size <<= 1)
+        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+            for (uint32_t i = tid; i < P; i += kSelThreads) {
+                const uint32_t o = i ^ stride;
+                if (o > i) {
+                    const unsigned long long x = js[i], y = js[o];
+                    if ((i & size) == 0 ? x > y : x < y) {
+                        js[i] = y;
+                        js[o] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+}
+
+// PER: bins per thread (B <= PER kSelThreads)
+template <int PER>
+__global__ void __launch_bounds__(kSelThreads) k_gen_select(const GenArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t hist[kSelDigits], tmp[33], s_digit, s_above, s_in;
+    const uint32_t s = a.req_base + blockIdx.x, tid = threadIdx.x, B = a.B, lane = tid & 31u;
+    const SelLayout Ly = sel_layout(B, a.kprime, a.zcap);
+    uint32_t* table = reinterpret_cast<uint32_t*>(smem + Ly.table);
+    unsigned long long* js = reinterpret_cast<unsigned long long*>(smem + Ly.js);  // (index, bin) of J
+    uint32_t* zs = reinterpret_cast<uint32_t*>(smem + Ly.zi);
+    uint32_t* dup = reinterpret_cast<uint32_t*>(smem + Ly.dup);
     uint32_t* zi = a.zidx + (size_t)s * a.zcap;
     double2* zv = a.zval + (size_t)s * a.zcap;
-    for (uint32_t e = tid; e < nz; e += kThreads) {
-        const uint32_t key = zi[e];
-        const uint32_t pos = e + lower_bound_u32(topi, nJ, key);
-        out_idx[pos] = key;
-        out_val[pos] = zv[e];
+    const double2* ew = a.est_w + (size_t)s * B;
+    // the candidates, and zhat's indices for the merge
+    uint32_t cand[PER];
+    unsigned long long mag[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const uint32_t j = tid + (uint32_t)i * kSelThreads;
+        cand[i] = j < B ? a.L[(size_t)s * B + j] : kNoIndex;
+        mag[i] = j < B ? reinterpret_cast<const unsigned long long*>(a.est_mag)[(size_t)s * B + j] : 0ull;
     }
-    for (uint32_t c = tid; c < nJ; c += kThreads) {
-        const uint32_t pos = c + upper_bound_u32(zi, nz, topi[c]);
-        out_idx[pos] = topi[c];
-        out_val[pos] = topv[c];
-    }
+    const uint32_t nz = min(a.zcount[s], a.zcap);
+    for (uint32_t e = tid; e < nz; e += kSelThreads) zs[e] = zi[e];
+    for (uint32_t h = tid; h < Ly.H; h += kSelThreads) table[h] = kNoIndex;
+    hist[tid] = 0;
     __syncthreads();
-    const uint32_t tot = nz + nJ;
-    for (uint32_t p = tid; p < tot; p += kThreads) {
-        const uint32_t idx = out_idx[p];
-        uint32_t kp = 0;
-        if (p == 0 || out_idx[p - 1] != idx) {
-            if (p + 1 < tot && out_idx[p + 1] == idx) {
-                out_val[p] = make_double2(out_val[p].x + out_val[p + 1].x, out_val[p].y + out_val[p + 1].y);
+    // L without repetitions: the first to claim an index keeps it (at most B of H >= 2 B places taken)
+    uint32_t state = 0, kept = 0;  // bit i: candidate i still undecided; in J
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        if (cand[i] == kNoIndex) continue;
+        uint32_t h = (cand[i] * 2654435769u) >> (__clz((int)Ly.H) + 1);  // the product's top log2 H bits
+        for (;;) {
+            const uint32_t old = atomicCAS(&table[h], kNoIndex, cand[i]);
+            if (old == kNoIndex) {
+                state |= 1u << i;
+                break;
             }
-            kp = 1;
+            if (old == cand[i]) break;
+            h = (h + 1) & (Ly.H - 1);
         }
-        keep[p] = kp;
+    }
+    uint32_t nL;
+    sel_scan((uint32_t)__popc((int)state), tmp, &nL);
+    // J: the k' first by (mag2 descending, index ascending).  Digits of 10 bits from the top of the key
+    // (mag2, ~index); a digit's histogram over the undecided candidates tells which value holds the
+    // k'-th, those above it are in J, those below are not
+    if (nL <= a.kprime) {
+        kept = state;
+    } else {
+        uint32_t need = a.kprime;
+        for (uint32_t pass = 0;; ++pass) {
+            uint32_t dg[PER];
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                // 64 bits of mag2 as 6 x 10 + 4, then 32 of ~index as 3 x 10 + 2
+                if (pass < 7)
+                    dg[i] = pass < 6 ? (uint32_t)(mag[i] >> (54 - 10 * pass)) & 1023u : (uint32_t)mag[i] & 15u;
+                else
+                    dg[i] = pass < 10 ? (~cand[i] >> (22 - 10 * (pass - 7))) & 1023u : ~cand[i] & 3u;
+                const bool in = (state >> i) & 1u;
+                const unsigned act = __ballot_sync(0xffffffffu, in);
+                if (in) {  // one shared-memory atomic per digit value and warp
+                    const unsigned same = __match_any_sync(act, dg[i]);
+                    if (lane == (uint32_t)__ffs((int)same) - 1u) atomicAdd(&hist[dg[i]], (uint32_t)__popc((int)same));
+                }
+            }
+            __syncthreads();
+            const uint32_t d = kSelDigits - 1 - tid, c = hist[d];
+            uint32_t tot;
+            const uint32_t above = sel_scan(c, tmp, &tot);
+            hist[d] = 0;  // for the next pass
+            if (above < need && need <= above + c) {
+                s_digit = d;
+                s_above = above;
+                s_in = c;
+            }
+            __syncthreads();
+            const uint32_t digit = s_digit;
+            const bool all = s_in == need - s_above;  // the whole digit value belongs to J
+            need -= s_above;
+#pragma unroll
+            for (int i = 0; i < PER; ++i)
+                if ((state >> i) & 1u) {
+                    if (dg[i] > digit || (all && dg[i] == digit)) kept |= 1u << i;
+                    if (dg[i] != digit || all) state &= ~(1u << i);
+                }
+            if (all) break;  // the keys are distinct, so the last digit at the latest ends it
+            __syncthreads();  // s_digit, s_above, s_in are rewritten by the next pass
+        }
+    }
+    uint32_t nJ;
+    uint32_t at = sel_scan((uint32_t)__popc((int)kept), tmp, &nJ);
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if ((kept >> i) & 1u) js[at++] = ((unsigned long long)cand[i] << 32) | (tid + (uint32_t)i * kSelThreads);
+    __syncthreads();
+    sel_sort(js, nJ);
+    // zhat <- zhat + w_J; nothing is dropped in the general case.  An entry of J already in zhat is added
+    // to it (zhat first); the others go to c - (repeated ones before c) + (zhat entries below)
+    auto jidx = [&](uint32_t c) { return (uint32_t)(js[c] >> 32); };
+    uint32_t ndup = 0;  // J's repeated entries, counted before each
+    for (uint32_t c0 = 0; c0 < nJ; c0 += kSelThreads) {
+        const uint32_t c = c0 + tid;
+        uint32_t rep = 0;
+        if (c < nJ) {
+            const uint32_t key = jidx(c), ub = upper_bound_u32(zs, nz, key);
+            rep = ub > 0 && zs[ub - 1] == key ? 1u : 0u;
+        }
+        uint32_t tot;
+        const uint32_t before = sel_scan(rep, tmp, &tot);
+        if (c < nJ) dup[c] = (ndup + before) | (rep << 31);
+        ndup += tot;
     }
     __syncthreads();
-    const uint32_t newcount = block_exclusive_scan(keep, tot, scan);
     const bool last = a.last_round != 0;
-    for (uint32_t p = tid; p < tot; p += kThreads) {
-        const uint32_t pos = keep[p];
-        const uint32_t nxt = p + 1 < tot ? keep[p + 1] : newcount;
-        if (nxt == pos) continue;
+    const uint32_t newcount = nz + nJ - ndup;
+    auto put = [&](uint32_t pos, uint32_t key, double2 v) {
         if (pos < a.zcap) {
-            zi[pos] = out_idx[p];
-            zv[pos] = out_val[p];
+            zi[pos] = key;
+            zv[pos] = v;
         }
         if (last && pos < a.out_cap) {
-            a.out_idx[(size_t)s * a.out_cap + pos] = out_idx[p];
-            a.out_val[(size_t)s * a.out_cap + pos] = out_val[p];
+            a.out_idx[(size_t)s * a.out_cap + pos] = key;
+            a.out_val[(size_t)s * a.out_cap + pos] = v;
         }
+    };
+    // zhat moves up in place: each pass of kSelThreads entries from the top is read before it is
+    // written, and writes only at or above the places it read
+    for (uint32_t done = 0; done < nz; done += kSelThreads) {
+        const uint32_t e = nz - 1 - done - tid;
+        const bool mine = done + tid < nz;
+        uint32_t key = 0, pos = 0;
+        double2 v = make_double2(0.0, 0.0);
+        if (mine) {
+            key = zs[e];
+            v = zv[e];
+            uint32_t lo = 0, hi = nJ;  // entries of J below key
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (jidx(mid) < key) lo = mid + 1; else hi = mid;
+            }
+            const uint32_t d = lo < nJ ? dup[lo] : ndup;
+            pos = e + lo - (d & 0x7FFFFFFFu);
+            if (lo < nJ && jidx(lo) == key) {
+                const double2 w = ew[(uint32_t)js[lo]];
+                v = make_double2(v.x + w.x, v.y + w.y);
+            }
+        }
+        __syncthreads();
+        if (mine) put(pos, key, v);
     }
-    __syncthreads();
+    for (uint32_t c = tid; c < nJ; c += kSelThreads) {
+        const uint32_t d = dup[c];
+        if (d >> 31) continue;
+        const uint32_t key = jidx(c);
+        put(c - d + upper_bound_u32(zs, nz, key), key, ew[(uint32_t)js[c]]);
+    }
     if (tid == 0) {
         const bool overflow = newcount > a.zcap;
         if (overflow) a.zflag[s] = 1;
         a.zcount[s] = overflow ? a.zcap : newcount;
         if (last) {
-            const uint32_t kept = overflow ? a.zcap : newcount;
-            a.out_count[s] = kept < a.out_cap ? kept : a.out_cap;
-            a.out_flag[s] = (a.zflag[s] || kept > a.out_cap) ? SFFT_ERR_CAPACITY : SFFT_OK;
+            const uint32_t count = overflow ? a.zcap : newcount;
+            a.out_count[s] = count < a.out_cap ? count : a.out_cap;
+            a.out_flag[s] = (a.zflag[s] || count > a.out_cap) ? SFFT_ERR_CAPACITY : SFFT_OK;
         }
     }
 }
@@ -918,10 +1041,29 @@ __global__ void __launch_bounds__(kThreads) k_locate_votes(const VoteArgs a) {
     }
 }
 
+struct EstLayout {
+    size_t w, mag, perm, keep, scan, total;
+    uint32_t P;
+};
+__host__ __device__ inline EstLayout est_layout(uint32_t m) {
+    EstLayout L;
+    size_t off = 0;
+    uint32_t P = 1;
+    while (P < m) P <<= 1;
+    L.P = P;
+    L.w = gtake(&off, (size_t)m * 16);
+    L.mag = gtake(&off, (size_t)m * 8);
+    L.perm = gtake(&off, (size_t)P * 4);
+    L.keep = gtake(&off, (size_t)m * 4);
+    L.scan = gtake(&off, (size_t)(kThreads + 8) * 4);
+    L.total = off;
+    return L;
+}
+
 __global__ void __launch_bounds__(kThreads) k_estimate_from_bins(const EstArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t tid = threadIdx.x;
-    const EstLayout Ly = est_layout(a.nL > 0 ? a.nL : 1, a.kprime > 0 ? a.kprime : 1, 1);
+    const EstLayout Ly = est_layout(a.nL > 0 ? a.nL : 1);
     double2* wv = reinterpret_cast<double2*>(smem + Ly.w);
     double* mag = reinterpret_cast<double*>(smem + Ly.mag);
     uint32_t* perm = reinterpret_cast<uint32_t*>(smem + Ly.perm);
@@ -929,9 +1071,8 @@ __global__ void __launch_bounds__(kThreads) k_estimate_from_bins(const EstArgs a
     uint32_t* scan = reinterpret_cast<uint32_t*>(smem + Ly.scan);
     const uint32_t logNp = (uint32_t)(63 - __clzll((long long)a.n)) - a.logB;
     for (uint32_t c = tid; c < a.nL; c += kThreads) {
-        const double2 w = estimate_one(a.L[c], a.nrep, a.sig, a.bb, a.aa,
-                                       [&](uint32_t q, uint32_t j) { return a.u[(size_t)q * a.B + j]; }, (uint32_t)a.n,
-                                       a.nmask, logNp, a.wtab, a.est_gmin, a.tw, a.tw_shift);
+        const double2 w = estimate_one(a.L[c], a.nrep, a.sig, a.bb, a.aa, a.u, a.B, (uint32_t)a.n, a.nmask, logNp, a.wtab,
+                                       a.est_gmin, a.tw, a.tw_shift);
         wv[c] = w;
         mag[c] = __dadd_rn(__dmul_rn(w.x, w.x), __dmul_rn(w.y, w.y));
     }
@@ -956,25 +1097,22 @@ __global__ void __launch_bounds__(kThreads) k_estimate_from_bins(const EstArgs a
 // ------------------------------------------------------------------------------------------------
 // launchers
 // ------------------------------------------------------------------------------------------------
-cudaError_t general_set_smem(size_t finish, size_t locate, size_t estimate) {
+static cudaError_t raise_smem(const void* kernel, size_t bytes, size_t* lim) {
+    if (bytes <= *lim) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) *lim = bytes;
+    return e;
+}
+cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate) {
     static std::mutex mu;  // plans may be created from several threads
     std::lock_guard<std::mutex> lk(mu);
-    static size_t lim[4] = {0, 0, 0, 0};
-    cudaError_t e = cudaSuccess;
-    if (finish > lim[1] && (e = cudaFuncSetAttribute(k_gen_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)finish)) == cudaSuccess)
-        lim[1] = finish;
-    if (e != cudaSuccess) return e;
-    if (locate > lim[2] && (e = cudaFuncSetAttribute(k_gen_locate, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)locate)) == cudaSuccess)
-        lim[2] = locate;
-    if (e != cudaSuccess) return e;
-    if (estimate > lim[3]) {
-        e = cudaFuncSetAttribute(k_gen_estimate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)estimate);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_estimate_from_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)estimate);
-        if (e == cudaSuccess) lim[3] = estimate;
-    }
+    static size_t lim[6] = {0, 0, 0, 0, 0, 0};
+    cudaError_t e = raise_smem((const void*)k_gen_finish, finish, &lim[0]);
+    if (e == cudaSuccess) e = raise_smem((const void*)k_gen_locate, locate, &lim[1]);
+    if (e == cudaSuccess) e = raise_smem((const void*)k_gen_select<1>, select, &lim[2]);
+    if (e == cudaSuccess) e = raise_smem((const void*)k_gen_select<2>, select, &lim[3]);
+    if (e == cudaSuccess) e = raise_smem((const void*)k_gen_select<4>, select, &lim[4]);
+    if (e == cudaSuccess) e = raise_smem((const void*)k_estimate_from_bins, estimate, &lim[5]);
     return e;
 }
 
@@ -1001,10 +1139,15 @@ cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const General
     if (e != cudaSuccess) return e;
     k_gen_finish<<<dim3(r.ngroups, batch), kThreads, r.fin_global ? 0 : r.smem_finish, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_gen_locate<<<dim3((r.B * r.t + kThreads - 1) / kThreads, batch), kThreads, 0, st>>>(a);
+    const uint32_t nb = kThreads / r.t;  // bins per CTA
+    k_gen_locate<<<dim3((r.B + nb - 1) / nb, batch), kThreads, r.smem_locate, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const uint32_t E = r.est_global ? 1u : (r.B + kThreads - 1) / kThreads;
-    k_gen_estimate<<<dim3(E, batch), kThreads, r.est_global ? 0 : r.smem_estimate, st>>>(a);
+    if (r.B <= kSelThreads)
+        k_gen_select<1><<<batch, kSelThreads, r.smem_select, st>>>(a);
+    else if (r.B <= 2 * kSelThreads)
+        k_gen_select<2><<<batch, kSelThreads, r.smem_select, st>>>(a);
+    else
+        k_gen_select<4><<<batch, kSelThreads, r.smem_select, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1014,8 +1157,8 @@ cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st) {
-    const size_t smem = est_layout(a.nL > 0 ? a.nL : 1, a.kprime > 0 ? a.kprime : 1, 1).total;
-    cudaError_t e = general_set_smem(0, 0, smem);
+    const size_t smem = est_layout(a.nL > 0 ? a.nL : 1).total;
+    cudaError_t e = general_set_smem(0, 0, 0, smem);
     if (e != cudaSuccess) return e;
     k_estimate_from_bins<<<1, kThreads, smem, st>>>(a);
     return cudaGetLastError();

@@ -388,13 +388,10 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
         r.taps_off = taps_off;
         r.wtab_off = wtab_off;
         r.smem_finish = general_finish_smem(r.B, p.z_cap);
-        r.smem_locate = general_locate_smem(r.B);
-        r.smem_estimate = general_estimate_smem(r.B, r.kprime, p.z_cap);
-        // arrays beyond kFinSmemMax go to device memory, one slice per CTA: the finish's per (request,
-        // group), the estimate's per request (its launch then gives each request a single CTA)
+        r.smem_locate = general_locate_smem(r.npairs, r.t, p.R_est);
+        r.smem_select = general_select_smem(r.B, r.kprime, p.z_cap);
+        // finish arrays beyond kFinSmemMax go to device memory, one slice per (request, group)
         r.fin_global = r.smem_finish > kFinSmemMax;
-        r.est_global = r.smem_estimate > kFinSmemMax;
-        if (r.smem_locate > 200 * 1024) return SFFT_ERR_K_RANGE;
         const uint64_t Np = p.n / B;
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, p.alpha0, p.delta, r.T, pl->taps_host.data() + taps_off);

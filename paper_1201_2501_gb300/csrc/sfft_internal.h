@@ -211,8 +211,8 @@ struct GeneralRound {
     uint64_t beta_lo[kMaxLevels] = {}, beta_hi[kMaxLevels] = {};
     uint32_t npairs = 0, ngroups = 0, nhash = 0;
     size_t taps_off = 0, wtab_off = 0;
-    size_t smem_finish = 0, smem_locate = 0, smem_estimate = 0;
-    bool fin_global = false, est_global = false;  // arrays too large for shared memory: in d_gfin / d_gest
+    size_t smem_finish = 0, smem_locate = 0, smem_select = 0;
+    bool fin_global = false;       // the finish's arrays are too large for shared memory: in d_gfin
     bool perm = false;             // the pairs read the permuted copy x_{sigma m} (written first)
 };
 
@@ -239,18 +239,14 @@ struct GenArgs {
     uint32_t tw_shift;
     float2* part;          // [batch][ngroups][2][B]: the folds
     size_t part_stride;    // elements per request
-    uint32_t* ecount;      // [batch] arrival counters of the estimate CTAs (zero between launches)
-    double2* est_w;        // [batch][B] candidates' estimates shared by a request's estimate CTAs
+    double2* est_w;        // [batch][B] the bins' candidates' estimates
     double* est_mag;       // [batch][B] their squared magnitudes
     unsigned char* fin_scratch;  // k_gen_finish arrays in device memory: [batch][ngroups][fin_stride], or null
     size_t fin_stride;
-    unsigned char* est_scratch;  // k_gen_estimate arrays in device memory: [batch][est_stride], or null
-    size_t est_stride;
     double2* bins;         // [batch][nhash][B]  (hashing 2g, 2g+1: pair g; 2 npairs + q: estimate q)
-    double* phase;         // [batch][npairs][B] phase(u_a conj(u_{a+beta})) / 2 pi
+    uint32_t* phase;       // [batch][npairs][B] phase(u_a conj(u_{a+beta})) in units of 2^-32 of a turn
     size_t bins_stride, phase_stride;  // elements per request
-    uint32_t* L;           // [batch][B] candidate frequencies
-    uint32_t* nL;          // [batch]
+    uint32_t* L;           // [batch][B] the bins' candidate frequencies (kNoIndex: none)
     uint32_t* zidx;        // [batch][zcap]
     double2* zval;
     uint32_t* zcount;
@@ -309,11 +305,10 @@ struct sfft_plan_s {
     std::vector<sfft::ExactRound> rounds;
     std::vector<sfft::GeneralRound> grounds;  // general mode
     double2* d_bins = nullptr;
-    double* d_phase = nullptr;
+    uint32_t* d_phase = nullptr;
     uint32_t* d_L = nullptr;  // general mode: per round r, [max_batch][B_r] candidates
     double2* d_tw = nullptr;  // general mode: FP64 twiddle factor tables (2^tw_shift + n / 2^tw_shift)
     uint32_t tw_shift = 0;
-    uint32_t* d_nL = nullptr;
     float2* d_xperm = nullptr;  // general mode, rounds with perm: [max_batch][n] permuted signals
     // general mode: per round r, [max_batch][B_r] estimates; then per round [max_batch][B_r] magnitudes
     double2* d_estw = nullptr;
@@ -327,7 +322,7 @@ struct sfft_plan_s {
     void* d_part = nullptr;
     size_t part_bytes = 0;
     size_t part_stride = 0;  // elements of the partial-fold buffer owned by one request
-    // arrival counters, zero between launches: exact [2 R][max_batch]; general [max_batch]
+    // exact mode: arrival counters [2 R][max_batch], zero between launches
     uint32_t* d_counter = nullptr;
     std::vector<sfft::ExactArgs> rdesc;  // [R] round blocks of the one-launch exact path
     std::vector<size_t> chan_off;        // exact FP32: round t's partial folds in a channel slot's area
@@ -352,8 +347,6 @@ struct sfft_plan_s {
     // general mode, per round r with fin_global: [max_batch][ngroups_r][gfin_stride]
     unsigned char* d_gfin = nullptr;
     size_t gfin_stride = 0, gfin_groups = 0;  // gfin_groups: ngroups summed over those rounds
-    unsigned char* d_gest = nullptr;  // general mode: [max_batch][gest_stride]
-    size_t gest_stride = 0;
     size_t dev_bytes = 0;          // device memory allocated at plan creation
     uint64_t samples = 0;          // samples one transform gathers (all rounds, all hashings)
     // internal streams: a batch is split into groups whose rounds run on their own streams
@@ -420,9 +413,9 @@ cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1, ui
 // general mode (sfft_general.cu, sfft_host.cu)
 sfft_status build_general_schedule(sfft_plan_s* pl);
 size_t general_finish_smem(uint32_t B, uint32_t zcap);
-size_t general_locate_smem(uint32_t B);
-size_t general_estimate_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
-cudaError_t general_set_smem(size_t finish, size_t locate, size_t estimate);
+size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est);
+size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
+cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate);
 cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st);
 cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);

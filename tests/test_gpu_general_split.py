@@ -2,7 +2,8 @@
 
 * the gather's residue blocks (B below, at and above 256, up to 4096) and its pairs per CTA (1, 2 or 4
   with the size of the call): bins against the oracle's FP64 HashToBins within 2e-5 of the hashing's
-  largest bin (FP32 folds), and every request bit-identical to the same request run alone.
+  largest bin (FP32 folds), and every request bit-identical to the same request run alone;
+* the per-bin candidates and the selection of the k' largest: replayed by the oracle.
 """
 import numpy as np
 import pytest
@@ -75,4 +76,49 @@ def test_gather_bins_match_oracle_at_every_split(sf, m, k, batch):
         c = int(cnt[s])
         assert int(one[2][0]) == c and int(one[3][0]) == int(flag[s])
         assert torch.equal(one[0][0, :c], idx[s, :c]) and torch.equal(one[1][0, :c], val[s, :c])
+    plan.close()
+
+
+# (log2 n, k, bins per k, batch): one, two and four bins per thread of the selection (B up to 1024, 2048,
+# 4096), k' = 3 k above the sort's one key per thread (k = 512) and above B (every candidate is kept)
+@pytest.mark.parametrize("m,k,bpk,batch", [(12, 100, 8.0, 3), (13, 256, 8.0, 2), (14, 512, 8.0, 2), (12, 64, 2.0, 2),
+                                           (8, 2, 8.0, 1)])
+def test_candidates_and_selection_match_oracle(sf, m, k, bpk, batch):
+    """Rounds 0 and 1 replayed by the oracle on the pipeline's own bins: regions, bottoms and candidates
+    bit for bit, the kept indices bit for bit, values within 1e-12 of the largest."""
+    n, seed = 1 << m, 17
+    f = general_fields(n, k, bins_per_k=bpk, z_cap=min(4096, max(8 * k, 64)))
+    P = oracle_params(f)
+    x = torch.as_tensor(np.stack(_signals(n, k, batch))).cuda()
+    plan = _plan(sf, f, batch)
+    ks, Bs = oracle.general_rounds(P)
+    for r in range(min(2, len(Bs))):
+        _, tr = sf.sfft_execute_trace(plan, x, seed, f["z_cap"], r)
+        torch.cuda.synchronize()
+        tr = {key: v.cpu().numpy() for key, v in tr.items()}
+        B = Bs[r]
+        _, _, dmax = oracle.locate_geometry(P, B)
+        npairs = dmax * P.R_loc
+        for s in range(batch):
+            bins = tr["bins"][s][..., 0] + 1j * tr["bins"][s][..., 1]
+            d = [oracle.locate_draws(P, seed, s, r, B, D, q) for D in range(1, dmax + 1) for q in range(P.R_loc)]
+            olfp, ovalid, ocand = oracle.locate_replay(P, B, d[0]["sigma"], d[0]["b"], [e["beta"] for e in d],
+                                                       bins[0:2 * npairs:2], bins[1:2 * npairs:2])
+            assert np.array_equal(tr["valid"][s], ovalid)
+            assert np.array_equal(tr["regions"][s].view(np.uint64), olfp)
+            want = np.where(ocand == oracle.BOTTOM, np.uint64(0xFFFFFFFF), ocand).astype(np.uint32)
+            assert np.array_equal(tr["cand"][s].view(np.uint32), want)
+            e = [oracle.estimate_draws(P, seed, s, r, q) for q in range(P.R_est)]
+            wi, wv = oracle.estimate_from_bins(P, B, P.alpha0, [q["sigma"] for q in e], [q["b"] for q in e],
+                                               [q["a"] for q in e], bins[2 * npairs:2 * npairs + P.R_est],
+                                               np.unique(ocand[ocand != oracle.BOTTOM]), 3 * ks[r])
+            nb, na = int(tr["zcount_before"][s]), int(tr["zcount_after"][s])
+            zb, za = tr["zval_before"][s], tr["zval_after"][s]
+            merged = dict(zip(tr["zidx_before"][s][:nb].view(np.uint32).tolist(), zb[:nb, 0] + 1j * zb[:nb, 1]))
+            for i, v in zip(wi.astype(np.int64).tolist(), wv):
+                merged[i] = merged[i] + v if i in merged else v
+            keys = sorted(merged)[:f["z_cap"]]
+            assert tr["zidx_after"][s][:na].view(np.uint32).tolist() == keys
+            got, ref = za[:na, 0] + 1j * za[:na, 1], np.array([merged[i] for i in keys])
+            assert np.max(np.abs(got - ref), initial=0.0) <= 1e-12 * max(1.0, float(np.max(np.abs(ref), initial=0.0)))
     plan.close()
