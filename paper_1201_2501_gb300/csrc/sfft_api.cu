@@ -67,7 +67,6 @@ void free_plan(sfft_plan_s* pl) {
         if (pl->ev_reqs[i]) cudaEventDestroy(pl->ev_reqs[i]);
     }
     cudaFree(pl->d_fin);
-    cudaFree(pl->d_gfin);
     cudaFree(pl->d_stage);
     cudaFree(pl->d_out_idx);
     cudaFree(pl->d_out_val);
@@ -228,12 +227,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         if (r.B > maxB) maxB = r.B;
         if (r.ngroups > max_groups) max_groups = r.ngroups;
         sum_B += r.B;
-        if (r.fin_global) {
-            pl->gfin_stride = std::max(pl->gfin_stride, (r.smem_finish + 255) & ~size_t(255));
-            pl->gfin_groups += r.ngroups;  // each such round has its own region
-        } else {
-            fs_max = r.smem_finish > fs_max ? r.smem_finish : fs_max;
-        }
+        fs_max = r.smem_finish > fs_max ? r.smem_finish : fs_max;
         ls_max = r.smem_locate > ls_max ? r.smem_locate : ls_max;
         ss_max = r.smem_select > ss_max ? r.smem_select : ss_max;
     }
@@ -280,7 +274,6 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     // one-launch path forms a round's bins in the CTA's shared memory), and a request's decodes run one
     // after another (round t + 1's waits for round t's arrival on the request's second counter)
     if (pl->fin_stride) SFFT_ALLOC(pl->d_fin, pl->fin_stride * max_batch);
-    if (pl->gfin_stride) SFFT_ALLOC(pl->d_gfin, pl->gfin_stride * pl->gfin_groups * max_batch);
     if (general) {
         SFFT_ALLOC(pl->d_bins, pl->bins_stride * max_batch * sizeof(double2));
         SFFT_ALLOC(pl->d_phase, pl->phase_stride * max_batch * sizeof(uint32_t));
@@ -422,12 +415,10 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
     SFFT_CUDA(cudaMemsetAsync(plan->d_zflag, 0, batch * sizeof(int32_t), st), "clear flags");
     const uint32_t R = (uint32_t)plan->grounds.size();
     // stream groups may run different rounds at once, so every round has its own regions: candidates,
-    // estimates and magnitudes from max_batch boff[r], device-memory finish arrays from
-    // max_batch foff[r] slices
-    std::vector<size_t> boff(R + 1, 0), foff(R + 1, 0);
+    // estimates and magnitudes from max_batch boff[r]
+    std::vector<size_t> boff(R + 1, 0);
     for (uint32_t r = 0; r < R; ++r) {
         boff[r + 1] = boff[r] + plan->grounds[r].B;
-        foff[r + 1] = foff[r] + (plan->grounds[r].fin_global ? plan->grounds[r].ngroups : 0);
     }
     uint32_t groups = plan->nstreams;
     if (groups > batch) groups = batch;
@@ -467,6 +458,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.logB = gr.logB;
             a.T = gr.T;
             a.rtaps = gr.rtaps;
+            a.nzmax = gr.nzmax;
             a.batch = batch;
             a.dmax = gr.dmax;
             a.t = gr.t;
@@ -492,9 +484,6 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.est_w = plan->d_estw + (size_t)plan->max_batch * boff[r];
             a.est_mag = reinterpret_cast<double*>(plan->d_estw + (size_t)plan->max_batch * boff[R]) +
                         (size_t)plan->max_batch * boff[r];
-            a.fin_scratch =
-                gr.fin_global ? plan->d_gfin + (size_t)plan->max_batch * foff[r] * plan->gfin_stride : nullptr;
-            a.fin_stride = plan->gfin_stride;
             a.bins = plan->d_bins;
             a.phase = plan->d_phase;
             a.bins_stride = plan->bins_stride;

@@ -44,6 +44,11 @@ __device__ __forceinline__ C cmul(C a, C b) {
     r.y = a.x * b.y + a.y * b.x;
     return r;
 }
+// b w with each product and sum rounded as written in any context (a compiler may otherwise merge the
+// product into the sums of an unrolled FFT pass): the roundings of cmul where it is not merged
+__device__ __forceinline__ float2 cmul_rn(float2 b, float2 w) {
+    return make_float2(__fmaf_rn(b.x, w.x, -__fmul_rn(b.y, w.y)), __fmaf_rn(b.x, w.y, __fmul_rn(b.y, w.x)));
+}
 // acc + a * b
 template <typename C>
 __device__ __forceinline__ C cfma(C a, C b, C acc) {
@@ -233,10 +238,9 @@ __device__ inline void rank_sort(const uint32_t* idx, const double2* val, uint32
 // in place in shared memory, all rows together, one barrier per stage.  Butterfly arithmetic and
 // twiddle values are the same in both forms.  Ends with a barrier.
 template <typename R>
-__device__ void block_fft_rows(typename Cx<R>::T* a, uint32_t H, uint32_t logB) {
+__device__ __forceinline__ void fft_first_stages(typename Cx<R>::T* a, uint32_t H, uint32_t logB) {
     using C = typename Cx<R>::T;
     const uint32_t B = 1u << logB;
-    const uint32_t halfB = B >> 1;
     const uint32_t total = H * B, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t S = logB < 5 ? logB : 5;
     __syncthreads();  // the rows are in place
@@ -264,6 +268,15 @@ __device__ void block_fft_rows(typename Cx<R>::T* a, uint32_t H, uint32_t logB) 
         }
     }
     __syncthreads();
+}
+
+template <typename R>
+__device__ void block_fft_rows(typename Cx<R>::T* a, uint32_t H, uint32_t logB) {
+    using C = typename Cx<R>::T;
+    const uint32_t B = 1u << logB;
+    const uint32_t halfB = B >> 1;
+    fft_first_stages<R>(a, H, logB);
+    const uint32_t S = logB < 5 ? logB : 5;
     for (uint32_t st = S + 1; st <= logB; ++st) {
         const uint32_t half = 1u << (st - 1);
         for (uint32_t idx = threadIdx.x; idx < H * halfB; idx += kThreads) {

@@ -259,97 +259,311 @@ __global__ void __launch_bounds__(kThreads, 2) k_gen_gather(const GenArgs a) {
 // ------------------------------------------------------------------------------------------------
 // 2. finish the bins of one hashing group
 // ------------------------------------------------------------------------------------------------
+// One CTA per (hashing group, request): the fold's B-point FFTs, then the recovered coefficients are
+// subtracted in FP64, entry by entry in index order, and a pair's phases are formed.  zhat's entries
+// are placed by bin with a stable counting split (per-warp counters, no sort), up to kFinSlab of them at
+// a time, so that every array stays on chip whatever zhat holds.  Bound by latency in the first round,
+// by FP64 (1/64 of the FP32 rate) once zhat has many entries: per entry and hashing four products, and
+// one chain of subtractions per (bin, hashing, component).  Measured alone at n = 2^20, k = 500 (last
+// round: 16 bins, about 2000 entries): 110 us before, with bin lists sorted by insertion, one thread
+// per bin and arrays in device memory.  Whole calls: 943 -> 640 us there (batch 5), 1155 -> 963 us at
+// n = 2^22, k = 256, batch 8.
+constexpr uint32_t kFinSlab = 2048;  // entries of zhat handled at once (8 per thread)
+constexpr uint32_t kFinPer = kFinSlab / kThreads;
 struct GenFinLayout {
-    size_t U, ent_idx, ent_bin, ent_sub, bin_cnt, bin_start, bin_list, scan, total;
+    size_t U, term, slot, cnt, start, ub, scan, total;
 };
 __host__ __device__ inline size_t gtake(size_t* off, size_t bytes) {
     const size_t o = (*off + 15) & ~size_t(15);
     *off = o + bytes;
     return o;
 }
-__host__ __device__ inline GenFinLayout gen_fin_layout(uint32_t B, uint32_t zcap) {
+// warps that count a slab (each its own counters): 8 up to B = 1024
+__host__ __device__ inline uint32_t fin_segments(uint32_t B) {
+    return B <= 1024 ? 8u : 8192u / B;
+}
+// nzmax: the most entries zhat can have when the round starts
+__host__ __device__ inline GenFinLayout gen_fin_layout(uint32_t B, uint32_t nzmax) {
     GenFinLayout L;
+    const uint32_t ns = nzmax < kFinSlab ? nzmax : kFinSlab;
     size_t off = 0;
     L.U = gtake(&off, (size_t)2 * B * 8);
-    L.ent_idx = gtake(&off, (size_t)zcap * 4);
-    L.ent_bin = gtake(&off, (size_t)zcap * 4);
-    L.ent_sub = gtake(&off, (size_t)zcap * 2 * 16);
-    L.bin_cnt = gtake(&off, (size_t)(B + 1) * 4);
-    L.bin_start = gtake(&off, (size_t)(B + 1) * 4);
-    L.bin_list = gtake(&off, (size_t)zcap * 4);
+    L.term = gtake(&off, (size_t)ns * 2 * 16);
+    L.slot = gtake(&off, (size_t)ns * 4);
+    L.cnt = gtake(&off, ns ? (size_t)fin_segments(B) * B * 2 : 0);
+    L.start = gtake(&off, ns ? (size_t)(B + 1) * 4 : 0);
+    L.ub = gtake(&off, ns && B < (uint32_t)kThreads ? (size_t)4 * B * 8 : 0);
     L.scan = gtake(&off, (size_t)(kThreads + 8) * 4);
     L.total = off;
     return L;
 }
-size_t general_finish_smem(uint32_t B, uint32_t zcap) { return gen_fin_layout(B, zcap).total; }
+size_t general_finish_smem(uint32_t B, uint32_t nzmax) { return gen_fin_layout(B, nzmax).total; }
+
+// (double)v, on the integer units for a zero or normal v
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t f = __float_as_uint(v), m = f & 0x7FFFFFFFu;
+    if (m - 0x00800000u >= 0x7F000000u && m != 0) return (double)v;  // denormal, infinite or NaN
+    const uint32_t hi = (f & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(f << 29));
+}
+// a x + b y rounded once from a sum good to ~2^-46 (exact products, their sum and its error)
+__device__ __forceinline__ float dot2(float a, float x, float b, float y) {
+    const float p = __fmul_rn(a, x), pe = __fmaf_rn(a, x, -p);
+    const float q = __fmul_rn(b, y), qe = __fmaf_rn(b, y, -q);
+    const float s = __fadd_rn(p, q), t = __fsub_rn(s, p);
+    const float e = __fadd_rn(__fsub_rn(p, __fsub_rn(s, t)), __fsub_rn(q, t));
+    return __fadd_rn(s, __fadd_rn(e, __fadd_rn(pe, qe)));
+}
+
+// Stages st + 1 .. st + N of an FFT of H rows: a thread takes the 2^N elements those stages mix, so that
+// one pass over shared memory and one barrier serve N stages.  Ends with a barrier.
+template <int N>
+__device__ __forceinline__ void fft_pass(float2* a, uint32_t H, uint32_t logB, uint32_t st) {
+    constexpr int M = 1 << N;
+    const uint32_t half = 1u << st, groups = 1u << (logB - N);
+    auto butterflies = [&](float2* row, const float2* w) {
+        float2 v[M];
+#pragma unroll
+        for (int e = 0; e < M; ++e) v[e] = row[(uint32_t)e << st];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int e = 0; e < M; ++e)
+                if (!(e & (1 << k))) {
+                    const float2 bv = cmul_rn(v[e | (1 << k)], w[(1 << k) - 1 + (e & ((1 << k) - 1))]);
+                    const float2 av = v[e];
+                    v[e] = cadd(av, bv);
+                    v[e | (1 << k)] = csub(av, bv);
+                }
+#pragma unroll
+        for (int e = 0; e < M; ++e) row[(uint32_t)e << st] = v[e];
+    };
+    // the twiddles of stage st + 1 + k at position lo: exp(-i pi (lo + f half) / (half 2^k)), f < 2^k
+    auto twiddles = [&](uint32_t lo, float2* w) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int f = 0; f < (1 << k); ++f) {
+                float sn, cs;
+                sincospif(-(float)(lo + ((uint32_t)f << st)) / (float)(half << k), &sn, &cs);
+                w[(1 << k) - 1 + f] = mkc(cs, sn);
+            }
+    };
+    float2 w[M - 1];
+    if (groups >= (uint32_t)kThreads) {  // every thread has a position: its twiddles serve all rows
+        for (uint32_t q = threadIdx.x; q < groups; q += kThreads) {
+            const uint32_t lo = q & (half - 1);
+            twiddles(lo, w);
+            for (uint32_t h = 0; h < H; ++h) butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
+        }
+    } else {
+        for (uint32_t i = threadIdx.x; i < H * groups; i += kThreads) {
+            const uint32_t h = i >> (logB - N), q = i & (groups - 1), lo = q & (half - 1);
+            twiddles(lo, w);
+            butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
+        }
+    }
+    __syncthreads();
+}
+
+// block_fft_rows with the stages past the fifth taken two or three per pass: as many as leave every
+// thread a group of elements (B = 2048, two rows: two barriers instead of six, and a third of the
+// sincospif).  The same butterflies, so the same bits.
+__device__ void fft_rows_by_passes(float2* a, uint32_t H, uint32_t logB) {
+    fft_first_stages<float>(a, H, logB);
+    for (uint32_t st = logB < 5 ? logB : 5; st < logB;) {
+        const uint32_t left = logB - st;
+        if (left >= 3 && left != 4 && (H << (logB - 3)) >= (uint32_t)kThreads) {
+            fft_pass<3>(a, H, logB, st);
+            st += 3;
+        } else if (left >= 2 && (H << (logB - 2)) >= (uint32_t)kThreads) {
+            fft_pass<2>(a, H, logB, st);
+            st += 2;
+        } else {
+            fft_pass<1>(a, H, logB, st);
+            st += 1;
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t s = a.req_base + blockIdx.y, g = blockIdx.x, tid = threadIdx.x;
+    const uint32_t s = a.req_base + blockIdx.y, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ReqView rq = gen_req(a, s);
     const HashDesc h = group_desc(a, rq.seed, rq.id, g);
     const uint32_t B = a.B;
-    const GenFinLayout Ly = gen_fin_layout(B, a.zcap);
-    // the arrays live in shared memory, or in this (request, group)'s slice of fin_scratch when large
-    unsigned char* fb = a.fin_scratch ? a.fin_scratch + ((size_t)s * a.ngroups + g) * a.fin_stride : smem;
-    float2* U = reinterpret_cast<float2*>(fb + Ly.U);
-    uint32_t* ent_idx = reinterpret_cast<uint32_t*>(fb + Ly.ent_idx);
-    uint32_t* ent_bin = reinterpret_cast<uint32_t*>(fb + Ly.ent_bin);
-    double2* ent_sub = reinterpret_cast<double2*>(fb + Ly.ent_sub);
-    uint32_t* bin_cnt = reinterpret_cast<uint32_t*>(fb + Ly.bin_cnt);
-    uint32_t* bin_start = reinterpret_cast<uint32_t*>(fb + Ly.bin_start);
-    uint32_t* bin_list = reinterpret_cast<uint32_t*>(fb + Ly.bin_list);
-    uint32_t* scan = reinterpret_cast<uint32_t*>(fb + Ly.scan);
+    const GenFinLayout Ly = gen_fin_layout(B, a.nzmax);
+    float2* U = reinterpret_cast<float2*>(smem + Ly.U);
+    double2* term = reinterpret_cast<double2*>(smem + Ly.term);       // [slot][2]: by bin, then by index
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + Ly.slot);     // an entry's bin, then its place in term
+    uint16_t* cnt = reinterpret_cast<uint16_t*>(smem + Ly.cnt);       // [segment][B]
+    uint32_t* start = reinterpret_cast<uint32_t*>(smem + Ly.start);   // first place of each bin
+    double* ub = reinterpret_cast<double*>(smem + Ly.ub);             // B < kThreads: [hashing][component][B]
+    uint32_t* scan = reinterpret_cast<uint32_t*>(smem + Ly.scan);
     const uint32_t logNp = (uint32_t)(63 - __clzll((long long)a.n)) - a.logB;
     // step 3: the fold, bit-reversed, B-point FFT per hashing
     const float2* part = a.part + (size_t)s * a.part_stride + (size_t)g * 2 * B;
     const uint32_t shift_br = 32u - a.logB;
     for (uint32_t i = tid; i < h.H * B; i += kThreads) {
-        const uint32_t hh = i / B, r = i - hh * B;
-        U[hh * B + (__brev(r) >> shift_br)] = __ldcg(part + (size_t)hh * B + r);
+        const uint32_t r = i & (B - 1);
+        U[i - r + (__brev(r) >> shift_br)] = __ldcg(part + i);
     }
-    // step 4 terms of the recovered coefficients: W(-o(i)) zhat_i w^{a_h sigma i}
-    const uint32_t nz = min(a.zcount[s], a.zcap);
-    for (uint32_t e = tid; e < nz; e += kThreads) {
-        const uint32_t i = a.zidx[(size_t)s * a.zcap + e];
-        ent_idx[e] = i;
-        uint32_t jb;
-        const int32_t o = gen_offset((h.sigma * (i - h.b)) & a.nmask, (uint32_t)a.n, a.nmask, logNp, &jb);
-        ent_bin[e] = jb;
-        const double gain = a.wtab[o < 0 ? -o : o];
-        const double2 z = a.zval[(size_t)s * a.zcap + e];
-        const double2 gz = make_double2(gain * z.x, gain * z.y);
-        for (uint32_t hh = 0; hh < h.H; ++hh) {
-            const double2 w = root_pow<float>((h.a[hh] * h.sigma * i) & a.nmask, a.nmask);
-            ent_sub[2 * e + hh] = make_double2(gz.x * w.x - gz.y * w.y, gz.x * w.y + gz.y * w.x);
-        }
-    }
-    __syncthreads();
-    block_fft_rows<float>(U, h.H, a.logB);
-    bucket_entries(ent_bin, nz, B, bin_cnt, bin_start, bin_list, scan);
+    const uint32_t nz = min(a.zcount[s], a.nzmax);
+    const uint32_t* zidx = a.zidx + (size_t)s * a.zcap;
+    const double2* zval = a.zval + (size_t)s * a.zcap;
+    fft_rows_by_passes(U, h.H, a.logB);
     double2* bins = a.bins + (size_t)s * a.bins_stride;
-    for (uint32_t j = tid; j < B; j += kThreads) {
-        double2 u[2];
-        for (uint32_t hh = 0; hh < h.H; ++hh) {
-            const float2 v = U[hh * B + j];
-            u[hh] = make_double2((double)v.x, (double)v.y);
-        }
-        for (uint32_t xx = bin_start[j]; xx < bin_start[j + 1]; ++xx) {
-            const uint32_t e = bin_list[xx];
-            for (uint32_t hh = 0; hh < h.H; ++hh) {
-                u[hh].x -= ent_sub[2 * e + hh].x;
-                u[hh].y -= ent_sub[2 * e + hh].y;
+    uint32_t* phase = a.phase + (size_t)s * a.phase_stride + (size_t)g * B;
+    const float two_over_n = 2.0f / (float)a.n;
+    const uint32_t row0 = hash_index(a, g, 0);
+    // a bin after the last entry: stored, and c_j for a pair: an FP32 arctangent of the product
+    // u_j conj(u'_j) (the vote arcs are s pi wide and the FP32 bins carry ~1e-6 of phase noise), in units
+    // of 2^-32 of a turn; z is the product rounded to float
+    auto store_phase = [&](uint32_t j, float zx, float zy) {
+        phase[j] = (uint32_t)__double2int_rn(widen(atan2f(zy, zx)) * (4294967296.0 * 0.15915494309189533576888));
+    };
+    if (nz == 0) {
+        for (uint32_t j = tid; j < B; j += kThreads) {
+            const float2 u = U[j];
+            bins[(size_t)row0 * B + j] = make_double2(widen(u.x), widen(u.y));
+            if (h.H == 2) {
+                const float2 v = U[B + j];
+                bins[(size_t)(row0 + 1) * B + j] = make_double2(widen(v.x), widen(v.y));
+                float zx = dot2(u.x, v.x, u.y, v.y), zy = dot2(u.y, v.x, -u.x, v.y);
+                const float mag = fabsf(zx) + fabsf(zy);
+                if (!(mag > 1e-30f && mag < 1e38f)) {  // beyond the range of the exact products' errors
+                    const double2 z = mul_conj_rn(make_double2(widen(u.x), widen(u.y)),
+                                                  make_double2(widen(v.x), widen(v.y)));
+                    zx = (float)z.x;
+                    zy = (float)z.y;
+                }
+                store_phase(j, zx, zy);
             }
         }
-        for (uint32_t hh = 0; hh < h.H; ++hh) bins[(size_t)hash_index(a, g, hh) * B + j] = u[hh];
-        // LocateInner's c_j: an FP32 arctangent of the FP64 product (the vote arcs are s pi wide and
-        // the FP32 bins carry ~1e-6 of phase noise; GB300 runs FP64 at 1/64 of the FP32 rate), kept in
-        // units of 2^-32 of a turn
-        if (h.H == 2) {
-            const double2 z = mul_conj_rn(u[0], u[1]);
-            a.phase[(size_t)s * a.phase_stride + (size_t)g * B + j] =
-                (uint32_t)__double2int_rn((double)atan2f((float)z.y, (float)z.x) * (4294967296.0 * 0.15915494309189533576888));
+        return;
+    }
+    const uint32_t nseg = fin_segments(B), slab = min(a.nzmax, kFinSlab);
+    for (uint32_t z0 = 0; z0 < nz; z0 += slab) {
+        const uint32_t m = min(slab, nz - z0);
+        const bool first = z0 == 0, last = z0 + m == nz;
+        // step 4 terms: W(-o(i)) zhat_i w^{a_h sigma i}
+        double2 gz[kFinPer];
+        uint32_t si[kFinPer];
+#pragma unroll
+        for (uint32_t q = 0; q < kFinPer; ++q) {
+            const uint32_t e = tid + q * kThreads;
+            if (e < m) {
+                const uint32_t i = zidx[z0 + e];
+                uint32_t jb;
+                const int32_t o = gen_offset((h.sigma * (i - h.b)) & a.nmask, (uint32_t)a.n, a.nmask, logNp, &jb);
+                slot[e] = jb;
+                si[q] = h.sigma * i;
+                const double gain = a.wtab[o < 0 ? -o : o];
+                const double2 z = zval[z0 + e];
+                gz[q] = make_double2(gain * z.x, gain * z.y);
+            }
         }
+        for (uint32_t i = tid; i < nseg * B / 2; i += kThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0;
+        __syncthreads();
+        // places by (bin, entry): warp w < nseg counts its share of the slab per bin, the counts are
+        // summed over bins and warps, and the warp's entries take their places in order
+        const uint32_t per = ((m + nseg - 1) / nseg + 31u) & ~31u, e_beg = warp * per, e_end = min(m, e_beg + per);
+        uint16_t* mine = cnt + (size_t)warp * B;
+        if (warp < nseg)
+            for (uint32_t e0 = e_beg; e0 < e_end; e0 += 32) {
+                const bool in = e0 + lane < e_end;
+                const uint32_t b = in ? slot[e0 + lane] : kNoIndex;
+                const unsigned same = __match_any_sync(0xffffffffu, b);
+                if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(mine[b] + __popc((int)same));
+                __syncwarp();
+            }
+        __syncthreads();
+        for (uint32_t j = tid; j < B; j += kThreads) {
+            uint32_t run = 0;
+            for (uint32_t w = 0; w < nseg; ++w) {
+                const uint32_t c = cnt[w * B + j];
+                cnt[w * B + j] = (uint16_t)run;
+                run += c;
+            }
+            start[j] = run;
+        }
+        __syncthreads();
+        block_exclusive_scan(start, B, scan);  // ends with a barrier
+        if (tid == 0) start[B] = m;
+        if (warp < nseg)
+            for (uint32_t e0 = e_beg; e0 < e_end; e0 += 32) {
+                const bool in = e0 + lane < e_end;
+                const uint32_t b = in ? slot[e0 + lane] : kNoIndex;
+                const unsigned same = __match_any_sync(0xffffffffu, b);
+                uint32_t base = 0;
+                if (in) {
+                    base = mine[b];
+                    slot[e0 + lane] = start[b] + base + (uint32_t)__popc((int)(same & ((1u << lane) - 1u)));
+                }
+                __syncwarp();
+                if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(base + __popc((int)same));
+                __syncwarp();
+            }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t q = 0; q < kFinPer; ++q) {
+            const uint32_t e = tid + q * kThreads;
+            if (e < m) {
+                const uint32_t at = slot[e];
+                for (uint32_t hh = 0; hh < h.H; ++hh) {
+                    const uint32_t ex = (h.a[hh] * si[q]) & a.nmask;
+                    const int32_t es = ex > (a.nmask >> 1) ? (int32_t)((int64_t)ex - (int64_t)a.n) : (int32_t)ex;
+                    float sn, cs;
+                    sincospif((float)es * two_over_n, &sn, &cs);
+                    const double wx = widen(cs), wy = widen(-sn);
+                    term[2 * at + hh] = make_double2(gz[q].x * wx - gz[q].y * wy, gz[q].x * wy + gz[q].y * wx);
+                }
+            }
+        }
+        __syncthreads();
+        if (B < (uint32_t)kThreads) {
+            // few bins with long lists: one thread per (component, hashing, bin)
+            for (uint32_t i = tid; i < 2 * h.H * B; i += kThreads) {
+                const uint32_t j = i & (B - 1), c = (i >> a.logB) & 1u, hh = i >> (a.logB + 1);
+                const double* tc = reinterpret_cast<const double*>(term + hh) + c;
+                double u = first ? widen(c ? U[hh * B + j].y : U[hh * B + j].x) : ub[i];
+                for (uint32_t x = start[j], x1 = start[j + 1]; x < x1; ++x) u -= tc[4 * x];
+                ub[i] = u;
+            }
+            __syncthreads();
+            if (last)
+                for (uint32_t j = tid; j < B; j += kThreads) {
+                    const double2 u = make_double2(ub[j], ub[B + j]);
+                    bins[(size_t)row0 * B + j] = u;
+                    if (h.H == 2) {
+                        const double2 v = make_double2(ub[2 * B + j], ub[3 * B + j]);
+                        bins[(size_t)(row0 + 1) * B + j] = v;
+                        const double2 z = mul_conj_rn(u, v);
+                        store_phase(j, (float)z.x, (float)z.y);
+                    }
+                }
+        } else {
+            for (uint32_t j = tid; j < B; j += kThreads) {
+                const uint32_t x0 = start[j], x1 = start[j + 1];
+                double2 u[2];
+                for (uint32_t hh = 0; hh < h.H; ++hh) {
+                    const float2 v = U[hh * B + j];
+                    u[hh] = first ? make_double2(widen(v.x), widen(v.y)) : bins[(size_t)(row0 + hh) * B + j];
+                }
+                for (uint32_t x = x0; x < x1; ++x)
+                    for (uint32_t hh = 0; hh < h.H; ++hh) {
+                        const double2 t = term[2 * x + hh];
+                        u[hh].x -= t.x;
+                        u[hh].y -= t.y;
+                    }
+                for (uint32_t hh = 0; hh < h.H; ++hh) bins[(size_t)(row0 + hh) * B + j] = u[hh];
+                if (h.H == 2 && last) {
+                    const double2 z = mul_conj_rn(u[0], u[1]);
+                    store_phase(j, (float)z.x, (float)z.y);
+                }
+            }
+        }
+        if (!last) __syncthreads();  // the arrays are filled again
     }
 }
 
@@ -1137,7 +1351,7 @@ cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const General
         k_gen_gather<1><<<grid, kThreads, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_gen_finish<<<dim3(r.ngroups, batch), kThreads, r.fin_global ? 0 : r.smem_finish, st>>>(a);
+    k_gen_finish<<<dim3(r.ngroups, batch), kThreads, r.smem_finish, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const uint32_t nb = kThreads / r.t;  // bins per CTA
     k_gen_locate<<<dim3((r.B + nb - 1) / nb, batch), kThreads, r.smem_locate, st>>>(a);

@@ -353,6 +353,7 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
     if (p.z_cap > 4096) return SFFT_ERR_INVALID_ARG;
     const uint32_t tp = t / 4, logtp = ceil_log2(tp);
     size_t taps_off = 0, wtab_off = 0;
+    uint64_t kept = 0;
     for (uint64_t kr = p.k; kr >= 1; kr /= 4) {
         GeneralRound r;
         r.kr = (uint32_t)kr;
@@ -387,11 +388,11 @@ sfft_status build_general_schedule(sfft_plan_s* pl) {
         r.nhash = 2 * r.npairs + p.R_est;
         r.taps_off = taps_off;
         r.wtab_off = wtab_off;
-        r.smem_finish = general_finish_smem(r.B, p.z_cap);
+        r.nzmax = (uint32_t)std::min<uint64_t>(p.z_cap, kept);  // what the rounds before can have kept
+        kept += r.kprime;
+        r.smem_finish = general_finish_smem(r.B, r.nzmax);
         r.smem_locate = general_locate_smem(r.npairs, r.t, p.R_est);
         r.smem_select = general_select_smem(r.B, r.kprime, p.z_cap);
-        // finish arrays beyond kFinSmemMax go to device memory, one slice per (request, group)
-        r.fin_global = r.smem_finish > kFinSmemMax;
         const uint64_t Np = p.n / B;
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, p.alpha0, p.delta, r.T, pl->taps_host.data() + taps_off);

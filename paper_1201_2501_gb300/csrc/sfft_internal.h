@@ -212,7 +212,7 @@ struct GeneralRound {
     uint32_t npairs = 0, ngroups = 0, nhash = 0;
     size_t taps_off = 0, wtab_off = 0;
     size_t smem_finish = 0, smem_locate = 0, smem_select = 0;
-    bool fin_global = false;       // the finish's arrays are too large for shared memory: in d_gfin
+    uint32_t nzmax = 0;            // the most entries zhat can have when the round starts
     bool perm = false;             // the pairs read the permuted copy x_{sigma m} (written first)
 };
 
@@ -229,6 +229,7 @@ struct GenArgs {
     uint32_t B, logB;
     int64_t T;
     uint32_t rtaps;        // taps per range of the fold's summation order (see k_gen_gather)
+    uint32_t nzmax;        // the most entries zhat can have when the round starts
     uint32_t batch;        // requests of the whole call (its stream groups together)
     uint32_t dmax, t, logtp, R_loc, R_est, npairs, ngroups, nhash, kprime;
     uint64_t beta_lo[kMaxLevels], beta_hi[kMaxLevels];
@@ -241,8 +242,6 @@ struct GenArgs {
     size_t part_stride;    // elements per request
     double2* est_w;        // [batch][B] the bins' candidates' estimates
     double* est_mag;       // [batch][B] their squared magnitudes
-    unsigned char* fin_scratch;  // k_gen_finish arrays in device memory: [batch][ngroups][fin_stride], or null
-    size_t fin_stride;
     double2* bins;         // [batch][nhash][B]  (hashing 2g, 2g+1: pair g; 2 npairs + q: estimate q)
     uint32_t* phase;       // [batch][npairs][B] phase(u_a conj(u_{a+beta})) in units of 2^-32 of a turn
     size_t bins_stride, phase_stride;  // elements per request
@@ -344,9 +343,6 @@ struct sfft_plan_s {
     // finisher arrays of the exact rounds with fin_global: per such round, [max_batch][fin_stride]
     unsigned char* d_fin = nullptr;
     size_t fin_stride = 0;
-    // general mode, per round r with fin_global: [max_batch][ngroups_r][gfin_stride]
-    unsigned char* d_gfin = nullptr;
-    size_t gfin_stride = 0, gfin_groups = 0;  // gfin_groups: ngroups summed over those rounds
     size_t dev_bytes = 0;          // device memory allocated at plan creation
     uint64_t samples = 0;          // samples one transform gathers (all rounds, all hashings)
     // internal streams: a batch is split into groups whose rounds run on their own streams
@@ -412,7 +408,7 @@ cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1, ui
                           uint32_t count, uint32_t* out, cudaStream_t st);
 // general mode (sfft_general.cu, sfft_host.cu)
 sfft_status build_general_schedule(sfft_plan_s* pl);
-size_t general_finish_smem(uint32_t B, uint32_t zcap);
+size_t general_finish_smem(uint32_t B, uint32_t nzmax);
 size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est);
 size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
 cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate);

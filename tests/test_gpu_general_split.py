@@ -80,19 +80,22 @@ def test_gather_bins_match_oracle_at_every_split(sf, m, k, batch):
 
 
 # (log2 n, k, bins per k, batch): one, two and four bins per thread of the selection (B up to 1024, 2048,
-# 4096), k' = 3 k above the sort's one key per thread (k = 512) and above B (every candidate is kept)
+# 4096), k' = 3 k above the sort's one key per thread (k = 512) and above B (every candidate is kept);
+# zhat beyond the 2048 entries the finish takes at once, with many and with few bins (k = 1000)
 @pytest.mark.parametrize("m,k,bpk,batch", [(12, 100, 8.0, 3), (13, 256, 8.0, 2), (14, 512, 8.0, 2), (12, 64, 2.0, 2),
-                                           (8, 2, 8.0, 1)])
+                                           (8, 2, 8.0, 1), (14, 1000, 4.0, 2)])
 def test_candidates_and_selection_match_oracle(sf, m, k, bpk, batch):
-    """Rounds 0 and 1 replayed by the oracle on the pipeline's own bins: regions, bottoms and candidates
-    bit for bit, the kept indices bit for bit, values within 1e-12 of the largest."""
+    """Every round replayed by the oracle on the pipeline's own bins: regions, bottoms and candidates
+    bit for bit, the kept indices bit for bit, values within 1e-12 of the largest; the bins after the
+    subtraction of zhat within 2e-5 of the hashing's largest bin before it (FP32 folds)."""
     n, seed = 1 << m, 17
     f = general_fields(n, k, bins_per_k=bpk, z_cap=min(4096, max(8 * k, 64)))
     P = oracle_params(f)
-    x = torch.as_tensor(np.stack(_signals(n, k, batch))).cuda()
+    xs = _signals(n, k, batch)
+    x = torch.as_tensor(np.stack(xs)).cuda()
     plan = _plan(sf, f, batch)
     ks, Bs = oracle.general_rounds(P)
-    for r in range(min(2, len(Bs))):
+    for r in range(len(Bs)):
         _, tr = sf.sfft_execute_trace(plan, x, seed, f["z_cap"], r)
         torch.cuda.synchronize()
         tr = {key: v.cpu().numpy() for key, v in tr.items()}
@@ -114,6 +117,12 @@ def test_candidates_and_selection_match_oracle(sf, m, k, bpk, batch):
                                                np.unique(ocand[ocand != oracle.BOTTOM]), 3 * ks[r])
             nb, na = int(tr["zcount_before"][s]), int(tr["zcount_after"][s])
             zb, za = tr["zval_before"][s], tr["zval_after"][s]
+            zi, zc = tr["zidx_before"][s][:nb].view(np.uint32).astype(np.uint64), zb[:nb, 0] + 1j * zb[:nb, 1]
+            for row, h in [(0, (d[0]["sigma"], d[0]["a"], d[0]["b"])), (2 * npairs, (e[0]["sigma"], e[0]["a"], e[0]["b"])),
+                           (2 * npairs - 1, (d[-1]["sigma"], (d[-1]["a"] + d[-1]["beta"]) % n, d[-1]["b"]))]:
+                x64 = xs[s].astype(np.complex128)
+                scale = np.max(np.abs(oracle.hash_to_bins(x64, *h, B, P.alpha0, P.delta)))
+                assert np.max(np.abs(bins[row] - oracle.hash_to_bins(x64, *h, B, P.alpha0, P.delta, zi, zc))) <= 2e-5 * scale
             merged = dict(zip(tr["zidx_before"][s][:nb].view(np.uint32).tolist(), zb[:nb, 0] + 1j * zb[:nb, 1]))
             for i, v in zip(wi.astype(np.int64).tolist(), wv):
                 merged[i] = merged[i] + v if i in merged else v
