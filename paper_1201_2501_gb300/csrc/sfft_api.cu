@@ -218,10 +218,14 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         }
         if (chan_elems > part_elems) part_elems = chan_elems;
     }
-    for (const GeneralRound& r : pl->grounds) {
+    if (pl->grounds.size() > kMaxGenRounds) {
+        free_plan(pl);
+        return SFFT_ERR_K_RANGE;
+    }
+    for (GeneralRound& r : pl->grounds) {  // every round's folds live at once: one gather serves all rounds
         pl->samples += (uint64_t)r.nhash * (2 * (uint64_t)r.T + 1);
-        const size_t e = (size_t)r.ngroups * 2 * r.B;
-        if (e > part_elems) part_elems = e;
+        r.part_off = part_elems;
+        part_elems += (size_t)r.ngroups * 2 * r.B;
         if ((size_t)r.nhash * r.B > pl->bins_stride) pl->bins_stride = (size_t)r.nhash * r.B;
         if ((size_t)r.npairs * r.B > pl->phase_stride) pl->phase_stride = (size_t)r.npairs * r.B;
         if (r.B > maxB) maxB = r.B;
@@ -281,9 +285,9 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         pl->tw_shift = (ilog2_host(p->n) + 1) / 2;
         SFFT_ALLOC(pl->d_tw, ((size_t(1) << pl->tw_shift) + (p->n >> pl->tw_shift)) * sizeof(double2));
         SFFT_ALLOC(pl->d_estw, (size_t)max_batch * sum_B * (sizeof(double2) + sizeof(double)));
-        bool perm = false;
-        for (const GeneralRound& r : pl->grounds) perm = perm || r.perm;
-        if (perm) SFFT_ALLOC(pl->d_xperm, (size_t)max_batch * p->n * sizeof(float2));
+        size_t perm = 0;
+        for (const GeneralRound& r : pl->grounds) perm += r.perm ? 1 : 0;
+        if (perm) SFFT_ALLOC(pl->d_xperm, perm * max_batch * p->n * sizeof(float2));
     }
 #undef SFFT_ALLOC
     auto fail = [&](cudaError_t err, const char* what) {
@@ -432,22 +436,15 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
         const uint32_t r0 = (uint32_t)((uint64_t)batch * g / groups);
         const uint32_t r1 = (uint32_t)((uint64_t)batch * (g + 1) / groups);
         cudaStream_t gs = groups > 1 ? plan->aux[g] : st;
+        GenArgs args[kMaxGenRounds];
+        size_t nperm = 0;
         for (uint32_t r = 0; r < R; ++r) {
             const GeneralRound& gr = plan->grounds[r];
             const bool traced = tr && tr->round == r;
-            if (traced) {
-                SFFT_CUDA(cudaMemcpyAsync(tr->d_zidx_before, plan->d_zidx, batch * zc * 4, cudaMemcpyDeviceToDevice, gs),
-                          "trace");
-                SFFT_CUDA(cudaMemcpyAsync(tr->d_zval_before, plan->d_zval, batch * zc * 16, cudaMemcpyDeviceToDevice,
-                                          gs),
-                          "trace");
-                SFFT_CUDA(cudaMemcpyAsync(tr->d_zcount_before, plan->d_zcount, batch * 4, cudaMemcpyDeviceToDevice, gs),
-                          "trace");
-            }
-            GenArgs a;
+            GenArgs& a = args[r];
             std::memset(&a, 0, sizeof(a));
             a.x = reinterpret_cast<const float2*>(d_x);
-            a.xperm = gr.perm ? plan->d_xperm : nullptr;
+            a.xperm = gr.perm ? plan->d_xperm + (nperm++) * plan->max_batch * p.n : nullptr;
             a.reqs = d_reqs;
             a.n = p.n;
             a.nmask = (uint32_t)(p.n - 1);
@@ -479,7 +476,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.wtab = plan->d_wtab + gr.wtab_off;
             a.tw = plan->d_tw;
             a.tw_shift = plan->tw_shift;
-            a.part = reinterpret_cast<float2*>(plan->d_part);
+            a.part = reinterpret_cast<float2*>(plan->d_part) + gr.part_off;
             a.part_stride = plan->part_stride;
             a.est_w = plan->d_estw + (size_t)plan->max_batch * boff[r];
             a.est_mag = reinterpret_cast<double*>(plan->d_estw + (size_t)plan->max_batch * boff[R]) +
@@ -503,6 +500,21 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             if (traced) {
                 a.dbg_lfp = tr->d_regions;
                 a.dbg_valid = tr->d_valid;
+            }
+        }
+        SFFT_CUDA(launch_general_gather(args, plan->grounds.data(), R, r1 - r0, gs), "general gather");
+        for (uint32_t r = 0; r < R; ++r) {
+            const GeneralRound& gr = plan->grounds[r];
+            const bool traced = tr && tr->round == r;
+            const GenArgs& a = args[r];
+            if (traced) {
+                SFFT_CUDA(cudaMemcpyAsync(tr->d_zidx_before, plan->d_zidx, batch * zc * 4, cudaMemcpyDeviceToDevice, gs),
+                          "trace");
+                SFFT_CUDA(cudaMemcpyAsync(tr->d_zval_before, plan->d_zval, batch * zc * 16, cudaMemcpyDeviceToDevice,
+                                          gs),
+                          "trace");
+                SFFT_CUDA(cudaMemcpyAsync(tr->d_zcount_before, plan->d_zcount, batch * 4, cudaMemcpyDeviceToDevice, gs),
+                          "trace");
             }
             SFFT_CUDA(launch_general_round(a, r1 - r0, gr, gs), "general round");
             if (traced) {

@@ -4,11 +4,12 @@
 //
 // The hashings of one round are non-adaptive (the intuition of Sec. 4.1): every LocateInner pair
 // (a, a + beta) of every level and every EstimateValues hashing is known before any vote is counted.
-// So a round is four launches for the whole batch (five with the permuted copy):
+// Nor do the samples of any round depend on zhat.  So a batch is one gather for all rounds, then three
+// launches per round:
 //   0. k_gen_permute  (rounds whose LocateInner pairs gather >= 2n samples) every request: x_{sigma m}
 //                     for all m under the round's sigma, so that the pairs read it in order;
-//   1. k_gen_gather   every (residue block, hashings, request): permuted gather, window, modulation,
-//                     fold mod B (HashToBins steps 1-2);
+//   1. k_gen_gather   every (round, residue block, hashings, request): permuted gather, window,
+//                     modulation, fold mod B (HashToBins steps 1-2);
 //   2. k_gen_finish   every (hashing group, request): the fold's B-point FFT
 //                     (step 3), recovered coefficients subtracted in FP64 (step 4), bins stored;
 //                     for a LocateInner pair also c_j = phase(u_j / u'_j);
@@ -138,17 +139,16 @@ __global__ void __launch_bounds__(kThreads) k_gen_permute(const GenArgs a) {
 // are added in thread order), and the ranges' sums are added in range order.
 template <int NH>
 __device__ __forceinline__ void gather_residues(const GenArgs& a, const float2* __restrict__ x, uint32_t xmul,
-                                                uint32_t xmask, uint32_t sb, const uint32_t* ah, uint32_t nh,
+                                                uint32_t xmask, uint32_t sb, const uint32_t* ah, uint32_t nh, uint32_t blk,
                                                 float2* __restrict__ out, float2 (*red)[kThreads]) {
     constexpr int TB = NH >= 8 ? 2 : (NH == 4 ? 4 : (NH == 2 ? 8 : 16));  // taps per batch of loads
     const uint32_t tid = threadIdx.x, B = a.B;
     const uint32_t step = B > (uint32_t)kThreads ? B : (uint32_t)kThreads;  // a thread's taps are step apart
-    const uint32_t k0 = blockIdx.x * kThreads + tid;
+    const uint32_t first = blk * kThreads, k0 = first + tid;
     const uint32_t ntot = (uint32_t)(2 * a.T + 1);
     const uint32_t t0 = (uint32_t)(int32_t)(-a.T) + k0;  // first tap, mod 2^32
     const uint32_t nt = a.rtaps / step;                  // a thread's taps per range (a power of two if there are several)
     const bool several = ntot > a.rtaps;
-    const uint32_t first = blockIdx.x * kThreads;
     const uint32_t mend = first < ntot ? (ntot - first + step - 1) / step : 0;  // batches end here for every thread
     float2 acc[NH], sum[NH];
     uint32_t xi[NH];
@@ -226,21 +226,11 @@ __device__ __forceinline__ void gather_residues(const GenArgs& a, const float2* 
     }
 }
 
-// Grid (residue blocks, EstimateValues hashings then blocks of P pairs, requests).
+// P pairs from g0 on (the round's last block may hold fewer)
 template <int P>
-__global__ void __launch_bounds__(kThreads, 2) k_gen_gather(const GenArgs a) {
-    __shared__ float2 red[2 * P][kThreads];
-    const uint32_t s = a.req_base + blockIdx.z;
-    const ReqView rq = gen_req(a, s);
-    float2* part = a.part + (size_t)s * a.part_stride;
-    if (blockIdx.y < a.R_est) {
-        const uint32_t g = a.npairs + blockIdx.y;
-        const HashDesc h = group_desc(a, rq.seed, rq.id, g);
-        gather_residues<1>(a, static_cast<const float2*>(rq.x), h.sigma, rq.xmask, h.sigma * h.b, h.a, 1,
-                           part + (size_t)g * 2 * a.B, red);
-        return;
-    }
-    const uint32_t g0 = (blockIdx.y - a.R_est) * P, np = min((uint32_t)P, a.npairs - g0);
+__device__ __forceinline__ void gather_pairs(const GenArgs& a, const ReqView& rq, uint32_t s, uint32_t g0, uint32_t blk,
+                                             float2* part, float2 (*red)[kThreads]) {
+    const uint32_t np = min((uint32_t)P, a.npairs - g0);
     // a round with a permuted copy reads xperm[(t - a) mod n] = x_{sigma (t - a)} in order
     const bool perm = a.xperm != nullptr;
     uint32_t sigma, b, ah[2 * P];
@@ -253,7 +243,47 @@ __global__ void __launch_bounds__(kThreads, 2) k_gen_gather(const GenArgs a) {
         ah[2 * p + 1] = (uint32_t)((ah[2 * p] + beta) & a.nmask);
     }
     gather_residues<2 * P>(a, perm ? a.xperm + (size_t)s * a.n : static_cast<const float2*>(rq.x), perm ? 1u : sigma,
-                           perm ? a.nmask : rq.xmask, sigma * b, ah, 2 * np, part + (size_t)g0 * 2 * a.B, red);
+                           perm ? a.nmask : rq.xmask, sigma * b, ah, 2 * np, blk, part + (size_t)g0 * 2 * a.B, red);
+}
+
+// Every round's hashings in one launch (their samples do not depend on zhat): grid (CTAs of all
+// rounds, requests), request by request so that a signal and its copies stay in L2; a round's CTAs
+// are its EstimateValues hashings, then its blocks of P pairs, residue blocks fastest.  The small
+// rounds' few CTAs run beside the first round's.  Whole calls, against one gather per round: n = 2^22,
+// k = 256, batch 8: 774 us, was 963; n = 2^18, k = 50, one request: 132 us, was 150; n = 2^26, k = 64,
+// batch 4: 603 us, was 670 (26.3 M random sectors of HBM: 44 G/s).
+template <int NR>
+struct GatherParams {
+    uint32_t R;
+    uint32_t seg[NR + 1];  // first CTA of each round
+    uint32_t P[NR];        // pairs per CTA: 1, 2 or 4
+    GenArgs r[NR];
+};
+template <int NR>
+__global__ void __launch_bounds__(kThreads, 2) k_gen_gather(const __grid_constant__ GatherParams<NR> gp) {
+    __shared__ float2 red[8][kThreads];
+    uint32_t r = 0;
+    while (r + 1 < gp.R && blockIdx.x >= gp.seg[r + 1]) ++r;
+    const GenArgs& a = gp.r[r];
+    const uint32_t s = a.req_base + blockIdx.y;
+    const uint32_t blocks = a.B > (uint32_t)kThreads ? a.B / kThreads : 1u;
+    const uint32_t local = blockIdx.x - gp.seg[r], blk = local % blocks, y = local / blocks;
+    const ReqView rq = gen_req(a, s);
+    float2* part = a.part + (size_t)s * a.part_stride;
+    if (y < a.R_est) {
+        const uint32_t g = a.npairs + y;
+        const HashDesc h = group_desc(a, rq.seed, rq.id, g);
+        gather_residues<1>(a, static_cast<const float2*>(rq.x), h.sigma, rq.xmask, h.sigma * h.b, h.a, 1, blk,
+                           part + (size_t)g * 2 * a.B, red);
+        return;
+    }
+    const uint32_t P = gp.P[r], g0 = (y - a.R_est) * P;
+    if (P == 4)
+        gather_pairs<4>(a, rq, s, g0, blk, part, red);
+    else if (P == 2)
+        gather_pairs<2>(a, rq, s, g0, blk, part, red);
+    else
+        gather_pairs<1>(a, rq, s, g0, blk, part, red);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1330,27 +1360,38 @@ cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t
     return e;
 }
 
-cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st) {
-    if (r.perm) {
-        const uint64_t per = (uint64_t)kThreads * 8, blocks = (a.n + per - 1) / per;
-        k_gen_permute<<<dim3((uint32_t)(blocks < 65535 ? blocks : 65535), batch), kThreads, 0, st>>>(a);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+template <int NR>
+static cudaError_t launch_gather_nr(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st) {
+    GatherParams<NR> gp;
+    gp.R = R;
+    gp.seg[0] = 0;
+    for (uint32_t r = 0; r < R; ++r) {
+        // pairs per CTA: as many as leave the chip (152 SMs, 2 CTAs each) two waves of CTAs over the
+        // whole call, so that a tap's window product serves more hashings
+        const uint32_t blocks = g[r].B > (uint32_t)kThreads ? g[r].B / kThreads : 1u;
+        const uint64_t pairs = (uint64_t)blocks * g[r].npairs * a[r].batch;
+        gp.P[r] = pairs >= 4 * 608 ? 4u : (pairs >= 2 * 608 ? 2u : 1u);
+        gp.seg[r + 1] = gp.seg[r] + blocks * (a[r].R_est + (g[r].npairs + gp.P[r] - 1) / gp.P[r]);
+        gp.r[r] = a[r];
     }
-    // pairs per gather CTA: as many as leave the chip (152 SMs, 2 CTAs each) two waves of CTAs over the
-    // whole call, so that a tap's window product serves more hashings
-    const uint32_t blocks = r.B > (uint32_t)kThreads ? r.B / kThreads : 1u;
-    const uint64_t pairs = (uint64_t)blocks * r.npairs * a.batch;
-    const uint32_t P = pairs >= 4 * 608 ? 4u : (pairs >= 2 * 608 ? 2u : 1u);
-    const dim3 grid(blocks, a.R_est + (r.npairs + P - 1) / P, batch);
-    if (P == 4)
-        k_gen_gather<4><<<grid, kThreads, 0, st>>>(a);
-    else if (P == 2)
-        k_gen_gather<2><<<grid, kThreads, 0, st>>>(a);
-    else
-        k_gen_gather<1><<<grid, kThreads, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    k_gen_gather<NR><<<dim3(gp.seg[R], batch), kThreads, 0, st>>>(gp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_general_gather(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st) {
+    if (R == 0 || R > kMaxGenRounds) return cudaErrorInvalidValue;
+    for (uint32_t r = 0; r < R; ++r)
+        if (g[r].perm) {
+            const uint64_t per = (uint64_t)kThreads * 8, blocks = (a[r].n + per - 1) / per;
+            k_gen_permute<<<dim3((uint32_t)(blocks < 65535 ? blocks : 65535), batch), kThreads, 0, st>>>(a[r]);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+    return R <= 6 ? launch_gather_nr<6>(a, g, R, batch, st) : launch_gather_nr<kMaxGenRounds>(a, g, R, batch, st);
+}
+
+cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st) {
+    cudaError_t e;
     k_gen_finish<<<dim3(r.ngroups, batch), kThreads, r.smem_finish, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const uint32_t nb = kThreads / r.t;  // bins per CTA

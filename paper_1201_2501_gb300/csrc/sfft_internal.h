@@ -200,6 +200,7 @@ constexpr int kMaxLevels = 16;   // LocateSignal levels D_max
 constexpr int kMaxRloc = 15;     // LocateInner rounds per level
 constexpr int kMaxRest = 15;     // EstimateValues hashings
 constexpr int kMaxT = 32;        // regions per level t
+constexpr uint32_t kMaxGenRounds = 16;  // rounds of a general plan (k_r falls by 4 from k <= n / 4 < 2^29)
 constexpr int kFracBits = 16;    // fixed-point fraction bits of region positions
 
 struct GeneralRound {
@@ -214,6 +215,7 @@ struct GeneralRound {
     size_t smem_finish = 0, smem_locate = 0, smem_select = 0;
     uint32_t nzmax = 0;            // the most entries zhat can have when the round starts
     bool perm = false;             // the pairs read the permuted copy x_{sigma m} (written first)
+    size_t part_off = 0;           // the round's folds in a request's region (elements)
 };
 
 // Kernel argument block of the general-mode kernels of one round (passed by value).
@@ -238,7 +240,7 @@ struct GenArgs {
     const double* wtab;
     const double2* tw;     // FP64 twiddles w^e = tw[e mod 2^tw_shift] tw[2^tw_shift + (e >> tw_shift)]
     uint32_t tw_shift;
-    float2* part;          // [batch][ngroups][2][B]: the folds
+    float2* part;          // [batch][ngroups][2][B]: the round's folds
     size_t part_stride;    // elements per request
     double2* est_w;        // [batch][B] the bins' candidates' estimates
     double* est_mag;       // [batch][B] their squared magnitudes
@@ -308,7 +310,7 @@ struct sfft_plan_s {
     uint32_t* d_L = nullptr;  // general mode: per round r, [max_batch][B_r] candidates
     double2* d_tw = nullptr;  // general mode: FP64 twiddle factor tables (2^tw_shift + n / 2^tw_shift)
     uint32_t tw_shift = 0;
-    float2* d_xperm = nullptr;  // general mode, rounds with perm: [max_batch][n] permuted signals
+    float2* d_xperm = nullptr;  // general mode, per round with perm: [max_batch][n] permuted signals
     // general mode: per round r, [max_batch][B_r] estimates; then per round [max_batch][B_r] magnitudes
     double2* d_estw = nullptr;
     size_t bins_stride = 0, phase_stride = 0;
@@ -412,6 +414,8 @@ size_t general_finish_smem(uint32_t B, uint32_t nzmax);
 size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est);
 size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
 cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate);
+// the gathers of every round (and the permuted copies they read), then per round the rest
+cudaError_t launch_general_gather(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st);
 cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st);
 cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);
