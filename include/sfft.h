@@ -295,15 +295,15 @@ sfft_status sfft_autotune(const sfft_params* base, uint32_t batch, double snr_db
                           sfft_params* best, sfft_tune_entry* report, uint32_t report_cap, uint32_t* n_report);
 
 /* ---------------------------------------------------------------------------------------------- */
-/* Mixed batches in one persistent launch                                                          */
+/* Mixed batches in one launch                                                                     */
 /* ---------------------------------------------------------------------------------------------- */
 /*
  * A batch plan groups exact-mode plans of any (n, k) (one precision) so that a batch mixing them runs
- * as ONE persistent launch: CTAs take (request, round, chunk) items from a device queue, and the CTA
- * that finishes a request's round (Algorithm 1's loop) queues that request's next round at once, so
- * rounds of different requests overlap with no launch boundary between them.  Results are those of
- * sfft_execute_requests on each request's own plan, bit for bit.  The batch plan owns a workspace for
- * max_requests requests; the plans must outlive it.
+ * as ONE launch (two, side by side, where plans with z_cap above 256 are mixed with others): the
+ * gathers of every request and round (Algorithm 1's loop) are in the grid at once, and the decodes of a
+ * request's rounds follow one another as their bins arrive, with no launch boundary between them.
+ * Results are those of sfft_execute_requests on each request's own plan, bit for bit.  The batch plan
+ * owns a workspace for max_requests requests; the plans must outlive it.
  * Errors: INVALID_ARG (null, nplans == 0, a general-mode plan, mixed precisions), OOM, CUDA.
  */
 typedef struct sfft_batch_plan_s* sfft_batch_plan;
@@ -315,8 +315,7 @@ sfft_status sfft_batch_plan_destroy(sfft_batch_plan bp);
  * Run nreq (<= max_requests) requests: request r uses plans[h_plan_of[r]] and h_reqs[r] (signal, seed,
  * id, period).  Outputs as for sfft_execute (slot r, capacity cap).  The host tables are staged in
  * page-locked memory owned by the batch plan (two buffers, so consecutive calls on one stream do not
- * wait for each other).  A request whose queue item was not published within about a second (a
- * malfunction, never expected) ends with d_flag = SFFT_ERR_TIMEOUT.
+ * wait for each other).
  * Errors: INVALID_ARG (null, nreq out of range, a plan index or request that is out of range), CUDA.
  */
 sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, const sfft_request* h_reqs,
@@ -324,10 +323,10 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
                                uint32_t* d_count, int32_t* d_flag);
 
 /*
- * Check of the persistent launch's bounded wait: one CTA of the batch kernel takes a queue item that
- * nothing ever publishes.  Its wait gives up after about a second, it sets the launch's error flag and
- * returns; the call synchronises `stream` and returns SFFT_ERR_TIMEOUT when the flag was set (the
- * expected outcome) or SFFT_OK if the wait did not give up.  The device stays usable either way.
+ * Check of a bounded device wait: one thread waits for a word that nothing ever publishes.  Its wait
+ * gives up after about a second, it sets an error flag and returns; the call synchronises `stream` and
+ * returns SFFT_ERR_TIMEOUT when the flag was set (the expected outcome) or SFFT_OK if the wait did not
+ * give up.  The device stays usable either way.  (No launch of this library waits on another CTA.)
  * Errors: OOM, CUDA.
  */
 sfft_status sfft_persistent_wait_check(void* stream);

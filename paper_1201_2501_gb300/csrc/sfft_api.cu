@@ -104,6 +104,11 @@ ExactArgs base_args(const sfft_plan_s* pl, const ExactRound& r, uint32_t t) {
         a.shift64[l + 1] = r.shift[l];
     }
     a.chunks = r.chunks;
+    a.owner = r.owner ? 1 : 0;
+    a.ring = r.ring;
+    a.gctas = r.owner ? r.B / (uint32_t)kThreads : r.chunks;
+    a.large = r.large ? 1 : 0;
+    a.large_smem = kLargeSmem;
     a.ctaps = r.ctaps;
     a.stage = r.stage;
     a.maxshift = (uint32_t)r.shift[r.nshift - 1];
@@ -113,7 +118,7 @@ ExactArgs base_args(const sfft_plan_s* pl, const ExactRound& r, uint32_t t) {
     a.winv = a.wtab + (p.n / r.B) / 2 + 1;  // the exact schedule stores 1 / W(o) after W(o)
     a.part = pl->d_part;
     a.part_stride = pl->part_stride;
-    a.fin_scratch = r.fin_global ? pl->d_fin : nullptr;
+    a.fin_scratch = r.fin_bytes ? pl->d_fin : nullptr;
     a.fin_stride = pl->fin_stride;
     a.counter = pl->d_counter;
     a.zidx = pl->d_zidx;
@@ -201,10 +206,10 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     for (const ExactRound& r : pl->rounds) {
         pl->samples += 2 * (uint64_t)r.T + 1 + r.shift[r.nshift - 1];
         part_off.push_back(part_elems);
-        part_elems += (size_t)r.chunks * (1 + r.nshift) * r.B;
+        part_elems += (size_t)(r.owner ? 1 : r.chunks) * (1 + r.nshift) * r.B;
         if (r.smem > max_smem) max_smem = r.smem;
         if (r.B > maxB) maxB = r.B;
-        if (r.fin_global && r.fin_bytes > pl->fin_stride) pl->fin_stride = (r.fin_bytes + 255) & ~size_t(255);
+        if (r.fin_bytes > pl->fin_stride) pl->fin_stride = (r.fin_bytes + 255) & ~size_t(255);
     }
     if (!general && !fp64) {  // the partial folds of a multi-channel batch (sfft_execute_channels)
         size_t chan_elems = 0;
@@ -238,7 +243,10 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     pl->part_stride = part_elems;
     pl->max_B = maxB;
     pl->max_groups = max_groups;
-    pl->part_bytes = part_elems * (size_t)max_batch * (fp64 ? 16 : 8);
+    // sfft_hash_to_bins folds any round by chunks
+    size_t single = 0;
+    for (const ExactRound& r : pl->rounds) single = std::max(single, (size_t)r.chunks * r.B);
+    pl->part_bytes = std::max(part_elems * max_batch, single) * (fp64 ? 16 : 8);
     cudaError_t e = cudaSuccess;
 #define SFFT_ALLOC(ptr, bytes)                                        \
     do {                                                              \
@@ -336,7 +344,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         if ((e = cudaEventCreateWithFlags(&pl->ev_join[i], cudaEventDisableTiming)) != cudaSuccess)
             return fail(e, "create event");
     }
-    if (!general && (e = set_exact_smem_limit(max_smem, fp64)) != cudaSuccess) return fail(e, "shared memory limit");
+    if (!general && (e = set_exact_smem_limit(max_smem, fp64, pl->rounds[0].large)) != cudaSuccess) return fail(e, "shared memory limit");
     if (general && (e = general_set_smem(fs_max, ls_max, ss_max, 0)) != cudaSuccess)
         return fail(e, "shared memory limit");
     // The gather reads one 8- or 16-byte sample per 32-byte sector at random; ask L2 not to widen
@@ -621,6 +629,7 @@ static sfft_status execute_channels(sfft_plan plan, const void* d_x, uint32_t ch
         a.req_base = 0;
         a.part = static_cast<unsigned char*>(plan->d_part) + plan->chan_off[t] * sizeof(float2);
         a.chunks = plan->chan_chunks[t];
+        a.owner = 0;
         a.out_idx = d_idx;
         a.out_val = reinterpret_cast<double2*>(d_val);
         a.out_cap = cap;
@@ -815,6 +824,9 @@ sfft_status sfft_hash_to_bins(sfft_plan plan, uint32_t t, const void* d_x, uint6
     args.a[0] = 0;
     args.maxshift = 0;
     args.stage = r.ctaps;
+    args.owner = 0;
+    args.gctas = r.chunks;
+    args.fin_scratch = r.fin_global ? plan->d_fin : nullptr;
     args.bins_only = 1;
     args.e_sigma = (uint32_t)sigma;
     args.e_b = (uint32_t)b;
@@ -827,7 +839,7 @@ sfft_status sfft_hash_to_bins(sfft_plan plan, uint32_t t, const void* d_x, uint6
                                                                 (fp64 ? 16 : 8);
     const size_t fs = exact_finish_smem(r.B, 1, args.zcap, fp64);
     const size_t smem = gs > fs ? gs : fs;
-    SFFT_CUDA(set_exact_smem_limit(smem > r.smem ? smem : r.smem, fp64), "shared memory limit");
+    SFFT_CUDA(set_exact_smem_limit(smem, fp64, r.large), "shared memory limit");
     SFFT_CUDA(launch_exact_round(args, 1, smem, st, fp64), "hash to bins");
     return SFFT_OK;
 }
@@ -943,42 +955,39 @@ sfft_status sfft_estimate_from_bins(sfft_plan plan, uint32_t r, uint32_t nrep, c
 }  // extern "C"
 
 // ------------------------------------------------------------------------------------------------
-// Batch plans: mixed exact-mode requests in one persistent launch
+// Batch plans: mixed exact-mode requests in one launch
 // ------------------------------------------------------------------------------------------------
 struct sfft_batch_plan_s {
     std::vector<sfft_plan> plans;
-    std::vector<uint32_t> rd0, rounds, chunks0, items_of;  // per plan: first descriptor, rounds,
-                                                          // round-0 chunks, items of a request
+    std::vector<uint32_t> rd0;         // per plan: its first descriptor
     bool fp64 = false;
-    uint32_t max_req = 0;
-    size_t max_items = 0;         // items of the largest batch the workspace holds
+    uint32_t max_req = 0, max_rounds = 0;
+    size_t smem[2] = {0, 0};           // dynamic shared memory of the plans without and with finish_large
     ExactArgs* d_rdesc = nullptr;
-    unsigned char* d_ctl = nullptr;  // [reqs | rd0 | rounds | head, tail, error | flags] of one call
-    unsigned long long* d_items = nullptr;
+    unsigned char* d_ctl = nullptr;    // the tables of one call (CtlLayout)
     unsigned char* d_part = nullptr;
     size_t part_stride = 0;
     uint32_t* d_counter = nullptr;
     uint32_t* d_zidx = nullptr;
     double2* d_zval = nullptr;
     size_t z_stride = 0;
-    uint32_t* d_zcount = nullptr;
-    int32_t* d_zflag = nullptr;
+    uint32_t* d_zstate = nullptr;      // [2][max_req]: counts, then flags
     unsigned char* d_fin = nullptr;
     size_t fin_stride = 0;
-    size_t smem = 0;
-    int ctas = 0;
     size_t ctl_bytes = 0;
-    unsigned char* h_stage[2] = {nullptr, nullptr};  // page-locked copies of the control block + items
+    unsigned char* h_stage[2] = {nullptr, nullptr};  // page-locked copies of the tables
     cudaEvent_t ev[2] = {nullptr, nullptr};
     int cur = 0;
+    cudaStream_t side = nullptr;       // plans with finish_large run here, beside the others
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 namespace {
 
 struct CtlLayout {
-    size_t reqs, rd0, rounds, ctr, flags, items, total;
+    size_t reqs, rd0, rounds, seg, who, total;
 };
-CtlLayout ctl_layout(uint32_t nreq, size_t items0) {
+CtlLayout ctl_layout(uint32_t nreq, size_t nseg) {
     CtlLayout L;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -989,9 +998,8 @@ CtlLayout ctl_layout(uint32_t nreq, size_t items0) {
     L.reqs = take((size_t)nreq * sizeof(ReqDesc));
     L.rd0 = take((size_t)nreq * 4);
     L.rounds = take((size_t)nreq * 4);
-    L.ctr = take(16);
-    L.flags = take((size_t)nreq * 4);
-    L.items = take(items0 * 8);
+    L.seg = take(nseg * 4);
+    L.who = take(nseg * 4);
     L.total = off;
     return L;
 }
@@ -1000,18 +1008,19 @@ void free_batch_plan(sfft_batch_plan_s* bp) {
     if (!bp) return;
     cudaFree(bp->d_rdesc);
     cudaFree(bp->d_ctl);
-    cudaFree(bp->d_items);
     cudaFree(bp->d_part);
     cudaFree(bp->d_counter);
     cudaFree(bp->d_zidx);
     cudaFree(bp->d_zval);
-    cudaFree(bp->d_zcount);
-    cudaFree(bp->d_zflag);
+    cudaFree(bp->d_zstate);
     cudaFree(bp->d_fin);
     for (int i = 0; i < 2; ++i) {
         cudaFreeHost(bp->h_stage[i]);
         if (bp->ev[i]) cudaEventDestroy(bp->ev[i]);
     }
+    if (bp->side) cudaStreamDestroy(bp->side);
+    if (bp->ev_fork) cudaEventDestroy(bp->ev_fork);
+    if (bp->ev_join) cudaEventDestroy(bp->ev_join);
     delete bp;
 }
 
@@ -1027,7 +1036,6 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
     for (uint32_t i = 0; i < nplans; ++i) {
         if (!plans[i] || plans[i]->p.mode != SFFT_EXACT) return SFFT_ERR_INVALID_ARG;
         if (plans[i]->p.precision != plans[0]->p.precision) return SFFT_ERR_INVALID_ARG;
-        if (plans[i]->rounds.size() > 255) return SFFT_ERR_INVALID_ARG;
     }
     auto* bp = new (std::nothrow) sfft_batch_plan_s();
     if (!bp) return SFFT_ERR_OOM;
@@ -1036,94 +1044,81 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
     bp->max_req = max_requests;
     const size_t csize = bp->fp64 ? 16 : 8;
     std::vector<ExactArgs> rdesc;
-    uint32_t max_items_req = 0, max_chunks0 = 0;
+    size_t max_ctas_req = 0;
+    bool kinds[2] = {false, false};
     for (sfft_plan pl : bp->plans) {
         bp->rd0.push_back((uint32_t)rdesc.size());
         const uint32_t R = (uint32_t)pl->rounds.size();
-        bp->rounds.push_back(R);
-        uint32_t items = 0;
+        bp->max_rounds = std::max(bp->max_rounds, R);
+        size_t ctas = 0;
         for (uint32_t t = 0; t < R; ++t) {
             const ExactRound& r = pl->rounds[t];
-            if (r.chunks > 0xFFFFu) {
-                free_batch_plan(bp);
-                return SFFT_ERR_K_RANGE;
-            }
-            ExactArgs a = base_args(pl, r, t);
-            a.first_round = t == 0;
-            a.last_round = t + 1 == R;
+            ExactArgs a = pl->rdesc[t];  // its folds where the plan has them, in the request's own region
+            a.part_bytes = (size_t)(static_cast<unsigned char*>(a.part) - static_cast<unsigned char*>(pl->d_part));
             rdesc.push_back(a);
-            items += r.chunks;
-            bp->smem = std::max(bp->smem, r.smem);
-            if (r.fin_global) bp->fin_stride = std::max(bp->fin_stride, (r.fin_bytes + 255) & ~size_t(255));
+            ctas += a.gctas;
+            const int kind = r.large ? 1 : 0;
+            kinds[kind] = true;
+            bp->smem[kind] = std::max(bp->smem[kind], r.smem);
+            bp->fin_stride = std::max(bp->fin_stride, (r.fin_bytes + 255) & ~size_t(255));
         }
-        bp->chunks0.push_back(pl->rounds[0].chunks);
-        bp->items_of.push_back(items);
-        max_items_req = std::max(max_items_req, items);
-        max_chunks0 = std::max(max_chunks0, pl->rounds[0].chunks);
+        max_ctas_req = std::max(max_ctas_req, ctas);
         bp->part_stride = std::max(bp->part_stride, ((pl->part_stride * csize) + 255) & ~size_t(255));
         bp->z_stride = std::max(bp->z_stride, (size_t)pl->p.z_cap);
     }
-    bp->max_items = (size_t)max_items_req * max_requests;
-    if (bp->max_items >= (size_t)1 << 32) {
+    if (max_ctas_req * max_requests >= (size_t)1 << 32) {
         free_batch_plan(bp);
         return SFFT_ERR_INVALID_ARG;
     }
-    bp->ctl_bytes = ctl_layout(max_requests, (size_t)max_chunks0 * max_requests).total;
+    bp->ctl_bytes = ctl_layout(max_requests, (size_t)bp->max_rounds * max_requests).total;
+    const size_t counter_bytes = (size_t)max_requests * 2 * kMaxRounds * 4;
     bool ok = cudaMalloc((void**)&bp->d_rdesc, rdesc.size() * sizeof(ExactArgs)) == cudaSuccess &&
               cudaMalloc((void**)&bp->d_ctl, bp->ctl_bytes) == cudaSuccess &&
-              cudaMalloc((void**)&bp->d_items, bp->max_items * 8) == cudaSuccess &&
               cudaMalloc((void**)&bp->d_part, bp->part_stride * max_requests) == cudaSuccess &&
-              cudaMalloc((void**)&bp->d_counter, (size_t)max_requests * 4) == cudaSuccess &&
+              cudaMalloc((void**)&bp->d_counter, counter_bytes) == cudaSuccess &&
               cudaMalloc((void**)&bp->d_zidx, bp->z_stride * max_requests * 4) == cudaSuccess &&
               cudaMalloc((void**)&bp->d_zval, bp->z_stride * max_requests * 16) == cudaSuccess &&
-              cudaMalloc((void**)&bp->d_zcount, (size_t)max_requests * 4) == cudaSuccess &&
-              cudaMalloc((void**)&bp->d_zflag, (size_t)max_requests * 4) == cudaSuccess &&
+              cudaMalloc((void**)&bp->d_zstate, (size_t)max_requests * 8) == cudaSuccess &&
               (bp->fin_stride == 0 || cudaMalloc((void**)&bp->d_fin, bp->fin_stride * max_requests) == cudaSuccess) &&
               cudaMallocHost((void**)&bp->h_stage[0], bp->ctl_bytes) == cudaSuccess &&
               cudaMallocHost((void**)&bp->h_stage[1], bp->ctl_bytes) == cudaSuccess &&
               cudaEventCreateWithFlags(&bp->ev[0], cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&bp->ev[1], cudaEventDisableTiming) == cudaSuccess;
+    if (ok && kinds[0] && kinds[1])
+        ok = cudaStreamCreateWithFlags(&bp->side, cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&bp->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&bp->ev_join, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
         set_last_error(std::string("batch plan: ") + cudaGetErrorString(cudaGetLastError()));
         free_batch_plan(bp);
         return SFFT_ERR_OOM;
     }
     cudaError_t e = cudaMemcpy(bp->d_rdesc, rdesc.data(), rdesc.size() * sizeof(ExactArgs), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(bp->d_counter, 0, (size_t)max_requests * 4);
+    if (e == cudaSuccess) e = cudaMemset(bp->d_counter, 0, counter_bytes);
+    for (int kind = 0; kind < 2; ++kind)
+        if (e == cudaSuccess && kinds[kind]) e = set_batch_smem_limit(bp->smem[kind], bp->fp64, kind != 0);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         set_last_error(std::string("batch plan: ") + cudaGetErrorString(e));
         free_batch_plan(bp);
         return SFFT_ERR_CUDA;
-    }
-    bp->ctas = exact_persistent_ctas(bp->smem, bp->fp64);
-    if (bp->ctas <= 0) {
-        set_last_error("batch plan: no CTA of the persistent kernel fits on the device");
-        free_batch_plan(bp);
-        return SFFT_ERR_K_RANGE;
     }
     *out = bp;
     return SFFT_OK;
 }
 
 sfft_status sfft_persistent_wait_check(void* stream) {
-    // control block: items[1] (never published), head, tail, error
-    unsigned char* d = nullptr;
+    unsigned char* d = nullptr;  // the word, the error flag
     if (cudaMalloc((void**)&d, 64) != cudaSuccess) {
         cudaGetLastError();
         return SFFT_ERR_OOM;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    PersistArgs a;
-    std::memset(&a, 0, sizeof(a));
-    a.items = reinterpret_cast<unsigned long long*>(d);
-    a.head = reinterpret_cast<uint32_t*>(d + 16);
-    a.tail = a.head + 1;
-    a.error = reinterpret_cast<int32_t*>(a.head + 2);
-    a.total = 1;
+    int32_t* flag = reinterpret_cast<int32_t*>(d + 16);
     int32_t err = 0;
     cudaError_t e = cudaMemsetAsync(d, 0, 64, st);
-    if (e == cudaSuccess) e = launch_exact_persistent(a, 1, 0, st, false);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, a.error, sizeof(err), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = launch_wait_check(reinterpret_cast<const uint32_t*>(d), flag, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, flag, sizeof(err), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaFree(d);
     if (e != cudaSuccess) {
@@ -1148,71 +1143,68 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
     if (nreq == 0 || nreq > bp->max_req) return SFFT_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t align = bp->fp64 ? 16 : 8;
-    size_t items0 = 0, total = 0;
+    size_t nseg = 0;
     for (uint32_t r = 0; r < nreq; ++r) {
         const uint32_t p = h_plan_of[r];
         if (p >= bp->plans.size() || !h_reqs[r].d_x || ((uintptr_t)h_reqs[r].d_x % align) != 0)
             return SFFT_ERR_INVALID_ARG;
         const uint32_t per = h_reqs[r].period;
         if (per != 0 && (!is_pow2(per) || per > bp->plans[p]->p.n)) return SFFT_ERR_INVALID_ARG;
-        items0 += bp->chunks0[p];
-        total += bp->items_of[p];
+        nseg += bp->plans[p]->rounds.size();
     }
-    // stage the control block in this call's page-locked buffer (its previous copy has completed)
+    // the call's tables in this call's page-locked buffer (its previous copy has completed)
     const int cur = bp->cur;
     bp->cur ^= 1;
     SFFT_CUDA(cudaEventSynchronize(bp->ev[cur]), "staging buffer");
     unsigned char* h = bp->h_stage[cur];
-    const CtlLayout L = ctl_layout(nreq, items0);
+    const CtlLayout L = ctl_layout(nreq, nseg);
     ReqDesc* reqs = reinterpret_cast<ReqDesc*>(h + L.reqs);
     uint32_t* rd0 = reinterpret_cast<uint32_t*>(h + L.rd0);
     uint32_t* rounds = reinterpret_cast<uint32_t*>(h + L.rounds);
-    uint32_t* ctr = reinterpret_cast<uint32_t*>(h + L.ctr);
-    int32_t* flags = reinterpret_cast<int32_t*>(h + L.flags);
-    unsigned long long* items = reinterpret_cast<unsigned long long*>(h + L.items);
-    size_t q = 0;
+    uint32_t* seg = reinterpret_cast<uint32_t*>(h + L.seg);
+    uint32_t* who = reinterpret_cast<uint32_t*>(h + L.who);
     for (uint32_t r = 0; r < nreq; ++r) {
-        const uint32_t p = h_plan_of[r];
         std::memcpy(&reqs[r], &h_reqs[r], sizeof(ReqDesc));
-        rd0[r] = bp->rd0[p];
-        rounds[r] = bp->rounds[p];
-        flags[r] = SFFT_ERR_TIMEOUT;  // overwritten by the request's last round
-        for (uint32_t c = 0; c < bp->chunks0[p]; ++c)
-            items[q++] = (1ull << 63) | ((unsigned long long)r << 24) | c;
+        rd0[r] = bp->rd0[h_plan_of[r]];
+        rounds[r] = (uint32_t)bp->plans[h_plan_of[r]]->rounds.size();
     }
-    ctr[0] = 0;                 // head
-    ctr[1] = (uint32_t)items0;  // tail
-    ctr[2] = 0;                 // error
-    ctr[3] = 0;
+    // the CTAs of each kind of plan, round by round: the first rounds' decodes start the chains
+    uint64_t ctas[2] = {0, 0};
+    size_t seg0[3] = {0, 0, 0};
+    for (int kind = 0; kind < 2; ++kind) {
+        size_t q = seg0[kind];
+        for (uint32_t t = 0; t < bp->max_rounds; ++t)
+            for (uint32_t r = 0; r < nreq; ++r) {
+                const sfft_plan pl = bp->plans[h_plan_of[r]];
+                if (t >= pl->rounds.size() || (pl->rounds[0].large ? 1 : 0) != kind) continue;
+                seg[q] = (uint32_t)ctas[kind];
+                who[q++] = t << 24 | r;
+                ctas[kind] += pl->rdesc[t].gctas;
+            }
+        seg0[kind + 1] = q;
+        if (ctas[kind] > 0x7FFFFFFFull) {
+            set_last_error("batch: more than 2^31 - 1 CTAs");
+            return SFFT_ERR_CUDA;
+        }
+    }
     unsigned char* d = bp->d_ctl;
-    SFFT_CUDA(cudaMemcpyAsync(d, h, L.items, cudaMemcpyHostToDevice, st), "copy control block");
-    SFFT_CUDA(cudaMemcpyAsync(bp->d_items, h + L.items, items0 * 8, cudaMemcpyHostToDevice, st), "copy items");
+    SFFT_CUDA(cudaMemcpyAsync(d, h, L.total, cudaMemcpyHostToDevice, st), "copy tables");
     SFFT_CUDA(cudaEventRecord(bp->ev[cur], st), "staging event");
-    if (total > items0)
-        SFFT_CUDA(cudaMemsetAsync(bp->d_items + items0, 0, (total - items0) * 8, st), "clear items");
-    SFFT_CUDA(cudaMemcpyAsync(d_flag, d + L.flags, (size_t)nreq * 4, cudaMemcpyDeviceToDevice, st), "flags");
-    SFFT_CUDA(cudaMemsetAsync(d_count, 0, (size_t)nreq * 4, st), "counts");
-    SFFT_CUDA(cudaMemsetAsync(bp->d_zcount, 0, (size_t)nreq * 4, st), "clear zhat");
-    SFFT_CUDA(cudaMemsetAsync(bp->d_zflag, 0, (size_t)nreq * 4, st), "clear flags");
-    PersistArgs a;
+    SFFT_CUDA(cudaMemsetAsync(bp->d_zstate, 0, (size_t)bp->max_req * 8, st), "clear zhat");
+    BatchArgs a;
     std::memset(&a, 0, sizeof(a));
     a.rdesc = bp->d_rdesc;
     a.reqs = reinterpret_cast<const ReqDesc*>(d + L.reqs);
     a.req_rd0 = reinterpret_cast<const uint32_t*>(d + L.rd0);
     a.req_rounds = reinterpret_cast<const uint32_t*>(d + L.rounds);
-    a.items = bp->d_items;
-    a.head = reinterpret_cast<uint32_t*>(d + L.ctr);
-    a.tail = a.head + 1;
-    a.error = reinterpret_cast<int32_t*>(a.head + 2);
-    a.total = (uint32_t)total;
     a.part = bp->d_part;
     a.part_stride = bp->part_stride;
     a.counter = bp->d_counter;
     a.zidx = bp->d_zidx;
     a.zval = bp->d_zval;
     a.z_stride = bp->z_stride;
-    a.zcount = bp->d_zcount;
-    a.zflag = bp->d_zflag;
+    a.zcount = bp->d_zstate;
+    a.zflag = reinterpret_cast<int32_t*>(bp->d_zstate + bp->max_req);
     a.fin = bp->d_fin;
     a.fin_stride = bp->fin_stride;
     a.out_idx = d_idx;
@@ -1220,8 +1212,22 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
     a.out_cap = cap;
     a.out_count = d_count;
     a.out_flag = d_flag;
-    const uint32_t ctas = (uint32_t)std::min<size_t>((size_t)bp->ctas, total);
-    SFFT_CUDA(launch_exact_persistent(a, ctas, bp->smem, st, bp->fp64), "persistent launch");
+    const bool both = ctas[0] != 0 && ctas[1] != 0;
+    if (both) {
+        SFFT_CUDA(cudaEventRecord(bp->ev_fork, st), "fork");
+        SFFT_CUDA(cudaStreamWaitEvent(bp->side, bp->ev_fork, 0), "fork");
+    }
+    for (int kind = 1; kind >= 0; --kind) {  // the longer chains first
+        a.seg = reinterpret_cast<const uint32_t*>(d + L.seg) + seg0[kind];
+        a.seg_who = reinterpret_cast<const uint32_t*>(d + L.who) + seg0[kind];
+        a.nseg = (uint32_t)(seg0[kind + 1] - seg0[kind]);
+        SFFT_CUDA(launch_exact_batch(a, (uint32_t)ctas[kind], bp->smem[kind], both && kind ? bp->side : st, bp->fp64, kind != 0),
+                  "mixed batch");
+    }
+    if (both) {
+        SFFT_CUDA(cudaEventRecord(bp->ev_join, bp->side), "join");
+        SFFT_CUDA(cudaStreamWaitEvent(st, bp->ev_join, 0), "join");
+    }
     return SFFT_OK;
 }
 

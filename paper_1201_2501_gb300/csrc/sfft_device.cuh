@@ -297,6 +297,133 @@ __device__ void block_fft_rows(typename Cx<R>::T* a, uint32_t H, uint32_t logB) 
     }
 }
 
+// dst[0..len) <- src[0..len) (another CTA's stores), eight loads in flight per thread
+template <typename C>
+__device__ __forceinline__ void load_rows(C* dst, const C* src, uint32_t len) {
+    constexpr uint32_t N = sizeof(C) == 8 ? 8 : 4;
+    for (uint32_t i0 = threadIdx.x; i0 < len; i0 += kThreads * N) {
+        C v[N];
+#pragma unroll
+        for (uint32_t q = 0; q < N; ++q)
+            if (i0 + q * kThreads < len) v[q] = __ldcg(src + i0 + q * kThreads);
+#pragma unroll
+        for (uint32_t q = 0; q < N; ++q)
+            if (i0 + q * kThreads < len) dst[i0 + q * kThreads] = v[q];
+    }
+}
+
+// Stages st + 1 .. st + N of an FFT of H rows: a thread takes the 2^N elements those stages mix, so that
+// one pass over shared memory and one barrier serve N stages.  Ends with a barrier.
+template <int N>
+__device__ __forceinline__ void fft_pass(float2* a, uint32_t H, uint32_t logB, uint32_t st) {
+    constexpr int M = 1 << N;
+    const uint32_t half = 1u << st, groups = 1u << (logB - N);
+    auto butterflies = [&](float2* row, const float2* w) {
+        float2 v[M];
+#pragma unroll
+        for (int e = 0; e < M; ++e) v[e] = row[(uint32_t)e << st];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int e = 0; e < M; ++e)
+                if (!(e & (1 << k))) {
+                    const float2 bv = cmul_rn(v[e | (1 << k)], w[(1 << k) - 1 + (e & ((1 << k) - 1))]);
+                    const float2 av = v[e];
+                    v[e] = cadd(av, bv);
+                    v[e | (1 << k)] = csub(av, bv);
+                }
+#pragma unroll
+        for (int e = 0; e < M; ++e) row[(uint32_t)e << st] = v[e];
+    };
+    // the twiddles of stage st + 1 + k at position lo: exp(-i pi (lo + f half) / (half 2^k)), f < 2^k
+    auto twiddles = [&](uint32_t lo, float2* w) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int f = 0; f < (1 << k); ++f) {
+                float sn, cs;  // (a quotient by a power of two: the product with its inverse is exact)
+                sincospif(-(float)(lo + ((uint32_t)f << st)) * __int_as_float((int)(127u - st - (uint32_t)k) << 23), &sn, &cs);
+                w[(1 << k) - 1 + f] = mkc(cs, sn);
+            }
+    };
+    float2 w[M - 1];
+    if (groups >= (uint32_t)kThreads) {  // every thread has a position: its twiddles serve all rows
+        for (uint32_t q = threadIdx.x; q < groups; q += kThreads) {
+            const uint32_t lo = q & (half - 1);
+            twiddles(lo, w);
+            for (uint32_t h = 0; h < H; ++h) butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
+        }
+    } else {
+        for (uint32_t i = threadIdx.x; i < H * groups; i += kThreads) {
+            const uint32_t h = i >> (logB - N), q = i & (groups - 1), lo = q & (half - 1);
+            twiddles(lo, w);
+            butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
+        }
+    }
+    __syncthreads();
+}
+
+// The first five stages of rows of 32 or more elements (fft_first_stages, four groups of 32 elements per
+// warp at a time: the shuffles of one group hide those of the others).
+__device__ __forceinline__ void fft_first_five(float2* a, uint32_t total) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    __syncthreads();  // the rows are in place
+    float ts, tc;
+    sincospif(-(float)(lane & 15u) / 16.0f, &ts, &tc);  // exp(-i pi k / 16), k = lane mod 16
+    float2 w[5];
+#pragma unroll
+    for (int st = 1; st <= 5; ++st) {
+        const int pos = (int)(lane & ((1u << (st - 1)) - 1u));
+        w[st - 1] = make_float2(__shfl_sync(0xffffffffu, tc, pos << (5 - st)), __shfl_sync(0xffffffffu, ts, pos << (5 - st)));
+    }
+    constexpr uint32_t G = 4;
+    for (uint32_t g0 = warp * 32u; g0 < total; g0 += (uint32_t)kThreads * G) {
+        float2 v[G];
+#pragma unroll
+        for (uint32_t g = 0; g < G; ++g)
+            v[g] = g0 + g * kThreads < total ? a[g0 + g * kThreads + lane] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int st = 1; st <= 5; ++st) {
+            const int half = 1 << (st - 1);
+            const bool upper = (lane & (uint32_t)half) != 0;
+#pragma unroll
+            for (uint32_t g = 0; g < G; ++g) {
+                const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[g].x, half), __shfl_xor_sync(0xffffffffu, v[g].y, half));
+                const float2 bv = cmul_rn(upper ? v[g] : p, w[st - 1]), av = upper ? p : v[g];
+                v[g] = upper ? make_float2(__fsub_rn(av.x, bv.x), __fsub_rn(av.y, bv.y))
+                             : make_float2(__fadd_rn(av.x, bv.x), __fadd_rn(av.y, bv.y));
+            }
+        }
+#pragma unroll
+        for (uint32_t g = 0; g < G; ++g)
+            if (g0 + g * kThreads < total) a[g0 + g * kThreads + lane] = v[g];
+    }
+    __syncthreads();
+}
+
+// block_fft_rows with the stages past the fifth taken two or three per pass: as many as leave every
+// thread a group of elements (B = 2048, two rows: two barriers instead of six, and a third of the
+// sincospif).  The same butterflies, so the same bits.
+__device__ inline void fft_rows_by_passes(float2* a, uint32_t H, uint32_t logB) {
+    if (logB >= 5)
+        fft_first_five(a, H << logB);
+    else
+        fft_first_stages<float>(a, H, logB);
+    for (uint32_t st = logB < 5 ? logB : 5; st < logB;) {
+        const uint32_t left = logB - st;
+        if (left >= 3 && left != 4 && (H << (logB - 3)) >= (uint32_t)kThreads) {
+            fft_pass<3>(a, H, logB, st);
+            st += 3;
+        } else if (left >= 2 && (H << (logB - 2)) >= (uint32_t)kThreads) {
+            fft_pass<2>(a, H, logB, st);
+            st += 2;
+        } else {
+            fft_pass<1>(a, H, logB, st);
+            st += 1;
+        }
+    }
+}
+
 // Bucket the nz entries of zhat by bin: bin_start[B+1] (exclusive prefix), bin_list (entry ids of
 // each bin, ascending).  ent_bin must be filled.
 __device__ inline void bucket_entries(const uint32_t* ent_bin, uint32_t nz, uint32_t B, uint32_t* bin_cnt,

@@ -13,8 +13,8 @@
 // k_exact_step runs every round of the batch in one launch: the sample positions of all rounds are
 // known up front (sigma, b come from the counter-based draws, never from zhat), so all chunks are
 // gathered at once and only the finishers are ordered, round t's by the arrival of round t - 1's.
-// k_exact_round runs one round (single-hashing entry points and the persistent queue reuse its
-// pieces).  Every reduction has a fixed order and no floating-point atomics exist, so results are
+// k_exact_batch does the same for requests of different plans; k_exact_round runs one round (the
+// single-hashing entry points).  Every reduction has a fixed order and no floating-point atomics exist, so results are
 // bit-reproducible.
 #include <cuda_runtime.h>
 
@@ -36,6 +36,12 @@ __device__ __forceinline__ const float* taps_of<float>(const ExactArgs& a) {
 template <>
 __device__ __forceinline__ const double* taps_of<double>(const ExactArgs& a) {
     return a.taps64;
+}
+
+// samples in flight per thread of gather_owner
+template <typename R>
+__host__ __device__ constexpr uint32_t owner_loads() {
+    return sizeof(R) == sizeof(float) ? 16 : 8;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -82,6 +88,15 @@ size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
     return fin_layout(B, H, zcap, fp64 ? 16 : 8).total;
 }
 size_t exact_gather_smem(uint32_t stage, bool fp64) { return (size_t)stage * (fp64 ? 16 : 8); }
+size_t exact_owner_smem(uint32_t ring, bool fp64) {  // samples and taps of every thread
+    return (size_t)kThreads * (fp64 ? ring * 16 + owner_loads<double>() * 8 : ring * 8 + owner_loads<float>() * 4);
+}
+// samples a thread of gather_owner keeps: those of a batch of loads and of the longest shift
+uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64) {
+    uint32_t r = 1;
+    while (r < (fp64 ? owner_loads<double>() : owner_loads<float>()) + maxshift / B) r <<= 1;
+    return r;
+}
 
 // ------------------------------------------------------------------------------------------------
 // Location and estimation of one bin (NoiselessSparseFFTInner's loop body)
@@ -182,6 +197,13 @@ __device__ void fill_ctx_round(DecodeCtx& d, const ExactArgs& a, uint32_t sigma,
 // ladder keeps a tolerance of at least tau_dec per level and GB300 issues FP64 at 1/64 of FP32, so FP64
 // arithmetic there would cost most of the finisher's time and change no decision outside a
 // measure-zero band at the thresholds.
+// kDirect: the bin's entries are ent_*[x], x < nbin, instead of ent_*[list[x]]; a decode is returned
+// before its window gain is read, with the signed offset o in *oi, and a re-estimate with its x there.
+__device__ __forceinline__ uint32_t index_at(const DecodeCtx& d, uint32_t j, int32_t o) {
+    const uint32_t p = (j * d.Np + (uint32_t)o) & d.nmask;
+    return (d.sigma_inv * ((p + d.sb) & d.nmask)) & d.nmask;
+}
+template <bool kDirect>
 __device__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list, uint32_t nbin,
                                const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
                                double* ginv, bool* above) {
@@ -200,7 +222,7 @@ __device__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u,
         uint32_t matches = 0, who = 0;
         double gw = 1.0;
         for (uint32_t x = 0; x < nbin; ++x) {
-            const uint32_t e = list[x];
+            const uint32_t e = kDirect ? x : list[x];
             const uint32_t i = ent_idx[e];
             const double gain = ent_gain[e];
             if (!(gain >= d.gmin)) continue;
@@ -213,7 +235,7 @@ __device__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u,
             }
             if (ok) {
                 ++matches;
-                who = i;
+                who = kDirect ? x : i;
                 gw = gain;
             }
         }
@@ -240,11 +262,13 @@ __device__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u,
     const uint32_t q = (uint32_t)c;
     const uint32_t dd = (q + d.Np - (d.sb & (d.Np - 1)) + (d.Np >> 1)) & (d.Np - 1);
     const int32_t o = (int32_t)dd - (int32_t)(d.Np >> 1);
-    const uint32_t p = (j * d.Np + (uint32_t)o) & d.nmask;
-    const uint32_t si = (p + d.sb) & d.nmask;
-    const uint32_t i = (d.sigma_inv * si) & d.nmask;
+    const uint32_t i = index_at(d, j, o);
     for (uint32_t l = 0; l < L; ++l)
         if (fabs(cmag<double>(u[l + 1]) - mag0) > d.iso_tol * mag0) return 0;
+    if (kDirect) {
+        *oi = (uint32_t)o;
+        return 1;
+    }
     const double gain = d.wtab[o < 0 ? -o : o];
     if (!(gain >= d.gmin)) return 0;
     *oi = i;
@@ -266,6 +290,7 @@ __device__ __forceinline__ float pow2_f(int e) { return __int_as_float((127 + e)
 
 // Every loop over hashings is unrolled to kMaxHash with compile-time indices, so u[] and the
 // phases stay in registers.
+template <bool kDirect>
 __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, const float2* u, const uint32_t* list,
                                                uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain,
                                                uint32_t* oi, double* gout, double* ginv, bool* above) {
@@ -288,7 +313,7 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
         uint32_t matches = 0, who = 0;
         double gw = 1.0;
         for (uint32_t x = 0; x < nbin; ++x) {
-            const uint32_t e = list[x];
+            const uint32_t e = kDirect ? x : list[x];
             const uint32_t i = ent_idx[e];
             const double gain = ent_gain[e];
             if (!(gain >= d.gmin)) continue;
@@ -304,7 +329,7 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
             }
             if (ok) {
                 ++matches;
-                who = i;
+                who = kDirect ? x : i;
                 gw = gain;
             }
         }
@@ -342,12 +367,14 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
     const uint32_t q = c;
     const uint32_t dd = (q + d.Np - (d.sb & (d.Np - 1)) + (d.Np >> 1)) & (d.Np - 1);
     const int32_t o = (int32_t)dd - (int32_t)(d.Np >> 1);
-    const uint32_t p = (j * d.Np + (uint32_t)o) & d.nmask;
-    const uint32_t si = (p + d.sb) & d.nmask;
-    const uint32_t i = (d.sigma_inv * si) & d.nmask;
+    const uint32_t i = index_at(d, j, o);
 #pragma unroll
     for (int l = 0; l < kMaxHash - 1; ++l)
         if ((uint32_t)l < L && fabsf(hypotf(u[l + 1].x, u[l + 1].y) - mag0) > d.iso_tol_f * mag0) return 0;
+    if (kDirect) {
+        *oi = (uint32_t)o;
+        return 1;
+    }
     const uint32_t oa = (uint32_t)(o < 0 ? -o : o);
     const double gain = d.wtab[oa];
     const double gi = d.winv ? d.winv[oa] : 0.0;  // loaded beside the gain: one memory latency for both
@@ -358,15 +385,17 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
     return 1;
 }
 
+template <bool kDirect = false>
 __device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list,
                                           uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
                                           double* gout, double* ginv, bool* above) {
-    return decode_bin_fp64(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    return decode_bin_fp64<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
 }
+template <bool kDirect = false>
 __device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const float2* u, const uint32_t* list,
                                           uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
                                           double* gout, double* ginv, bool* above) {
-    return decode_bin_fp32(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    return decode_bin_fp32<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
 }
 
 // Bin j's hashings after the subtraction of zhat, for the decisions: u_h = U_h - sum over the bin's
@@ -499,6 +528,92 @@ __device__ void gather_fold(const ExactArgs& a, const void* xrow, uint32_t xmask
     }
 }
 
+// The same fold with a CTA owning kThreads residues of the round (rounds of kOwnerB bins or more): one
+// residue per thread, which folds all its taps, so that no partial fold leaves the CTA (B = 4096 has
+// about 140 chunks, whose partial folds one CTA would have to add).  The ladder's shifts are multiples
+// of B, so the samples of every hashing's tap t, x_{sigma (t - a_h)}, are the thread's own: it keeps the
+// last ones in its column of shared memory and needs no barrier.  Order of the sums: that of the
+// chunks (a residue's taps of a chunk from zero, then the chunks in order), so the bits are the same.
+// Bound by random sectors (16 in flight per thread in FP32, 8 in FP64).
+template <typename R>
+__device__ __forceinline__ void gather_owner(const ExactArgs& a, const void* xrow, uint32_t xmask, uint32_t s,
+                                             uint32_t blk, uint32_t sigma, uint32_t b, unsigned char* smem) {
+    using C = typename Cx<R>::T;
+    constexpr uint32_t kLoads = owner_loads<R>();
+    const uint32_t tid = threadIdx.x, B = a.B, H = a.H, nmask = a.nmask;
+    C* ring = reinterpret_cast<C*>(smem) + tid;  // [a.ring][kThreads], this thread's column
+    R* tap = reinterpret_cast<R*>(reinterpret_cast<C*>(smem) + a.ring * kThreads) + tid;  // [kLoads][kThreads]
+    const uint32_t rmask = a.ring - 1u;
+    const C* __restrict__ x = reinterpret_cast<const C*>(xrow);
+    const R* __restrict__ taps = taps_of<R>(a);
+    const uint32_t first = blk * kThreads, i0 = first + tid;   // first tap -T + i0, then every B-th
+    const uint32_t ntot = (uint32_t)(2 * a.T + 1);
+    const uint32_t mend = first < ntot ? (ntot - first + B - 1) / B : 0;  // taps per thread, rounded up for all
+    const uint32_t mine = i0 < ntot ? (ntot - i0 + B - 1) / B : 0;        // this thread's
+    const uint32_t nt = a.ctaps > B ? a.ctaps / B : 1u;        // a thread's taps per chunk
+    const uint32_t t0 = (uint32_t)(int32_t)(-a.T) + i0;
+    const uint32_t dmax = a.maxshift / B;                      // sample j of the thread: t0 + (j - dmax) B
+    uint32_t dl[kMaxHash];                                     // hashing h's tap m takes sample m + dl[h]
+    C acc[kMaxHash], sum[kMaxHash];
+#pragma unroll
+    for (int h = 0; h < kMaxHash; ++h) {
+        dl[h] = dmax - ((uint32_t)h < H ? a.a[h] / B : 0u);
+        acc[h] = sum[h] = mkc((R)0, (R)0);
+    }
+    uint32_t xi = sigma * (t0 - a.maxshift);
+    const uint32_t xstep = sigma * B, sb = sigma * b, estep = sb * B;
+    uint32_t e = sb * t0;
+    const R inv_half_n = (R)2 / (R)a.n;
+    for (uint32_t j = 0; j < dmax; ++j) {
+        ring[(j & rmask) * kThreads] = ldg_c(x + (xi & xmask));
+        xi += xstep;
+    }
+    for (uint32_t m0 = 0; m0 < mend; m0 += kLoads) {
+        {
+            C v[kLoads];
+            R g[kLoads];  // the taps in the same batch: alone, their latency would be paid tap by tap
+#pragma unroll
+            for (uint32_t u = 0; u < kLoads; ++u)
+                if (m0 + u < mine) {
+                    v[u] = ldg_c(x + ((xi + u * xstep) & xmask));
+                    const int32_t t = (int32_t)(t0 + (m0 + u) * B);
+                    g[u] = taps[t < 0 ? -t : t];
+                }
+            xi += kLoads * xstep;
+#pragma unroll
+            for (uint32_t u = 0; u < kLoads; ++u)
+                if (m0 + u < mine) {
+                    ring[((m0 + u + dmax) & rmask) * kThreads] = v[u];
+                    tap[u * kThreads] = g[u];
+                }
+        }
+        const uint32_t mb = min(m0 + kLoads, mine);
+        // (kept a short loop: unrolled, its code is fetched from L2 once per SM for as long as it runs)
+#pragma unroll 1
+        for (uint32_t m = m0; m < mb; ++m, e += estep) {
+            if (m != 0 && (m & (nt - 1)) == 0) {
+#pragma unroll
+                for (int h = 0; h < kMaxHash; ++h) {
+                    sum[h] = cadd(sum[h], acc[h]);
+                    acc[h] = mkc((R)0, (R)0);
+                }
+            }
+            const int32_t es = (int32_t)((e & nmask) << (__clz((int)nmask) & 31)) >> (__clz((int)nmask) & 31);
+            R sn, cs;
+            sincospi_r((R)es * inv_half_n, &sn, &cs);
+            const R g = tap[(m - m0) * kThreads];
+            const C gt = mkc(g * cs, -g * sn);
+#pragma unroll
+            for (int h = 0; h < kMaxHash; ++h)
+                if ((uint32_t)h < H) acc[h] = cfma(gt, ring[((m + dl[h]) & rmask) * kThreads], acc[h]);
+        }
+    }
+    C* area = reinterpret_cast<C*>(a.part) + (size_t)s * a.part_stride + (__brev(t0 & (B - 1)) >> (32u - a.logB));
+#pragma unroll
+    for (int h = 0; h < kMaxHash; ++h)
+        if ((uint32_t)h < H) area[(size_t)h * B] = cadd(sum[h], acc[h]);  // bit-reversed, as the bin FFT takes it
+}
+
 // Step 2 across chunks: U[h][brev(r)] = sum over chunks c, in order, of part[c][h][r].  Each thread
 // takes E elements of up to CM chunks with all their loads in flight at once (CM >= chunks), else
 // one element at a time in batches of 16.
@@ -563,7 +678,11 @@ __device__ void sum_partials(const C* part, uint32_t chunks, uint32_t H, uint32_
 // the first H B entries of the request's partial-fold area of the round; kFinDecode starts from there.
 enum FinPart { kFinBins = 1, kFinDecode = 2, kFinAll = 3 };
 
-template <typename R>
+__device__ __forceinline__ void fft_rows(float2* U, uint32_t H, uint32_t logB) { fft_rows_by_passes(U, H, logB); }
+__device__ __forceinline__ void fft_rows(double2* U, uint32_t H, uint32_t logB) { block_fft_rows<double>(U, H, logB); }
+
+// LARGE: the bins of a plan decoded by finish_large (many bins: FFT stages by passes)
+template <typename R, bool LARGE = false>
 __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uint32_t b, unsigned char* smem,
                              int part = kFinAll, bool carry = false, bool bins_here = false,
                              const uint32_t* next_ctr = nullptr) {
@@ -596,8 +715,14 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
 
     // steps 2 (across chunks) and 3: partial folds summed in chunk order, bit-reversed, FFT
     if (part & kFinBins) {
-        sum_partials(area, a.chunks, H, a.logB, U);
-        block_fft_rows<R>(U, H, a.logB);  // starts and ends with a barrier
+        if (LARGE && a.owner)
+            load_rows(U, area, H * B);  // whole folds, bit-reversed
+        else
+            sum_partials(area, a.chunks, H, a.logB, U);
+        if (LARGE)
+            fft_rows(U, H, a.logB);
+        else
+            block_fft_rows<R>(U, H, a.logB);  // starts and ends with a barrier
         if (!(part & kFinDecode)) {  // every partial fold has been read: the area takes the bins
             for (uint32_t i = tid; i < H * B; i += kThreads) area[i] = U[i];
             return false;
@@ -895,6 +1020,496 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
     return next_ready;
 }
 
+// ------------------------------------------------------------------------------------------------
+// The decode of a round of a plan whose zhat may hold more than kCarry entries
+// ------------------------------------------------------------------------------------------------
+// The same steps and the same order of every sum as finish_round's decode, with arrays sized by what
+// zhat holds and by what was decoded instead of by their capacities, so that they stay on chip (device
+// memory only when they do not fit a.large_smem bytes): the entries' terms lie by bin (stable counting
+// split with per-warp counters), the bins are read straight from the round's area, and the candidates
+// are sorted by a bitonic network.  Bound by latency (about 40 barriers, 80 with a sort).  Measured with
+// gather_owner at n = 2^24, k = 1000, batch 12: 592 us a call, was 1005 (arrays sized by capacity in
+// device memory, long bin lists sorted by insertion, one CTA per SM, 140 partial folds per round).
+struct LargeLayout {
+    size_t e_idx, pre, key, cval, start, slot, s_idx, s_gain, s_t0, s_tf, cnt, out_idx, out_val, keep, scan, total;
+};
+__host__ __device__ inline uint32_t split_segments(uint32_t B) { return B <= 1024 ? 8u : 8192u / B; }
+// nz entries, up to B candidates, tot merged entries; the merge's arrays take the place of the entries'
+__host__ __device__ inline LargeLayout large_layout(uint32_t B, uint32_t H, uint32_t nz, uint32_t tot, bool fp64,
+                                                    bool val_on_chip) {
+    LargeLayout L;
+    size_t off = 0;
+    const uint32_t P = B < 1024 ? 1024 : B;  // the sort's keys, padded
+    L.scan = fin_take(&off, (size_t)(kThreads + 8) * 4);
+    L.e_idx = fin_take(&off, (size_t)nz * 4);
+    // the decoded bins share their place with the split's counters
+    const size_t cnt = nz ? (size_t)split_segments(B) * B * 2 : 0, pre = (size_t)B * 8;
+    L.pre = L.cnt = fin_take(&off, pre > cnt ? pre : cnt);
+    L.key = fin_take(&off, (size_t)P * 8);
+    L.cval = fin_take(&off, val_on_chip ? (size_t)B * 16 : 0);
+    const size_t shared = off;
+    L.start = fin_take(&off, (size_t)(B + 1) * 4);
+    L.slot = fin_take(&off, (size_t)nz * 4);
+    L.s_idx = fin_take(&off, (size_t)nz * 4);
+    L.s_gain = fin_take(&off, (size_t)nz * 8);
+    L.s_t0 = fin_take(&off, (size_t)nz * 16);
+    L.s_tf = fin_take(&off, (size_t)nz * H * (fp64 ? 16 : 8));
+    const size_t end = off;
+    off = shared;
+    L.out_idx = fin_take(&off, (size_t)tot * 4);
+    L.out_val = fin_take(&off, (size_t)tot * 16);
+    L.keep = fin_take(&off, (size_t)(tot + 1) * 4);
+    L.total = off > end ? off : end;
+    return L;
+}
+// device-memory slice of a request: the candidates' values, then everything at its largest
+size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
+    return (size_t)B * 16 + large_layout(B, H, zcap, zcap + B, fp64, false).total;
+}
+
+// place[e] <- the rank of entry e in (bin, index) order, from place[e] = its bin; start[j] <- the first
+// rank of bin j (start[B] = nz).  cnt: split_segments(B) x B counters.
+__device__ void split_by_bin(uint32_t* place, uint32_t nz, uint32_t B, uint16_t* cnt, uint32_t* start, uint32_t* scan) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nseg = split_segments(B);
+    for (uint32_t i = tid; i < nseg * B / 2; i += kThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0;
+    __syncthreads();
+    const uint32_t per = ((nz + nseg - 1) / nseg + 31u) & ~31u, beg = warp * per, end = min(nz, beg + per);
+    uint16_t* mine = cnt + (size_t)warp * B;
+    if (warp < nseg)
+        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
+            const bool in = e0 + lane < end;
+            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
+            const unsigned same = __match_any_sync(0xffffffffu, b);
+            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(mine[b] + __popc((int)same));
+            __syncwarp();
+        }
+    __syncthreads();
+    for (uint32_t j = tid; j < B; j += kThreads) {
+        uint32_t run = 0;
+        for (uint32_t w = 0; w < nseg; ++w) {
+            const uint32_t c = cnt[w * B + j];
+            cnt[w * B + j] = (uint16_t)run;
+            run += c;
+        }
+        start[j] = run;
+    }
+    __syncthreads();
+    block_exclusive_scan(start, B, scan);  // ends with a barrier
+    if (tid == 0) start[B] = nz;
+    if (warp < nseg)
+        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
+            const bool in = e0 + lane < end;
+            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
+            const unsigned same = __match_any_sync(0xffffffffu, b);
+            uint32_t base = 0;
+            if (in) {
+                base = mine[b];
+                place[e0 + lane] = start[b] + base + (uint32_t)__popc((int)(same & ((1u << lane) - 1u)));
+            }
+            __syncwarp();
+            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(base + __popc((int)same));
+            __syncwarp();
+        }
+    __syncthreads();
+}
+
+// whether decode_bin goes beyond its first test on a bin whose subtracted u_0 is u
+__device__ __forceinline__ bool worth_decoding(const DecodeCtx& d, float2 u, bool entries) {
+    const float m = hypotf(u.x, u.y);
+    return m > d.thr_f || (entries && m > d.ref_lo_f && m <= d.ref_hi_f);
+}
+__device__ __forceinline__ bool worth_decoding(const DecodeCtx& d, double2 u, bool entries) {
+    const double m = cmag<double>(u);
+    return m > d.thr || (entries && m > d.ref_lo * d.thr && m <= d.ref_hi * d.thr);
+}
+
+// Ascending sort of the nw distinct keys (key holds max(1024, pow2(nw)) words): up to 1024 as four per
+// thread, exchanged in registers (strides 1, 2), by shuffles (4 to 64) and through shared memory (128 on:
+// 6 exchanges), more by the network in memory.
+__device__ __forceinline__ void sort_keys(unsigned long long* key, uint32_t nw) {
+    const uint32_t tid = threadIdx.x;
+    uint32_t P = 2;
+    while (P < nw) P <<= 1;
+    if (P <= 4 * (uint32_t)kThreads) {
+        unsigned long long k[4];
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) k[q] = 4 * tid + q < nw ? key[4 * tid + q] : ~0ull;
+        for (uint32_t size = 2; size <= P; size <<= 1) {
+            for (uint32_t stride = size >> 1; stride > 2; stride >>= 1) {
+                if (stride >= 128) {
+                    __syncthreads();
+#pragma unroll
+                    for (uint32_t q = 0; q < 4; ++q) key[4 * tid + q] = k[q];
+                    __syncthreads();
+                }
+#pragma unroll
+                for (uint32_t q = 0; q < 4; ++q) {
+                    const uint32_t i = 4 * tid + q;
+                    const unsigned long long o =
+                        stride >= 128 ? key[i ^ stride] : __shfl_xor_sync(0xffffffffu, k[q], (int)(stride >> 2));
+                    if ((((i & stride) == 0) == ((i & size) == 0)) == (o < k[q])) k[q] = o;
+                }
+            }
+#pragma unroll
+            for (uint32_t stride = 2; stride > 0; stride >>= 1)
+                if (stride < size)
+#pragma unroll
+                    for (uint32_t q = 0; q < 4; ++q)
+                        if (!(q & stride)) {
+                            const unsigned long long x = k[q], y = k[q | stride];
+                            const bool up = ((4 * tid + q) & size) == 0;
+                            if (up == (x > y)) {
+                                k[q] = y;
+                                k[q | stride] = x;
+                            }
+                        }
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (4 * tid + q < nw) key[4 * tid + q] = k[q];
+        __syncthreads();
+        return;
+    }
+    for (uint32_t p = nw + tid; p < P; p += kThreads) key[p] = ~0ull;
+    __syncthreads();
+    for (uint32_t size = 2; size <= P; size <<= 1)
+        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+            for (uint32_t i = tid; i < P / 2; i += kThreads) {
+                const uint32_t lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+                const unsigned long long x = key[lo], y = key[hi];
+                if ((lo & size) == 0 ? x > y : x < y) {
+                    key[lo] = y;
+                    key[hi] = x;
+                }
+            }
+            __syncthreads();
+        }
+}
+
+template <typename R>
+__device__ __forceinline__ bool finish_large(const ExactArgs& a, uint32_t s, uint32_t sigma, uint32_t b,
+                                          unsigned char* smem, const uint32_t* next_ctr) {
+    using C = typename Cx<R>::T;
+    constexpr bool f32 = sizeof(C) == sizeof(float2);
+    const uint32_t tid = threadIdx.x, B = a.B, H = a.H;
+    __shared__ uint32_t s_nw, s_pre, s_list, s_above, s_kept, s_next_ready;
+    __shared__ DecodeCtx d;
+    C* area = reinterpret_cast<C*>(a.part) + (size_t)s * a.part_stride;  // the round's bins
+    __syncthreads();  // the bins, when this CTA stored them
+    if (tid == kThreads - 1) s_next_ready = next_ctr != nullptr && acquire_is(next_ctr, 1u) ? 1u : 0u;
+    if (tid == kThreads - 2) fill_ctx_round(d, a, sigma, b);
+    if (tid == 0) {
+        s_nw = 0;
+        s_pre = 0;
+        s_list = 0;
+        s_above = 0;
+        s_kept = 0;
+    }
+    // zhat is read through L2: in the one-launch path another CTA of this launch may have written it
+    uint32_t* zi = a.zidx + (size_t)s * a.zcap;
+    double2* zv = a.zval + (size_t)s * a.zcap;
+    const uint32_t nz = min(__ldcg(a.zcount + s), a.zcap);
+    unsigned char* slice = a.fin_scratch + (size_t)s * a.fin_stride;
+    const bool val_on_chip = B <= 512;
+    LargeLayout Ly = large_layout(B, H, nz, 0, !f32, val_on_chip);
+    unsigned char* mem = smem;
+    if (Ly.total > a.large_smem) {
+        mem = slice + (size_t)B * 16;
+        Ly = large_layout(B, H, a.zcap, a.zcap + B, !f32, false);
+    }
+    double2* cval = mem == smem && val_on_chip ? reinterpret_cast<double2*>(smem + Ly.cval) : reinterpret_cast<double2*>(slice);
+    uint32_t* scan = reinterpret_cast<uint32_t*>(mem + Ly.scan);
+    uint32_t* e_idx = reinterpret_cast<uint32_t*>(mem + Ly.e_idx);
+    uint2* pre = reinterpret_cast<uint2*>(mem + Ly.pre);
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(mem + Ly.key);
+    uint32_t* start = reinterpret_cast<uint32_t*>(mem + Ly.start);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(mem + Ly.slot);
+    uint32_t* s_idx = reinterpret_cast<uint32_t*>(mem + Ly.s_idx);
+    double* s_gain = reinterpret_cast<double*>(mem + Ly.s_gain);
+    double2* s_t0 = reinterpret_cast<double2*>(mem + Ly.s_t0);
+    C* s_tf = reinterpret_cast<C*>(mem + Ly.s_tf);
+    // the entries by bin
+    const uint32_t Np = (uint32_t)(a.n >> a.logB), logNp = ilog2_u32(Np);
+    // (the first four per thread have their gains and values requested here, to arrive during the split)
+    double gv[4];
+    double2 vv[4];
+    for (uint32_t e0 = tid; e0 < nz; e0 += 4 * kThreads) {
+        uint32_t iv[4];
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (e0 + q * kThreads < nz) {
+                iv[q] = __ldcg(zi + e0 + q * kThreads);
+                if (e0 == tid) vv[q] = __ldcg(zv + e0 + q * kThreads);
+            }
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (e0 + q * kThreads < nz) {
+                e_idx[e0 + q * kThreads] = iv[q];
+                uint32_t jb;
+                const int32_t o = offset_of((sigma * (iv[q] - b)) & a.nmask, Np, logNp, a.nmask, &jb);
+                slot[e0 + q * kThreads] = jb;
+                if (e0 == tid) gv[q] = a.wtab[o < 0 ? -o : o];
+            }
+    }
+    __syncthreads();
+    const bool next_ready = s_next_ready != 0;
+    if (nz != 0)
+        split_by_bin(slot, nz, B, reinterpret_cast<uint16_t*>(mem + Ly.cnt), start, scan);
+    else
+        for (uint32_t j = tid; j <= B; j += kThreads) start[j] = 0;
+    // step 4 terms: W(-o(i)) zhat_i w^{a_h sigma i}, as finish_round forms them
+    for (uint32_t e0 = tid; e0 < nz; e0 += 4 * kThreads) {
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (e0 != tid && e0 + q * kThreads < nz) {
+                uint32_t jb;
+                const int32_t o = offset_of((sigma * (e_idx[e0 + q * kThreads] - b)) & a.nmask, Np, logNp, a.nmask, &jb);
+                gv[q] = a.wtab[o < 0 ? -o : o];
+                vv[q] = __ldcg(zv + e0 + q * kThreads);
+            }
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) {
+            if (e0 + q * kThreads >= nz) break;
+            const uint32_t i = e_idx[e0 + q * kThreads], at = slot[e0 + q * kThreads];
+            s_idx[at] = i;
+            s_gain[at] = gv[q];
+            const double2 gz = make_double2(gv[q] * vv[q].x, gv[q] * vv[q].y);
+            s_t0[at] = gz;  // hashing 0 has offset 0: w^0 = 1
+            const float2 g = make_float2((float)gz.x, (float)gz.y);
+            const float two_over_n = 2.0f * d.inv_n_f;
+            for (uint32_t h = 0; h < H; ++h) {
+                const uint32_t ex = (a.a[h] * sigma * i) & a.nmask;
+                C w;
+                if (f32) {
+                    const int32_t es = ex > (a.nmask >> 1) ? (int32_t)((int64_t)ex - (int64_t)a.n) : (int32_t)ex;
+                    float sn, cs;
+                    sincospif((float)es * two_over_n, &sn, &cs);
+                    w.x = g.x * cs + g.y * sn;
+                    w.y = g.y * cs - g.x * sn;
+                } else {
+                    double2 r = gz;
+                    if (ex != 0) {
+                        const double2 tw = root_pow<R>(ex, a.nmask);
+                        r = make_double2(gz.x * tw.x - gz.y * tw.y, gz.x * tw.y + gz.y * tw.x);
+                    }
+                    w.x = r.x;
+                    w.y = r.y;
+                }
+                s_tf[at * H + h] = w;
+            }
+        }
+    }
+    __syncthreads();
+    // the bins that may hold something: above thr (J), or with entries and a residual in the window of a
+    // re-estimation.  Their list takes the place of the keys; only they are decoded.
+    uint32_t* jl = reinterpret_cast<uint32_t*>(key);
+    for (uint32_t b0 = 0; b0 < B; b0 += 4 * kThreads) {  // the same trips for every lane (full-warp ballots)
+        const uint32_t j0 = b0 + tid;
+        C uv[4];
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (j0 + q * kThreads < B) uv[q] = __ldcg(area + j0 + q * kThreads);
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q) {
+            const uint32_t j = j0 + q * kThreads;
+            bool want = false;
+            if (j < B) {
+                C u = uv[q];
+                const uint32_t x0 = start[j], x1 = start[j + 1];
+                for (uint32_t x = x0; x < x1; ++x) {
+                    u.x -= s_tf[x * H].x;
+                    u.y -= s_tf[x * H].y;
+                }
+                want = worth_decoding(d, u, x1 != x0);
+            }
+            const unsigned mw = __ballot_sync(0xffffffffu, want);
+            uint32_t base = 0;
+            if ((tid & 31u) == 0 && mw) base = atomicAdd(&s_list, (uint32_t)__popc((int)mw));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (want) jl[base + (uint32_t)__popc((int)(mw & ((1u << (tid & 31u)) - 1u)))] = j;
+        }
+    }
+    __syncthreads();
+    // step 4 and the decode, one listed bin per thread
+    const uint32_t nlist = s_list;
+    for (uint32_t c = tid; c < nlist; c += kThreads) {
+        const uint32_t j = jl[c], x0 = start[j], nbin = start[j + 1] - x0;
+        C u[kMaxHash];
+#pragma unroll
+        for (int h = 0; h < kMaxHash; ++h) {
+            u[h] = mkc((R)0, (R)0);
+            if ((uint32_t)h < H) u[h] = __ldcg(area + (size_t)h * B + j);
+        }
+        for (uint32_t x = x0; x < x0 + nbin; ++x) {
+#pragma unroll
+            for (int h = 0; h < kMaxHash; ++h)
+                if ((uint32_t)h < H) {
+                    u[h].x -= s_tf[x * H + h].x;
+                    u[h].y -= s_tf[x * H + h].y;
+                }
+        }
+        // a decoded bin, its gain still to be read: its offset, or the entry re-estimated
+        uint32_t where = 0;
+        bool above;
+        double g0, g1;
+        const int kind = decode_bin<true>(d, j, u, nullptr, nbin, s_idx + x0, s_gain + x0, &where, &g0, &g1, &above);
+        const unsigned m = __activemask();
+        const unsigned ma = __ballot_sync(m, above), mw = __ballot_sync(m, kind != 0);
+        const uint32_t lane = tid & 31u, leader = (uint32_t)__ffs((int)m) - 1u;
+        uint32_t base = 0;
+        if (lane == leader) {
+            if (ma) atomicAdd(&s_above, (uint32_t)__popc((int)ma));
+            if (mw) base = atomicAdd(&s_pre, (uint32_t)__popc((int)mw));
+        }
+        base = __shfl_sync(m, base, (int)leader);
+        if (kind != 0)
+            pre[base + (uint32_t)__popc((int)(mw & ((1u << lane) - 1u)))] =
+                make_uint2(kind == 1 ? where : x0 + where, j | (kind == 2 ? 0x80000000u : 0u));
+    }
+    __syncthreads();
+    // the decoded bins' gains and values: u_0 in FP64, in the entries' order, times 1 / W(-o) or over W(-o)
+    const uint32_t npre = s_pre;
+    for (uint32_t c = tid; c < npre; c += kThreads) {
+        const uint2 pr = pre[c];
+        const uint32_t j = pr.y & 0x7FFFFFFFu;
+        const bool known = (pr.y >> 31) != 0;
+        const int32_t o = (int32_t)pr.x;
+        const uint32_t oa = (uint32_t)(o < 0 ? -o : o);
+        const C v = __ldcg(area + j);
+        const double gain = known ? s_gain[pr.x] : a.wtab[oa];
+        const double ginv = f32 && !known && d.winv ? d.winv[oa] : 0.0;
+        const bool kept = known || gain >= d.gmin;
+        const unsigned m = __activemask();
+        const unsigned mk = __ballot_sync(m, kept && !known), mw = __ballot_sync(m, kept);
+        const uint32_t lane = tid & 31u, leader = (uint32_t)__ffs((int)m) - 1u;
+        uint32_t base = 0;
+        if (lane == leader) {
+            if (mk) atomicAdd(&s_kept, (uint32_t)__popc((int)mk));
+            if (mw) base = atomicAdd(&s_nw, (uint32_t)__popc((int)mw));
+        }
+        base = __shfl_sync(m, base, (int)leader);
+        if (kept) {
+            const uint32_t at = base + (uint32_t)__popc((int)(mw & ((1u << lane) - 1u)));
+            double2 u0 = make_double2((double)v.x, (double)v.y);
+            for (uint32_t x = start[j]; x < start[j + 1]; ++x) {
+                u0.x -= s_t0[x].x;
+                u0.y -= s_t0[x].y;
+            }
+            const uint32_t oi = known ? s_idx[pr.x] : index_at(d, j, o);
+            key[at] = ((unsigned long long)oi << 32) | at;
+            cval[at] = f32 && !known && d.winv ? make_double2(u0.x * ginv, u0.y * ginv)
+                                               : make_double2(u0.x / gain, u0.y / gain);
+        }
+    }
+    __syncthreads();
+    const uint32_t nw = s_nw;
+    const bool last = a.last_round != 0;
+    const uint32_t tot = nz + nw;
+    if (mem == smem) {  // the merge's arrays, in place of the entries' where they fit
+        Ly = large_layout(B, H, nz, tot, !f32, val_on_chip);
+        if (Ly.total > a.large_smem) {
+            mem = slice + (size_t)B * 16;
+            Ly = large_layout(B, H, a.zcap, a.zcap + B, !f32, false);
+        }
+    }
+    uint32_t* out_idx = reinterpret_cast<uint32_t*>(mem + Ly.out_idx);
+    double2* out_val = reinterpret_cast<double2*>(mem + Ly.out_val);
+    uint32_t* keep = reinterpret_cast<uint32_t*>(mem + Ly.keep);
+    uint32_t newcount = nz;
+    if (nw == 0) {
+        // nothing decoded: zhat stays as it is
+        if (last)
+            for (uint32_t e = tid; e < nz && e < a.out_cap; e += kThreads) {
+                a.out_idx[(size_t)s * a.out_cap + e] = e_idx[e];
+                a.out_val[(size_t)s * a.out_cap + e] = __ldcg(zv + e);
+            }
+    } else {
+        // the candidates by index (distinct: a decode lies in its own bin)
+        if (nw <= (uint32_t)kThreads) {
+            unsigned long long k = 0;
+            uint32_t r = 0;
+            if (tid < nw) {
+                k = key[tid];
+                for (uint32_t q = 0; q < nw; ++q) r += key[q] < k ? 1u : 0u;
+            }
+            __syncthreads();
+            if (tid < nw) key[r] = k;
+            __syncthreads();
+        } else {
+            sort_keys(key, nw);
+        }
+        // merge what into zhat (zhat first on equal indices), then drop entries below prune * thr
+        for (uint32_t e = tid; e < nz; e += kThreads) {
+            const unsigned long long k = (unsigned long long)e_idx[e] << 32;
+            uint32_t lo = 0, hi = nw;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (key[mid] < k) lo = mid + 1; else hi = mid;
+            }
+            out_idx[e + lo] = e_idx[e];
+            out_val[e + lo] = __ldcg(zv + e);
+        }
+        for (uint32_t c = tid; c < nw; c += kThreads) {
+            const uint32_t idx = (uint32_t)(key[c] >> 32);
+            const uint32_t pos = c + upper_bound_u32(e_idx, nz, idx);
+            out_idx[pos] = idx;
+            out_val[pos] = cval[(uint32_t)key[c]];
+        }
+        __syncthreads();
+        for (uint32_t p = tid; p < tot; p += kThreads) {
+            uint32_t kp = 0;
+            const uint32_t idx = out_idx[p];
+            if (p == 0 || out_idx[p - 1] != idx) {
+                double2 v = out_val[p];
+                if (p + 1 < tot && out_idx[p + 1] == idx) {
+                    v.x += out_val[p + 1].x;
+                    v.y += out_val[p + 1].y;
+                    out_val[p] = v;  // the duplicate at p + 1 is never a head and is not written
+                }
+                if (f32)
+                    kp = hypotf((float)v.x, (float)v.y) < a.drop_f ? 0u : 1u;
+                else
+                    kp = cmag<R>(v) < a.prune * a.thr ? 0u : 1u;
+            }
+            keep[p] = kp;
+        }
+        __syncthreads();
+        newcount = block_exclusive_scan(keep, tot, scan);
+        for (uint32_t p = tid; p < tot; p += kThreads) {
+            const uint32_t pos = keep[p];
+            const uint32_t nxt = p + 1 < tot ? keep[p + 1] : newcount;
+            if (nxt == pos) continue;
+            const uint32_t idx = out_idx[p];
+            const double2 v = out_val[p];
+            if (pos < a.zcap) {
+                zi[pos] = idx;
+                zv[pos] = v;
+            }
+            if (last && pos < a.out_cap) {
+                a.out_idx[(size_t)s * a.out_cap + pos] = idx;
+                a.out_val[(size_t)s * a.out_cap + pos] = v;
+            }
+        }
+    }
+    if (tid == 0) {
+        const bool overflow = newcount > a.zcap;
+        const uint32_t count = overflow ? a.zcap : newcount;
+        if (overflow) a.zflag[s] = 1;
+        if (nw != 0) a.zcount[s] = count;
+        if (last) {
+            a.out_count[s] = count < a.out_cap ? count : a.out_cap;
+            int32_t flag = SFFT_OK;
+            if (__ldcg(a.zflag + s) || count > a.out_cap)
+                flag = SFFT_ERR_CAPACITY;
+            else if (s_above > s_kept)
+                flag = SFFT_ERR_NOT_CONVERGED;
+            a.out_flag[s] = flag;
+        }
+    }
+    return next_ready;
+}
+
 #ifndef SFFT_ROUND_MIN_BLOCKS
 #define SFFT_ROUND_MIN_BLOCKS 2  // resident CTAs per SM the register budget is sized for
 #endif
@@ -927,17 +1542,17 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_round
 // counter2 (an acquire load that overlaps its own loads): when those bins have arrived, this chain is
 // the last party of that round and goes on without an arrival of its own.  (seed, id) name the
 // request's draws.
-template <typename R, int NR>
+template <typename R, int NR, bool LARGE>
 __device__ __forceinline__ void decode_chain(const StepParams<NR>& sp, uint32_t t, const ExactArgs* a, uint32_t s,
                                              uint64_t seed, uint32_t id, uint32_t sigma, uint32_t b,
                                              unsigned char* smem) {
     if (t > 0 && arrive_pair(a->counter2 + s) == 0) return;
-    bool bins_here = a->fin_scratch == nullptr;  // the bins just formed are in this CTA's shared memory
+    bool bins_here = true;  // the bins just formed are in this CTA's shared memory
     for (bool carried = false;; carried = true) {
         const uint32_t* next_ctr = t + 1 < sp.R ? sp.r[t + 1].counter2 + s : nullptr;
         const bool next_ready =
-            finish_round<R>(*a, s, sigma, b, a->fin_scratch ? a->fin_scratch + (size_t)s * a->fin_stride : smem,
-                            kFinDecode, carried, bins_here, next_ctr);
+            LARGE ? finish_large<R>(*a, s, sigma, b, smem, next_ctr)
+                  : finish_round<R>(*a, s, sigma, b, smem, kFinDecode, carried, bins_here, next_ctr);
         if (threadIdx.x == 0) a->counter2[s] = 0;  // both arrivals of round t have happened (or none, t = 0)
         if (t + 1 >= sp.R) break;
         a = &sp.r[++t];
@@ -952,7 +1567,7 @@ __device__ __forceinline__ void decode_chain(const StepParams<NR>& sp, uint32_t 
     }
 }
 
-template <typename R, int NR>
+template <typename R, int NR, bool LARGE>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_step(const __grid_constant__ StepParams<NR> sp) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t tid = threadIdx.x;
@@ -960,17 +1575,20 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_step(
     while (t + 1 < sp.R && blockIdx.x >= sp.seg[t + 1]) ++t;
     const ExactArgs* a = &sp.r[t];
     const uint32_t local = blockIdx.x - sp.seg[t];
-    const uint32_t c = local % a->chunks;
-    const uint32_t s = a->req_base + local / a->chunks;
+    const uint32_t c = local % a->gctas;
+    const uint32_t s = a->req_base + local / a->gctas;
     const ReqView rq = req_view(a->reqs, a->x, a->n * sizeof(typename Cx<R>::T), a->seed, s, a->nmask);
     uint32_t sigma, b;
     exact_hash(rq.seed, rq.id, t, a->nmask, &sigma, &b);
-    gather_fold<R>(*a, rq.x, rq.xmask, s, c, sigma, b, smem);
-    if (arrive(a->counter + s, a->chunks) == 0) return;
+    if (LARGE && a->owner)
+        gather_owner<R>(*a, rq.x, rq.xmask, s, c, sigma, b, smem);
+    else
+        gather_fold<R>(*a, rq.x, rq.xmask, s, c, sigma, b, smem);
+    if (arrive(a->counter + s, a->gctas) == 0) return;
     // the round's bins, in this CTA's shared memory (the gather's staging area holds H B values)
-    finish_round<R>(*a, s, sigma, b, smem, kFinBins);
+    finish_round<R, LARGE>(*a, s, sigma, b, smem, kFinBins);
     if (tid == 0) a->counter[s] = 0;  // every chunk of round t has arrived
-    decode_chain<R, NR>(sp, t, a, s, rq.seed, rq.id, sigma, b, smem);
+    decode_chain<R, NR, LARGE>(sp, t, a, s, rq.seed, rq.id, sigma, b, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1072,7 +1690,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_bins(c
 
 // The decodes: one CTA per channel slot runs them in round order (zhat of round t feeds round t + 1).
 // If the gather flagged a copy that never landed, every slot reports SFFT_ERR_TIMEOUT instead.
-template <int NR>
+template <int NR, bool LARGE>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode(const __grid_constant__ StepParams<NR> sp,
                                                                                 uint64_t seed, uint32_t id,
                                                                                 const uint32_t* error) {
@@ -1090,135 +1708,119 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode
         const ExactArgs& a = sp.r[t];
         uint32_t sigma, b;
         exact_hash(seed, id, t, a.nmask, &sigma, &b);
-        finish_round<float>(a, s, sigma, b, a.fin_scratch ? a.fin_scratch + (size_t)s * a.fin_stride : smem,
-                            kFinDecode, t > 0);
+        if (LARGE)
+            finish_large<float>(a, s, sigma, b, smem, nullptr);
+        else
+            finish_round<float>(a, s, sigma, b, smem, kFinDecode, t > 0);
         __syncthreads();  // zhat of round t is read by round t + 1 (same CTA)
     }
 }
 
 // ------------------------------------------------------------------------------------------------
-// Persistent path: one launch, a device queue of (request, round, chunk) items
+// Mixed batches: requests of different plans in one launch
 // ------------------------------------------------------------------------------------------------
-constexpr unsigned long long kItemValid = 1ull << 63;
-constexpr uint32_t kSpinLimit = 1u << 23;  // x ~128 ns: a wait gives up after about a second
-
-__device__ __forceinline__ unsigned long long pack_item(uint32_t r, uint32_t t, uint32_t c) {
-    return kItemValid | ((unsigned long long)r << 24) | ((unsigned long long)t << 16) | c;
-}
-__device__ __forceinline__ unsigned long long load_acquire(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void store_release(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-#ifndef SFFT_PERSIST_MIN_BLOCKS
-#define SFFT_PERSIST_MIN_BLOCKS 2  // resident CTAs per SM the register budget is sized for
-#endif
-
-template <typename R>
-__global__ void __launch_bounds__(kThreads, SFFT_PERSIST_MIN_BLOCKS) k_exact_persistent(const PersistArgs pa) {
+// The scheme of k_exact_step over requests that each have their own plan: the gathers of every round of
+// every request are in the grid from the start, round by round (segment i = the CTAs of one (round,
+// request)), the decodes are chained by arrival counters and nothing waits.  A round's argument block
+// comes from device memory, its per-request fields are pointed at the request's own workspace.  Against
+// the device queue it replaces, where a request's next round was gathered only after the last one's
+// decode: 452 us, was 880 (96 requests of six plans, n = 2^16 .. 2^22).
+template <typename R, bool LARGE>
+__global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_batch(const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) ExactArgs sa;
-    __shared__ unsigned long long s_item;
     const uint32_t tid = threadIdx.x;
-    for (;;) {
-        // take the next item and wait (bounded) until it is published
-        if (tid == 0) {
-            const uint32_t slot = atomicAdd(pa.head, 1u);
-            unsigned long long it = 0;
-            if (slot < pa.total) {
-                for (uint32_t spin = 0;; ++spin) {
-                    it = load_acquire(pa.items + slot);
-                    if (it & kItemValid) break;
-                    if (spin >= kSpinLimit) {
-                        atomicExch(pa.error, 1);
-                        it = 0;
-                        break;
-                    }
-                    __nanosleep(128);
-                }
-            }
-            s_item = it;
-        }
-        __syncthreads();
-        const unsigned long long it = s_item;
-        if (!it) return;
-        const uint32_t r = (uint32_t)((it >> 24) & 0xFFFFFFFFull), t = (uint32_t)((it >> 16) & 0xFFu),
-                       c = (uint32_t)(it & 0xFFFFu);
-        // the (plan, round) argument block, then the request's own workspace as slot 0
-        {
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(pa.rdesc + pa.req_rd0[r] + t);
-            uint32_t* dst = reinterpret_cast<uint32_t*>(&sa);
-            for (uint32_t w = tid; w < sizeof(ExactArgs) / 4; w += kThreads) dst[w] = src[w];
-        }
+    // the segment of this CTA: the last whose first CTA is not above it, kThreads probes at a time
+    uint32_t lo = 0, len = ba.nseg;
+    while (len > 1) {
+        const uint32_t stride = (len + kThreads - 1) / kThreads, i = tid * stride;
+        const uint32_t n = (uint32_t)__syncthreads_count(i < len && ba.seg[lo + i] <= blockIdx.x);
+        lo += (n - 1) * stride;
+        len = min(stride, len - (n - 1) * stride);
+    }
+    const uint32_t c = blockIdx.x - ba.seg[lo], who = ba.seg_who[lo];
+    const uint32_t r = who & 0xFFFFFFu;
+    uint32_t t = who >> 24;
+    uint32_t* const counters = ba.counter + (size_t)r * 2 * kMaxRounds;  // per round; then the second ones
+    const uint32_t rounds = ba.req_rounds[r];
+    auto load_round = [&](uint32_t round) {
+        __syncthreads();  // every reader of the block is done
+        const uint32_t* src = reinterpret_cast<const uint32_t*>(ba.rdesc + ba.req_rd0[r] + round);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(&sa);
+        for (uint32_t w = tid; w < sizeof(ExactArgs) / 4; w += kThreads) dst[w] = src[w];
         __syncthreads();
         if (tid == 0) {
-            sa.reqs = pa.reqs + r;
+            sa.reqs = ba.reqs + r;
             sa.req_base = 0;
-            sa.part = pa.part + (size_t)r * pa.part_stride;
+            sa.part = ba.part + (size_t)r * ba.part_stride + sa.part_bytes;
             sa.part_stride = 0;
-            sa.counter = pa.counter + r;
-            sa.zidx = pa.zidx + (size_t)r * pa.z_stride;
-            sa.zval = pa.zval + (size_t)r * pa.z_stride;
-            sa.zcount = pa.zcount + r;
-            sa.zflag = pa.zflag + r;
-            sa.fin_scratch = sa.fin_scratch ? pa.fin + (size_t)r * pa.fin_stride : nullptr;
+            sa.counter = counters + round;
+            sa.counter2 = counters + kMaxRounds + round;
+            sa.zidx = ba.zidx + (size_t)r * ba.z_stride;
+            sa.zval = ba.zval + (size_t)r * ba.z_stride;
+            sa.zcount = ba.zcount + r;
+            sa.zflag = ba.zflag + r;
+            sa.fin_scratch = ba.fin + (size_t)r * ba.fin_stride;
             sa.fin_stride = 0;
-            sa.out_idx = pa.out_idx + (size_t)r * pa.out_cap;
-            sa.out_val = pa.out_val + (size_t)r * pa.out_cap;
-            sa.out_cap = pa.out_cap;
-            sa.out_count = pa.out_count + r;
-            sa.out_flag = pa.out_flag + r;
+            sa.out_idx = ba.out_idx + (size_t)r * ba.out_cap;
+            sa.out_val = ba.out_val + (size_t)r * ba.out_cap;
+            sa.out_cap = ba.out_cap;
+            sa.out_count = ba.out_count + r;
+            sa.out_flag = ba.out_flag + r;
         }
         __syncthreads();
-        const ExactArgs& a = sa;
-        const ReqView rq = req_view(a.reqs, nullptr, 0, 0, 0, a.nmask);
-        uint32_t sigma, b;
-        exact_hash(rq.seed, rq.id, a.round, a.nmask, &sigma, &b);
-        gather_fold<R>(a, rq.x, rq.xmask, 0, c, sigma, b, smem);
-        if (arrive(a.counter, a.chunks)) {
-            finish_round<R>(a, 0, sigma, b, a.fin_scratch ? a.fin_scratch : smem);
-            __syncthreads();  // every thread's zhat and output stores precede thread 0's release
-            if (tid == 0) {
-                __threadfence();
-                *a.counter = 0;
-                if (t + 1 < pa.req_rounds[r]) {  // publish the request's next round
-                    const uint32_t nch = pa.rdesc[pa.req_rd0[r] + t + 1].chunks;
-                    const uint32_t base = atomicAdd(pa.tail, nch);
-                    for (uint32_t q = 0; q < nch; ++q) store_release(pa.items + base + q, pack_item(r, t + 1, q));
-                }
-            }
-        }
-        __syncthreads();  // sa and the shared arrays are rewritten by the next item
-    }
-}
-
-int exact_persistent_ctas(size_t smem, bool fp64) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e;
-    if (fp64) {
-        e = cudaFuncSetAttribute(k_exact_persistent<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_exact_persistent<double>, kThreads, smem);
-    } else {
-        e = cudaFuncSetAttribute(k_exact_persistent<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_exact_persistent<float>, kThreads, smem);
-    }
-    if (e != cudaSuccess) return 0;
-    return sms * per;
-}
-
-cudaError_t launch_exact_persistent(const PersistArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64) {
-    if (fp64)
-        k_exact_persistent<double><<<ctas, kThreads, smem, st>>>(a);
+    };
+    load_round(t);
+    const ReqView rq = req_view(sa.reqs, nullptr, 0, 0, 0, sa.nmask);
+    uint32_t sigma, b;
+    exact_hash(rq.seed, rq.id, t, sa.nmask, &sigma, &b);
+    if (LARGE && sa.owner)
+        gather_owner<R>(sa, rq.x, rq.xmask, 0, c, sigma, b, smem);
     else
-        k_exact_persistent<float><<<ctas, kThreads, smem, st>>>(a);
+        gather_fold<R>(sa, rq.x, rq.xmask, 0, c, sigma, b, smem);
+    if (arrive(sa.counter, sa.gctas) == 0) return;
+    finish_round<R, LARGE>(sa, 0, sigma, b, smem, kFinBins);
+    if (tid == 0) *sa.counter = 0;
+    if (t > 0 && arrive_pair(sa.counter2) == 0) return;
+    // the decodes from round t on (as decode_chain)
+    for (bool first = true;; first = false) {
+        const uint32_t* next_ctr = t + 1 < rounds ? counters + kMaxRounds + t + 1 : nullptr;
+        const bool next_ready = LARGE ? finish_large<R>(sa, 0, sigma, b, smem, next_ctr)
+                                      : finish_round<R>(sa, 0, sigma, b, smem, kFinDecode, !first, first, next_ctr);
+        if (tid == 0) *sa.counter2 = 0;
+        if (++t >= rounds) break;
+        if (!next_ready && arrive_pair(counters + kMaxRounds + t) == 0) break;
+        load_round(t);
+        exact_hash(rq.seed, rq.id, t, sa.nmask, &sigma, &b);
+    }
+}
+
+cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, bool large) {
+    if (ctas == 0) return cudaSuccess;
+    if (fp64 && large)
+        k_exact_batch<double, true><<<ctas, kThreads, smem, st>>>(a);
+    else if (fp64)
+        k_exact_batch<double, false><<<ctas, kThreads, smem, st>>>(a);
+    else if (large)
+        k_exact_batch<float, true><<<ctas, kThreads, smem, st>>>(a);
+    else
+        k_exact_batch<float, false><<<ctas, kThreads, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+// A bounded wait for a word that nothing publishes: it gives up after about a second and says so.
+constexpr uint32_t kSpinLimit = 1u << 23;  // x ~128 ns
+__global__ void k_wait_check(const uint32_t* word, int32_t* error) {
+    for (uint32_t spin = 0; !acquire_is(word, 1u); ++spin) {
+        if (spin >= kSpinLimit) {
+            atomicExch(error, 1);
+            return;
+        }
+        __nanosleep(128);
+    }
+}
+cudaError_t launch_wait_check(const uint32_t* word, int32_t* error, cudaStream_t st) {
+    k_wait_check<<<1, 1, 0, st>>>(word, error);
     return cudaGetLastError();
 }
 
@@ -1357,7 +1959,10 @@ static cudaError_t launch_chan_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
     if (after && (e = cudaEventRecord(after, st)) != cudaSuccess) return e;
     k_chan_bins<NR><<<sp.seg[R], kThreads, smem, st>>>(sp, seed, id);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_chan_decode<NR><<<C, kThreads, smem, st>>>(sp, seed, id, error);
+    if (rounds[0].large)
+        k_chan_decode<NR, true><<<C, kThreads, smem, st>>>(sp, seed, id, error);
+    else
+        k_chan_decode<NR, false><<<C, kThreads, smem, st>>>(sp, seed, id, error);
     return cudaGetLastError();
 }
 
@@ -1370,31 +1975,57 @@ cudaError_t launch_exact_channels(const ExactArgs* rounds, uint32_t R, uint32_t 
     return launch_chan_nr<32>(rounds, R, C, x, seed, id, smem, error, st, before, after);
 }
 
-cudaError_t set_exact_smem_limit(size_t bytes, bool fp64) {
+template <typename R, bool LARGE>
+static cudaError_t raise_exact_smem(size_t bytes, size_t* cur) {
+    if (bytes <= *cur) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    auto raise = [&](const void* kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    raise((const void*)k_exact_step<R, 8, LARGE>);
+    raise((const void*)k_exact_step<R, 16, LARGE>);
+    raise((const void*)k_exact_step<R, 32, LARGE>);
+    if constexpr (sizeof(R) == sizeof(float)) {
+        raise((const void*)k_chan_decode<8, LARGE>);
+        raise((const void*)k_chan_decode<16, LARGE>);
+        raise((const void*)k_chan_decode<32, LARGE>);
+    }
+    if (e == cudaSuccess) *cur = bytes;
+    return e;
+}
+cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, bool large) {
     static std::mutex mu;  // plans may be created from several threads
     std::lock_guard<std::mutex> lk(mu);
-    static size_t limit[2] = {0, 0};
-    size_t& cur = limit[fp64 ? 1 : 0];
-    if (bytes <= cur) return cudaSuccess;
-    cudaError_t e;
-    const int b = (int)bytes;
+    static size_t limit[2][2] = {{0, 0}, {0, 0}}, single[2] = {0, 0};
+    cudaError_t e = fp64 ? (large ? raise_exact_smem<double, true>(bytes, &limit[1][1])
+                                  : raise_exact_smem<double, false>(bytes, &limit[1][0]))
+                         : (large ? raise_exact_smem<float, true>(bytes, &limit[0][1])
+                                  : raise_exact_smem<float, false>(bytes, &limit[0][0]));
+    size_t& cur = single[fp64 ? 1 : 0];  // the kernels that serve both kinds of plan
+    auto raise = [&](const void* kernel) {
+        if (e == cudaSuccess && bytes > cur)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
     if (fp64) {
-        e = cudaFuncSetAttribute(k_exact_round<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<double, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<double, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<double, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+        raise((const void*)k_exact_round<double>);
     } else {
-        e = cudaFuncSetAttribute(k_exact_round<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<float, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<float, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_exact_step<float, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_bins<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_bins<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_bins<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_decode<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_decode<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chan_decode<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+        raise((const void*)k_exact_round<float>);
+        raise((const void*)k_chan_bins<8>);
+        raise((const void*)k_chan_bins<16>);
+        raise((const void*)k_chan_bins<32>);
     }
+    if (e == cudaSuccess && bytes > cur) cur = bytes;
+    return e;
+}
+cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, bool large) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lk(mu);
+    static size_t limit[2][2] = {{0, 0}, {0, 0}};
+    size_t& cur = limit[fp64 ? 1 : 0][large ? 1 : 0];
+    if (bytes <= cur) return cudaSuccess;
+    const void* k = fp64 ? (large ? (const void*)k_exact_batch<double, true> : (const void*)k_exact_batch<double, false>)
+                         : (large ? (const void*)k_exact_batch<float, true> : (const void*)k_exact_batch<float, false>);
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) cur = bytes;
     return e;
 }
@@ -1415,17 +2046,22 @@ static cudaError_t launch_step_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
     sp.R = R;
     sp.seg[0] = 0;
     for (uint32_t t = 0; t < R; ++t) {
-        const uint64_t end = (uint64_t)sp.seg[t] + (uint64_t)rounds[t].chunks * batch;
+        const uint64_t end = (uint64_t)sp.seg[t] + (uint64_t)rounds[t].gctas * batch;
         if (end > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;  // grid limit
         sp.seg[t + 1] = (uint32_t)end;
         sp.r[t] = rounds[t];
     }
     const uint32_t ctas = sp.seg[R];
     if (ctas == 0) return cudaSuccess;
-    if (fp64)
-        k_exact_step<double, NR><<<ctas, kThreads, smem, st>>>(sp);
+    const bool large = rounds[0].large != 0;  // of the whole plan
+    if (fp64 && large)
+        k_exact_step<double, NR, true><<<ctas, kThreads, smem, st>>>(sp);
+    else if (fp64)
+        k_exact_step<double, NR, false><<<ctas, kThreads, smem, st>>>(sp);
+    else if (large)
+        k_exact_step<float, NR, true><<<ctas, kThreads, smem, st>>>(sp);
     else
-        k_exact_step<float, NR><<<ctas, kThreads, smem, st>>>(sp);
+        k_exact_step<float, NR, false><<<ctas, kThreads, smem, st>>>(sp);
     return cudaGetLastError();
 }
 

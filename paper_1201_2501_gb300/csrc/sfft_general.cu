@@ -219,7 +219,8 @@ __device__ __forceinline__ void gather_residues(const GenArgs& a, const float2* 
     }
     end_range();
     if (B >= (uint32_t)kThreads || tid < B) {
-        const uint32_t r = t0 & (B - 1);
+        // in bit-reversed order, as the bin FFT takes them
+        const uint32_t r = __brev(t0 & (B - 1)) >> (32u - a.logB);
 #pragma unroll
         for (int h = 0; h < NH; ++h)
             if ((uint32_t)h < nh) out[(size_t)h * B + r] = sum[h];
@@ -345,77 +346,6 @@ __device__ __forceinline__ float dot2(float a, float x, float b, float y) {
     return __fadd_rn(s, __fadd_rn(e, __fadd_rn(pe, qe)));
 }
 
-// Stages st + 1 .. st + N of an FFT of H rows: a thread takes the 2^N elements those stages mix, so that
-// one pass over shared memory and one barrier serve N stages.  Ends with a barrier.
-template <int N>
-__device__ __forceinline__ void fft_pass(float2* a, uint32_t H, uint32_t logB, uint32_t st) {
-    constexpr int M = 1 << N;
-    const uint32_t half = 1u << st, groups = 1u << (logB - N);
-    auto butterflies = [&](float2* row, const float2* w) {
-        float2 v[M];
-#pragma unroll
-        for (int e = 0; e < M; ++e) v[e] = row[(uint32_t)e << st];
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-#pragma unroll
-            for (int e = 0; e < M; ++e)
-                if (!(e & (1 << k))) {
-                    const float2 bv = cmul_rn(v[e | (1 << k)], w[(1 << k) - 1 + (e & ((1 << k) - 1))]);
-                    const float2 av = v[e];
-                    v[e] = cadd(av, bv);
-                    v[e | (1 << k)] = csub(av, bv);
-                }
-#pragma unroll
-        for (int e = 0; e < M; ++e) row[(uint32_t)e << st] = v[e];
-    };
-    // the twiddles of stage st + 1 + k at position lo: exp(-i pi (lo + f half) / (half 2^k)), f < 2^k
-    auto twiddles = [&](uint32_t lo, float2* w) {
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-#pragma unroll
-            for (int f = 0; f < (1 << k); ++f) {
-                float sn, cs;
-                sincospif(-(float)(lo + ((uint32_t)f << st)) / (float)(half << k), &sn, &cs);
-                w[(1 << k) - 1 + f] = mkc(cs, sn);
-            }
-    };
-    float2 w[M - 1];
-    if (groups >= (uint32_t)kThreads) {  // every thread has a position: its twiddles serve all rows
-        for (uint32_t q = threadIdx.x; q < groups; q += kThreads) {
-            const uint32_t lo = q & (half - 1);
-            twiddles(lo, w);
-            for (uint32_t h = 0; h < H; ++h) butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
-        }
-    } else {
-        for (uint32_t i = threadIdx.x; i < H * groups; i += kThreads) {
-            const uint32_t h = i >> (logB - N), q = i & (groups - 1), lo = q & (half - 1);
-            twiddles(lo, w);
-            butterflies(a + (h << logB) + ((q >> st) << (st + N)) + lo, w);
-        }
-    }
-    __syncthreads();
-}
-
-// block_fft_rows with the stages past the fifth taken two or three per pass: as many as leave every
-// thread a group of elements (B = 2048, two rows: two barriers instead of six, and a third of the
-// sincospif).  The same butterflies, so the same bits.
-__device__ void fft_rows_by_passes(float2* a, uint32_t H, uint32_t logB) {
-    fft_first_stages<float>(a, H, logB);
-    for (uint32_t st = logB < 5 ? logB : 5; st < logB;) {
-        const uint32_t left = logB - st;
-        if (left >= 3 && left != 4 && (H << (logB - 3)) >= (uint32_t)kThreads) {
-            fft_pass<3>(a, H, logB, st);
-            st += 3;
-        } else if (left >= 2 && (H << (logB - 2)) >= (uint32_t)kThreads) {
-            fft_pass<2>(a, H, logB, st);
-            st += 2;
-        } else {
-            fft_pass<1>(a, H, logB, st);
-            st += 1;
-        }
-    }
-}
-
 __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t s = a.req_base + blockIdx.y, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -431,13 +361,8 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     double* ub = reinterpret_cast<double*>(smem + Ly.ub);             // B < kThreads: [hashing][component][B]
     uint32_t* scan = reinterpret_cast<uint32_t*>(smem + Ly.scan);
     const uint32_t logNp = (uint32_t)(63 - __clzll((long long)a.n)) - a.logB;
-    // step 3: the fold, bit-reversed, B-point FFT per hashing
-    const float2* part = a.part + (size_t)s * a.part_stride + (size_t)g * 2 * B;
-    const uint32_t shift_br = 32u - a.logB;
-    for (uint32_t i = tid; i < h.H * B; i += kThreads) {
-        const uint32_t r = i & (B - 1);
-        U[i - r + (__brev(r) >> shift_br)] = __ldcg(part + i);
-    }
+    // step 3: the fold (bit-reversed), B-point FFT per hashing
+    load_rows(U, a.part + (size_t)s * a.part_stride + (size_t)g * 2 * B, h.H * B);
     const uint32_t nz = min(a.zcount[s], a.nzmax);
     const uint32_t* zidx = a.zidx + (size_t)s * a.zcap;
     const double2* zval = a.zval + (size_t)s * a.zcap;

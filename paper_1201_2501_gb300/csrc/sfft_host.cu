@@ -269,6 +269,7 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
     pl->taps_host.clear();
     pl->wtab_host.clear();
     size_t taps_off = 0, wtab_off = 0;
+    bool large = false;
     for (uint32_t t = 0; t < R; ++t) {
         ExactRound r;
         uint64_t kt = ((uint64_t)p.k + (uint64_t(1) << t) - 1) >> t;
@@ -307,11 +308,15 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
         const size_t gs = exact_gather_smem(r.stage, fp64) + (size_t)(1 + r.nshift) * (B > (uint64_t)kThreads ? B : kThreads) *
                                                               (fp64 ? 16 : 8);
         const size_t fs = exact_finish_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
-        // a finisher that does not fit next to the gather's staging keeps its arrays in device memory
-        r.fin_bytes = fs;
+        // finish_round's arrays beyond kFinSmemMax live in device memory (the single-hashing call); the
+        // transform's decode is finish_large there, and wherever zhat may outgrow what a decode keeps on
+        // chip for the next one
         r.fin_global = fs > kFinSmemMax;
-        r.smem = r.fin_global ? gs : (gs > fs ? gs : fs);
-        if (r.smem > 200 * 1024) return SFFT_ERR_K_RANGE;
+        if ((r.fin_global ? gs : (gs > fs ? gs : fs)) > 200 * 1024) return SFFT_ERR_K_RANGE;
+        large = large || r.fin_global || p.z_cap > kCarry;
+        r.fin_bytes = r.fin_global ? fs : 0;
+        r.smem = fs;
+        r.smem_gather = std::max(gs, (size_t)(1 + r.nshift) * r.B * (fp64 ? 16 : 8));
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, r.alpha, p.delta, r.T, pl->taps_host.data() + taps_off);
         pl->wtab_host.resize(wtab_off + 2 * (Np / 2 + 1));
@@ -326,6 +331,16 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
         taps_off += (size_t)r.T + 1;
         wtab_off += 2 * (Np / 2 + 1);
         pl->rounds.push_back(r);
+    }
+    for (ExactRound& r : pl->rounds) {  // one kind of decode for the whole plan
+        r.large = large;
+        // gather_owner where it has two CTAs or more per request: below, its one CTA walks the window alone
+        r.ring = exact_owner_ring(r.shift[r.nshift - 1], r.B, fp64);
+        r.owner = large && r.B >= 2 * (uint32_t)kThreads && r.ring <= 32;
+        if (r.owner)
+            r.smem_gather = std::max(exact_owner_smem(r.ring, fp64), (size_t)(1 + r.nshift) * r.B * (fp64 ? 16 : 8));
+        r.smem = std::max(r.smem_gather, large ? (size_t)kLargeSmem : r.smem);
+        if (large) r.fin_bytes = std::max(r.fin_bytes, exact_large_bytes(r.B, 1 + r.nshift, p.z_cap, fp64));
     }
     pl->wtab_len = wtab_off;
     return SFFT_OK;

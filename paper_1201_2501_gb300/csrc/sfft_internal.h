@@ -15,6 +15,7 @@ constexpr int kThreads = 256;     // threads per CTA of every kernel
 constexpr int kChunkTaps = 2048;  // taps per CTA in the gather phase (8 per thread)
 constexpr int kMaxHash = 4;       // hashings per exact round: a = 0 plus up to 3 ladder shifts
 constexpr uint32_t kCarry = 256;  // zhat entries an exact finisher keeps on chip for the next round
+constexpr uint32_t kLargeSmem = 104 * 1024;  // shared memory of finish_large: two CTAs per SM
 constexpr uint32_t kMaxB = 4096;  // largest B of the fused exact round
 constexpr uint32_t kNoIndex = 0xFFFFFFFFu;
 constexpr size_t kFinSmemMax = 160 * 1024;  // largest on-chip finisher of the exact round
@@ -46,8 +47,12 @@ struct ExactRound {
     size_t wtab_off = 0;      // offset of this round's W(o), o = 0..n/2B, in the W table (exact rounds:
                               // followed by 1 / W(o) for the same o)
     size_t smem = 0;          // dynamic shared memory of the round kernel
-    bool fin_global = false;  // the finisher's arrays do not fit on chip: they live in d_fin
-    size_t fin_bytes = 0;     // size of the finisher's arrays of one request
+    size_t smem_gather = 0;   // of which the gather and the bins need this
+    bool fin_global = false;  // the arrays of finish_round do not fit on chip: they live in d_fin
+    bool large = false;       // the transform's decode is finish_large (the same for all of a plan's rounds)
+    bool owner = false;       // gather_owner folds the round (a CTA per kThreads residues)
+    uint32_t ring = 0;        // samples a thread of gather_owner keeps
+    size_t fin_bytes = 0;     // device memory a request's decode may need
 };
 
 // Kernel argument block of the exact round (passed by value).
@@ -66,6 +71,10 @@ struct ExactArgs {
     uint32_t a[kMaxHash];      // a[0] = 0, a[l] = beta_l
     uint64_t shift64[kMaxHash];
     uint32_t chunks, stage, maxshift;
+    uint32_t gctas;            // gather CTAs of the round per request: its chunks, or B / kThreads (owner)
+    uint32_t owner, ring;      // fold by gather_owner, with this many samples kept per thread
+    uint32_t large;            // decode by finish_large
+    uint32_t large_smem;       // its dynamic shared memory
     uint32_t ctaps;            // taps per CTA: chunk c gathers taps [-T + c ctaps, -T + (c + 1) ctaps)
     const float* taps32;
     const double* taps64;
@@ -74,6 +83,7 @@ struct ExactArgs {
     void* part;                // partial fold sums: request s owns [s part_stride, (s + 1) part_stride),
                                // laid out [chunks][H][B] complex R (requests may be in different rounds)
     size_t part_stride;
+    size_t part_bytes;         // mixed batches: where the round's folds start in a request's region
     uint32_t* counter;         // [batch] arrival counters (zero between launches)
     uint32_t* counter2;        // [batch] the one-launch path's second counters: round t's decode starts
                                // once its bins are ready and round t - 1's decode is done
@@ -93,8 +103,9 @@ struct ExactArgs {
     uint32_t out_cap;
     uint32_t* out_count;
     int32_t* out_flag;
-    // the finisher's arrays: in shared memory (fin_scratch null) or, for large B and zcap, in the
-    // global region [s fin_stride, (s + 1) fin_stride) of fin_scratch (only one CTA per request uses it)
+    // device memory for the decode's arrays, [s fin_stride, (s + 1) fin_stride) of fin_scratch (only one
+    // CTA per request uses it): what finish_large cannot keep on chip; all of finish_round's where the
+    // single-hashing call sets it
     unsigned char* fin_scratch;
     size_t fin_stride;
     // single-hashing mode (sfft_hash_to_bins): explicit (sigma, b), bins written to ubins, no decode
@@ -144,36 +155,32 @@ struct ChanParams {
     ExactArgs r[NR];          // round blocks; part at the round's channel layout, chunks = its chunks
 };
 
-// The persistent exact path: requests of different plans (n, k, schedule) in one launch, their
-// rounds driven by a device work queue.  Item = (request, round, chunk); the CTA that finishes a
-// request's round publishes the chunks of its next round.  rdesc holds one argument block per
-// (plan, round) with the plan's tables; the per-request fields are pointed at the request's own
-// workspace (as slot 0) by the kernel.
-struct PersistArgs {
+// Mixed batches: requests of different plans (n, k, schedule) in one launch (two where plans of both
+// kinds of decode are mixed).  rdesc holds one argument block per (plan, round) with the plan's tables;
+// the per-request fields are pointed at the request's own workspace by the kernel.
+struct BatchArgs {
     const ExactArgs* rdesc;         // [sum of the plans' rounds]
     const ReqDesc* reqs;            // [nreq]
     const uint32_t* req_rd0;        // [nreq] index in rdesc of the request's round 0
     const uint32_t* req_rounds;     // [nreq]
-    unsigned long long* items;      // [total] (bit 63: published)
-    uint32_t* head;                 // items taken
-    uint32_t* tail;                 // items reserved
-    uint32_t total;
+    const uint32_t* seg;            // [nseg] first CTA of each (round, request)
+    const uint32_t* seg_who;        // [nseg] round << 24 | request
+    uint32_t nseg;
     unsigned char* part;            // [nreq][part_stride] bytes
     size_t part_stride;
-    uint32_t* counter;              // [nreq] (zero between rounds)
+    uint32_t* counter;              // [nreq][2][kMaxRounds] (zero between launches)
     uint32_t* zidx;                 // [nreq][z_stride]
     double2* zval;
     size_t z_stride;
     uint32_t* zcount;               // [nreq]
     int32_t* zflag;                 // [nreq]
-    unsigned char* fin;             // [nreq][fin_stride] bytes (rounds with fin_global)
+    unsigned char* fin;             // [nreq][fin_stride] bytes (finish_large)
     size_t fin_stride;
     uint32_t* out_idx;              // [nreq][out_cap]
     double2* out_val;
     uint32_t out_cap;
     uint32_t* out_count;            // [nreq]
     int32_t* out_flag;              // [nreq]
-    int32_t* error;                 // set when a wait for an item ran out
 };
 
 struct DecodeArgs {
@@ -342,7 +349,7 @@ struct sfft_plan_s {
     sfft::ReqDesc* h_reqs[2] = {nullptr, nullptr};
     cudaEvent_t ev_reqs[2] = {nullptr, nullptr};
     int reqs_cur = 0;
-    // finisher arrays of the exact rounds with fin_global: per such round, [max_batch][fin_stride]
+    // device memory of the exact rounds' decodes with fin_bytes: [max_batch][fin_stride]
     unsigned char* d_fin = nullptr;
     size_t fin_stride = 0;
     size_t dev_bytes = 0;          // device memory allocated at plan creation
@@ -402,9 +409,9 @@ cudaError_t launch_exact_step(const ExactArgs* rounds, uint32_t R, uint32_t batc
 cudaError_t launch_exact_channels(const ExactArgs* rounds, uint32_t R, uint32_t C, const void* x, uint64_t seed,
                                   uint32_t id, size_t smem, uint32_t* error, cudaStream_t st, cudaEvent_t before,
                                   cudaEvent_t after);
-// persistent path: CTAs that fit on the device at `smem`, and the launch
-int exact_persistent_ctas(size_t smem, bool fp64);
-cudaError_t launch_exact_persistent(const PersistArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64);
+// mixed batches, and the check of a bounded wait
+cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, bool large);
+cudaError_t launch_wait_check(const uint32_t* word, int32_t* error, cudaStream_t st);
 cudaError_t launch_exact_decode(const DecodeArgs& a, cudaStream_t st);
 cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                           uint32_t count, uint32_t* out, cudaStream_t st);
@@ -421,5 +428,9 @@ cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);
 size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 size_t exact_gather_smem(uint32_t stage, bool fp64);
-cudaError_t set_exact_smem_limit(size_t bytes, bool fp64);
+size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
+uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64);
+size_t exact_owner_smem(uint32_t ring, bool fp64);
+cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, bool large);
+cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, bool large);
 }  // namespace sfft

@@ -440,7 +440,7 @@ class Graph:
 
 
 class BatchPlan:
-    """Exact-mode plans of any (n, k) run together in one persistent launch (``sfft_batch_*``)."""
+    """Exact-mode plans of any (n, k) run together in one launch (``sfft_batch_*``)."""
 
     def __init__(self, plans, max_requests: int):
         self.plans = list(plans)  # the plans must outlive the batch plan

@@ -1,0 +1,74 @@
+"""Exact-mode plans whose zhat may hold more than 256 entries (their rounds fold by residue blocks where B
+is 512 or more, and decode with arrays sized by what was found) against the FP64 oracle, at the edges of
+their ranges, and the same requests in a mixed batch.
+
+Supports, counts and flags bit for bit; values within 1e-9 (FP64 data) or 1e-5 (FP32 data) of |X| = 1.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1201_2501_gb300 import workloads
+from tests.common import exact_fields, oracle_params
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def sf():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1201_2501_gb300 import build, sfft
+
+    build.build()
+    sfft.lib()
+    return sfft
+
+
+def _params(sf, f, prec):
+    p = sf.sfft_params_default(f["n"], f["k"], f["mode"])
+    for name, _ in sf.SfftParams._fields_:
+        if name in f:
+            setattr(p, name, f[name])
+    p.precision = prec
+    return p
+
+
+# smallest such plan (z_cap 260); a capacity below k (CAPACITY, the smallest indices kept); FP64 at few
+# samples; the longest ladder shifts (8 B, B = 1024); B = 4096; entries beyond shared memory (device
+# memory in their place); chunks of 256 and of 8192 taps
+@pytest.mark.parametrize("m,k,prec,batch,over", [
+    (16, 65, 0, 3, {}), (16, 400, 1, 2, dict(z_cap=300)), (14, 100, 1, 2, dict(delta=1e-8)),
+    (22, 130, 0, 2, dict(tau_dec=5e-3)), (18, 1000, 0, 2, {}),
+    (20, 1500, 0, 1, dict(bins_per_k=2.5, z_cap=4096)), (16, 130, 0, 2, dict(chunk_taps=256)),
+    (16, 130, 1, 2, dict(chunk_taps=8192))])
+def test_large_plans_match_oracle(sf, m, k, prec, batch, over):
+    n, seed = 1 << m, 33
+    f = exact_fields(n, k, **{key: v for key, v in over.items() if key != "chunk_taps"})
+    P = oracle_params(f)
+    p = _params(sf, f, prec)
+    p.chunk_taps = over.get("chunk_taps", 2048)
+    dt = np.complex128 if prec else np.complex64
+    sigs = [workloads.exact_sparse(n, k, workloads.seed_for(2, 700 + i), dtype=dt) for i in range(batch)]
+    x = torch.as_tensor(np.stack([s.x for s in sigs])).cuda()
+    plan, cap = sf.Plan(p, batch), f["z_cap"]
+    small = sf.Plan(_params(sf, exact_fields(1 << 14, 8), prec), 1)
+    idx, val, cnt, flag = [o.cpu().numpy() for o in sf.sfft_execute(plan, x, seed, cap)]
+    bp = sf.BatchPlan([small, plan], batch + 1)
+    xs = [x[r] for r in range(batch)]
+    extra = torch.as_tensor(workloads.exact_sparse(1 << 14, 8, 5, dtype=dt).x).cuda()
+    mixed = [o.cpu().numpy() for o in bp.execute([1] * batch + [0], xs + [extra], [seed] * (batch + 1),
+                                                 list(range(batch)) + [0], cap)]
+    for r, s in enumerate(sigs):
+        oi, ov, of = oracle.sfft_exact(P, s.x.astype(np.complex128), seed, r)
+        of = {0: sf.SFFT_OK, 1: sf.SFFT_ERR_NOT_CONVERGED, 2: sf.SFFT_ERR_CAPACITY}[of]
+        c = int(cnt[r])
+        assert np.array_equal(idx[r, :c].view(np.uint32).astype(np.int64), oi.astype(np.int64))
+        assert int(flag[r]) == of
+        assert np.max(np.abs(val[r, :c, 0] + 1j * val[r, :c, 1] - ov), initial=0.0) < (1e-9 if prec else 1e-5)
+        assert int(mixed[2][r]) == c and int(mixed[3][r]) == of
+        assert np.array_equal(mixed[0][r, :c], idx[r, :c]) and np.array_equal(mixed[1][r, :c], val[r, :c])
+    for q in (bp, plan, small):
+        q.close()
