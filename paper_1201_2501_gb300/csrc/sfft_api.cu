@@ -116,6 +116,9 @@ ExactArgs base_args(const sfft_plan_s* pl, const ExactRound& r, uint32_t t) {
     a.taps64 = pl->d_taps64 + r.taps_off;
     a.wtab = pl->d_wtab + r.wtab_off;
     a.winv = a.wtab + (p.n / r.B) / 2 + 1;  // the exact schedule stores 1 / W(o) after W(o)
+    a.tw = pl->d_tw;
+    a.tw_shift = pl->tw_shift;
+    a.logn = ilog2_host(p.n);
     a.part = pl->d_part;
     a.part_stride = pl->part_stride;
     a.fin_scratch = r.fin_bytes ? pl->d_fin : nullptr;
@@ -286,12 +289,14 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     // one-launch path forms a round's bins in the CTA's shared memory), and a request's decodes run one
     // after another (round t + 1's waits for round t's arrival on the request's second counter)
     if (pl->fin_stride) SFFT_ALLOC(pl->d_fin, pl->fin_stride * max_batch);
+    if (general || fp64) {
+        pl->tw_shift = (ilog2_host(p->n) + 1) / 2;
+        SFFT_ALLOC(pl->d_tw, ((size_t(1) << pl->tw_shift) + (p->n >> pl->tw_shift)) * sizeof(double2));
+    }
     if (general) {
         SFFT_ALLOC(pl->d_bins, pl->bins_stride * max_batch * sizeof(double2));
         SFFT_ALLOC(pl->d_phase, pl->phase_stride * max_batch * sizeof(uint32_t));
         SFFT_ALLOC(pl->d_L, sum_B * max_batch * sizeof(uint32_t));
-        pl->tw_shift = (ilog2_host(p->n) + 1) / 2;
-        SFFT_ALLOC(pl->d_tw, ((size_t(1) << pl->tw_shift) + (p->n >> pl->tw_shift)) * sizeof(double2));
         SFFT_ALLOC(pl->d_estw, (size_t)max_batch * sum_B * (sizeof(double2) + sizeof(double)));
         size_t perm = 0;
         for (const GeneralRound& r : pl->grounds) perm += r.perm ? 1 : 0;
@@ -308,9 +313,12 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
     if ((e = cudaMemcpy(pl->d_taps64, pl->taps_host.data(), ntaps * sizeof(double), cudaMemcpyHostToDevice)) !=
         cudaSuccess)
         return fail(e, "upload taps");
-    if (general) {  // twiddle factor tables of the FP64 estimates
+    if (general || fp64) {  // twiddle factor tables of the FP64 estimates, or of the FP64 data path
         std::vector<double2> tw;
-        twiddle_tables_host(p->n, pl->tw_shift, &tw);
+        if (general)
+            twiddle_tables_host(p->n, pl->tw_shift, &tw);
+        else
+            twiddle_tables_exact_host(p->n, pl->tw_shift, &tw);
         if ((e = cudaMemcpy(pl->d_tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice)) != cudaSuccess)
             return fail(e, "upload twiddle tables");
     }

@@ -103,6 +103,21 @@ __device__ __forceinline__ double2 root_pow(uint32_t e, uint32_t nmask) {
     return make_double2((double)c, -(double)s);
 }
 
+// w^e = exp(-2 pi i e / n) for an exact exponent e in [0, n) from two tables of FP64 factors,
+// exp(-2 pi i (e mod 2^sh) / n) and exp(-2 pi i 2^sh (e >> sh) / n): one complex product (a few ulp
+// from a direct evaluation) instead of an FP64 sincospi, which GB300 runs at 1/64 of the FP32 rate
+__device__ __forceinline__ double2 root_pow_tab(uint32_t e, const double2* tw, uint32_t sh) {
+    const double2 lo = tw[e & ((1u << sh) - 1u)], hi = tw[(1u << sh) + (e >> sh)];
+    return make_double2(hi.x * lo.x - hi.y * lo.y, hi.x * lo.y + hi.y * lo.x);
+}
+
+// The same from tables whose first part holds the factors minus one: w^e = h + h (l - 1), where the small
+// second term's rounding is lost in the sum's (error below 1 ulp, against 2 of the plain product).
+__device__ __forceinline__ double2 root_pow_fine(uint32_t e, const double2* tw, uint32_t sh) {
+    const double2 d = tw[e & ((1u << sh) - 1u)], h = tw[(1u << sh) + (e >> sh)];
+    return make_double2(fma(h.x, d.x, fma(-h.y, d.y, h.x)), fma(h.x, d.y, fma(h.y, d.x, h.y)));
+}
+
 // phase(z) / 2 pi in [0, 1)
 template <typename R>
 __device__ __forceinline__ double phase01(double2 z);
@@ -290,6 +305,27 @@ __device__ void block_fft_rows(typename Cx<R>::T* a, uint32_t H, uint32_t logB) 
             const C w = mkc(cs, sn);
             const C bv = cmul(a[i1], w);
             const C av = a[i0];
+            a[i0] = cadd(av, bv);
+            a[i1] = csub(av, bv);
+        }
+        __syncthreads();
+    }
+}
+
+// block_fft_rows in FP64 with its twiddles from the factor tables (n = 2^logn): an FP64 sincospi costs
+// about 45 operations of a pipe that issues at 1/64 of the FP32 rate, a butterfly 8, and thread pairs
+// that exchange by shuffles would each form the whole product.  exp(-i pi pos / half) = w^{pos n / (2 half)}.
+__device__ inline void fft_rows_fp64(double2* a, uint32_t H, uint32_t logB, uint32_t logn, const double2* tw, uint32_t sh) {
+    const uint32_t halfB = (1u << logB) >> 1;
+    __syncthreads();
+    for (uint32_t st = 1; st <= logB; ++st) {
+        const uint32_t half = 1u << (st - 1);
+        for (uint32_t idx = threadIdx.x; idx < H * halfB; idx += kThreads) {
+            const uint32_t h = idx >> (logB - 1), k = idx & (halfB - 1), pos = k & (half - 1);
+            const uint32_t i0 = (h << logB) + ((k >> (st - 1)) << st) + pos, i1 = i0 + half, e = pos << (logn - st);
+            const double2 w = logn - st >= sh ? tw[(1u << sh) + (e >> sh)] : root_pow_fine(e, tw, sh);
+            const double2 b = a[i1], av = a[i0];
+            const double2 bv = make_double2(b.x * w.x - b.y * w.y, b.x * w.y + b.y * w.x);
             a[i0] = cadd(av, bv);
             a[i1] = csub(av, bv);
         }

@@ -98,6 +98,27 @@ uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64) {
     return r;
 }
 
+// g w^e of a tap, w = exp(-2 pi i / n), e = sigma b t (taken mod n): a sincospif in FP32; from the factor
+// tables in FP64, whose sincospi took most of the FP64 gather's time.  With the bins' FFT and the
+// subtraction terms from the tables and the decisions in guarded FP32 (decode_bin_guarded): n = 2^20,
+// k = 64, batch 16: 142 us a call, was 230; n = 2^14, k = 8, one request: 48 us, was 76.
+__device__ __forceinline__ float2 tap_factor(const ExactArgs& a, float g, uint32_t ex, float two_over_n) {
+    const uint32_t e = ex & a.nmask;
+    const int32_t es = e > (a.nmask >> 1) ? (int32_t)((int64_t)e - (int64_t)a.n) : (int32_t)e;
+    float sn, cs;
+    sincospif((float)es * two_over_n, &sn, &cs);
+    return make_float2(g * cs, -g * sn);
+}
+__device__ __forceinline__ double2 tap_factor(const ExactArgs& a, double g, uint32_t ex, double /*two_over_n*/) {
+    const double2 w = root_pow_fine(ex & a.nmask, a.tw, a.tw_shift);
+    return make_double2(g * w.x, g * w.y);
+}
+// w^e of a subtraction term in the precision of the data path
+template <typename R>
+__device__ __forceinline__ double2 term_root(const ExactArgs& a, uint32_t e) {
+    return sizeof(R) == sizeof(float) ? root_pow<float>(e, a.nmask) : root_pow_fine(e, a.tw, a.tw_shift);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Location and estimation of one bin (NoiselessSparseFFTInner's loop body)
 // ------------------------------------------------------------------------------------------------
@@ -204,7 +225,7 @@ __device__ __forceinline__ uint32_t index_at(const DecodeCtx& d, uint32_t j, int
     return (d.sigma_inv * ((p + d.sb) & d.nmask)) & d.nmask;
 }
 template <bool kDirect>
-__device__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list, uint32_t nbin,
+__device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list, uint32_t nbin,
                                const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
                                double* ginv, bool* above) {
     const double mag0 = cmag<double>(u[0]);
@@ -385,11 +406,87 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
     return 1;
 }
 
+// The FP64 data path's decisions, taken in FP32 wherever FP64 must agree.  The rounding of a subtracted
+// bin to FP32, hypotf and atan2f move a magnitude by less than 3e-7 of itself and a phase by less than
+// 2.5e-7 of a turn; a comparison or rounding that lies within several times that of its boundary (kMagGuard,
+// kPhaseGuard32) is not taken and the whole bin goes through decode_bin_fp64.  Every other one has the same
+// outcome in both, so the decode is that of decode_bin_fp64 (about 200 FP64 operations per bin and warp at
+// 1/64 of the FP32 rate).  Values stay in FP64.
+constexpr float kMagGuard = 2e-6f, kPhaseGuard32 = 1e-6f;
+// -1: m < t, 1: m > t, 0: too close
+__device__ __forceinline__ int cmp_guarded(float m, float t) {
+    const float g = kMagGuard * t;
+    return m > t + g ? 1 : (m < t - g ? -1 : 0);
+}
+constexpr int kUndecided = -1;
+template <bool kDirect>
+__device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list,
+                                                  uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain,
+                                                  uint32_t* oi, double* gout, double* ginv, bool* above) {
+    float2 v[kMaxHash];
+    const uint32_t L = d.H - 1;
+#pragma unroll
+    for (int h = 0; h < kMaxHash; ++h)
+        v[h] = (uint32_t)h < d.H ? make_float2((float)u[h].x, (float)u[h].y) : make_float2(0.f, 0.f);
+    *ginv = 0.0;
+    *above = false;
+    const float mag0 = hypotf(v[0].x, v[0].y);
+    // thresholds and magnitudes that FP32 holds to full precision only
+    if (!(d.thr_f > 1e-15f && d.thr_f < 1e15f && mag0 < 1e18f)) return kUndecided;
+    const int over = cmp_guarded(mag0, d.thr_f);
+    if (over == 0) return kUndecided;
+    if (over < 0) {
+        if (nbin == 0) return 0;
+        const int lo = cmp_guarded(mag0, d.ref_lo_f), hi = cmp_guarded(mag0, d.ref_hi_f);
+        return lo < 0 || hi > 0 ? 0 : kUndecided;  // (a re-estimation is decided in FP64)
+    }
+    *above = true;
+    float ml[kMaxHash - 1], th[kMaxHash - 1];
+#pragma unroll
+    for (int l = 0; l < kMaxHash - 1; ++l)
+        if ((uint32_t)l < L) {
+            ml[l] = hypotf(v[l + 1].x, v[l + 1].y);
+            th[l] = phase01_f(mul_conj_f(v[0], v[l + 1]));
+        }
+    // location ladder, coarsest shift first: each rounding has to stay clear of a half
+    uint32_t c = 0, logM = 0;
+#pragma unroll
+    for (int l = kMaxHash - 2; l >= 0; --l) {
+        if ((uint32_t)l >= L) continue;
+        const uint32_t logMp = d.logNp - d.logR[l], logRatio = logMp - logM;  // from logM = 0: the coarsest, c = 0
+        const float y = th[l] * pow2_f((int)logRatio) - __uint2float_rn(c) * pow2_f(-(int)logM);
+        const float f = y - floorf(y);
+        if (!(fabsf(f - 0.5f) > kPhaseGuard32 * (pow2_f((int)logRatio) + 1.0f))) return kUndecided;
+        c += ((uint32_t)__float2int_rd(y + 0.5f) & ((1u << logRatio) - 1u)) << logM;
+        logM = logMp;
+    }
+    const uint32_t dd = (c + d.Np - (d.sb & (d.Np - 1)) + (d.Np >> 1)) & (d.Np - 1);
+    const int32_t o = (int32_t)dd - (int32_t)(d.Np >> 1);
+#pragma unroll
+    for (int l = 0; l < kMaxHash - 1; ++l)
+        if ((uint32_t)l < L) {
+            const float df = fabsf(ml[l] - mag0), t = d.iso_tol_f * mag0, g = kMagGuard * (mag0 + ml[l]);
+            if (df > t + g) return 0;
+            if (!(df < t - g)) return kUndecided;
+        }
+    if (kDirect) {
+        *oi = (uint32_t)o;
+        return 1;
+    }
+    const double gain = d.wtab[o < 0 ? -o : o];
+    if (!(gain >= d.gmin)) return 0;
+    *oi = index_at(d, j, o);
+    *gout = gain;
+    return 1;
+}
+
 template <bool kDirect = false>
 __device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list,
                                           uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
                                           double* gout, double* ginv, bool* above) {
-    return decode_bin_fp64<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    const int kind = decode_bin_guarded<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    return kind != kUndecided ? kind
+                              : decode_bin_fp64<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
 }
 template <bool kDirect = false>
 __device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const float2* u, const uint32_t* list,
@@ -493,11 +590,7 @@ __device__ void gather_fold(const ExactArgs& a, const void* xrow, uint32_t xmask
     for (uint32_t k = tid; k < ntap; k += kThreads) {
         const int32_t t = (int32_t)t_lo + (int32_t)k;
         const R g = taps[t < 0 ? -t : t];
-        const uint32_t e = (sb * (uint32_t)t) & a.nmask;
-        const int32_t es = e > (a.nmask >> 1) ? (int32_t)((int64_t)e - (int64_t)a.n) : (int32_t)e;
-        R sn, cs;
-        sincospi_r((R)es * inv_half_n, &sn, &cs);
-        const C gt = mkc(g * cs, -g * sn);
+        const C gt = tap_factor(a, g, sb * (uint32_t)t, inv_half_n);
         const uint32_t si = k + a.maxshift;
         if (!big) {
 #pragma unroll
@@ -540,7 +633,7 @@ __device__ __forceinline__ void gather_owner(const ExactArgs& a, const void* xro
                                              uint32_t blk, uint32_t sigma, uint32_t b, unsigned char* smem) {
     using C = typename Cx<R>::T;
     constexpr uint32_t kLoads = owner_loads<R>();
-    const uint32_t tid = threadIdx.x, B = a.B, H = a.H, nmask = a.nmask;
+    const uint32_t tid = threadIdx.x, B = a.B, H = a.H;
     C* ring = reinterpret_cast<C*>(smem) + tid;  // [a.ring][kThreads], this thread's column
     R* tap = reinterpret_cast<R*>(reinterpret_cast<C*>(smem) + a.ring * kThreads) + tid;  // [kLoads][kThreads]
     const uint32_t rmask = a.ring - 1u;
@@ -598,11 +691,7 @@ __device__ __forceinline__ void gather_owner(const ExactArgs& a, const void* xro
                     acc[h] = mkc((R)0, (R)0);
                 }
             }
-            const int32_t es = (int32_t)((e & nmask) << (__clz((int)nmask) & 31)) >> (__clz((int)nmask) & 31);
-            R sn, cs;
-            sincospi_r((R)es * inv_half_n, &sn, &cs);
-            const R g = tap[(m - m0) * kThreads];
-            const C gt = mkc(g * cs, -g * sn);
+            const C gt = tap_factor(a, tap[(m - m0) * kThreads], e, inv_half_n);
 #pragma unroll
             for (int h = 0; h < kMaxHash; ++h)
                 if ((uint32_t)h < H) acc[h] = cfma(gt, ring[((m + dl[h]) & rmask) * kThreads], acc[h]);
@@ -612,6 +701,16 @@ __device__ __forceinline__ void gather_owner(const ExactArgs& a, const void* xro
 #pragma unroll
     for (int h = 0; h < kMaxHash; ++h)
         if ((uint32_t)h < H) area[(size_t)h * B] = cadd(sum[h], acc[h]);  // bit-reversed, as the bin FFT takes it
+}
+
+// |v| < prune thr in FP64, by FP32 where that is clear of the bound
+__device__ __forceinline__ bool dropped(double2 v, const ExactArgs& a) {
+    const float f = hypotf((float)v.x, (float)v.y);
+    if (a.drop_f > 1e-25f && a.drop_f < 1e25f && f < 1e18f) {
+        const int c = cmp_guarded(f, a.drop_f);
+        if (c != 0) return c < 0;
+    }
+    return cmag<double>(v) < a.prune * a.thr;
 }
 
 // Step 2 across chunks: U[h][brev(r)] = sum over chunks c, in order, of part[c][h][r].  Each thread
@@ -678,8 +777,17 @@ __device__ void sum_partials(const C* part, uint32_t chunks, uint32_t H, uint32_
 // the first H B entries of the request's partial-fold area of the round; kFinDecode starts from there.
 enum FinPart { kFinBins = 1, kFinDecode = 2, kFinAll = 3 };
 
-__device__ __forceinline__ void fft_rows(float2* U, uint32_t H, uint32_t logB) { fft_rows_by_passes(U, H, logB); }
-__device__ __forceinline__ void fft_rows(double2* U, uint32_t H, uint32_t logB) { block_fft_rows<double>(U, H, logB); }
+template <bool LARGE>
+__device__ __forceinline__ void fft_rows(const ExactArgs& a, float2* U) {
+    if (LARGE)
+        fft_rows_by_passes(U, a.H, a.logB);
+    else
+        block_fft_rows<float>(U, a.H, a.logB);
+}
+template <bool LARGE>
+__device__ __forceinline__ void fft_rows(const ExactArgs& a, double2* U) {
+    fft_rows_fp64(U, a.H, a.logB, a.logn, a.tw, a.tw_shift);
+}
 
 // LARGE: the bins of a plan decoded by finish_large (many bins: FFT stages by passes)
 template <typename R, bool LARGE = false>
@@ -719,10 +827,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
             load_rows(U, area, H * B);  // whole folds, bit-reversed
         else
             sum_partials(area, a.chunks, H, a.logB, U);
-        if (LARGE)
-            fft_rows(U, H, a.logB);
-        else
-            block_fft_rows<R>(U, H, a.logB);  // starts and ends with a barrier
+        fft_rows<LARGE>(a, U);  // starts and ends with a barrier
         if (!(part & kFinDecode)) {  // every partial fold has been read: the area takes the bins
             for (uint32_t i = tid; i < H * B; i += kThreads) area[i] = U[i];
             return false;
@@ -794,7 +899,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
             double2 t0 = gz;  // hashing 0 has offset 0 in the transform's rounds: w^0 = 1
             const uint32_t e0 = (a0 * sigma * i) & a.nmask;
             if (e0 != 0) {
-                const double2 w = root_pow<R>(e0, a.nmask);
+                const double2 w = term_root<R>(a, e0);
                 t0 = make_double2(gz.x * w.x - gz.y * w.y, gz.x * w.y + gz.y * w.x);
             }
             ent_sub[e] = t0;
@@ -842,7 +947,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         for (uint32_t q = tid; q < nz * H; q += kThreads) {
             const uint32_t e = q / H, h = q - e * H;
             const uint32_t i = ent_idx[e];
-            const double2 w = root_pow<R>(((a.a_base + a.a[h]) * sigma * i) & a.nmask, a.nmask);
+            const double2 w = term_root<R>(a, ((a.a_base + a.a[h]) * sigma * i) & a.nmask);
             const double2 gz = make_double2(ent_gain[e] * ent_val[e].x, ent_gain[e] * ent_val[e].y);
             const double2 t = make_double2(gz.x * w.x - gz.y * w.y, gz.x * w.y + gz.y * w.x);
             ent_sub[q] = t;
@@ -973,7 +1078,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
             if (f32)
                 kp = hypotf((float)v.x, (float)v.y) < a.drop_f ? 0u : 1u;
             else
-                kp = cmag<R>(v) < a.prune * a.thr ? 0u : 1u;
+                kp = dropped(v, a) ? 0u : 1u;
         }
         keep[p] = kp;
     }
@@ -1119,6 +1224,12 @@ __device__ __forceinline__ bool worth_decoding(const DecodeCtx& d, float2 u, boo
     return m > d.thr_f || (entries && m > d.ref_lo_f && m <= d.ref_hi_f);
 }
 __device__ __forceinline__ bool worth_decoding(const DecodeCtx& d, double2 u, bool entries) {
+    const float f = hypotf((float)u.x, (float)u.y);
+    if (d.thr_f > 1e-25f && d.thr_f < 1e25f && f < 1e18f) {  // clear of every bound: as decode_bin_guarded
+        if (cmp_guarded(f, d.thr_f) > 0) return true;
+        if (cmp_guarded(f, d.thr_f) < 0 && (!entries || cmp_guarded(f, d.ref_hi_f) > 0 || cmp_guarded(f, d.ref_lo_f) < 0))
+            return false;
+    }
     const double m = cmag<double>(u);
     return m > d.thr || (entries && m > d.ref_lo * d.thr && m <= d.ref_hi * d.thr);
 }
@@ -1290,7 +1401,7 @@ __device__ __forceinline__ bool finish_large(const ExactArgs& a, uint32_t s, uin
                 } else {
                     double2 r = gz;
                     if (ex != 0) {
-                        const double2 tw = root_pow<R>(ex, a.nmask);
+                        const double2 tw = term_root<R>(a, ex);
                         r = make_double2(gz.x * tw.x - gz.y * tw.y, gz.x * tw.y + gz.y * tw.x);
                     }
                     w.x = r.x;
@@ -1470,7 +1581,7 @@ __device__ __forceinline__ bool finish_large(const ExactArgs& a, uint32_t s, uin
                 if (f32)
                     kp = hypotf((float)v.x, (float)v.y) < a.drop_f ? 0u : 1u;
                 else
-                    kp = cmag<R>(v) < a.prune * a.thr ? 0u : 1u;
+                    kp = dropped(v, a) ? 0u : 1u;
             }
             keep[p] = kp;
         }

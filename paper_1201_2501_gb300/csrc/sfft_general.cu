@@ -638,14 +638,6 @@ __device__ void locate_bin(uint32_t t, uint32_t nrep, const uint64_t* beta, Phas
 // ------------------------------------------------------------------------------------------------
 // w_i = median_q Re e_q + i median_q Im e_q over the hashings q whose window gain at i is >= est_gmin,
 // e_q = u^{(q)}_{h_q(i)} w^{-a_q sigma_q i} / W(-o_q(i)); lower median; 0 when no hashing qualifies.
-// w^e = exp(-2 pi i e / n) for an exact exponent e in [0, n) from two tables of FP64 factors,
-// exp(-2 pi i (e mod 2^sh) / n) and exp(-2 pi i 2^sh (e >> sh) / n): one complex product (a few ulp
-// from a direct evaluation) instead of an FP64 sincospi, which GB300 runs at 1/64 of the FP32 rate
-__device__ __forceinline__ double2 root_pow_tab(uint32_t e, const double2* tw, uint32_t sh) {
-    const double2 lo = tw[e & ((1u << sh) - 1u)], hi = tw[(1u << sh) + (e >> sh)];
-    return make_double2(hi.x * lo.x - hi.y * lo.y, hi.x * lo.y + hi.y * lo.x);
-}
-
 // e_q of candidate i under one hashing (sigma, b, a) with bins u; false where the window gain is too small
 __device__ __forceinline__ bool estimate_term(uint32_t i, uint32_t sigma, uint32_t b, uint32_t a, const double2* u,
                                               uint32_t n, uint32_t nmask, uint32_t logNp, const double* wtab, double gmin,

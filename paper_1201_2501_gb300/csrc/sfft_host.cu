@@ -220,6 +220,24 @@ void twiddle_tables_host(uint64_t n, uint32_t sh, std::vector<double2>* out) {
     for (uint64_t a = 0; a < hi; ++a) (*out)[lo + a] = root_of_unity(a << sh, n);
 }
 
+void twiddle_tables_exact_host(uint64_t n, uint32_t sh, std::vector<double2>* out) {
+    const uint64_t lo = uint64_t(1) << sh, hi = n >> sh;
+    const long double two_pi = 6.283185307179586476925286766559005768L;
+    auto root = [&](uint64_t m) {
+        const long double th = two_pi * (long double)m / (long double)n;
+        return make_double2((double)cosl(th), (double)-sinl(th));
+    };
+    out->resize(lo + hi);
+    for (uint64_t b = 0; b < lo; ++b) {  // cos - 1 = -2 sin^2 of the half angle
+        const long double half = sinl(two_pi * (long double)b / (long double)n / 2);
+        (*out)[b] = make_double2((double)(-2 * half * half), root(b).y);
+    }
+    for (uint64_t a = 0; a < hi; ++a) (*out)[lo + a] = root(a << sh);
+    // the quarter turns exactly
+    for (int q = 1; q < 4 && hi >= 4; ++q)
+        (*out)[lo + hi / 4 * q] = make_double2(q == 2 ? -1.0 : 0.0, q == 1 ? -1.0 : (q == 3 ? 1.0 : 0.0));
+}
+
 void window_gprime_host(uint64_t n, uint32_t B, double alpha, double delta, uint64_t len, double* W) {
     const double nn = (double)n, z = std::sqrt(2.0 * std::log(1.0 / delta));
     const double C = (1.0 - alpha / 2.0) / (2.0 * (double)B), sf = alpha / (4.0 * (double)B * z);

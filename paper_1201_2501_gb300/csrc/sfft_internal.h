@@ -80,6 +80,8 @@ struct ExactArgs {
     const double* taps64;
     const double* wtab;
     const double* winv;        // 1 / W(o) for the same o (null: the decode divides by W(o))
+    const double2* tw;         // FP64 data path: w^e = (1 + tw[e mod 2^tw_shift]) tw[2^tw_shift + (e >> tw_shift)]
+    uint32_t tw_shift, logn;
     void* part;                // partial fold sums: request s owns [s part_stride, (s + 1) part_stride),
                                // laid out [chunks][H][B] complex R (requests may be in different rounds)
     size_t part_stride;
@@ -315,7 +317,7 @@ struct sfft_plan_s {
     double2* d_bins = nullptr;
     uint32_t* d_phase = nullptr;
     uint32_t* d_L = nullptr;  // general mode: per round r, [max_batch][B_r] candidates
-    double2* d_tw = nullptr;  // general mode: FP64 twiddle factor tables (2^tw_shift + n / 2^tw_shift)
+    double2* d_tw = nullptr;  // general mode, exact FP64: twiddle factor tables (2^tw_shift + n / 2^tw_shift)
     uint32_t tw_shift = 0;
     float2* d_xperm = nullptr;  // general mode, per round with perm: [max_batch][n] permuted signals
     // general mode: per round r, [max_batch][B_r] estimates; then per round [max_batch][B_r] magnitudes
@@ -392,6 +394,8 @@ inline uint32_t ilog2_host(uint64_t v) {  // v a power of two
 // FP64 twiddle factor tables for n = 2^L and split sh: out[b] = exp(-2 pi i b / n), b < 2^sh, then
 // out[2^sh + a] = exp(-2 pi i a 2^sh / n), a < n / 2^sh
 void twiddle_tables_host(uint64_t n, uint32_t sh, std::vector<double2>* out);
+// the same less one in the first part (root_pow_fine), every entry rounded from extended precision
+void twiddle_tables_exact_host(uint64_t n, uint32_t sh, std::vector<double2>* out);
 void window_table_host(uint64_t n, const double* g, int64_t T, uint64_t len, double* W);
 int64_t window_halfwidth(uint32_t B, double alpha, double delta);
 void draw_exact_host(uint64_t seed, uint32_t request, uint32_t round, uint64_t n, uint64_t* sigma, uint64_t* b);

@@ -72,3 +72,51 @@ def test_large_plans_match_oracle(sf, m, k, prec, batch, over):
         assert np.array_equal(mixed[0][r, :c], idx[r, :c]) and np.array_equal(mixed[1][r, :c], val[r, :c])
     for q in (bp, plan, small):
         q.close()
+
+
+@pytest.mark.parametrize("m,k,t", [(14, 8, 0), (18, 64, 0), (22, 64, 1), (20, 128, 0)])
+def test_fp64_decisions_at_their_boundaries(sf, m, k, t):
+    """The FP64 data path takes a decision in FP32 only where FP64 agrees: bins whose magnitude, isolation,
+    ladder rounding or re-estimation window lies 1e-12 to 1e-2 (relative) from its boundary, on both
+    sides, decode as the oracle's FP64 does, bit for bit (values within 1e-12)."""
+    n = 1 << m
+    f = exact_fields(n, k)
+    P = oracle_params(f)
+    plan = sf.Plan(_params(sf, f, 1), 1)
+    info = plan.round_info(t, seed=5)
+    B, shifts = info["B"], info["shifts"]
+    Np, L = n // B, len(shifts)
+    rng = np.random.default_rng(m + t)
+    near = lambda size: rng.choice([-1, 1], size) * 10.0 ** rng.uniform(-12, -2, size)
+    for trial in range(24):
+        sigma, b = int(rng.integers(0, n)) | 1, int(rng.integers(0, n))
+        mag = np.where(rng.random(B) < 0.5, P.thr * (1 + near(B)), 10.0 ** rng.uniform(-0.5, 1, B))
+        u = np.zeros((1 + L, B), dtype=np.complex128)
+        u[0] = mag * np.exp(2j * np.pi * rng.random(B))
+        c, M = np.zeros(B), 1.0
+        for l in range(L - 1, -1, -1):  # coarsest first: th 2^logRatio - c / M close to a half-integer, or not
+            ratio = Np / (shifts[l] // B) / M
+            y = np.floor(rng.random(B) * ratio) + np.where(rng.random(B) < 0.5, 0.5 + near(B), 0.3 * rng.uniform(-1, 1, B))
+            th = (y + c / M) / ratio
+            c = c + M * (np.floor(y + 0.5) % ratio)
+            M *= ratio
+            size = np.where(rng.random(B) < 0.5, 1 + rng.choice([-1, 1], B) * P.iso_tol * (1 + near(B)), 1.0)
+            u[l + 1] = u[0] * size * np.exp(-2j * np.pi * th)
+        known = np.sort(rng.choice(n, size=max(2, B // 4), replace=False)).astype(np.uint32)
+        for i in known:
+            j, _ = oracle.bin_offset((sigma * (int(i) - b)) % n, n, B)
+            edge = rng.choice([P.ref_lo, P.ref_hi]) * P.thr * (1 + float(near(1)[0]))
+            for h, be in enumerate([0] + list(shifts)):
+                u[h, j] = edge * np.exp(-2j * np.pi * ((be * sigma * int(i)) % n) / n)
+        widx, wval, aux = sf.sfft_exact_decode(plan, t, sigma, b, torch.as_tensor(np.stack([u.real, u.imag], -1)).cuda(),
+                                               torch.as_tensor(known.astype(np.int32)).cuda())
+        torch.cuda.synchronize()
+        cnt, nab, nkept = [int(v) for v in aux.cpu().numpy()]
+        oi, ov, oab, okept = oracle.exact_decode(P, B, info["alpha"], sigma, b, shifts, u, known.astype(np.uint64),
+                                                 with_kept=True)
+        order = np.argsort(oi)
+        assert (nab, nkept) == (oab, okept)
+        assert np.array_equal(widx.cpu().numpy()[:cnt].astype(np.uint32).astype(np.int64), oi[order].astype(np.int64))
+        v = wval.cpu().numpy()[:cnt]
+        assert np.max(np.abs(v[:, 0] + 1j * v[:, 1] - ov[order]) / np.maximum(1.0, np.abs(ov[order])), initial=0.0) <= 1e-12
+    plan.close()
