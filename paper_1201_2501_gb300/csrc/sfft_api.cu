@@ -30,6 +30,11 @@ sfft_status cuda_fail(cudaError_t e, const char* what) {
 
 bool is_pow2(uint64_t v) { return v && !(v & (v - 1)); }
 
+// the counts and flags of requests [0, batch) (the counts of the others with them)
+cudaError_t clear_zhat(const sfft_plan_s* pl, uint32_t batch, cudaStream_t st) {
+    return cudaMemsetAsync(pl->d_zcount, 0, ((size_t)pl->max_batch + batch) * sizeof(uint32_t), st);
+}
+
 sfft_status validate(const sfft_params* p) {
     if (!p) return SFFT_ERR_INVALID_ARG;
     if (!is_pow2(p->n) || p->n < 64 || p->n > (uint64_t(1) << 30)) return SFFT_ERR_N_NOT_POW2;
@@ -58,7 +63,6 @@ void free_plan(sfft_plan_s* pl) {
     cudaFree(pl->d_zidx);
     cudaFree(pl->d_zval);
     cudaFree(pl->d_zcount);
-    cudaFree(pl->d_zflag);
     cudaFree(pl->d_ubins);
     cudaFree(pl->d_aux);
     cudaFree(pl->d_reqs);
@@ -106,7 +110,7 @@ ExactArgs base_args(const sfft_plan_s* pl, const ExactRound& r, uint32_t t) {
     a.chunks = r.chunks;
     a.owner = r.owner ? 1 : 0;
     a.ring = r.ring;
-    a.gctas = r.owner ? r.B / (uint32_t)kThreads : r.chunks;
+    a.gctas = r.owner ? r.B / kOwnerRes : r.chunks;
     a.large = r.large ? 1 : 0;
     a.large_smem = kLargeSmem;
     a.ctaps = r.ctaps;
@@ -271,8 +275,8 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
 
     SFFT_ALLOC(pl->d_zidx, (size_t)max_batch * p->z_cap * sizeof(uint32_t));
     SFFT_ALLOC(pl->d_zval, (size_t)max_batch * p->z_cap * sizeof(double2));
-    SFFT_ALLOC(pl->d_zcount, (size_t)max_batch * sizeof(uint32_t));
-    SFFT_ALLOC(pl->d_zflag, (size_t)max_batch * sizeof(int32_t));
+    SFFT_ALLOC(pl->d_zcount, (size_t)max_batch * 2 * sizeof(uint32_t));
+    pl->d_zflag = reinterpret_cast<int32_t*>(pl->d_zcount + max_batch);
     SFFT_ALLOC(pl->d_ubins, (size_t)maxB * kMaxHash * sizeof(double2));
     SFFT_ALLOC(pl->d_aux, 64 * sizeof(uint32_t));
     SFFT_ALLOC(pl->d_reqs, (size_t)max_batch * sizeof(ReqDesc));
@@ -431,8 +435,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
                                    uint32_t* d_idx, double* d_val, uint32_t cap, uint32_t* d_count, int32_t* d_flag,
                                    const sfft_general_trace* tr = nullptr) {
     const sfft_params& p = plan->p;
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zcount, 0, batch * sizeof(uint32_t), st), "clear zhat");
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zflag, 0, batch * sizeof(int32_t), st), "clear flags");
+    SFFT_CUDA(clear_zhat(plan, batch, st), "clear zhat");
     const uint32_t R = (uint32_t)plan->grounds.size();
     // stream groups may run different rounds at once, so every round has its own regions: candidates,
     // estimates and magnitudes from max_batch boff[r]
@@ -566,8 +569,7 @@ sfft_status sfft::execute_batch(sfft_plan plan, const void* d_x, const ReqDesc* 
     if (plan->p.mode == SFFT_GENERAL)
         return execute_general(plan, d_x, d_reqs, batch, seed, st, d_idx, d_val, cap, d_count, d_flag);
     const bool fp64 = plan->p.precision == SFFT_FP64;
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zcount, 0, batch * sizeof(uint32_t), st), "clear zhat");
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zflag, 0, batch * sizeof(int32_t), st), "clear flags");
+    SFFT_CUDA(clear_zhat(plan, batch, st), "clear zhat");
     const uint32_t R = (uint32_t)plan->rounds.size();
     // One launch per group covers every round (k_exact_step).  Requests are independent, so the batch
     // may be cut into groups on separate streams: one group's last finishers overlap the next group's
@@ -624,8 +626,7 @@ static sfft_status execute_channels(sfft_plan plan, const void* d_x, uint32_t ch
         return SFFT_ERR_INVALID_ARG;
     if (channels == 0 || channels % 32 || channels > kChanMaxC || channels > plan->max_batch || ((uintptr_t)d_x & 15))
         return SFFT_ERR_INVALID_ARG;
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zcount, 0, channels * sizeof(uint32_t), st), "clear zhat");
-    SFFT_CUDA(cudaMemsetAsync(plan->d_zflag, 0, channels * sizeof(int32_t), st), "clear flags");
+    SFFT_CUDA(clear_zhat(plan, channels, st), "clear zhat");
     const uint32_t R = (uint32_t)plan->rounds.size();
     ExactArgs rounds[kMaxRounds];
     for (uint32_t t = 0; t < R; ++t) {

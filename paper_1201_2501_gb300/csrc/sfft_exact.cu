@@ -38,6 +38,7 @@ __device__ __forceinline__ const double* taps_of<double>(const ExactArgs& a) {
     return a.taps64;
 }
 
+static_assert(kThreads / kOwnerRes >= kMaxHash, "a thread per (residue, hashing)");
 // samples in flight per thread of gather_owner
 template <typename R>
 __host__ __device__ constexpr uint32_t owner_loads() {
@@ -48,8 +49,7 @@ __host__ __device__ constexpr uint32_t owner_loads() {
 // shared-memory layout of the finishing phase
 // ------------------------------------------------------------------------------------------------
 struct FinLayout {
-    size_t U, ent_idx, ent_bin, ent_val, ent_gain, ent_sub, ent_sub_f, bin_cnt, bin_start, bin_list, cand_idx, cand_bin, cand_gain,
-        cand_val, srt_idx, srt_val, out_idx, out_val, keep, scan;
+    size_t U, ent_idx, ent_bin, ent_val, ent_gain, ent_sub, ent_sub_f, mask, bin_cnt, bin_start, bin_list, cand_idx, cand_val, srt_idx, srt_val, out_idx, out_val, keep, scan;
     size_t total;
 };
 __host__ __device__ inline size_t fin_take(size_t* off, size_t bytes) {
@@ -57,7 +57,8 @@ __host__ __device__ inline size_t fin_take(size_t* off, size_t bytes) {
     *off = o + bytes;
     return o;
 }
-__host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t zcap, uint32_t csize) {
+// masks: the entries of each bin as bits (the transform's decode), instead of as lists
+__host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t zcap, uint32_t csize, bool masks = false) {
     FinLayout L;
     size_t off = 0;
     L.U = fin_take(&off, (size_t)H * B * csize);
@@ -67,12 +68,12 @@ __host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t
     L.ent_gain = fin_take(&off, (size_t)zcap * 8);
     L.ent_sub = fin_take(&off, (size_t)zcap * H * 16);
     L.ent_sub_f = fin_take(&off, (size_t)zcap * H * 8);
-    L.bin_cnt = fin_take(&off, (size_t)(B + 1) * 4);
-    L.bin_start = fin_take(&off, (size_t)(B + 1) * 4);
-    L.bin_list = fin_take(&off, (size_t)zcap * 4);
+    L.mask = fin_take(&off, masks ? (size_t)B * ((zcap + 31) / 32) * 4 : 0);
+    L.bin_cnt = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
+    L.bin_start = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
+    L.bin_list = fin_take(&off, masks ? 0 : (size_t)zcap * 4);
     L.cand_idx = fin_take(&off, (size_t)B * 4);
-    L.cand_bin = fin_take(&off, (size_t)B * 4);
-    L.cand_gain = fin_take(&off, (size_t)B * 8);
+    if (!masks) fin_take(&off, (size_t)B * 12);
     L.cand_val = fin_take(&off, (size_t)B * 16);
     L.srt_idx = fin_take(&off, (size_t)B * 4);
     L.srt_val = fin_take(&off, (size_t)B * 16);
@@ -87,15 +88,21 @@ __host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t
 size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
     return fin_layout(B, H, zcap, fp64 ? 16 : 8).total;
 }
-size_t exact_gather_smem(uint32_t stage, bool fp64) { return (size_t)stage * (fp64 ? 16 : 8); }
-size_t exact_owner_smem(uint32_t ring, bool fp64) {  // samples and taps of every thread
-    return (size_t)kThreads * (fp64 ? ring * 16 + owner_loads<double>() * 8 : ring * 8 + owner_loads<float>() * 4);
+size_t exact_decode_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
+    return fin_layout(B, H, zcap, fp64 ? 16 : 8, true).total;
 }
-// samples a thread of gather_owner keeps: those of a batch of loads and of the longest shift
+size_t exact_gather_smem(uint32_t stage, bool fp64) { return (size_t)stage * (fp64 ? 16 : 8); }
+constexpr uint32_t owner_batch(bool fp64) {  // taps of a residue per batch
+    return (fp64 ? owner_loads<double>() : owner_loads<float>()) * (kThreads / kOwnerRes);
+}
+size_t exact_owner_smem(uint32_t ring, bool fp64) {  // samples and factors
+    return (size_t)(ring + owner_batch(fp64)) * kOwnerRes * (fp64 ? 16 : 8);
+}
+// samples gather_owner keeps of a residue: those of a batch and of the longest shift (0: too many)
 uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64) {
     uint32_t r = 1;
-    while (r < (fp64 ? owner_loads<double>() : owner_loads<float>()) + maxshift / B) r <<= 1;
-    return r;
+    while (r < owner_batch(fp64) + maxshift / B) r <<= 1;
+    return r <= 2 * owner_batch(fp64) ? r : 0;
 }
 
 // g w^e of a tap, w = exp(-2 pi i / n), e = sigma b t (taken mod n): a sincospif in FP32; from the factor
@@ -218,15 +225,49 @@ __device__ void fill_ctx_round(DecodeCtx& d, const ExactArgs& a, uint32_t sigma,
 // ladder keeps a tolerance of at least tau_dec per level and GB300 issues FP64 at 1/64 of FP32, so FP64
 // arithmetic there would cost most of the finisher's time and change no decision outside a
 // measure-zero band at the thresholds.
-// kDirect: the bin's entries are ent_*[x], x < nbin, instead of ent_*[list[x]]; a decode is returned
-// before its window gain is read, with the signed offset o in *oi, and a re-estimate with its x there.
+// The zhat entries hashed to a bin, in ascending order of their ids e: f(e) for each.  kDirect: ids count
+// from the bin's first place, and a decode is returned before its window gain is read, with the signed
+// offset o in *oi, or with the id of the entry a re-estimate corrects.
+struct ListEntries {
+    static constexpr bool kDirect = false;
+    const uint32_t* list;
+    uint32_t count;
+    __device__ __forceinline__ bool any() const { return count != 0; }
+    template <typename F>
+    __device__ __forceinline__ void each(F f) const {
+        for (uint32_t x = 0; x < count; ++x) f(list[x]);
+    }
+};
+struct RunEntries {
+    static constexpr bool kDirect = true;
+    uint32_t count;
+    __device__ __forceinline__ bool any() const { return count != 0; }
+    template <typename F>
+    __device__ __forceinline__ void each(F f) const {
+        for (uint32_t x = 0; x < count; ++x) f(x);
+    }
+};
+struct MaskEntries {  // bit e mod 32 of words[(e / 32) stride]
+    static constexpr bool kDirect = false;
+    const uint32_t* words;
+    uint32_t stride, nwords;
+    __device__ __forceinline__ bool any() const {
+        uint32_t m = 0;
+        for (uint32_t w = 0; w < nwords; ++w) m |= words[w * stride];
+        return m != 0;
+    }
+    template <typename F>
+    __device__ __forceinline__ void each(F f) const {
+        for (uint32_t w = 0; w < nwords; ++w)
+            for (uint32_t m = words[w * stride]; m != 0; m &= m - 1u) f(w * 32u + (uint32_t)__ffs((int)m) - 1u);
+    }
+};
 __device__ __forceinline__ uint32_t index_at(const DecodeCtx& d, uint32_t j, int32_t o) {
     const uint32_t p = (j * d.Np + (uint32_t)o) & d.nmask;
     return (d.sigma_inv * ((p + d.sb) & d.nmask)) & d.nmask;
 }
-template <bool kDirect>
-__device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list, uint32_t nbin,
-                               const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
+template <typename Ents>
+__device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const Ents ents, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
                                double* ginv, bool* above) {
     const double mag0 = cmag<double>(u[0]);
     *ginv = 0.0;  // the FP64 path divides
@@ -234,7 +275,7 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
     *above = false;
     if (!(mag0 > d.thr)) {
         // re-estimation of a known value: exactly one entry of the bin must explain the residual
-        if (nbin == 0 || !(mag0 > d.ref_lo * d.thr && mag0 <= d.ref_hi * d.thr)) return 0;
+        if (!ents.any() || !(mag0 > d.ref_lo * d.thr && mag0 <= d.ref_hi * d.thr)) return 0;
         double th[kMaxHash];
         for (uint32_t l = 0; l < L; ++l) {
             if (fabs(cmag<double>(u[l + 1]) - mag0) > 0.25 * mag0) return 0;
@@ -242,11 +283,10 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
         }
         uint32_t matches = 0, who = 0;
         double gw = 1.0;
-        for (uint32_t x = 0; x < nbin; ++x) {
-            const uint32_t e = kDirect ? x : list[x];
+        ents.each([&](uint32_t e) {
             const uint32_t i = ent_idx[e];
             const double gain = ent_gain[e];
-            if (!(gain >= d.gmin)) continue;
+            if (!(gain >= d.gmin)) return;
             bool ok = true;
             for (uint32_t l = 0; l < L && ok; ++l) {
                 const uint32_t ph = (d.shift[l] * d.sigma * i) & d.nmask;
@@ -256,10 +296,10 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
             }
             if (ok) {
                 ++matches;
-                who = kDirect ? x : i;
+                who = Ents::kDirect ? e : i;
                 gw = gain;
             }
-        }
+        });
         if (matches != 1) return 0;
         *oi = who;
         *gout = gw;
@@ -286,7 +326,7 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
     const uint32_t i = index_at(d, j, o);
     for (uint32_t l = 0; l < L; ++l)
         if (fabs(cmag<double>(u[l + 1]) - mag0) > d.iso_tol * mag0) return 0;
-    if (kDirect) {
+    if (Ents::kDirect) {
         *oi = (uint32_t)o;
         return 1;
     }
@@ -311,9 +351,9 @@ __device__ __forceinline__ float pow2_f(int e) { return __int_as_float((127 + e)
 
 // Every loop over hashings is unrolled to kMaxHash with compile-time indices, so u[] and the
 // phases stay in registers.
-template <bool kDirect>
-__device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, const float2* u, const uint32_t* list,
-                                               uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain,
+template <typename Ents>
+__device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, const float2* u, const Ents& ents,
+                                               const uint32_t* ent_idx, const double* ent_gain,
                                                uint32_t* oi, double* gout, double* ginv, bool* above) {
     const float mag0 = hypotf(u[0].x, u[0].y);
     *ginv = 0.0;
@@ -321,7 +361,7 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
     *above = false;
     if (!(mag0 > d.thr_f)) {
         // re-estimation of a known value: exactly one entry of the bin must explain the residual
-        if (nbin == 0 || !(mag0 > d.ref_lo_f && mag0 <= d.ref_hi_f)) return 0;
+        if (!ents.any() || !(mag0 > d.ref_lo_f && mag0 <= d.ref_hi_f)) return 0;
         float th[kMaxHash - 1];
 #pragma unroll
         for (int l = 0; l < kMaxHash - 1; ++l) {
@@ -333,11 +373,10 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
         }
         uint32_t matches = 0, who = 0;
         double gw = 1.0;
-        for (uint32_t x = 0; x < nbin; ++x) {
-            const uint32_t e = kDirect ? x : list[x];
+        ents.each([&](uint32_t e) {
             const uint32_t i = ent_idx[e];
             const double gain = ent_gain[e];
-            if (!(gain >= d.gmin)) continue;
+            if (!(gain >= d.gmin)) return;
             bool ok = true;
 #pragma unroll
             for (int l = 0; l < kMaxHash - 1; ++l) {
@@ -350,10 +389,10 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
             }
             if (ok) {
                 ++matches;
-                who = kDirect ? x : i;
+                who = Ents::kDirect ? e : i;
                 gw = gain;
             }
-        }
+        });
         if (matches != 1) return 0;
         *oi = who;
         *gout = gw;
@@ -392,7 +431,7 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
 #pragma unroll
     for (int l = 0; l < kMaxHash - 1; ++l)
         if ((uint32_t)l < L && fabsf(hypotf(u[l + 1].x, u[l + 1].y) - mag0) > d.iso_tol_f * mag0) return 0;
-    if (kDirect) {
+    if (Ents::kDirect) {
         *oi = (uint32_t)o;
         return 1;
     }
@@ -419,9 +458,8 @@ __device__ __forceinline__ int cmp_guarded(float m, float t) {
     return m > t + g ? 1 : (m < t - g ? -1 : 0);
 }
 constexpr int kUndecided = -1;
-template <bool kDirect>
-__device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list,
-                                                  uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain,
+template <typename Ents>
+__device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j, const double2* u, const Ents& ents,
                                                   uint32_t* oi, double* gout, double* ginv, bool* above) {
     float2 v[kMaxHash];
     const uint32_t L = d.H - 1;
@@ -436,7 +474,7 @@ __device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j
     const int over = cmp_guarded(mag0, d.thr_f);
     if (over == 0) return kUndecided;
     if (over < 0) {
-        if (nbin == 0) return 0;
+        if (!ents.any()) return 0;
         const int lo = cmp_guarded(mag0, d.ref_lo_f), hi = cmp_guarded(mag0, d.ref_hi_f);
         return lo < 0 || hi > 0 ? 0 : kUndecided;  // (a re-estimation is decided in FP64)
     }
@@ -469,7 +507,7 @@ __device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j
             if (df > t + g) return 0;
             if (!(df < t - g)) return kUndecided;
         }
-    if (kDirect) {
+    if (Ents::kDirect) {
         *oi = (uint32_t)o;
         return 1;
     }
@@ -480,65 +518,62 @@ __device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j
     return 1;
 }
 
-template <bool kDirect = false>
-__device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const double2* u, const uint32_t* list,
-                                          uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
+template <typename Ents>
+__device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const double2* u, const Ents& ents,
+                                          const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
                                           double* gout, double* ginv, bool* above) {
-    const int kind = decode_bin_guarded<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
-    return kind != kUndecided ? kind
-                              : decode_bin_fp64<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    const int kind = decode_bin_guarded(d, j, u, ents, oi, gout, ginv, above);
+    return kind != kUndecided ? kind : decode_bin_fp64(d, j, u, ents, ent_idx, ent_gain, oi, gout, ginv, above);
 }
-template <bool kDirect = false>
-__device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const float2* u, const uint32_t* list,
-                                          uint32_t nbin, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
+template <typename Ents>
+__device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const float2* u, const Ents& ents,
+                                          const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi,
                                           double* gout, double* ginv, bool* above) {
-    return decode_bin_fp32<kDirect>(d, j, u, list, nbin, ent_idx, ent_gain, oi, gout, ginv, above);
+    return decode_bin_fp32(d, j, u, ents, ent_idx, ent_gain, oi, gout, ginv, above);
 }
 
 // Bin j's hashings after the subtraction of zhat, for the decisions: u_h = U_h - sum over the bin's
 // entries e (in list order) of sub[e H + h], in the data path's precision (FP64 terms and sums for
 // the FP64 path; the terms rounded to FP32 and summed in FP32 for the FP32 path, whose bins carry
 // ~1e-6 of rounding).  The values of decoded bins are formed separately from subtracted_u0 in FP64.
-__device__ __forceinline__ void subtracted_bin(const double2* U, uint32_t B, uint32_t H, uint32_t j,
-                                               const uint32_t* list, uint32_t nbin, const double2* sub,
-                                               const float2* /*sub_f*/, double2* u) {
+template <typename Ents>
+__device__ __forceinline__ void subtracted_bin(const double2* U, uint32_t B, uint32_t H, uint32_t j, const Ents& ents,
+                                               const double2* sub, const float2* /*sub_f*/, double2* u) {
     for (uint32_t h = 0; h < H; ++h) {
         double2 w = U[h * B + j];
-        for (uint32_t x = 0; x < nbin; ++x) {
-            const uint32_t e = list[x];
+        ents.each([&](uint32_t e) {
             w.x -= sub[e * H + h].x;
             w.y -= sub[e * H + h].y;
-        }
+        });
         u[h] = w;
     }
 }
-__device__ __forceinline__ void subtracted_bin(const float2* U, uint32_t B, uint32_t H, uint32_t j,
-                                               const uint32_t* list, uint32_t nbin, const double2* /*sub*/,
-                                               const float2* sub_f, float2* u) {
+template <typename Ents>
+__device__ __forceinline__ void subtracted_bin(const float2* U, uint32_t B, uint32_t H, uint32_t j, const Ents& ents,
+                                               const double2* /*sub*/, const float2* sub_f, float2* u) {
 #pragma unroll
     for (int h = 0; h < kMaxHash; ++h) u[h] = (uint32_t)h < H ? U[h * B + j] : make_float2(0.0f, 0.0f);
-    for (uint32_t x = 0; x < nbin; ++x) {
-        const float2* t = sub_f + list[x] * H;
+    ents.each([&](uint32_t e) {
+        const float2* t = sub_f + e * H;
 #pragma unroll
         for (int h = 0; h < kMaxHash; ++h)
             if ((uint32_t)h < H) {
                 u[h].x -= t[h].x;
                 u[h].y -= t[h].y;
             }
-    }
+    });
 }
 // u_0 of bin j after the subtraction, in FP64 (the first row of subtracted_bin, same order); entry e's
 // FP64 term of hashing 0 is sub[e * stride]
-template <typename C>
-__device__ __forceinline__ double2 subtracted_u0(const C* U, uint32_t stride, uint32_t j, const uint32_t* list,
-                                                 uint32_t nbin, const double2* sub) {
+template <typename C, typename Ents>
+__device__ __forceinline__ double2 subtracted_u0(const C* U, uint32_t stride, uint32_t j, const Ents& ents,
+                                                 const double2* sub) {
     const C v = U[j];
     double2 w = make_double2((double)v.x, (double)v.y);
-    for (uint32_t x = 0; x < nbin; ++x) {
-        const uint32_t e = list[x];
+    ents.each([&](uint32_t e) {
         w.x -= sub[e * stride].x;
         w.y -= sub[e * stride].y;
-    }
+    });
     return w;
 }
 
@@ -621,86 +656,81 @@ __device__ void gather_fold(const ExactArgs& a, const void* xrow, uint32_t xmask
     }
 }
 
-// The same fold with a CTA owning kThreads residues of the round (rounds of kOwnerB bins or more): one
-// residue per thread, which folds all its taps, so that no partial fold leaves the CTA (B = 4096 has
-// about 140 chunks, whose partial folds one CTA would have to add).  The ladder's shifts are multiples
-// of B, so the samples of every hashing's tap t, x_{sigma (t - a_h)}, are the thread's own: it keeps the
-// last ones in its column of shared memory and needs no barrier.  Order of the sums: that of the
-// chunks (a residue's taps of a chunk from zero, then the chunks in order), so the bits are the same.
-// Bound by random sectors (16 in flight per thread in FP32, 8 in FP64).
+// The same fold with a CTA owning kOwnerRes residues of the round (rounds of kThreads bins or more of
+// large plans), so that no partial fold leaves the CTA (B = 4096 has about 140 chunks, whose partial folds
+// one CTA would have to add).  Four threads load a residue's taps, a batch of loads ahead of the fold; the
+// taps' factors are formed once into shared memory, and thread (residue, h) folds hashing h.  The ladder's
+// shifts are multiples of B, so the samples of every hashing's tap t, x_{sigma (t - a_h)}, are the
+// residue's own: the last ones stay in its column of the ring.  Order of the sums: that of the chunks (a
+// residue's taps of a chunk from zero, then the chunks in order), so the bits are the same.
+// Bound by random sectors.  64 residues a CTA, not 256: at n = 2^22, k = 227, batch 33 round 0 then has
+// more CTAs than the chip has places and ends before the later rounds' gathers share the bandwidth.
 template <typename R>
 __device__ __forceinline__ void gather_owner(const ExactArgs& a, const void* xrow, uint32_t xmask, uint32_t s,
                                              uint32_t blk, uint32_t sigma, uint32_t b, unsigned char* smem) {
     using C = typename Cx<R>::T;
-    constexpr uint32_t kLoads = owner_loads<R>();
-    const uint32_t tid = threadIdx.x, B = a.B, H = a.H;
-    C* ring = reinterpret_cast<C*>(smem) + tid;  // [a.ring][kThreads], this thread's column
-    R* tap = reinterpret_cast<R*>(reinterpret_cast<C*>(smem) + a.ring * kThreads) + tid;  // [kLoads][kThreads]
+    constexpr uint32_t kLoads = owner_loads<R>(), kQ = kThreads / kOwnerRes, kBatch = kLoads * kQ;
+    const uint32_t lr = threadIdx.x & (kOwnerRes - 1), q = threadIdx.x / kOwnerRes, B = a.B, H = a.H;
+    C* ring = reinterpret_cast<C*>(smem) + lr;      // [a.ring][kOwnerRes], this residue's column
+    C* factor = ring + (size_t)a.ring * kOwnerRes;  // [kBatch][kOwnerRes]
     const uint32_t rmask = a.ring - 1u;
     const C* __restrict__ x = reinterpret_cast<const C*>(xrow);
     const R* __restrict__ taps = taps_of<R>(a);
-    const uint32_t first = blk * kThreads, i0 = first + tid;   // first tap -T + i0, then every B-th
+    const uint32_t first = blk * kOwnerRes, i0 = first + lr;  // first tap -T + i0, then every B-th
     const uint32_t ntot = (uint32_t)(2 * a.T + 1);
-    const uint32_t mend = first < ntot ? (ntot - first + B - 1) / B : 0;  // taps per thread, rounded up for all
-    const uint32_t mine = i0 < ntot ? (ntot - i0 + B - 1) / B : 0;        // this thread's
-    const uint32_t nt = a.ctaps > B ? a.ctaps / B : 1u;        // a thread's taps per chunk
+    const uint32_t mend = first < ntot ? (ntot - first + B - 1) / B : 0;  // taps per residue, rounded up for all
+    const uint32_t mine = i0 < ntot ? (ntot - i0 + B - 1) / B : 0;        // this one's
+    const uint32_t nt = a.ctaps > B ? a.ctaps / B : 1u;       // a residue's taps per chunk
     const uint32_t t0 = (uint32_t)(int32_t)(-a.T) + i0;
-    const uint32_t dmax = a.maxshift / B;                      // sample j of the thread: t0 + (j - dmax) B
-    uint32_t dl[kMaxHash];                                     // hashing h's tap m takes sample m + dl[h]
-    C acc[kMaxHash], sum[kMaxHash];
-#pragma unroll
-    for (int h = 0; h < kMaxHash; ++h) {
-        dl[h] = dmax - ((uint32_t)h < H ? a.a[h] / B : 0u);
-        acc[h] = sum[h] = mkc((R)0, (R)0);
-    }
-    uint32_t xi = sigma * (t0 - a.maxshift);
-    const uint32_t xstep = sigma * B, sb = sigma * b, estep = sb * B;
-    uint32_t e = sb * t0;
+    const uint32_t dmax = a.maxshift / B;                     // sample j of the residue: t0 + (j - dmax) B
+    const uint32_t dl = dmax - (q < H ? a.a[q] / B : 0u);     // hashing q's tap m takes sample m + dl
+    const uint32_t x0 = sigma * (t0 - a.maxshift), xstep = sigma * B, sb = sigma * b;
     const R inv_half_n = (R)2 / (R)a.n;
-    for (uint32_t j = 0; j < dmax; ++j) {
-        ring[(j & rmask) * kThreads] = ldg_c(x + (xi & xmask));
-        xi += xstep;
-    }
-    for (uint32_t m0 = 0; m0 < mend; m0 += kLoads) {
-        {
-            C v[kLoads];
-            R g[kLoads];  // the taps in the same batch: alone, their latency would be paid tap by tap
+    C acc = mkc((R)0, (R)0), sum = acc;
+    for (uint32_t j = q; j < dmax; j += kQ) ring[(j & rmask) * kOwnerRes] = ldg_c(x + ((x0 + j * xstep) & xmask));
+    C v[kLoads];
+    R g[kLoads];
+    auto load = [&](uint32_t m0) {
 #pragma unroll
-            for (uint32_t u = 0; u < kLoads; ++u)
-                if (m0 + u < mine) {
-                    v[u] = ldg_c(x + ((xi + u * xstep) & xmask));
-                    const int32_t t = (int32_t)(t0 + (m0 + u) * B);
-                    g[u] = taps[t < 0 ? -t : t];
-                }
-            xi += kLoads * xstep;
-#pragma unroll
-            for (uint32_t u = 0; u < kLoads; ++u)
-                if (m0 + u < mine) {
-                    ring[((m0 + u + dmax) & rmask) * kThreads] = v[u];
-                    tap[u * kThreads] = g[u];
-                }
-        }
-        const uint32_t mb = min(m0 + kLoads, mine);
-        // (kept a short loop: unrolled, its code is fetched from L2 once per SM for as long as it runs)
-#pragma unroll 1
-        for (uint32_t m = m0; m < mb; ++m, e += estep) {
-            if (m != 0 && (m & (nt - 1)) == 0) {
-#pragma unroll
-                for (int h = 0; h < kMaxHash; ++h) {
-                    sum[h] = cadd(sum[h], acc[h]);
-                    acc[h] = mkc((R)0, (R)0);
-                }
+        for (uint32_t u = 0; u < kLoads; ++u) {
+            const uint32_t m = m0 + q + u * kQ;
+            if (m < mine) {
+                v[u] = ldg_c(x + ((x0 + (m + dmax) * xstep) & xmask));
+                const int32_t t = (int32_t)(t0 + m * B);
+                g[u] = taps[t < 0 ? -t : t];
             }
-            const C gt = tap_factor(a, tap[(m - m0) * kThreads], e, inv_half_n);
-#pragma unroll
-            for (int h = 0; h < kMaxHash; ++h)
-                if ((uint32_t)h < H) acc[h] = cfma(gt, ring[((m + dl[h]) & rmask) * kThreads], acc[h]);
         }
-    }
-    C* area = reinterpret_cast<C*>(a.part) + (size_t)s * a.part_stride + (__brev(t0 & (B - 1)) >> (32u - a.logB));
+    };
+    load(0);
+    for (uint32_t m0 = 0; m0 < mend; m0 += kBatch) {
 #pragma unroll
-    for (int h = 0; h < kMaxHash; ++h)
-        if ((uint32_t)h < H) area[(size_t)h * B] = cadd(sum[h], acc[h]);  // bit-reversed, as the bin FFT takes it
+        for (uint32_t u = 0; u < kLoads; ++u) {
+            const uint32_t m = m0 + q + u * kQ;
+            if (m < mine) {
+                ring[((m + dmax) & rmask) * kOwnerRes] = v[u];
+                factor[(m - m0) * kOwnerRes] = tap_factor(a, g[u], sb * (t0 + m * B), inv_half_n);
+            }
+        }
+        __syncthreads();
+        if (m0 + kBatch < mend) load(m0 + kBatch);
+        if (q < H) {
+            const uint32_t mb = min(m0 + kBatch, mine);
+            // (a short loop: unrolled, its code is fetched from L2 by every SM for as long as it runs)
+#pragma unroll 2
+            for (uint32_t m = m0; m < mb; ++m) {
+                if (m != 0 && (m & (nt - 1)) == 0) {
+                    sum = cadd(sum, acc);
+                    acc = mkc((R)0, (R)0);
+                }
+                acc = cfma(factor[(m - m0) * kOwnerRes], ring[((m + dl) & rmask) * kOwnerRes], acc);
+            }
+        }
+        __syncthreads();  // the ring and the factors are written again
+    }
+    if (q < H) {  // bit-reversed, as the bin FFT takes it
+        C* area = reinterpret_cast<C*>(a.part) + (size_t)s * a.part_stride + (__brev(t0 & (B - 1)) >> (32u - a.logB));
+        area[(size_t)q * B] = cadd(sum, acc);
+    }
 }
 
 // |v| < prune thr in FP64, by FP32 where that is clear of the bound
@@ -797,7 +827,8 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
     using C = typename Cx<R>::T;
     const uint32_t tid = threadIdx.x;
     const uint32_t B = a.B, H = a.H;
-    const FinLayout Ly = fin_layout(B, H, a.zcap, sizeof(C));
+    const bool masks = !a.bins_only;
+    const FinLayout Ly = fin_layout(B, H, a.zcap, sizeof(C), masks);
     C* U = reinterpret_cast<C*>(smem + Ly.U);
     uint32_t* ent_idx = reinterpret_cast<uint32_t*>(smem + Ly.ent_idx);
     uint32_t* ent_bin = reinterpret_cast<uint32_t*>(smem + Ly.ent_bin);
@@ -805,12 +836,11 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
     double* ent_gain = reinterpret_cast<double*>(smem + Ly.ent_gain);
     double2* ent_sub = reinterpret_cast<double2*>(smem + Ly.ent_sub);
     float2* ent_sub_f = reinterpret_cast<float2*>(smem + Ly.ent_sub_f);
+    uint32_t* mask = reinterpret_cast<uint32_t*>(smem + Ly.mask);  // [word][B]: bit e mod 32 of word e / 32
     uint32_t* bin_cnt = reinterpret_cast<uint32_t*>(smem + Ly.bin_cnt);
     uint32_t* bin_start = reinterpret_cast<uint32_t*>(smem + Ly.bin_start);
     uint32_t* bin_list = reinterpret_cast<uint32_t*>(smem + Ly.bin_list);
     uint32_t* cand_idx = reinterpret_cast<uint32_t*>(smem + Ly.cand_idx);
-    uint32_t* cand_bin = reinterpret_cast<uint32_t*>(smem + Ly.cand_bin);
-    double* cand_gain = reinterpret_cast<double*>(smem + Ly.cand_gain);
     double2* cand_val = reinterpret_cast<double2*>(smem + Ly.cand_val);
     uint32_t* srt_idx = reinterpret_cast<uint32_t*>(smem + Ly.srt_idx);
     double2* srt_val = reinterpret_cast<double2*>(smem + Ly.srt_val);
@@ -848,6 +878,10 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
     }
     if (tid == kThreads - 1 && next_ctr != nullptr) s_next_ready = acquire_is(next_ctr, 1u) ? 1u : 0u;
 
+    if (masks) {
+        for (uint32_t i = tid; i < B * ((a.zcap + 31) / 32); i += kThreads) mask[i] = 0;
+        __syncthreads();  // (waits for nothing: the loads above are still on their way)
+    }
     // zhat of this request and its per-entry subtraction terms
     // zhat is read through L2 only: in the one-launch path another CTA of this launch wrote it
     // (the first entry of each thread is fetched together with the count)
@@ -891,7 +925,10 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         ent_val[e] = v;
         uint32_t jb;
         const int32_t o = offset_of((sigma * (i - b)) & a.nmask, Np, logNp, a.nmask, &jb);
-        ent_bin[e] = jb;
+        if (masks)
+            atomicOr(&mask[(e >> 5) * B + jb], 1u << (e & 31u));
+        else
+            ent_bin[e] = jb;
         const double gain = a.wtab[o < 0 ? -o : o];
         ent_gain[e] = gain;
         if (f32) {
@@ -928,8 +965,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
     __syncthreads();  // d, the entries and the counts
     // read here, before thread 0 can reach the next round's write
     const bool next_ready = next_ctr != nullptr && s_next_ready != 0;
-    // step 4 terms: W(-o(i)) zhat_i w^{a_h sigma i} for every (entry, hashing).  No barrier after this
-    // loop: bucket_entries starts with one before anything reads the terms.
+    // step 4 terms: W(-o(i)) zhat_i w^{a_h sigma i} for every (entry, hashing)
     if (f32) {
         if (!a.bins_only) {
             const float two_over_n = 2.0f * d.inv_n_f;  // exact: n is a power of two
@@ -955,24 +991,24 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         }
     }
     const uint32_t sub_stride = f32 ? 1u : H;  // where subtracted_u0 finds hashing 0's FP64 terms
-    bucket_entries(ent_bin, nz, B, bin_cnt, bin_start, bin_list, scan);
-
     if (a.bins_only) {  // single-hashing mode: the subtracted bins u_0 in FP64, no decode
+        bucket_entries(ent_bin, nz, B, bin_cnt, bin_start, bin_list, scan);  // (a barrier before the terms are read)
         for (uint32_t j = tid; j < B; j += kThreads)
             a.ubins[j] =
-                subtracted_u0(U, sub_stride, j, bin_list + bin_start[j], bin_start[j + 1] - bin_start[j], ent_sub);
+                subtracted_u0(U, sub_stride, j, ListEntries{bin_list + bin_start[j], bin_start[j + 1] - bin_start[j]},
+                              ent_sub);
         return false;
     }
+    __syncthreads();  // the terms
     // step 4 and the decode, one bin per thread: decisions in the data path's precision
     for (uint32_t j = tid; j < B; j += kThreads) {
         C u[kMaxHash];
-        const uint32_t* list = bin_list + bin_start[j];
-        const uint32_t nbin = bin_start[j + 1] - bin_start[j];
-        subtracted_bin(U, B, H, j, list, nbin, ent_sub, ent_sub_f, u);
+        const MaskEntries ents{mask + j, B, (nz + 31) / 32};
+        subtracted_bin(U, B, H, j, ents, ent_sub, ent_sub_f, u);
         uint32_t oi = 0;
         double gain = 1.0, ginv = 0.0;
         bool above;
-        const int kind = decode_bin(d, j, u, list, nbin, ent_idx, ent_gain, &oi, &gain, &ginv, &above);
+        const int kind = decode_bin(d, j, u, ents, ent_idx, ent_gain, &oi, &gain, &ginv, &above);
         // counts and candidate slots, one shared-memory atomic per warp and counter
         const unsigned m = __activemask();
         const unsigned ma = __ballot_sync(m, above), mk = __ballot_sync(m, kind == 1), mw = __ballot_sync(m, kind != 0);
@@ -987,11 +1023,9 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         if (kind != 0) {
             const uint32_t slot = base + (uint32_t)__popc((int)(mw & ((1u << lane) - 1u)));
             cand_idx[slot] = oi;
-            cand_bin[slot] = j;
-            cand_gain[slot] = gain;
             // its value: u_0 (step 4 in FP64) / W(-o), as a product with 1 / W(-o) from the table where
             // the decode read one (FP32 path), else as a quotient
-            const double2 u0 = subtracted_u0(U, sub_stride, j, list, nbin, ent_sub);
+            const double2 u0 = subtracted_u0(U, sub_stride, j, ents, ent_sub);
             if (f32 && kind == 1 && d.winv)
                 cand_val[slot] = make_double2(u0.x * ginv, u0.y * ginv);
             else
@@ -1064,35 +1098,19 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         }
     }
     __syncthreads();
-    for (uint32_t p = tid; p < tot; p += kThreads) {
-        uint32_t kp = 0;
-        const uint32_t idx = out_idx[p];
-        if (p == 0 || out_idx[p - 1] != idx) {
-            double2 v = out_val[p];
-            if (p + 1 < tot && out_idx[p + 1] == idx) {
-                v.x += out_val[p + 1].x;
-                v.y += out_val[p + 1].y;
-                out_val[p] = v;  // the duplicate at p + 1 is never a head and is not written
-            }
-            // |v| < prune thr, in the data path's precision (FP32: against prune thr rounded up)
-            if (f32)
-                kp = hypotf((float)v.x, (float)v.y) < a.drop_f ? 0u : 1u;
-            else
-                kp = dropped(v, a) ? 0u : 1u;
+    // a merged entry's fate: heads of equal indices take their duplicate's value, small ones are dropped
+    auto keep_merged = [&](uint32_t p, uint32_t idx, double2& v) -> bool {
+        if (p != 0 && out_idx[p - 1] == idx) return false;
+        if (p + 1 < tot && out_idx[p + 1] == idx) {
+            v.x += out_val[p + 1].x;
+            v.y += out_val[p + 1].y;
         }
-        keep[p] = kp;
-    }
-    __syncthreads();
-    const uint32_t newcount =
-        tot <= (uint32_t)kThreads ? block_exclusive_scan_flags(keep, tot, scan) : block_exclusive_scan(keep, tot, scan);
+        // |v| < prune thr, in the data path's precision (FP32: against prune thr rounded up)
+        return f32 ? !(hypotf((float)v.x, (float)v.y) < a.drop_f) : !dropped(v, a);
+    };
     uint32_t* zi = a.zidx + (size_t)s * a.zcap;
     double2* zv = a.zval + (size_t)s * a.zcap;
-    for (uint32_t p = tid; p < tot; p += kThreads) {
-        const uint32_t pos = keep[p];  // exclusive prefix of the keep flags: kept iff the next differs
-        const uint32_t nxt = p + 1 < tot ? keep[p + 1] : newcount;
-        if (nxt == pos) continue;
-        const uint32_t idx = out_idx[p];
-        const double2 v = out_val[p];
+    auto put = [&](uint32_t pos, uint32_t idx, double2 v) {
         if (pos < a.zcap) {
             zi[pos] = idx;
             zv[pos] = v;
@@ -1104,6 +1122,43 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         if (last && pos < a.out_cap) {
             a.out_idx[(size_t)s * a.out_cap + pos] = idx;
             a.out_val[(size_t)s * a.out_cap + pos] = v;
+        }
+    };
+    uint32_t newcount = 0;
+    if (tot <= (uint32_t)kThreads) {  // one merged entry per thread: a ballot and one barrier
+        uint32_t idx = 0;
+        double2 v = make_double2(0.0, 0.0);
+        bool kept = false;
+        if (tid < tot) {
+            idx = out_idx[tid];
+            v = out_val[tid];
+            kept = keep_merged(tid, idx, v);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, kept);
+        if ((tid & 31u) == 0) scan[tid >> 5] = (uint32_t)__popc((int)bal);
+        __syncthreads();
+        uint32_t off = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < (uint32_t)kThreads / 32u; ++w) {
+            const uint32_t c = scan[w];
+            off += w < (tid >> 5) ? c : 0u;
+            newcount += c;
+        }
+        if (kept) put(off + (uint32_t)__popc((int)(bal & ((1u << (tid & 31u)) - 1u))), idx, v);
+    } else {
+        for (uint32_t p = tid; p < tot; p += kThreads) {
+            const uint32_t idx = out_idx[p];
+            double2 v = out_val[p];
+            const bool kept = keep_merged(p, idx, v);
+            if (kept) out_val[p] = v;  // (a duplicate's value is read by its head only, and never written)
+            keep[p] = kept ? 1u : 0u;
+        }
+        __syncthreads();
+        newcount = block_exclusive_scan(keep, tot, scan);
+        for (uint32_t p = tid; p < tot; p += kThreads) {
+            const uint32_t pos = keep[p];  // exclusive prefix of the keep flags: kept iff the next differs
+            const uint32_t nxt = p + 1 < tot ? keep[p + 1] : newcount;
+            if (nxt != pos) put(pos, out_idx[p], out_val[p]);
         }
     }
     if (tid == 0) {
@@ -1464,7 +1519,7 @@ __device__ __forceinline__ bool finish_large(const ExactArgs& a, uint32_t s, uin
         uint32_t where = 0;
         bool above;
         double g0, g1;
-        const int kind = decode_bin<true>(d, j, u, nullptr, nbin, s_idx + x0, s_gain + x0, &where, &g0, &g1, &above);
+        const int kind = decode_bin(d, j, u, RunEntries{nbin}, s_idx + x0, s_gain + x0, &where, &g0, &g1, &above);
         const unsigned m = __activemask();
         const unsigned ma = __ballot_sync(m, above), mw = __ballot_sync(m, kind != 0);
         const uint32_t lane = tid & 31u, leader = (uint32_t)__ffs((int)m) - 1u;
@@ -1988,7 +2043,7 @@ __global__ void __launch_bounds__(kThreads) k_exact_decode(const DecodeArgs a) {
         uint32_t oi = 0;
         double gain = 1.0, ginv;  // this decode divides by the gain (its context has no 1 / W table)
         bool above;
-        const int kind = decode_bin(d, j, u, bin_list + bin_start[j], bin_start[j + 1] - bin_start[j], ent_idx,
+        const int kind = decode_bin(d, j, u, ListEntries{bin_list + bin_start[j], bin_start[j + 1] - bin_start[j]}, ent_idx,
                                     ent_gain, &oi, &gain, &ginv, &above);
         if (above) atomicAdd(&s_above, 1u);
         if (kind == 1) atomicAdd(&s_kept, 1u);

@@ -331,9 +331,9 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
         // chip for the next one
         r.fin_global = fs > kFinSmemMax;
         if ((r.fin_global ? gs : (gs > fs ? gs : fs)) > 200 * 1024) return SFFT_ERR_K_RANGE;
-        large = large || r.fin_global || p.z_cap > kCarry;
+        r.smem = p.z_cap > kCarry ? 0 : exact_decode_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
+        large = large || r.fin_global || p.z_cap > kCarry || r.smem > kFinSmemMax;
         r.fin_bytes = r.fin_global ? fs : 0;
-        r.smem = fs;
         r.smem_gather = std::max(gs, (size_t)(1 + r.nshift) * r.B * (fp64 ? 16 : 8));
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, r.alpha, p.delta, r.T, pl->taps_host.data() + taps_off);
@@ -352,9 +352,9 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
     }
     for (ExactRound& r : pl->rounds) {  // one kind of decode for the whole plan
         r.large = large;
-        // gather_owner where it has two CTAs or more per request: below, its one CTA walks the window alone
+        // gather_owner where a thread's taps are one residue's in every chunk (B >= kThreads)
         r.ring = exact_owner_ring(r.shift[r.nshift - 1], r.B, fp64);
-        r.owner = large && r.B >= 2 * (uint32_t)kThreads && r.ring <= 32;
+        r.owner = large && r.B >= (uint32_t)kThreads && r.ring != 0;
         if (r.owner)
             r.smem_gather = std::max(exact_owner_smem(r.ring, fp64), (size_t)(1 + r.nshift) * r.B * (fp64 ? 16 : 8));
         r.smem = std::max(r.smem_gather, large ? (size_t)kLargeSmem : r.smem);

@@ -16,6 +16,7 @@ constexpr int kChunkTaps = 2048;  // taps per CTA in the gather phase (8 per thr
 constexpr int kMaxHash = 4;       // hashings per exact round: a = 0 plus up to 3 ladder shifts
 constexpr uint32_t kCarry = 256;  // zhat entries an exact finisher keeps on chip for the next round
 constexpr uint32_t kLargeSmem = 104 * 1024;  // shared memory of finish_large: two CTAs per SM
+constexpr uint32_t kOwnerRes = 64;  // residues per CTA of gather_owner
 constexpr uint32_t kMaxB = 4096;  // largest B of the fused exact round
 constexpr uint32_t kNoIndex = 0xFFFFFFFFu;
 constexpr size_t kFinSmemMax = 160 * 1024;  // largest on-chip finisher of the exact round
@@ -50,8 +51,8 @@ struct ExactRound {
     size_t smem_gather = 0;   // of which the gather and the bins need this
     bool fin_global = false;  // the arrays of finish_round do not fit on chip: they live in d_fin
     bool large = false;       // the transform's decode is finish_large (the same for all of a plan's rounds)
-    bool owner = false;       // gather_owner folds the round (a CTA per kThreads residues)
-    uint32_t ring = 0;        // samples a thread of gather_owner keeps
+    bool owner = false;       // gather_owner folds the round (a CTA per kOwnerRes residues)
+    uint32_t ring = 0;        // samples gather_owner keeps of a residue
     size_t fin_bytes = 0;     // device memory a request's decode may need
 };
 
@@ -71,8 +72,8 @@ struct ExactArgs {
     uint32_t a[kMaxHash];      // a[0] = 0, a[l] = beta_l
     uint64_t shift64[kMaxHash];
     uint32_t chunks, stage, maxshift;
-    uint32_t gctas;            // gather CTAs of the round per request: its chunks, or B / kThreads (owner)
-    uint32_t owner, ring;      // fold by gather_owner, with this many samples kept per thread
+    uint32_t gctas;            // gather CTAs of the round per request: its chunks, or B / kOwnerRes (owner)
+    uint32_t owner, ring;      // fold by gather_owner, with this many samples kept of a residue
     uint32_t large;            // decode by finish_large
     uint32_t large_smem;       // its dynamic shared memory
     uint32_t ctaps;            // taps per CTA: chunk c gathers taps [-T + c ctaps, -T + (c + 1) ctaps)
@@ -341,7 +342,7 @@ struct sfft_plan_s {
     uint32_t* d_zidx = nullptr;
     double2* d_zval = nullptr;
     uint32_t* d_zcount = nullptr;
-    int32_t* d_zflag = nullptr;
+    int32_t* d_zflag = nullptr;  // behind the counts: one clear for both
     // single-step helpers
     double2* d_ubins = nullptr;
     uint32_t* d_aux = nullptr;
@@ -431,6 +432,7 @@ cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const General
 cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);
 size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
+size_t exact_decode_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 size_t exact_gather_smem(uint32_t stage, bool fp64);
 size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64);
