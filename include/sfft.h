@@ -299,7 +299,7 @@ sfft_status sfft_autotune(const sfft_params* base, uint32_t batch, double snr_db
 /* ---------------------------------------------------------------------------------------------- */
 /*
  * A batch plan groups exact-mode plans of any (n, k) (one precision) so that a batch mixing them runs
- * as ONE launch (two, side by side, where plans with z_cap above 256 are mixed with others): the
+ * as ONE launch (two, side by side, where plans with large zhat capacities are mixed with others): the
  * gathers of every request and round (Algorithm 1's loop) are in the grid at once, and the decodes of a
  * request's rounds follow one another as their bins arrive, with no launch boundary between them.
  * Results are those of sfft_execute_requests on each request's own plan, bit for bit.  The batch plan

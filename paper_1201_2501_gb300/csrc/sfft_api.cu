@@ -111,7 +111,7 @@ ExactArgs base_args(const sfft_plan_s* pl, const ExactRound& r, uint32_t t) {
     a.owner = r.owner ? 1 : 0;
     a.ring = r.ring;
     a.gctas = r.owner ? r.B / kOwnerRes : r.chunks;
-    a.large = r.large ? 1 : 0;
+    a.kind = (uint32_t)r.kind;
     a.large_smem = kLargeSmem;
     a.ctaps = r.ctaps;
     a.stage = r.stage;
@@ -356,7 +356,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         if ((e = cudaEventCreateWithFlags(&pl->ev_join[i], cudaEventDisableTiming)) != cudaSuccess)
             return fail(e, "create event");
     }
-    if (!general && (e = set_exact_smem_limit(max_smem, fp64, pl->rounds[0].large)) != cudaSuccess) return fail(e, "shared memory limit");
+    if (!general && (e = set_exact_smem_limit(max_smem, fp64, pl->rounds[0].kind)) != cudaSuccess) return fail(e, "shared memory limit");
     if (general && (e = general_set_smem(fs_max, ls_max, ss_max, 0)) != cudaSuccess)
         return fail(e, "shared memory limit");
     // The gather reads one 8- or 16-byte sample per 32-byte sector at random; ask L2 not to widen
@@ -848,7 +848,7 @@ sfft_status sfft_hash_to_bins(sfft_plan plan, uint32_t t, const void* d_x, uint6
                                                                 (fp64 ? 16 : 8);
     const size_t fs = exact_finish_smem(r.B, 1, args.zcap, fp64);
     const size_t smem = gs > fs ? gs : fs;
-    SFFT_CUDA(set_exact_smem_limit(smem, fp64, r.large), "shared memory limit");
+    SFFT_CUDA(set_round_smem_limit(smem, fp64), "shared memory limit");
     SFFT_CUDA(launch_exact_round(args, 1, smem, st, fp64), "hash to bins");
     return SFFT_OK;
 }
@@ -972,6 +972,7 @@ struct sfft_batch_plan_s {
     bool fp64 = false;
     uint32_t max_req = 0, max_rounds = 0;
     size_t smem[2] = {0, 0};           // dynamic shared memory of the plans without and with finish_large
+    int small_kind = 0;                // DecodeKind of the plans without
     ExactArgs* d_rdesc = nullptr;
     unsigned char* d_ctl = nullptr;    // the tables of one call (CtlLayout)
     unsigned char* d_part = nullptr;
@@ -1054,7 +1055,7 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
     const size_t csize = bp->fp64 ? 16 : 8;
     std::vector<ExactArgs> rdesc;
     size_t max_ctas_req = 0;
-    bool kinds[2] = {false, false};
+    bool kinds[2] = {false, false}, lists = false;
     for (sfft_plan pl : bp->plans) {
         bp->rd0.push_back((uint32_t)rdesc.size());
         const uint32_t R = (uint32_t)pl->rounds.size();
@@ -1066,9 +1067,12 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
             a.part_bytes = (size_t)(static_cast<unsigned char*>(a.part) - static_cast<unsigned char*>(pl->d_part));
             rdesc.push_back(a);
             ctas += a.gctas;
-            const int kind = r.large ? 1 : 0;
-            kinds[kind] = true;
-            bp->smem[kind] = std::max(bp->smem[kind], r.smem);
+            const int large = r.kind == kDecodeLarge ? 1 : 0;
+            kinds[large] = true;
+            lists = lists || r.kind == kDecodeLists;
+            // (plans with masks run with lists beside plans that need them: room for either)
+            bp->smem[large] = std::max(bp->smem[large], r.smem);
+            if (!large) bp->smem[0] = std::max(bp->smem[0], exact_finish_smem(r.B, 1 + r.nshift, pl->p.z_cap, bp->fp64));
             bp->fin_stride = std::max(bp->fin_stride, (r.fin_bytes + 255) & ~size_t(255));
         }
         max_ctas_req = std::max(max_ctas_req, ctas);
@@ -1104,8 +1108,9 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
     }
     cudaError_t e = cudaMemcpy(bp->d_rdesc, rdesc.data(), rdesc.size() * sizeof(ExactArgs), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(bp->d_counter, 0, counter_bytes);
-    for (int kind = 0; kind < 2; ++kind)
-        if (e == cudaSuccess && kinds[kind]) e = set_batch_smem_limit(bp->smem[kind], bp->fp64, kind != 0);
+    bp->small_kind = lists ? kDecodeLists : kDecodeMasks;
+    if (e == cudaSuccess && kinds[0]) e = set_batch_smem_limit(bp->smem[0], bp->fp64, bp->small_kind);
+    if (e == cudaSuccess && kinds[1]) e = set_batch_smem_limit(bp->smem[1], bp->fp64, kDecodeLarge);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         set_last_error(std::string("batch plan: ") + cudaGetErrorString(e));
@@ -1185,7 +1190,7 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
         for (uint32_t t = 0; t < bp->max_rounds; ++t)
             for (uint32_t r = 0; r < nreq; ++r) {
                 const sfft_plan pl = bp->plans[h_plan_of[r]];
-                if (t >= pl->rounds.size() || (pl->rounds[0].large ? 1 : 0) != kind) continue;
+                if (t >= pl->rounds.size() || (pl->rounds[0].kind == kDecodeLarge ? 1 : 0) != kind) continue;
                 seg[q] = (uint32_t)ctas[kind];
                 who[q++] = t << 24 | r;
                 ctas[kind] += pl->rdesc[t].gctas;
@@ -1230,7 +1235,8 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
         a.seg = reinterpret_cast<const uint32_t*>(d + L.seg) + seg0[kind];
         a.seg_who = reinterpret_cast<const uint32_t*>(d + L.who) + seg0[kind];
         a.nseg = (uint32_t)(seg0[kind + 1] - seg0[kind]);
-        SFFT_CUDA(launch_exact_batch(a, (uint32_t)ctas[kind], bp->smem[kind], both && kind ? bp->side : st, bp->fp64, kind != 0),
+        SFFT_CUDA(launch_exact_batch(a, (uint32_t)ctas[kind], bp->smem[kind], both && kind ? bp->side : st, bp->fp64,
+                                     kind ? (int)kDecodeLarge : bp->small_kind),
                   "mixed batch");
     }
     if (both) {

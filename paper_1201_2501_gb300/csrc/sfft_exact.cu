@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
+#include <type_traits>
 #include <stdint.h>
 
 #include "philox.cuh"
@@ -532,6 +533,15 @@ __device__ __forceinline__ int decode_bin(const DecodeCtx& d, uint32_t j, const 
     return decode_bin_fp32(d, j, u, ents, ent_idx, ent_gain, oi, gout, ginv, above);
 }
 
+__device__ __forceinline__ MaskEntries bin_entries(std::true_type, const uint32_t* words, uint32_t stride, uint32_t nwords,
+                                                   const uint32_t*, const uint32_t*) {
+    return MaskEntries{words, stride, nwords};
+}
+__device__ __forceinline__ ListEntries bin_entries(std::false_type, const uint32_t*, uint32_t, uint32_t, const uint32_t* list,
+                                                   const uint32_t* start) {
+    return ListEntries{list + start[0], start[1] - start[0]};
+}
+
 // Bin j's hashings after the subtraction of zhat, for the decisions: u_h = U_h - sum over the bin's
 // entries e (in list order) of sub[e H + h], in the data path's precision (FP64 terms and sums for
 // the FP64 path; the terms rounded to FP32 and summed in FP32 for the FP32 path, whose bins carry
@@ -819,15 +829,15 @@ __device__ __forceinline__ void fft_rows(const ExactArgs& a, double2* U) {
     fft_rows_fp64(U, a.H, a.logB, a.logn, a.tw, a.tw_shift);
 }
 
-// LARGE: the bins of a plan decoded by finish_large (many bins: FFT stages by passes)
-template <typename R, bool LARGE = false>
+// KIND (see DecodeKind): how the entries of a bin are found; kDecodeLarge only forms the bins here
+template <typename R, int KIND = kDecodeLists>
 __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uint32_t b, unsigned char* smem,
                              int part = kFinAll, bool carry = false, bool bins_here = false,
                              const uint32_t* next_ctr = nullptr) {
     using C = typename Cx<R>::T;
     const uint32_t tid = threadIdx.x;
     const uint32_t B = a.B, H = a.H;
-    const bool masks = !a.bins_only;
+    constexpr bool masks = KIND == kDecodeMasks;
     const FinLayout Ly = fin_layout(B, H, a.zcap, sizeof(C), masks);
     C* U = reinterpret_cast<C*>(smem + Ly.U);
     uint32_t* ent_idx = reinterpret_cast<uint32_t*>(smem + Ly.ent_idx);
@@ -853,11 +863,11 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
 
     // steps 2 (across chunks) and 3: partial folds summed in chunk order, bit-reversed, FFT
     if (part & kFinBins) {
-        if (LARGE && a.owner)
+        if (KIND == kDecodeLarge && a.owner)
             load_rows(U, area, H * B);  // whole folds, bit-reversed
         else
             sum_partials(area, a.chunks, H, a.logB, U);
-        fft_rows<LARGE>(a, U);  // starts and ends with a barrier
+        fft_rows<KIND == kDecodeLarge>(a, U);  // starts and ends with a barrier
         if (!(part & kFinDecode)) {  // every partial fold has been read: the area takes the bins
             for (uint32_t i = tid; i < H * B; i += kThreads) area[i] = U[i];
             return false;
@@ -991,19 +1001,21 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
         }
     }
     const uint32_t sub_stride = f32 ? 1u : H;  // where subtracted_u0 finds hashing 0's FP64 terms
-    if (a.bins_only) {  // single-hashing mode: the subtracted bins u_0 in FP64, no decode
+    if (masks)
+        __syncthreads();  // the terms
+    else
         bucket_entries(ent_bin, nz, B, bin_cnt, bin_start, bin_list, scan);  // (a barrier before the terms are read)
+    if (a.bins_only) {  // single-hashing mode: the subtracted bins u_0 in FP64, no decode
         for (uint32_t j = tid; j < B; j += kThreads)
             a.ubins[j] =
                 subtracted_u0(U, sub_stride, j, ListEntries{bin_list + bin_start[j], bin_start[j + 1] - bin_start[j]},
                               ent_sub);
         return false;
     }
-    __syncthreads();  // the terms
     // step 4 and the decode, one bin per thread: decisions in the data path's precision
     for (uint32_t j = tid; j < B; j += kThreads) {
         C u[kMaxHash];
-        const MaskEntries ents{mask + j, B, (nz + 31) / 32};
+        const auto ents = bin_entries(std::integral_constant<bool, masks>(), mask + j, B, (nz + 31) / 32, bin_list, bin_start + j);
         subtracted_bin(U, B, H, j, ents, ent_sub, ent_sub_f, u);
         uint32_t oi = 0;
         double gain = 1.0, ginv = 0.0;
@@ -1708,7 +1720,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_round
 // counter2 (an acquire load that overlaps its own loads): when those bins have arrived, this chain is
 // the last party of that round and goes on without an arrival of its own.  (seed, id) name the
 // request's draws.
-template <typename R, int NR, bool LARGE>
+template <typename R, int NR, int KIND>
 __device__ __forceinline__ void decode_chain(const StepParams<NR>& sp, uint32_t t, const ExactArgs* a, uint32_t s,
                                              uint64_t seed, uint32_t id, uint32_t sigma, uint32_t b,
                                              unsigned char* smem) {
@@ -1717,8 +1729,8 @@ __device__ __forceinline__ void decode_chain(const StepParams<NR>& sp, uint32_t 
     for (bool carried = false;; carried = true) {
         const uint32_t* next_ctr = t + 1 < sp.R ? sp.r[t + 1].counter2 + s : nullptr;
         const bool next_ready =
-            LARGE ? finish_large<R>(*a, s, sigma, b, smem, next_ctr)
-                  : finish_round<R>(*a, s, sigma, b, smem, kFinDecode, carried, bins_here, next_ctr);
+            KIND == kDecodeLarge ? finish_large<R>(*a, s, sigma, b, smem, next_ctr)
+                  : finish_round<R, KIND>(*a, s, sigma, b, smem, kFinDecode, carried, bins_here, next_ctr);
         if (threadIdx.x == 0) a->counter2[s] = 0;  // both arrivals of round t have happened (or none, t = 0)
         if (t + 1 >= sp.R) break;
         a = &sp.r[++t];
@@ -1733,7 +1745,7 @@ __device__ __forceinline__ void decode_chain(const StepParams<NR>& sp, uint32_t 
     }
 }
 
-template <typename R, int NR, bool LARGE>
+template <typename R, int NR, int KIND>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_step(const __grid_constant__ StepParams<NR> sp) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t tid = threadIdx.x;
@@ -1746,15 +1758,15 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_step(
     const ReqView rq = req_view(a->reqs, a->x, a->n * sizeof(typename Cx<R>::T), a->seed, s, a->nmask);
     uint32_t sigma, b;
     exact_hash(rq.seed, rq.id, t, a->nmask, &sigma, &b);
-    if (LARGE && a->owner)
+    if (KIND == kDecodeLarge && a->owner)
         gather_owner<R>(*a, rq.x, rq.xmask, s, c, sigma, b, smem);
     else
         gather_fold<R>(*a, rq.x, rq.xmask, s, c, sigma, b, smem);
     if (arrive(a->counter + s, a->gctas) == 0) return;
     // the round's bins, in this CTA's shared memory (the gather's staging area holds H B values)
-    finish_round<R, LARGE>(*a, s, sigma, b, smem, kFinBins);
+    finish_round<R, KIND>(*a, s, sigma, b, smem, kFinBins);
     if (tid == 0) a->counter[s] = 0;  // every chunk of round t has arrived
-    decode_chain<R, NR, LARGE>(sp, t, a, s, rq.seed, rq.id, sigma, b, smem);
+    decode_chain<R, NR, KIND>(sp, t, a, s, rq.seed, rq.id, sigma, b, smem);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1856,7 +1868,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_bins(c
 
 // The decodes: one CTA per channel slot runs them in round order (zhat of round t feeds round t + 1).
 // If the gather flagged a copy that never landed, every slot reports SFFT_ERR_TIMEOUT instead.
-template <int NR, bool LARGE>
+template <int NR, int KIND>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode(const __grid_constant__ StepParams<NR> sp,
                                                                                 uint64_t seed, uint32_t id,
                                                                                 const uint32_t* error) {
@@ -1874,10 +1886,10 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode
         const ExactArgs& a = sp.r[t];
         uint32_t sigma, b;
         exact_hash(seed, id, t, a.nmask, &sigma, &b);
-        if (LARGE)
+        if (KIND == kDecodeLarge)
             finish_large<float>(a, s, sigma, b, smem, nullptr);
         else
-            finish_round<float>(a, s, sigma, b, smem, kFinDecode, t > 0);
+            finish_round<float, KIND>(a, s, sigma, b, smem, kFinDecode, t > 0);
         __syncthreads();  // zhat of round t is read by round t + 1 (same CTA)
     }
 }
@@ -1891,7 +1903,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode
 // comes from device memory, its per-request fields are pointed at the request's own workspace.  Against
 // the device queue it replaces, where a request's next round was gathered only after the last one's
 // decode: 452 us, was 880 (96 requests of six plans, n = 2^16 .. 2^22).
-template <typename R, bool LARGE>
+template <typename R, int KIND>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_batch(const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) ExactArgs sa;
@@ -1940,19 +1952,20 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_batch
     const ReqView rq = req_view(sa.reqs, nullptr, 0, 0, 0, sa.nmask);
     uint32_t sigma, b;
     exact_hash(rq.seed, rq.id, t, sa.nmask, &sigma, &b);
-    if (LARGE && sa.owner)
+    if (KIND == kDecodeLarge && sa.owner)
         gather_owner<R>(sa, rq.x, rq.xmask, 0, c, sigma, b, smem);
     else
         gather_fold<R>(sa, rq.x, rq.xmask, 0, c, sigma, b, smem);
     if (arrive(sa.counter, sa.gctas) == 0) return;
-    finish_round<R, LARGE>(sa, 0, sigma, b, smem, kFinBins);
+    finish_round<R, KIND>(sa, 0, sigma, b, smem, kFinBins);
     if (tid == 0) *sa.counter = 0;
     if (t > 0 && arrive_pair(sa.counter2) == 0) return;
     // the decodes from round t on (as decode_chain)
     for (bool first = true;; first = false) {
         const uint32_t* next_ctr = t + 1 < rounds ? counters + kMaxRounds + t + 1 : nullptr;
-        const bool next_ready = LARGE ? finish_large<R>(sa, 0, sigma, b, smem, next_ctr)
-                                      : finish_round<R>(sa, 0, sigma, b, smem, kFinDecode, !first, first, next_ctr);
+        const bool next_ready = KIND == kDecodeLarge
+                                    ? finish_large<R>(sa, 0, sigma, b, smem, next_ctr)
+                                    : finish_round<R, KIND>(sa, 0, sigma, b, smem, kFinDecode, !first, first, next_ctr);
         if (tid == 0) *sa.counter2 = 0;
         if (++t >= rounds) break;
         if (!next_ready && arrive_pair(counters + kMaxRounds + t) == 0) break;
@@ -1961,16 +1974,21 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_batch
     }
 }
 
-cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, bool large) {
-    if (ctas == 0) return cudaSuccess;
-    if (fp64 && large)
-        k_exact_batch<double, true><<<ctas, kThreads, smem, st>>>(a);
-    else if (fp64)
-        k_exact_batch<double, false><<<ctas, kThreads, smem, st>>>(a);
-    else if (large)
-        k_exact_batch<float, true><<<ctas, kThreads, smem, st>>>(a);
+template <typename R>
+static void launch_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, int kind) {
+    if (kind == kDecodeLarge)
+        k_exact_batch<R, kDecodeLarge><<<ctas, kThreads, smem, st>>>(a);
+    else if (kind == kDecodeMasks)
+        k_exact_batch<R, kDecodeMasks><<<ctas, kThreads, smem, st>>>(a);
     else
-        k_exact_batch<float, false><<<ctas, kThreads, smem, st>>>(a);
+        k_exact_batch<R, kDecodeLists><<<ctas, kThreads, smem, st>>>(a);
+}
+cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, int kind) {
+    if (ctas == 0) return cudaSuccess;
+    if (fp64)
+        launch_batch<double>(a, ctas, smem, st, kind);
+    else
+        launch_batch<float>(a, ctas, smem, st, kind);
     return cudaGetLastError();
 }
 
@@ -2110,8 +2128,6 @@ static cudaError_t launch_chan_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
             const int full = (int)(kChanRows * kChanMaxC * sizeof(float2) + kChanRows * kMaxHash * sizeof(float2));
             cudaError_t e = cudaFuncSetAttribute(k_chan_gather<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, full);
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_chan_gather<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, full);
-            if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k_chan_gather<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, full);
             if (e != cudaSuccess) return e;
             set_to = (size_t)full;
@@ -2125,10 +2141,12 @@ static cudaError_t launch_chan_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
     if (after && (e = cudaEventRecord(after, st)) != cudaSuccess) return e;
     k_chan_bins<NR><<<sp.seg[R], kThreads, smem, st>>>(sp, seed, id);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (rounds[0].large)
-        k_chan_decode<NR, true><<<C, kThreads, smem, st>>>(sp, seed, id, error);
+    if (rounds[0].kind == kDecodeLarge)
+        k_chan_decode<NR, kDecodeLarge><<<C, kThreads, smem, st>>>(sp, seed, id, error);
+    else if (rounds[0].kind == kDecodeMasks)
+        k_chan_decode<NR, kDecodeMasks><<<C, kThreads, smem, st>>>(sp, seed, id, error);
     else
-        k_chan_decode<NR, false><<<C, kThreads, smem, st>>>(sp, seed, id, error);
+        k_chan_decode<NR, kDecodeLists><<<C, kThreads, smem, st>>>(sp, seed, id, error);
     return cudaGetLastError();
 }
 
@@ -2137,61 +2155,71 @@ cudaError_t launch_exact_channels(const ExactArgs* rounds, uint32_t R, uint32_t 
                                   cudaEvent_t after) {
     if (R == 0 || R > kMaxRounds || C == 0 || C % 32 || C > kChanMaxC || !error) return cudaErrorInvalidValue;
     if (R <= 8) return launch_chan_nr<8>(rounds, R, C, x, seed, id, smem, error, st, before, after);
-    if (R <= 16) return launch_chan_nr<16>(rounds, R, C, x, seed, id, smem, error, st, before, after);
     return launch_chan_nr<32>(rounds, R, C, x, seed, id, smem, error, st, before, after);
 }
 
-template <typename R, bool LARGE>
+template <typename R, int KIND>
 static cudaError_t raise_exact_smem(size_t bytes, size_t* cur) {
     if (bytes <= *cur) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     auto raise = [&](const void* kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    raise((const void*)k_exact_step<R, 8, LARGE>);
-    raise((const void*)k_exact_step<R, 16, LARGE>);
-    raise((const void*)k_exact_step<R, 32, LARGE>);
+    raise((const void*)k_exact_step<R, 8, KIND>);
+    raise((const void*)k_exact_step<R, 32, KIND>);
     if constexpr (sizeof(R) == sizeof(float)) {
-        raise((const void*)k_chan_decode<8, LARGE>);
-        raise((const void*)k_chan_decode<16, LARGE>);
-        raise((const void*)k_chan_decode<32, LARGE>);
+        raise((const void*)k_chan_decode<8, KIND>);
+        raise((const void*)k_chan_decode<32, KIND>);
     }
     if (e == cudaSuccess) *cur = bytes;
     return e;
 }
-cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, bool large) {
+template <typename R>
+static cudaError_t raise_exact_smem(size_t bytes, int kind, size_t* limits) {
+    if (kind == kDecodeLarge) return raise_exact_smem<R, kDecodeLarge>(bytes, limits + kind);
+    if (kind == kDecodeMasks) return raise_exact_smem<R, kDecodeMasks>(bytes, limits + kind);
+    return raise_exact_smem<R, kDecodeLists>(bytes, limits + kind);
+}
+// the kernels that serve every kind of plan
+cudaError_t set_round_smem_limit(size_t bytes, bool fp64) {
     static std::mutex mu;  // plans may be created from several threads
     std::lock_guard<std::mutex> lk(mu);
-    static size_t limit[2][2] = {{0, 0}, {0, 0}}, single[2] = {0, 0};
-    cudaError_t e = fp64 ? (large ? raise_exact_smem<double, true>(bytes, &limit[1][1])
-                                  : raise_exact_smem<double, false>(bytes, &limit[1][0]))
-                         : (large ? raise_exact_smem<float, true>(bytes, &limit[0][1])
-                                  : raise_exact_smem<float, false>(bytes, &limit[0][0]));
-    size_t& cur = single[fp64 ? 1 : 0];  // the kernels that serve both kinds of plan
+    static size_t limit[2] = {0, 0};
+    size_t& cur = limit[fp64 ? 1 : 0];
+    if (bytes <= cur) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
     auto raise = [&](const void* kernel) {
-        if (e == cudaSuccess && bytes > cur)
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     if (fp64) {
         raise((const void*)k_exact_round<double>);
     } else {
         raise((const void*)k_exact_round<float>);
         raise((const void*)k_chan_bins<8>);
-        raise((const void*)k_chan_bins<16>);
         raise((const void*)k_chan_bins<32>);
     }
-    if (e == cudaSuccess && bytes > cur) cur = bytes;
+    if (e == cudaSuccess) cur = bytes;
     return e;
 }
-cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, bool large) {
+cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, int kind) {
+    const cudaError_t e = set_round_smem_limit(bytes, fp64);
+    if (e != cudaSuccess) return e;
     static std::mutex mu;
     std::lock_guard<std::mutex> lk(mu);
-    static size_t limit[2][2] = {{0, 0}, {0, 0}};
-    size_t& cur = limit[fp64 ? 1 : 0][large ? 1 : 0];
+    static size_t limit[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    return fp64 ? raise_exact_smem<double>(bytes, kind, limit[1]) : raise_exact_smem<float>(bytes, kind, limit[0]);
+}
+cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, int kind) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lk(mu);
+    static size_t limit[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    size_t& cur = limit[fp64 ? 1 : 0][kind];
     if (bytes <= cur) return cudaSuccess;
-    const void* k = fp64 ? (large ? (const void*)k_exact_batch<double, true> : (const void*)k_exact_batch<double, false>)
-                         : (large ? (const void*)k_exact_batch<float, true> : (const void*)k_exact_batch<float, false>);
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const void* kernels[2][3] = {
+        {(const void*)k_exact_batch<float, 0>, (const void*)k_exact_batch<float, 1>, (const void*)k_exact_batch<float, 2>},
+        {(const void*)k_exact_batch<double, 0>, (const void*)k_exact_batch<double, 1>, (const void*)k_exact_batch<double, 2>}};
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernels[fp64 ? 1 : 0][kind], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) cur = bytes;
     return e;
 }
@@ -2205,6 +2233,22 @@ cudaError_t launch_exact_round(const ExactArgs& a, uint32_t batch, size_t smem, 
     return cudaGetLastError();
 }
 
+template <int NR, int KIND>
+static void launch_step_kind(const StepParams<NR>& sp, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64) {
+    if (fp64)
+        k_exact_step<double, NR, KIND><<<ctas, kThreads, smem, st>>>(sp);
+    else
+        k_exact_step<float, NR, KIND><<<ctas, kThreads, smem, st>>>(sp);
+}
+template <int NR>
+static void launch_step(const StepParams<NR>& sp, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, int kind) {
+    if (kind == kDecodeLarge)
+        launch_step_kind<NR, kDecodeLarge>(sp, ctas, smem, st, fp64);
+    else if (kind == kDecodeMasks)
+        launch_step_kind<NR, kDecodeMasks>(sp, ctas, smem, st, fp64);
+    else
+        launch_step_kind<NR, kDecodeLists>(sp, ctas, smem, st, fp64);
+}
 template <int NR>
 static cudaError_t launch_step_nr(const ExactArgs* rounds, uint32_t R, uint32_t batch, size_t smem, cudaStream_t st,
                                   bool fp64) {
@@ -2219,15 +2263,7 @@ static cudaError_t launch_step_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
     }
     const uint32_t ctas = sp.seg[R];
     if (ctas == 0) return cudaSuccess;
-    const bool large = rounds[0].large != 0;  // of the whole plan
-    if (fp64 && large)
-        k_exact_step<double, NR, true><<<ctas, kThreads, smem, st>>>(sp);
-    else if (fp64)
-        k_exact_step<double, NR, false><<<ctas, kThreads, smem, st>>>(sp);
-    else if (large)
-        k_exact_step<float, NR, true><<<ctas, kThreads, smem, st>>>(sp);
-    else
-        k_exact_step<float, NR, false><<<ctas, kThreads, smem, st>>>(sp);
+    launch_step<NR>(sp, ctas, smem, st, fp64, (int)rounds[0].kind);  // one kind for the whole plan
     return cudaGetLastError();
 }
 
@@ -2235,7 +2271,6 @@ cudaError_t launch_exact_step(const ExactArgs* rounds, uint32_t R, uint32_t batc
                               bool fp64) {
     if (R == 0 || R > kMaxRounds) return cudaErrorInvalidValue;
     if (R <= 8) return launch_step_nr<8>(rounds, R, batch, smem, st, fp64);
-    if (R <= 16) return launch_step_nr<16>(rounds, R, batch, smem, st, fp64);
     return launch_step_nr<32>(rounds, R, batch, smem, st, fp64);
 }
 

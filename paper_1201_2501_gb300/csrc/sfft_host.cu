@@ -287,7 +287,7 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
     pl->taps_host.clear();
     pl->wtab_host.clear();
     size_t taps_off = 0, wtab_off = 0;
-    bool large = false;
+    int kind = kDecodeMasks;
     for (uint32_t t = 0; t < R; ++t) {
         ExactRound r;
         uint64_t kt = ((uint64_t)p.k + (uint64_t(1) << t) - 1) >> t;
@@ -326,14 +326,16 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
         const size_t gs = exact_gather_smem(r.stage, fp64) + (size_t)(1 + r.nshift) * (B > (uint64_t)kThreads ? B : kThreads) *
                                                               (fp64 ? 16 : 8);
         const size_t fs = exact_finish_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
-        // finish_round's arrays beyond kFinSmemMax live in device memory (the single-hashing call); the
-        // transform's decode is finish_large there, and wherever zhat may outgrow what a decode keeps on
-        // chip for the next one
+        // finish_round's arrays beyond kFinSmemMax live in device memory (the single-hashing call)
         r.fin_global = fs > kFinSmemMax;
         if ((r.fin_global ? gs : (gs > fs ? gs : fs)) > 200 * 1024) return SFFT_ERR_K_RANGE;
-        r.smem = p.z_cap > kCarry ? 0 : exact_decode_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
-        large = large || r.fin_global || p.z_cap > kCarry || r.smem > kFinSmemMax;
+        const size_t ms = p.z_cap > kCarry ? 0 : exact_decode_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
+        if (r.fin_global || ms > kFinSmemMax)
+            kind = kDecodeLarge;
+        else if (p.z_cap > kCarry && kind != kDecodeLarge)
+            kind = kDecodeLists;
         r.fin_bytes = r.fin_global ? fs : 0;
+        r.smem = p.z_cap > kCarry ? fs : ms;
         r.smem_gather = std::max(gs, (size_t)(1 + r.nshift) * r.B * (fp64 ? 16 : 8));
         pl->taps_host.resize(taps_off + (size_t)r.T + 1);
         window_taps_host(p.n, r.B, r.alpha, p.delta, r.T, pl->taps_host.data() + taps_off);
@@ -351,7 +353,8 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
         pl->rounds.push_back(r);
     }
     for (ExactRound& r : pl->rounds) {  // one kind of decode for the whole plan
-        r.large = large;
+        const bool large = kind == kDecodeLarge;
+        r.kind = kind;
         // gather_owner where a thread's taps are one residue's in every chunk (B >= kThreads)
         r.ring = exact_owner_ring(r.shift[r.nshift - 1], r.B, fp64);
         r.owner = large && r.B >= (uint32_t)kThreads && r.ring != 0;

@@ -22,6 +22,13 @@ constexpr uint32_t kNoIndex = 0xFFFFFFFFu;
 constexpr size_t kFinSmemMax = 160 * 1024;  // largest on-chip finisher of the exact round
 constexpr uint32_t kMaxRounds = 32;         // rounds of an exact plan (ceil(log2 k) + 1 + extra)
 
+// How a plan's decodes find the zhat entries of a bin and where their arrays live (the same for all of a
+// plan's rounds).  Masks: one bit per entry and bin (z_cap up to kCarry; n = 2^22, k = 64, one request:
+// 44.5 us against 49.4 with lists).  Lists: bin lists beside arrays sized by z_cap (up to kFinSmemMax).
+// Large: finish_large (beyond that; on smaller plans its extra phases cost more than they give: n = 2^20,
+// k = 130, batch 8: 136 us against 111).
+enum DecodeKind { kDecodeMasks = 0, kDecodeLarge = 1, kDecodeLists = 2 };
+
 // Per-request descriptor of a launch (device table, optional).  Without a table, request s of a
 // launch reads row s of the batch and draws its hashings with the launch's seed and request index s;
 // with one, request s reads x, draws with (seed, id), so its result does not depend on which slot of
@@ -50,7 +57,7 @@ struct ExactRound {
     size_t smem = 0;          // dynamic shared memory of the round kernel
     size_t smem_gather = 0;   // of which the gather and the bins need this
     bool fin_global = false;  // the arrays of finish_round do not fit on chip: they live in d_fin
-    bool large = false;       // the transform's decode is finish_large (the same for all of a plan's rounds)
+    int kind = 0;             // DecodeKind of the plan
     bool owner = false;       // gather_owner folds the round (a CTA per kOwnerRes residues)
     uint32_t ring = 0;        // samples gather_owner keeps of a residue
     size_t fin_bytes = 0;     // device memory a request's decode may need
@@ -74,8 +81,8 @@ struct ExactArgs {
     uint32_t chunks, stage, maxshift;
     uint32_t gctas;            // gather CTAs of the round per request: its chunks, or B / kOwnerRes (owner)
     uint32_t owner, ring;      // fold by gather_owner, with this many samples kept of a residue
-    uint32_t large;            // decode by finish_large
-    uint32_t large_smem;       // its dynamic shared memory
+    uint32_t kind;             // DecodeKind
+    uint32_t large_smem;       // dynamic shared memory of finish_large
     uint32_t ctaps;            // taps per CTA: chunk c gathers taps [-T + c ctaps, -T + (c + 1) ctaps)
     const float* taps32;
     const double* taps64;
@@ -125,7 +132,7 @@ struct ExactArgs {
 // needs round t - 1's zhat: whichever arrives last at counter2 -- the bins part, or round t - 1's
 // decode -- runs it, then arrives at round t + 1's counter2.  Nobody waits.  The round
 // blocks (tables, workspace and this launch's signal and outputs) travel in the kernel parameters,
-// NR of them (8, 16 or 32: the smallest that holds the plan's rounds).
+// NR of them (8 or 32: the smallest that holds the plan's rounds).
 template <int NR>
 struct StepParams {
     uint32_t R;
@@ -415,7 +422,7 @@ cudaError_t launch_exact_channels(const ExactArgs* rounds, uint32_t R, uint32_t 
                                   uint32_t id, size_t smem, uint32_t* error, cudaStream_t st, cudaEvent_t before,
                                   cudaEvent_t after);
 // mixed batches, and the check of a bounded wait
-cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, bool large);
+cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, int kind);
 cudaError_t launch_wait_check(const uint32_t* word, int32_t* error, cudaStream_t st);
 cudaError_t launch_exact_decode(const DecodeArgs& a, cudaStream_t st);
 cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
@@ -437,6 +444,7 @@ size_t exact_gather_smem(uint32_t stage, bool fp64);
 size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64);
 size_t exact_owner_smem(uint32_t ring, bool fp64);
-cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, bool large);
-cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, bool large);
+cudaError_t set_round_smem_limit(size_t bytes, bool fp64);
+cudaError_t set_exact_smem_limit(size_t bytes, bool fp64, int kind);
+cudaError_t set_batch_smem_limit(size_t bytes, bool fp64, int kind);
 }  // namespace sfft
