@@ -266,6 +266,17 @@ def _oracle_general_worker(args):
     return dt, float(np.linalg.norm(X - Z) / np.sqrt(np.sum(np.sort(np.abs(X) ** 2)[: n - GEN_K])))
 
 
+def general_launches(sfft, plan):
+    """Kernels per stream group of a general-mode batch: a permuted copy for every round whose pairs gather
+    2n samples or more, one gather for all rounds, then three per round."""
+    n, copies = plan.params.n, 0
+    for r in range(plan.rounds):
+        i = sfft.general_round_info(plan, r)
+        pairs = i["dmax"] * plan.params.R_loc
+        copies += plan.params.permuted_copy == 0 and 2 * pairs * (2 * i["T"] + 1) >= 2 * n
+    return copies + 1 + 3 * plan.rounds
+
+
 def general_samples_per_transform(sfft, plan):
     """Samples one general-case transform gathers: every round's 2 R_loc D_max LocateInner hashings and
     R_est EstimateValues hashings, 2T + 1 each (one 32-byte sector per sample)."""
@@ -379,7 +390,7 @@ def run_general(args):
                          "bytes_per_transform": samples * 32, "samples_per_transform": samples,
                          "peak_kind": peak_kind},
             "e2e": e2e, "clocks": clk.summary(),
-            "gpu_launches": plan.rounds * 4 * min(params.streams or 4, batch) * args.steps,
+            "gpu_launches": general_launches(sfft, plan) * min(params.streams or 4, batch) * args.steps,
             "cpu_baseline": cpu,
         }
         print(json.dumps(line), flush=True)
@@ -612,7 +623,7 @@ def run_ours(args):
                        "precision": "complex64 gather/fold/bin FFT, FP64 subtraction and decode",
                        "l2": "inputs (8 GiB per GPU) exceed L2; no flush", "parallelism": f"replicas x{world}",
                        "support_exact_fraction": exact / batch,
-                       "path": "one persistent launch per step (device queue of request-round-chunk items)"
+                       "path": "one mixed-batch launch per step (sfft_batch_execute, all rounds)"
                                if args.path == "persistent" else "one kernel per step and stream group (all rounds)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": profiled_traffic() if batch == 256 else None,

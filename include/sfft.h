@@ -92,7 +92,7 @@ typedef struct sfft_params {
                               round's sigma) gather at least 2n samples first writes x_{sigma m} for
                               every m in [n] once per request, and those hashings read it in order
                               instead of at random (the same samples, so the same results; n complex64
-                              of device memory per request of max_batch); 1 -> never */
+                              of device memory per such round and request of max_batch); 1 -> never */
 } sfft_params;
 
 /* Fill *p with the library defaults for (n, k, mode); precision SFFT_FP32. */
@@ -150,8 +150,9 @@ sfft_status sfft_plan_taps(sfft_plan plan, uint32_t t, double* h_taps, uint64_t 
  *   d_count[r]                    number of entries written (<= cap)
  *   d_flag[r]                     sfft_status of the request: OK, NOT_CONVERGED or CAPACITY
  * Exact mode follows Algorithm 1: one kernel launch per stream group covers every round, since the
- * samples of all rounds are known before any is decoded; general mode follows Algorithms 2 and 3 with
- * four launches per round (five in a round that writes the permuted copy; see permuted_copy).
+ * samples of all rounds are known before any is decoded; general mode follows Algorithms 2 and 3 with,
+ * per stream group, one gather for all rounds (after a launch per permuted copy; see permuted_copy) and
+ * three launches per round.
  * Asynchronous on `stream`; the plan may run one call at a time.
  * Errors: INVALID_ARG (null pointer, batch out of range, cap == 0), CUDA (launch failure, including a
  * batch whose chunks would exceed 2^31 - 1 CTAs).
