@@ -30,6 +30,27 @@ sfft_status cuda_fail(cudaError_t e, const char* what) {
 
 bool is_pow2(uint64_t v) { return v && !(v & (v - 1)); }
 
+// part(0 .. parts - 1) queue work on the n streams `side` and on st, all of it after what st holds now; st
+// then goes on after all of it, also when a part fails: what has been launched by then still reads the
+// caller's signals and writes the outputs, so the caller's stream must not run ahead of it.  Returns the
+// first error.
+template <typename Part>
+sfft_status fork_join(cudaStream_t st, cudaEvent_t fork, const cudaStream_t* side, const cudaEvent_t* join, uint32_t n,
+                      uint32_t parts, Part part) {
+    sfft_status status = SFFT_OK;
+    auto check = [&](cudaError_t e, const char* what) {
+        if (e != cudaSuccess && status == SFFT_OK) status = cuda_fail(e, what);
+        return e == cudaSuccess;
+    };
+    uint32_t forked = 0;
+    if (n == 0 || check(cudaEventRecord(fork, st), "fork"))
+        while (forked < n && check(cudaStreamWaitEvent(side[forked], fork, 0), "fork")) ++forked;
+    for (uint32_t p = 0; p < parts && status == SFFT_OK; ++p) status = part(p);
+    for (uint32_t g = 0; g < forked; ++g)
+        if (check(cudaEventRecord(join[g], side[g]), "join")) check(cudaStreamWaitEvent(st, join[g], 0), "join");
+    return status;
+}
+
 // the counts and flags of requests [0, batch) (the counts of the others with them)
 cudaError_t clear_zhat(const sfft_plan_s* pl, uint32_t batch, cudaStream_t st) {
     return cudaMemsetAsync(pl->d_zcount, 0, ((size_t)pl->max_batch + batch) * sizeof(uint32_t), st);
@@ -446,12 +467,8 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
     uint32_t groups = plan->nstreams;
     if (groups > batch) groups = batch;
     if (tr) groups = 1;  // a trace records the whole batch's round on the caller's stream
-    if (groups > 1) {
-        SFFT_CUDA(cudaEventRecord(plan->ev_fork, st), "fork");
-        for (uint32_t g = 0; g < groups; ++g) SFFT_CUDA(cudaStreamWaitEvent(plan->aux[g], plan->ev_fork, 0), "fork");
-    }
     const size_t zc = p.z_cap;
-    for (uint32_t g = 0; g < groups; ++g) {
+    auto group = [&](uint32_t g) -> sfft_status {
         const uint32_t r0 = (uint32_t)((uint64_t)batch * g / groups);
         const uint32_t r1 = (uint32_t)((uint64_t)batch * (g + 1) / groups);
         cudaStream_t gs = groups > 1 ? plan->aux[g] : st;
@@ -551,12 +568,9 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
                           "trace");
             }
         }
-        if (groups > 1) {
-            SFFT_CUDA(cudaEventRecord(plan->ev_join[g], gs), "join");
-            SFFT_CUDA(cudaStreamWaitEvent(st, plan->ev_join[g], 0), "join");
-        }
-    }
-    return SFFT_OK;
+        return SFFT_OK;
+    };
+    return fork_join(st, plan->ev_fork, plan->aux, plan->ev_join, groups > 1 ? groups : 0, groups, group);
 }
 
 }  // extern "C"
@@ -578,11 +592,7 @@ sfft_status sfft::execute_batch(sfft_plan plan, const void* d_x, const ReqDesc* 
     uint32_t groups = plan->nstreams;
     if (groups > batch) groups = batch;
     if (batch < 8) groups = 1;
-    if (groups > 1) {
-        SFFT_CUDA(cudaEventRecord(plan->ev_fork, st), "fork");
-        for (uint32_t g = 0; g < groups; ++g) SFFT_CUDA(cudaStreamWaitEvent(plan->aux[g], plan->ev_fork, 0), "fork");
-    }
-    for (uint32_t g = 0; g < groups; ++g) {
+    auto group = [&](uint32_t g) -> sfft_status {
         const uint32_t r0 = (uint32_t)((uint64_t)batch * g / groups);
         const uint32_t r1 = (uint32_t)((uint64_t)batch * (g + 1) / groups);
         cudaStream_t gs = groups > 1 ? plan->aux[g] : st;
@@ -601,12 +611,9 @@ sfft_status sfft::execute_batch(sfft_plan plan, const void* d_x, const ReqDesc* 
             a.out_flag = d_flag;
         }
         SFFT_CUDA(launch_exact_step(rounds, R, r1 - r0, plan->step_smem, gs, fp64), "exact step");
-        if (groups > 1) {
-            SFFT_CUDA(cudaEventRecord(plan->ev_join[g], gs), "join");
-            SFFT_CUDA(cudaStreamWaitEvent(st, plan->ev_join[g], 0), "join");
-        }
-    }
-    return SFFT_OK;
+        return SFFT_OK;
+    };
+    return fork_join(st, plan->ev_fork, plan->aux, plan->ev_join, groups > 1 ? groups : 0, groups, group);
 }
 
 extern "C" {
@@ -1227,23 +1234,17 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
     a.out_count = d_count;
     a.out_flag = d_flag;
     const bool both = ctas[0] != 0 && ctas[1] != 0;
-    if (both) {
-        SFFT_CUDA(cudaEventRecord(bp->ev_fork, st), "fork");
-        SFFT_CUDA(cudaStreamWaitEvent(bp->side, bp->ev_fork, 0), "fork");
-    }
-    for (int kind = 1; kind >= 0; --kind) {  // the longer chains first
+    auto of_kind = [&](uint32_t part) -> sfft_status {
+        const int kind = part == 0 ? 1 : 0;  // the longer chains first
         a.seg = reinterpret_cast<const uint32_t*>(d + L.seg) + seg0[kind];
         a.seg_who = reinterpret_cast<const uint32_t*>(d + L.who) + seg0[kind];
         a.nseg = (uint32_t)(seg0[kind + 1] - seg0[kind]);
         SFFT_CUDA(launch_exact_batch(a, (uint32_t)ctas[kind], bp->smem[kind], both && kind ? bp->side : st, bp->fp64,
                                      kind ? (int)kDecodeLarge : bp->small_kind),
                   "mixed batch");
-    }
-    if (both) {
-        SFFT_CUDA(cudaEventRecord(bp->ev_join, bp->side), "join");
-        SFFT_CUDA(cudaStreamWaitEvent(st, bp->ev_join, 0), "join");
-    }
-    return SFFT_OK;
+        return SFFT_OK;
+    };
+    return fork_join(st, bp->ev_fork, &bp->side, &bp->ev_join, both ? 1 : 0, 2, of_kind);
 }
 
 }  // extern "C"

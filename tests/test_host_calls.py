@@ -1,0 +1,60 @@
+"""The host side of the C entry points, on a stand-in for the CUDA runtime (fake_runtime)."""
+import ctypes
+
+import pytest
+
+from paper_1201_2501_gb300 import sfft
+from tests import fake_runtime as fr
+
+STREAM = ctypes.c_void_p(0xABC000)
+
+
+@pytest.fixture(scope="module")
+def L(tmp_path_factory):
+    return fr.load(tmp_path_factory.mktemp("fake"))
+
+
+def _outputs():
+    return ctypes.c_void_p(0x1000), ctypes.c_void_p(0x2000), 64, ctypes.c_void_p(0x3000), ctypes.c_void_p(0x4000)
+
+
+def _run_mixed(L):
+    plans = [fr.plan(L, 1 << 14, 8), fr.plan(L, 1 << 16, 512)]  # one of each kind of decode
+    assert [s for s, _ in plans] == [0, 0]
+    handles = (ctypes.c_void_p * 2)(*[h for _, h in plans])
+    bp = ctypes.c_void_p()
+    assert L.sfft_batch_plan_create(handles, 2, 4, ctypes.byref(bp)) == 0
+    table = (sfft.SfftRequest * 2)()
+    for r in range(2):
+        table[r].d_x = 0x10000
+    call = lambda: L.sfft_batch_execute(bp, (ctypes.c_uint32 * 2)(0, 1), table, 2, STREAM, *_outputs())
+    return call, lambda: (L.sfft_batch_plan_destroy(bp), [L.sfft_plan_destroy(h) for _, h in plans])
+
+
+def _run_groups(L, mode):
+    s, h = fr.plan(L, 1 << 14, 8, mode, batch=16, streams=4)
+    assert s == 0
+    call = lambda: L.sfft_execute(h, ctypes.c_void_p(0x10000), 16, ctypes.c_uint64(5), STREAM, *_outputs())
+    return call, lambda: L.sfft_plan_destroy(h)
+
+
+@pytest.mark.parametrize("what", ["mixed", "exact", "general"])
+def test_a_launch_that_fails_leaves_nothing_running_unordered(L, what):
+    """A call that spreads its work over streams and fails at any of its launches returns SFFT_ERR_CUDA, and
+    the caller's stream still waits for every launch made before: the caller may free its arrays behind it."""
+    call, close = _run_mixed(L) if what == "mixed" else _run_groups(L, {"exact": 0, "general": 1}[what])
+    L.fake_reset()
+    assert call() == 0
+    st = hex(STREAM.value)
+    total = sum(c[0] == "launch" for c in fr.log(L))
+    assert total >= 2 and len({c[2] for c in fr.log(L) if c[0] == "launch"}) >= 2  # on several streams
+    assert fr.unordered(fr.log(L), st) == []
+    for good in range(total):
+        L.fake_reset()
+        L.fake_fail_launch(good)
+        assert call() == sfft.SFFT_ERR_CUDA
+        assert b"a call made to fail" in L.sfft_last_error()
+        assert sum(c[0] == "launch" for c in fr.log(L)) == good
+        assert fr.unordered(fr.log(L), st) == [], good
+    L.fake_reset()
+    close()
