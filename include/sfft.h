@@ -92,7 +92,8 @@ typedef struct sfft_params {
                               round's sigma) gather at least 2n samples first writes x_{sigma m} for
                               every m in [n] once per request, and those hashings read it in order
                               instead of at random (the same samples, so the same results; n complex64
-                              of device memory per such round and request of max_batch); 1 -> never */
+                              of device memory per such round and request of max_batch, or per request
+                              alone where the rounds take turns; see sfft_plan_create); 1 -> never */
 } sfft_params;
 
 /* Fill *p with the library defaults for (n, k, mode); precision SFFT_FP32. */
@@ -113,7 +114,9 @@ typedef struct sfft_plan_s* sfft_plan;
  * Build a plan: the round schedule, the flat-window taps of every round (Sec. 7, Lemma on window
  * construction), the exact window response table W(o), |o| <= n/2B, of every round, and a device
  * workspace for max_batch requests.  The only call that allocates device memory.  Runs on the
- * current CUDA device and synchronises it.
+ * current CUDA device and synchronises it.  A general-mode plan whose rounds, gathered all at once, would
+ * take more than 1/64 of the device's memory beyond what the largest round alone takes, or more than is
+ * free, is built to gather them one after another in the memory of one (slower, the same results).
  * Errors: INVALID_ARG (null, max_batch == 0, bad field), N_NOT_POW2, K_RANGE, OOM, CUDA.
  */
 sfft_status sfft_plan_create(const sfft_params* p, uint32_t max_batch, sfft_plan* out);
@@ -151,8 +154,8 @@ sfft_status sfft_plan_taps(sfft_plan plan, uint32_t t, double* h_taps, uint64_t 
  *   d_flag[r]                     sfft_status of the request: OK, NOT_CONVERGED or CAPACITY
  * Exact mode follows Algorithm 1: one kernel launch per stream group covers every round, since the
  * samples of all rounds are known before any is decoded; general mode follows Algorithms 2 and 3 with,
- * per stream group, one gather for all rounds (after a launch per permuted copy; see permuted_copy) and
- * three launches per round.
+ * per stream group, one gather for all rounds (one per round in a plan that gathers them in turn; after
+ * a launch per permuted copy; see permuted_copy) and three launches per round.
  * Asynchronous on `stream`; the plan may run one call at a time.
  * Errors: INVALID_ARG (null pointer, batch out of range, cap == 0), CUDA (launch failure, including a
  * batch whose chunks would exceed 2^31 - 1 CTAs).

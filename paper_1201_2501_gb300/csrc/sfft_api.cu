@@ -188,9 +188,23 @@ sfft_status sfft::validate_params(const sfft_params* p) {
     return SFFT_OK;
 }
 
+static sfft_status create(const sfft_params* p, uint32_t max_batch, const sfft_plan_s* tables, bool* by_round,
+                          sfft_plan* out);
+
 // Plan creation; with `tables` (a plan of the same parameters) its schedule and host window tables
 // are copied instead of computed again.
 sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sfft_plan_s* tables, sfft_plan* out) {
+    bool by_round = false;
+    const sfft_status st = create(p, max_batch, tables, &by_round, out);
+    if (st != SFFT_ERR_OOM || by_round || p->mode != SFFT_GENERAL) return st;
+    by_round = true;  // the memory of one round at a time may still be there
+    return create(p, max_batch, tables, &by_round, out);
+}
+
+// *by_round: a general plan's rounds are to share the memory of folds and permuted copies; set where the
+// plan does so by itself.
+static sfft_status create(const sfft_params* p, uint32_t max_batch, const sfft_plan_s* tables, bool* by_round,
+                          sfft_plan* out) {
     if (!out) return SFFT_ERR_INVALID_ARG;
     *out = nullptr;
     sfft_status st = validate(p);
@@ -255,10 +269,13 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         free_plan(pl);
         return SFFT_ERR_K_RANGE;
     }
+    size_t round_part = 0, copies = 0;  // general: folds of the largest round, rounds with a permuted copy
     for (GeneralRound& r : pl->grounds) {  // every round's folds live at once: one gather serves all rounds
         pl->samples += (uint64_t)r.nhash * (2 * (uint64_t)r.T + 1);
         r.part_off = part_elems;
         part_elems += (size_t)r.ngroups * 2 * r.B;
+        round_part = std::max(round_part, (size_t)r.ngroups * 2 * r.B);
+        copies += r.perm ? 1 : 0;
         if ((size_t)r.nhash * r.B > pl->bins_stride) pl->bins_stride = (size_t)r.nhash * r.B;
         if ((size_t)r.npairs * r.B > pl->phase_stride) pl->phase_stride = (size_t)r.npairs * r.B;
         if (r.B > maxB) maxB = r.B;
@@ -267,6 +284,21 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         fs_max = r.smem_finish > fs_max ? r.smem_finish : fs_max;
         ls_max = r.smem_locate > ls_max ? r.smem_locate : ls_max;
         ss_max = r.smem_select > ss_max ? r.smem_select : ss_max;
+    }
+    if (general) {
+        // Gathering all rounds at once is faster (see launch_general_gather) and holds every round's folds and
+        // permuted copies.  Where that takes more than 1/64 of the device's memory beyond the largest round's,
+        // or does not fit, the rounds are gathered one after another into the same memory.
+        size_t free_bytes = 0, total_bytes = 0;
+        cudaMemGetInfo(&free_bytes, &total_bytes);
+        const size_t extra = part_elems - round_part + (copies > 1 ? (copies - 1) * p->n : 0);
+        if (extra * max_batch * sizeof(float2) > total_bytes / 64) *by_round = true;
+        pl->by_round = *by_round;
+        if (pl->by_round) {
+            for (GeneralRound& r : pl->grounds) r.part_off = 0;
+            part_elems = round_part;
+            copies = std::min<size_t>(copies, 1);
+        }
     }
     pl->part_stride = part_elems;
     pl->max_B = maxB;
@@ -282,6 +314,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         pl->dev_bytes += (bytes);                                     \
         if (e != cudaSuccess) {                                       \
             set_last_error(std::string("cudaMalloc: ") + cudaGetErrorString(e)); \
+            cudaGetLastError(); /* not left for the next launch to report */ \
             free_plan(pl);                                            \
             return SFFT_ERR_OOM;                                      \
         }                                                             \
@@ -323,9 +356,7 @@ sfft_status sfft::plan_create(const sfft_params* p, uint32_t max_batch, const sf
         SFFT_ALLOC(pl->d_phase, pl->phase_stride * max_batch * sizeof(uint32_t));
         SFFT_ALLOC(pl->d_L, sum_B * max_batch * sizeof(uint32_t));
         SFFT_ALLOC(pl->d_estw, (size_t)max_batch * sum_B * (sizeof(double2) + sizeof(double)));
-        size_t perm = 0;
-        for (const GeneralRound& r : pl->grounds) perm += r.perm ? 1 : 0;
-        if (perm) SFFT_ALLOC(pl->d_xperm, perm * max_batch * p->n * sizeof(float2));
+        if (copies) SFFT_ALLOC(pl->d_xperm, copies * max_batch * p->n * sizeof(float2));
     }
 #undef SFFT_ALLOC
     auto fail = [&](cudaError_t err, const char* what) {
@@ -480,7 +511,8 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             GenArgs& a = args[r];
             std::memset(&a, 0, sizeof(a));
             a.x = reinterpret_cast<const float2*>(d_x);
-            a.xperm = gr.perm ? plan->d_xperm + (nperm++) * plan->max_batch * p.n : nullptr;
+            a.xperm = gr.perm ? plan->d_xperm + nperm * plan->max_batch * p.n : nullptr;
+            nperm += gr.perm && !plan->by_round ? 1 : 0;
             a.reqs = d_reqs;
             a.n = p.n;
             a.nmask = (uint32_t)(p.n - 1);
@@ -538,9 +570,11 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
                 a.dbg_valid = tr->d_valid;
             }
         }
-        SFFT_CUDA(launch_general_gather(args, plan->grounds.data(), R, r1 - r0, gs), "general gather");
+        if (!plan->by_round)
+            SFFT_CUDA(launch_general_gather(args, plan->grounds.data(), R, r1 - r0, gs), "general gather");
         for (uint32_t r = 0; r < R; ++r) {
             const GeneralRound& gr = plan->grounds[r];
+            if (plan->by_round) SFFT_CUDA(launch_general_gather(args + r, &gr, 1, r1 - r0, gs), "general gather");
             const bool traced = tr && tr->round == r;
             const GenArgs& a = args[r];
             if (traced) {

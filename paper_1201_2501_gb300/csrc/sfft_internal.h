@@ -327,7 +327,8 @@ struct sfft_plan_s {
     uint32_t* d_L = nullptr;  // general mode: per round r, [max_batch][B_r] candidates
     double2* d_tw = nullptr;  // general mode, exact FP64: twiddle factor tables (2^tw_shift + n / 2^tw_shift)
     uint32_t tw_shift = 0;
-    float2* d_xperm = nullptr;  // general mode, per round with perm: [max_batch][n] permuted signals
+    float2* d_xperm = nullptr;  // general mode, per round with perm (by_round: one): [max_batch][n] permuted signals
+    bool by_round = false;      // general mode: the rounds' folds and permuted copies share the largest one's memory
     // general mode: per round r, [max_batch][B_r] estimates; then per round [max_batch][B_r] magnitudes
     double2* d_estw = nullptr;
     size_t bins_stride = 0, phase_stride = 0;
@@ -433,7 +434,7 @@ size_t general_finish_smem(uint32_t B, uint32_t nzmax);
 size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est);
 size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
 cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate);
-// the gathers of every round (and the permuted copies they read), then per round the rest
+// the gathers of R rounds (and the permuted copies they read), then per round the rest
 cudaError_t launch_general_gather(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st);
 cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st);
 cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);

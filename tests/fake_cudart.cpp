@@ -16,7 +16,7 @@
 namespace {
 std::string g_log;
 std::map<const void*, size_t> g_allocs;
-size_t g_bytes = 0;
+size_t g_bytes = 0, g_memory = size_t(1) << 38;
 int g_fail_launch = -1;
 std::map<const void*, std::string>& names() {  // filled while the library's own objects are initialised
     static std::map<const void*, std::string> m;
@@ -58,11 +58,13 @@ void fake_reset() {
     g_fail_launch = -1;
     g_on_launch = nullptr;
     g_last = cudaSuccess;
+    g_memory = size_t(1) << 38;
 }
 const char* fake_log() { return g_log.c_str(); }
 void fake_fail_launch(int after) { g_fail_launch = after; }  // the launch after that many successful ones
 void fake_on_launch(LaunchFn f) { g_on_launch = f; }
 size_t fake_bytes() { return g_bytes; }
+void fake_memory(size_t bytes) { g_memory = bytes; }  // what the other users of the device leave of 2^38
 
 // kernels
 void** __cudaRegisterFatBinary(void*) {
@@ -103,6 +105,7 @@ cudaError_t cudaLaunchHostFunc(cudaStream_t, cudaHostFn_t, void*) { return cudaS
 
 // memory
 cudaError_t cudaMalloc(void** p, size_t bytes) {
+    if (g_bytes + bytes > g_memory) return g_last = cudaErrorMemoryAllocation;
     *p = mmap(nullptr, bytes ? bytes : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
     if (*p == MAP_FAILED) return g_last = cudaErrorMemoryAllocation;
     g_allocs[*p] = bytes ? bytes : 1;
@@ -145,7 +148,8 @@ cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
     return cudaSuccess;
 }
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) {
-    *f = *t = size_t(1) << 38;
+    *f = g_memory - g_bytes;
+    *t = size_t(1) << 38;
     return cudaSuccess;
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void*) {

@@ -58,3 +58,36 @@ def test_a_launch_that_fails_leaves_nothing_running_unordered(L, what):
         assert fr.unordered(fr.log(L), st) == [], good
     L.fake_reset()
     close()
+
+
+# per request of max_batch, the most device memory a general plan may take: what it took when the rounds
+# gathered one after another (bytes: (log2 n, k, fields) -> one request)
+GENERAL_BYTES = [(16, 16, dict(alpha0=0.25), 967_600), (15, 16, dict(bins_per_k=4.0), 529_600), (16, 64, {}, 2_520_700)]
+
+
+@pytest.mark.parametrize("m,k,fields,per", GENERAL_BYTES)
+def test_a_general_plan_takes_the_memory_of_one_round_where_it_has_to(L, m, k, fields, per):
+    """A plan for as many requests as fit when rounds take turns in the memory of one is built, by the size of
+    the plan alone or because other users hold the rest of the device, and runs; a smaller plan keeps one
+    gather for all rounds."""
+    def gathers(h, batch):
+        L.fake_reset()
+        assert L.sfft_execute(h, ctypes.c_void_p(0x10000), batch, ctypes.c_uint64(5), STREAM, *_outputs()) == 0
+        names = [c[1] for c in fr.log(L) if c[0] == "launch"]
+        assert sum("k_gen_select" in n for n in names) == L.sfft_plan_rounds(h)
+        return sum("k_gen_gather" in n for n in names)
+
+    L.fake_reset()
+    st, h = fr.plan(L, 1 << m, k, sfft.SFFT_GENERAL, batch=64, **fields)
+    at_once, rounds = L.fake_bytes(), L.sfft_plan_rounds(h)
+    assert st == 0 and gathers(h, 1) == 1 and rounds > 1
+    L.sfft_plan_destroy(h)
+    for batch, memory in (((1 << 38) // per, 1 << 38), (64, min(64 * per + (1 << 20), at_once - 1))):
+        L.fake_reset()
+        L.fake_memory(ctypes.c_size_t(memory))
+        st, h = fr.plan(L, 1 << m, k, sfft.SFFT_GENERAL, batch=batch, **fields)
+        assert st == 0, batch
+        assert L.fake_bytes() <= batch * per + (1 << 20)  # (the tables are the plan's, not a request's)
+        assert gathers(h, 1) == rounds
+        L.sfft_plan_destroy(h)
+    L.fake_reset()
