@@ -360,6 +360,18 @@ __device__ __forceinline__ float dot2(float a, float x, float b, float y) {
     const float e = __fadd_rn(__fsub_rn(p, __fsub_rn(s, t)), __fsub_rn(q, t));
     return __fadd_rn(s, __fadd_rn(e, __fadd_rn(pe, qe)));
 }
+// (z.x, z.y) for an FP32 arctangent: times a power of two where the larger part lies outside 2^-96 .. 2^124,
+// where float loses it (signals scaled below about 1e-15 or above 1e18); the phase stays.
+__device__ __forceinline__ float2 direction(double2 z) {
+    const uint32_t hx = (uint32_t)__double2hiint(z.x) & 0x7FFFFFFFu, hy = (uint32_t)__double2hiint(z.y) & 0x7FFFFFFFu;
+    const uint32_t e = max(hx, hy) >> 20;  // 1023 + the larger part's exponent
+    if (e - 927u > 220u && e - 1u < 2045u) {
+        const double scale = __hiloint2double((int)((2046u - e) << 20), 0);
+        z.x *= scale;
+        z.y *= scale;
+    }
+    return make_float2((float)z.x, (float)z.y);
+}
 
 __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -390,8 +402,8 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
     // a bin after the last entry: stored, and c_j for a pair: an FP32 arctangent of the product
     // u_j conj(u'_j) (the vote arcs are s pi wide and the FP32 bins carry ~1e-6 of phase noise), in units
     // of 2^-32 of a turn; z is the product rounded to float
-    auto store_phase = [&](uint32_t j, float zx, float zy) {
-        phase[j] = (uint32_t)__double2int_rn(widen(atan2f(zy, zx)) * (4294967296.0 * 0.15915494309189533576888));
+    auto store_phase = [&](uint32_t j, float2 z) {
+        phase[j] = (uint32_t)__double2int_rn(widen(atan2f(z.y, z.x)) * (4294967296.0 * 0.15915494309189533576888));
     };
     if (nz == 0) {
         for (uint32_t j = tid; j < B; j += kThreads) {
@@ -400,15 +412,11 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
             if (h.H == 2) {
                 const float2 v = U[B + j];
                 bins[(size_t)(row0 + 1) * B + j] = make_double2(widen(v.x), widen(v.y));
-                float zx = dot2(u.x, v.x, u.y, v.y), zy = dot2(u.y, v.x, -u.x, v.y);
-                const float mag = fabsf(zx) + fabsf(zy);
-                if (!(mag > 1e-30f && mag < 1e38f)) {  // beyond the range of the exact products' errors
-                    const double2 z = mul_conj_rn(make_double2(widen(u.x), widen(u.y)),
-                                                  make_double2(widen(v.x), widen(v.y)));
-                    zx = (float)z.x;
-                    zy = (float)z.y;
-                }
-                store_phase(j, zx, zy);
+                float2 z = make_float2(dot2(u.x, v.x, u.y, v.y), dot2(u.y, v.x, -u.x, v.y));
+                const float mag = fabsf(z.x) + fabsf(z.y);
+                if (!(mag > 1e-30f && mag < 1e38f))  // beyond the range of the exact products' errors
+                    z = direction(mul_conj_rn(make_double2(widen(u.x), widen(u.y)), make_double2(widen(v.x), widen(v.y))));
+                store_phase(j, z);
             }
         }
         return;
@@ -509,8 +517,7 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
                     if (h.H == 2) {
                         const double2 v = make_double2(ub[2 * B + j], ub[3 * B + j]);
                         bins[(size_t)(row0 + 1) * B + j] = v;
-                        const double2 z = mul_conj_rn(u, v);
-                        store_phase(j, (float)z.x, (float)z.y);
+                        store_phase(j, direction(mul_conj_rn(u, v)));
                     }
                 }
         } else {
@@ -529,8 +536,7 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
                     }
                 for (uint32_t hh = 0; hh < h.H; ++hh) bins[(size_t)(row0 + hh) * B + j] = u[hh];
                 if (h.H == 2 && last) {
-                    const double2 z = mul_conj_rn(u[0], u[1]);
-                    store_phase(j, (float)z.x, (float)z.y);
+                    store_phase(j, direction(mul_conj_rn(u[0], u[1])));
                 }
             }
         }
@@ -749,9 +755,9 @@ __device__ void sort_by_magnitude(const double* mag, const uint32_t* idx, uint32
 //
 // A vote compares the position e / M of beta (m + sigma b) with the arc of half width s / 2 around c_j,
 // both as 32-bit fractions of a turn: with M = n 2^F scaled to 2^64 the product wraps by itself and its
-// upper word is the position.  The pipeline's c_j comes from an FP32 arctangent of the FP64 product
-// u_j conj(u'_j): rounding the product to float and atan2f's few-ulp error move it by less than 2e-7 of
-// a turn, and the 32-bit fractions by less than 1e-9.  A vote within 2^-20 of a turn (about 1e-6) of an
+// upper word is the position.  The pipeline's c_j comes from an FP32 arctangent of the product
+// u_j conj(u'_j) (in FP64, or good to 2^-46): rounding it to float (see direction) and atan2f's few-ulp error
+// move it by less than 2e-7 of a turn, and the 32-bit fractions by less than 1e-9.  A vote within 2^-20 of a turn (about 1e-6) of an
 // arc end is decided by the FP64 test on the FP64 phase of the pair's stored bins; every other one is
 // farther than that error from the arc ends of either phase, so both give the same vote.
 constexpr int kLocBins = kThreads / 8;               // bins per CTA at the smallest t
