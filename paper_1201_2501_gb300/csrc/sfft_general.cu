@@ -815,8 +815,8 @@ __global__ void __launch_bounds__(kThreads) k_gen_locate(const GenArgs a) {
     const uint64_t M = uint64_t(1) << logM, mask = M - 1;
     const uint32_t sh = 64u - logM;
     const uint64_t sb_fp = ((uint64_t)((sigma * b) & a.nmask)) << kFracBits;
-    // half width of the vote arc, s / 2 of a turn (an arc of a whole turn or more takes every vote)
-    const uint32_t hw = a.s >= 1.0 ? 0xFFFFFFFFu - kPhaseGuard : (uint32_t)__double2uint_rn(a.s * 2147483648.0);
+    // half width of the vote arc, s / 2 of a turn (s = 1.5 takes every vote, as any larger s does)
+    const uint32_t hw = (uint32_t)__double2uint_rn((a.s > 1.5 ? 1.5 : a.s) * 2147483648.0);
     const double2* rbins = a.bins + (size_t)s * a.bins_stride;
     // the bin's region (start l_fp, width w_D) and its bottom flag live in registers, the same in every
     // lane of the bin's group (t divides 32)
