@@ -454,9 +454,9 @@ __device__ __forceinline__ int decode_bin_fp32(const DecodeCtx& d, uint32_t j, c
 // outcome in both, so the decode is that of decode_bin_fp64 (about 200 FP64 operations per bin and warp at
 // 1/64 of the FP32 rate).  Values stay in FP64.
 constexpr float kMagGuard = 2e-6f, kPhaseGuard32 = 1e-6f;
-// -1: m < t, 1: m > t, 0: too close
+// -1: m < t, 1: m > t, 0: too close (also among the denormal numbers, whose rounding is not relative)
 __device__ __forceinline__ int cmp_guarded(float m, float t) {
-    const float g = kMagGuard * t;
+    const float g = fmaf(kMagGuard, t, 1e-36f);
     return m > t + g ? 1 : (m < t - g ? -1 : 0);
 }
 constexpr int kUndecided = -1;
@@ -486,6 +486,7 @@ __device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j
     for (int l = 0; l < kMaxHash - 1; ++l)
         if ((uint32_t)l < L) {
             ml[l] = hypotf(v[l + 1].x, v[l + 1].y);
+            if (!(ml[l] > 1e-30f && ml[l] * mag0 > 1e-30f)) return kUndecided;  // the phase of a product FP32 holds
             th[l] = phase01_f(mul_conj_f(v[0], v[l + 1]));
         }
     // location ladder, coarsest shift first: each rounding has to stay clear of a half

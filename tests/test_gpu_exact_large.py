@@ -120,3 +120,103 @@ def test_fp64_decisions_at_their_boundaries(sf, m, k, t):
         v = wval.cpu().numpy()[:cnt]
         assert np.max(np.abs(v[:, 0] + 1j * v[:, 1] - ov[order]) / np.maximum(1.0, np.abs(ov[order])), initial=0.0) <= 1e-12
     plan.close()
+
+
+@pytest.mark.parametrize("m,k,t", [(14, 8, 0), (18, 64, 0), (22, 64, 1)])
+def test_fp64_decisions_on_magnitudes_below_fp32(sf, m, k, t):
+    """The same where FP32 holds a magnitude or a product of two only as a denormal number or not at all:
+    re-estimation windows at 1e-40 with residuals 1e-7 to 1e-3 (relative) from their ends, and ladder
+    hashings of 1e-38 to 1 of u_0 under an isolation tolerance that lets them pass."""
+    n = 1 << m
+    f = exact_fields(n, k, thr=1e-8, ref_lo=1e-32, ref_hi=4e-32, iso_tol=2.0)
+    P = oracle_params(f)
+    plan = sf.Plan(_params(sf, f, 1), 1)
+    info = plan.round_info(t, seed=5)
+    B, shifts = info["B"], info["shifts"]
+    Np, L = n // B, len(shifts)
+    rng = np.random.default_rng(m + t)
+    phases = lambda th: np.exp(-2j * np.pi * th)
+    for trial in range(16):
+        sigma, b = int(rng.integers(0, n)) | 1, int(rng.integers(0, n))
+        u = np.zeros((1 + L, B), dtype=np.complex128)
+        u[0] = 10.0 ** rng.uniform(-7.9, 0, B) * phases(rng.random(B))
+        c, M = np.zeros(B), 1.0
+        for l in range(L - 1, -1, -1):  # ladder roundings well away from a half-integer
+            ratio = Np / (shifts[l] // B) / M
+            y = np.floor(rng.random(B) * ratio) + 0.3 * rng.uniform(-1, 1, B)
+            c, M, th = c + M * (np.floor(y + 0.5) % ratio), M * ratio, (y + c / M) / ratio
+            u[l + 1] = u[0] * 10.0 ** rng.uniform(-38, 0, B) * phases(th)
+        known = np.sort(rng.choice(n, size=max(2, B // 4), replace=False)).astype(np.uint32)
+        for i in known:
+            j, _ = oracle.bin_offset((sigma * (int(i) - b)) % n, n, B)
+            off = float(rng.choice([-1, 1]) * 10.0 ** rng.uniform(-7, -3))
+            edge = rng.choice([P.ref_lo, P.ref_hi]) * P.thr * (1 + off) * phases(rng.random())
+            for h, be in enumerate([0] + list(shifts)):
+                u[h, j] = edge * phases(((be * sigma * int(i)) % n) / n)
+        widx, wval, aux = sf.sfft_exact_decode(plan, t, sigma, b, torch.as_tensor(np.stack([u.real, u.imag], -1)).cuda(),
+                                               torch.as_tensor(known.astype(np.int32)).cuda())
+        torch.cuda.synchronize()
+        cnt, nab, nkept = [int(v) for v in aux.cpu().numpy()]
+        oi, ov, oab, okept = oracle.exact_decode(P, B, info["alpha"], sigma, b, shifts, u, known.astype(np.uint64),
+                                                 with_kept=True)
+        order = np.argsort(oi)
+        assert (nab, nkept, cnt) == (oab, okept, len(oi))
+        assert np.array_equal(widx.cpu().numpy()[:cnt].astype(np.uint32).astype(np.int64), oi[order].astype(np.int64))
+        v = wval.cpu().numpy()[:cnt]
+        assert np.all(np.abs(v[:, 0] + 1j * v[:, 1] - ov[order]) <= 1e-12 * np.abs(ov[order]))
+    plan.close()
+
+
+@pytest.mark.parametrize("m,k", [(14, 8), (16, 130)])
+def test_fp64_pruning_at_its_bound(sf, m, k):
+    """|v| < prune thr is decided as FP64 decides it, also where FP32 cannot tell: with the bound a part in 1e9
+    above (dropped) and below (kept) the magnitude of the smallest entry (3/4 of the others'), in a decode on
+    chip and in one with arrays sized by what was found."""
+    n, seed = 1 << m, 33
+    f = exact_fields(n, k, delta=1e-8)
+    dt = np.complex128
+    s = workloads.exact_sparse(n, k, workloads.seed_for(2, 760), dtype=dt)
+    X = np.zeros(n, dtype=dt)
+    X[s.support] = s.values
+    weak = int(s.support[k // 2])
+    X[weak] *= 0.75
+    x = torch.as_tensor(np.fft.ifft(X)[None]).cuda()
+
+    def run(prune):
+        plan = sf.Plan(_params(sf, dict(f, prune=prune), 1), 1)
+        idx, val, cnt, flag = [o.cpu().numpy() for o in sf.sfft_execute(plan, x, seed, f["z_cap"])]
+        plan.close()
+        c = int(cnt[0])
+        return idx[0, :c].view(np.uint32).astype(np.int64), val[0, :c, 0] + 1j * val[0, :c, 1]
+
+    idx, val = run(f["prune"])
+    assert np.array_equal(idx, s.support)
+    size = float(np.abs(val[idx == weak])[0])
+    kept, _ = run(size * (1 - 1e-9) / f["thr"])
+    assert np.array_equal(kept, s.support)
+    dropped, _ = run(size * (1 + 1e-9) / f["thr"])
+    assert np.array_equal(dropped, s.support[s.support != weak])
+
+
+@pytest.mark.parametrize("m,k", [(14, 8), (16, 130), (14, 100)])
+def test_fp64_bins_at_the_threshold(sf, m, k):
+    """Whole transforms with thr = 1 of coefficients of magnitude 1: the bins' magnitudes lie within the window's
+    leakage (1e-8) of the threshold, on both sides, where FP32 cannot tell.  Supports, values and flags are the
+    oracle's, in a decode on chip and in those with arrays sized by what was found."""
+    n, seed, batch = 1 << m, 33, 3
+    f = exact_fields(n, k, delta=1e-8, thr=1.0)
+    P = oracle_params(f)
+    sigs = [workloads.exact_sparse(n, k, workloads.seed_for(2, 770 + i), dtype=np.complex128) for i in range(batch)]
+    plan = sf.Plan(_params(sf, f, 1), batch)
+    idx, val, cnt, flag = [o.cpu().numpy() for o in sf.sfft_execute(
+        plan, torch.as_tensor(np.stack([s.x for s in sigs])).cuda(), seed, f["z_cap"])]
+    plan.close()
+    missed = 0
+    for r, s in enumerate(sigs):
+        oi, ov, of = oracle.sfft_exact(P, s.x, seed, r)
+        c = int(cnt[r])
+        assert np.array_equal(idx[r, :c].view(np.uint32).astype(np.int64), oi.astype(np.int64))
+        assert int(flag[r]) == {0: sf.SFFT_OK, 1: sf.SFFT_ERR_NOT_CONVERGED}[of]
+        assert np.max(np.abs(val[r, :c, 0] + 1j * val[r, :c, 1] - ov), initial=0.0) < 1e-9
+        missed += k - c
+    assert 0 < missed < batch * k
