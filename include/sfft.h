@@ -327,10 +327,12 @@ sfft_status sfft_batch_execute(sfft_batch_plan bp, const uint32_t* h_plan_of, co
                                uint32_t* d_count, int32_t* d_flag);
 
 /*
- * Check of a bounded device wait: one thread waits for a word that nothing ever publishes.  Its wait
- * gives up after about a second, it sets an error flag and returns; the call synchronises `stream` and
- * returns SFFT_ERR_TIMEOUT when the flag was set (the expected outcome) or SFFT_OK if the wait did not
- * give up.  The device stays usable either way.  (No launch of this library waits on another CTA.)
+ * Check of the library's one wait on the device, that of the gather of sfft_execute_channels for its bulk
+ * copies (no launch waits on another CTA): one CTA runs that wait, with a shorter limit, on copies that never
+ * land.  It gives up twice after about half a second, sets the gather's error word and returns; the decode
+ * then reports it for 32 channel slots.  The call synchronises `stream` and returns SFFT_ERR_TIMEOUT when the
+ * wait gave up and every slot reads count 0 and SFFT_ERR_TIMEOUT (the expected outcome), SFFT_OK if the wait
+ * did not give up, SFFT_ERR_CUDA if a slot reads otherwise.  The device stays usable either way.
  * Errors: OOM, CUDA.
  */
 sfft_status sfft_persistent_wait_check(void* stream);

@@ -1163,25 +1163,43 @@ sfft_status sfft_batch_plan_create(const sfft_plan* plans, uint32_t nplans, uint
 }
 
 sfft_status sfft_persistent_wait_check(void* stream) {
-    unsigned char* d = nullptr;  // the word, the error flag
-    if (cudaMalloc((void**)&d, 64) != cudaSuccess) {
+    constexpr uint32_t kSlots = 32;
+    struct Report {
+        uint32_t error;
+        uint32_t count[kSlots];
+        int32_t flag[kSlots];
+    } h;
+    Report* d = nullptr;
+    if (cudaMalloc((void**)&d, sizeof(Report)) != cudaSuccess) {
         cudaGetLastError();
         return SFFT_ERR_OOM;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    int32_t* flag = reinterpret_cast<int32_t*>(d + 16);
-    int32_t err = 0;
-    cudaError_t e = cudaMemsetAsync(d, 0, 64, st);
-    if (e == cudaSuccess) e = launch_wait_check(reinterpret_cast<const uint32_t*>(d), flag, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&err, flag, sizeof(err), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    auto read = [&] {
+        const cudaError_t e = cudaMemcpyAsync(&h, d, sizeof(Report), cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+    };
+    // the slots hold what no decode writes
+    cudaError_t e = cudaMemsetAsync(d, 0x5A, sizeof(Report), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&d->error, 0, sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = launch_chan_wait_check(&d->error, st);
+    if (e == cudaSuccess) e = read();
+    const bool gave_up = e == cudaSuccess && h.error != 0;
+    if (gave_up) e = launch_chan_timeouts(&d->error, kSlots, d->count, d->flag, st);
+    if (gave_up && e == cudaSuccess) e = read();
     cudaFree(d);
     if (e != cudaSuccess) {
         set_last_error(std::string("wait check: ") + cudaGetErrorString(e));
         cudaGetLastError();
         return SFFT_ERR_CUDA;
     }
-    return err ? SFFT_ERR_TIMEOUT : SFFT_OK;
+    if (!gave_up) return SFFT_OK;
+    for (uint32_t s = 0; s < kSlots; ++s)
+        if (h.count[s] != 0 || h.flag[s] != SFFT_ERR_TIMEOUT) {
+            set_last_error("wait check: a slot does not report the wait that gave up");
+            return SFFT_ERR_CUDA;
+        }
+    return SFFT_ERR_TIMEOUT;
 }
 
 sfft_status sfft_batch_plan_destroy(sfft_batch_plan bp) {

@@ -1780,7 +1780,16 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_step(
 // per row (C contiguous complex values) into shared memory, then forms the rows' coefficients (one
 // row per lane) while the copies are in flight; once they have landed, thread ch folds channel ch in
 // row order.
-constexpr uint32_t kChanWaitLimit = 1u << 22;  // tries of a bounded wait (far beyond a second)
+constexpr uint32_t kChanWaitLimit = 1u << 22;  // tries of a bounded wait (3.8 us each: 16 s)
+// Every thread of a CTA: whether the copies that complete phase 0 of `bar` have landed, within `limit` tries.
+// If not (never expected), *error is set, and the copies get a second bounded wait, to end while their
+// shared memory is still this CTA's.
+__device__ __forceinline__ bool copies_landed(uint64_t* bar, uint32_t limit, uint32_t* error) {
+    if (mbar_wait(bar, 0, limit)) return true;
+    if (threadIdx.x == 0) atomicExch(error, 1u);
+    mbar_wait(bar, 0, limit);
+    return false;
+}
 template <int NR>
 __global__ void __launch_bounds__(kThreads) k_chan_gather(const __grid_constant__ ChanParams<NR> cp) {
     extern __shared__ __align__(16) unsigned char smem[];  // bulk copies need 16-byte alignment
@@ -1831,12 +1840,7 @@ __global__ void __launch_bounds__(kThreads) k_chan_gather(const __grid_constant_
         }
     }
     __syncthreads();  // the coefficients
-    if (!mbar_wait(&bar, 0, kChanWaitLimit)) {
-        // never expected: flag it, give the copies a second bounded wait, leave the partial sums alone
-        if (tid == 0) atomicExch(cp.error, 1u);
-        mbar_wait(&bar, 0, kChanWaitLimit);
-        return;
-    }
+    if (!copies_landed(&bar, kChanWaitLimit, cp.error)) return;  // (the partial sums stay as they are)
     for (uint32_t ch = tid; ch < C; ch += kThreads) {
         float2 acc[kMaxHash];
 #pragma unroll
@@ -1996,19 +2000,26 @@ cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, c
     return cudaGetLastError();
 }
 
-// A bounded wait for a word that nothing publishes: it gives up after about a second and says so.
-constexpr uint32_t kSpinLimit = 1u << 23;  // x ~128 ns
-__global__ void k_wait_check(const uint32_t* word, int32_t* error) {
-    for (uint32_t spin = 0; !acquire_is(word, 1u); ++spin) {
-        if (spin >= kSpinLimit) {
-            atomicExch(error, 1);
-            return;
-        }
-        __nanosleep(128);
-    }
+// The gather's wait where no copy ever lands: a barrier whose phase nothing completes.
+constexpr uint32_t kWaitCheckLimit = 1u << 17;  // half a second, twice
+__global__ void __launch_bounds__(kThreads) k_chan_wait_check(uint32_t limit, uint32_t* error) {
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x == 0) mbar_init(&bar, 1);
+    __syncthreads();
+    copies_landed(&bar, limit, error);
 }
-cudaError_t launch_wait_check(const uint32_t* word, int32_t* error, cudaStream_t st) {
-    k_wait_check<<<1, 1, 0, st>>>(word, error);
+cudaError_t launch_chan_wait_check(uint32_t* error, cudaStream_t st) {
+    k_chan_wait_check<<<1, kThreads, 0, st>>>(kWaitCheckLimit, error);
+    return cudaGetLastError();
+}
+// What the decodes of a channel batch report once the gather has set *error (which the caller has seen set:
+// there are no bins to decode).
+cudaError_t launch_chan_timeouts(const uint32_t* error, uint32_t slots, uint32_t* count, int32_t* flag, cudaStream_t st) {
+    StepParams<8> sp = {};
+    sp.R = 1;
+    sp.r[0].out_count = count;
+    sp.r[0].out_flag = flag;
+    k_chan_decode<8, kDecodeMasks><<<slots, kThreads, 0, st>>>(sp, 0, 0, error);
     return cudaGetLastError();
 }
 

@@ -422,9 +422,11 @@ cudaError_t launch_exact_step(const ExactArgs* rounds, uint32_t R, uint32_t batc
 cudaError_t launch_exact_channels(const ExactArgs* rounds, uint32_t R, uint32_t C, const void* x, uint64_t seed,
                                   uint32_t id, size_t smem, uint32_t* error, cudaStream_t st, cudaEvent_t before,
                                   cudaEvent_t after);
-// mixed batches, and the check of a bounded wait
+// mixed batches
 cudaError_t launch_exact_batch(const BatchArgs& a, uint32_t ctas, size_t smem, cudaStream_t st, bool fp64, int kind);
-cudaError_t launch_wait_check(const uint32_t* word, int32_t* error, cudaStream_t st);
+// the check of the channel gather's bounded wait: the wait, then what the slots report of it
+cudaError_t launch_chan_wait_check(uint32_t* error, cudaStream_t st);
+cudaError_t launch_chan_timeouts(const uint32_t* error, uint32_t slots, uint32_t* count, int32_t* flag, cudaStream_t st);
 cudaError_t launch_exact_decode(const DecodeArgs& a, cudaStream_t st);
 cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                           uint32_t count, uint32_t* out, cudaStream_t st);

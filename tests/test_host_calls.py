@@ -91,3 +91,19 @@ def test_a_general_plan_takes_the_memory_of_one_round_where_it_has_to(L, m, k, f
         assert gathers(h, 1) == rounds
         L.sfft_plan_destroy(h)
     L.fake_reset()
+
+
+def test_the_wait_check_reads_what_the_channel_slots_report(L):
+    """sfft_persistent_wait_check answers SFFT_ERR_TIMEOUT only when the channel gather's wait gave up and the
+    decode of every slot reported it: not when the wait ended, nor when the slots hold something else."""
+    gave_up = fr.LAUNCH_FN(lambda kernel, args: ctypes.memset(ctypes.cast(args[1], ctypes.POINTER(ctypes.c_void_p))[0], 1, 4)
+                           if b"wait_check" in kernel else None)
+    L.fake_reset()
+    assert L.sfft_persistent_wait_check(STREAM) == 0
+    assert not any("k_chan_decode" in c[1] for c in fr.log(L))
+    L.fake_reset()
+    L.fake_on_launch(gave_up)
+    assert L.sfft_persistent_wait_check(STREAM) == sfft.SFFT_ERR_CUDA
+    assert b"slot" in L.sfft_last_error()
+    assert any("k_chan_decode" in c[1] for c in fr.log(L))
+    L.fake_reset()
