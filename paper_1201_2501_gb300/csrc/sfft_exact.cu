@@ -486,9 +486,14 @@ __device__ __forceinline__ int decode_bin_guarded(const DecodeCtx& d, uint32_t j
     for (int l = 0; l < kMaxHash - 1; ++l)
         if ((uint32_t)l < L) {
             ml[l] = hypotf(v[l + 1].x, v[l + 1].y);
-            if (!(ml[l] > 1e-30f && ml[l] * mag0 > 1e-30f)) return kUndecided;  // the phase of a product FP32 holds
             th[l] = phase01_f(mul_conj_f(v[0], v[l + 1]));
         }
+    // a hashing far below u_0 passes a wide isolation tolerance only; FP32 may not hold its product's phase
+    if (d.iso_tol_f > 0.5f) {
+#pragma unroll
+        for (int l = 0; l < kMaxHash - 1; ++l)
+            if ((uint32_t)l < L && !(ml[l] > 1e-30f && ml[l] * mag0 > 1e-30f)) return kUndecided;
+    }
     // location ladder, coarsest shift first: each rounding has to stay clear of a half
     uint32_t c = 0, logM = 0;
 #pragma unroll
