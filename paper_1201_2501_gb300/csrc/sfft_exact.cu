@@ -69,13 +69,12 @@ __host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t
     L.ent_val = fin_take(&off, (size_t)zcap * 16);
     L.ent_gain = fin_take(&off, (size_t)zcap * 8);
     L.ent_sub = fin_take(&off, (size_t)zcap * H * 16);
-    L.ent_sub_f = fin_take(&off, (size_t)zcap * H * 8);
+    L.ent_sub_f = fin_take(&off, csize == 8 ? (size_t)zcap * H * 8 : 0);  // FP32 data path
     L.mask = fin_take(&off, masks ? (size_t)B * ((zcap + 31) / 32) * 4 : 0);
     L.bin_cnt = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
     L.bin_start = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
     L.bin_list = fin_take(&off, masks ? 0 : (size_t)zcap * 4);
     L.cand_idx = fin_take(&off, (size_t)B * 4);
-    if (!masks) fin_take(&off, (size_t)B * 12);
     L.cand_val = fin_take(&off, (size_t)B * 16);
     L.srt_idx = fin_take(&off, (size_t)B * 4);
     L.srt_val = fin_take(&off, (size_t)B * 16);
@@ -92,6 +91,15 @@ size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
 }
 size_t exact_decode_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
     return fin_layout(B, H, zcap, fp64 ? 16 : 8, true).total;
+}
+// What the bounds on a plan's arrays count beyond them: 12 bytes a bin for a decode by lists, 8 an entry and
+// hashing for FP64, arrays of earlier forms.  The bounds (kFinSmemMax, the refusal above 200 KB) were measured
+// with these, and a plan keeps its decode, or its refusal.
+size_t exact_finish_bound(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
+    return exact_finish_smem(B, H, zcap, fp64) + (size_t)B * 12 + (fp64 ? (size_t)zcap * H * 8 : 0);
+}
+size_t exact_decode_bound(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
+    return exact_decode_smem(B, H, zcap, fp64) + (fp64 ? (size_t)zcap * H * 8 : 0);
 }
 size_t exact_gather_smem(uint32_t stage, bool fp64) { return (size_t)stage * (fp64 ? 16 : 8); }
 constexpr uint32_t owner_batch(bool fp64) {  // taps of a residue per batch
@@ -215,21 +223,9 @@ __device__ void fill_ctx_round(DecodeCtx& d, const ExactArgs& a, uint32_t sigma,
     d.ref_tol_f = a.ref_tol_f;
 }
 
-// Decode of one bin (NoiselessSparseFFTInner's loop body).  u[0..H) are the bin's hashings after the
-// subtraction of zhat, in the precision R of the data path.  Returns 0 (nothing), 1 (a decode of J
-// kept) or 2 (a re-estimate of a known entry), with the index in *oi and the window gain that divides
-// u_0 in *gain (the caller forms the FP64 value; for a decode of the FP32 path *ginv is 1 / gain from
-// the table beside W, else 0, and the caller divides).  *above is set when |u_0| > thr.  The zhat entries
-// hashed to bin j are list[0..nbin) (entry ids), with indices ent_idx[] and window gains ent_gain[].
-//
-// The FP64 data path decides in FP64.  The FP32 path takes every decision (magnitudes, phases, the
-// location ladder, isolation and re-estimation tests) in FP32: its bins carry ~1e-6 of rounding, the
-// ladder keeps a tolerance of at least tau_dec per level and GB300 issues FP64 at 1/64 of FP32, so FP64
-// arithmetic there would cost most of the finisher's time and change no decision outside a
-// measure-zero band at the thresholds.
-// The zhat entries hashed to a bin, in ascending order of their ids e: f(e) for each.  kDirect: ids count
-// from the bin's first place, and a decode is returned before its window gain is read, with the signed
-// offset o in *oi, or with the id of the entry a re-estimate corrects.
+// The zhat entries hashed to a bin, in ascending order of their ids e: each(f) calls f(e) for every one.
+// kDirect: ids count from the bin's first place, and a decode is returned before its window gain is read, with
+// the signed offset o in *oi, or with the id of the entry a re-estimate corrects.
 struct ListEntries {
     static constexpr bool kDirect = false;
     const uint32_t* list;
@@ -268,6 +264,18 @@ __device__ __forceinline__ uint32_t index_at(const DecodeCtx& d, uint32_t j, int
     const uint32_t p = (j * d.Np + (uint32_t)o) & d.nmask;
     return (d.sigma_inv * ((p + d.sb) & d.nmask)) & d.nmask;
 }
+// Decode of one bin (NoiselessSparseFFTInner's loop body).  u[0..H) are the bin's hashings after the
+// subtraction of zhat, in the precision of the data path, `ents` its entries, with indices ent_idx[] and window
+// gains ent_gain[].  Returns 0 (nothing), 1 (a decode of J kept) or 2 (a re-estimate of a known entry), with
+// the index in *oi and the window gain that divides u_0 in *gout (the caller forms the FP64 value; for a decode
+// of the FP32 path *ginv is 1 / gain from the table beside W, else 0, and the caller divides).  *above is set
+// when |u_0| > thr.
+//
+// FP64 bins are decided as FP64 decides them: by decode_bin_guarded where FP32 must agree, else here.  FP32
+// bins take every decision (magnitudes, phases, the location ladder, isolation and re-estimation tests) in
+// FP32 (decode_bin_fp32): they carry ~1e-6 of rounding, the ladder keeps a tolerance of at least tau_dec per
+// level and GB300 issues FP64 at 1/64 of FP32, so FP64 arithmetic there would cost most of the finisher's time
+// and change no decision outside a measure-zero band at the thresholds.
 template <typename Ents>
 __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const Ents ents, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
                                double* ginv, bool* above) {
@@ -1002,9 +1010,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
             const uint32_t i = ent_idx[e];
             const double2 w = term_root<R>(a, ((a.a_base + a.a[h]) * sigma * i) & a.nmask);
             const double2 gz = make_double2(ent_gain[e] * ent_val[e].x, ent_gain[e] * ent_val[e].y);
-            const double2 t = make_double2(gz.x * w.x - gz.y * w.y, gz.x * w.y + gz.y * w.x);
-            ent_sub[q] = t;
-            ent_sub_f[q] = make_float2((float)t.x, (float)t.y);
+            ent_sub[q] = make_double2(gz.x * w.x - gz.y * w.y, gz.x * w.y + gz.y * w.x);
         }
     }
     const uint32_t sub_stride = f32 ? 1u : H;  // where subtracted_u0 finds hashing 0's FP64 terms

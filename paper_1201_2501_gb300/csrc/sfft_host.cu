@@ -327,10 +327,11 @@ sfft_status build_exact_schedule(sfft_plan_s* pl) {
                                                               (fp64 ? 16 : 8);
         const size_t fs = exact_finish_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
         // finish_round's arrays beyond kFinSmemMax live in device memory (the single-hashing call)
-        r.fin_global = fs > kFinSmemMax;
-        if ((r.fin_global ? gs : (gs > fs ? gs : fs)) > 200 * 1024) return SFFT_ERR_K_RANGE;
+        const size_t fbound = exact_finish_bound(r.B, 1 + r.nshift, p.z_cap, fp64);
+        r.fin_global = fbound > kFinSmemMax;
+        if ((r.fin_global ? gs : (gs > fbound ? gs : fbound)) > 200 * 1024) return SFFT_ERR_K_RANGE;
         const size_t ms = p.z_cap > kCarry ? 0 : exact_decode_smem(r.B, 1 + r.nshift, p.z_cap, fp64);
-        if (r.fin_global || ms > kFinSmemMax)
+        if (r.fin_global || (ms && exact_decode_bound(r.B, 1 + r.nshift, p.z_cap, fp64) > kFinSmemMax))
             kind = kDecodeLarge;
         else if (p.z_cap > kCarry && kind != kDecodeLarge)
             kind = kDecodeLists;

@@ -443,6 +443,8 @@ cudaError_t launch_locate_votes(const VoteArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_from_bins(const EstArgs& a, cudaStream_t st);
 size_t exact_finish_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 size_t exact_decode_smem(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
+size_t exact_finish_bound(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
+size_t exact_decode_bound(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 size_t exact_gather_smem(uint32_t stage, bool fp64);
 size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64);
 uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64);

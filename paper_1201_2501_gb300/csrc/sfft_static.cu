@@ -4,6 +4,7 @@
 // sums and the arrival counter live in a fixed array compiled into this library.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -103,7 +104,7 @@ extern "C" sfft_status sfft_hash_to_bins_static(uint64_t n, uint32_t B, int64_t 
     const size_t gs = exact_gather_smem(kChunkTaps, false) + (size_t)(B > (uint32_t)kThreads ? B : kThreads) * 8;
     const size_t fs = exact_finish_smem(B, 1, args.zcap, false);
     const size_t smem = gs > fs ? gs : fs;
-    if (smem > 200 * 1024) return SFFT_ERR_INVALID_ARG;
+    if (std::max(gs, exact_finish_bound(B, 1, args.zcap, false)) > 200 * 1024) return SFFT_ERR_INVALID_ARG;
     cudaError_t e = set_round_smem_limit(smem, false);
     if (e == cudaSuccess) e = cudaMemsetAsync(args.counter, 0, sizeof(uint32_t), (cudaStream_t)stream);
     if (e == cudaSuccess) e = launch_exact_round(args, 1, smem, (cudaStream_t)stream, false);
