@@ -119,10 +119,7 @@ __device__ __forceinline__ double2 root_pow_fine(uint32_t e, const double2* tw, 
 }
 
 // phase(z) / 2 pi in [0, 1)
-template <typename R>
-__device__ __forceinline__ double phase01(double2 z);
-template <>
-__device__ __forceinline__ double phase01<double>(double2 z) {
+__device__ __forceinline__ double phase01(double2 z) {
     double p = __ddiv_rn(atan2(z.y, z.x), 6.283185307179586476925286766559);
     if (p < 0.0) p += 1.0;
     if (p >= 1.0) p -= 1.0;
@@ -135,24 +132,7 @@ __device__ __forceinline__ double2 mul_conj_rn(double2 a, double2 b) {
     return make_double2(__dadd_rn(__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)),
                         __dsub_rn(__dmul_rn(a.y, b.x), __dmul_rn(a.x, b.y)));
 }
-template <>
-__device__ __forceinline__ double phase01<float>(double2 z) {
-    double p = (double)atan2f((float)z.y, (float)z.x) * 0.15915494309189533576888;
-    if (p < 0.0) p += 1.0;
-    if (p >= 1.0) p -= 1.0;
-    return p;
-}
-template <typename R>
-__device__ __forceinline__ double cmag(double2 z);
-template <>
-__device__ __forceinline__ double cmag<double>(double2 z) {
-    return hypot(z.x, z.y);
-}
-template <>
-__device__ __forceinline__ double cmag<float>(double2 z) {
-    return (double)hypotf((float)z.x, (float)z.y);
-}
-
+__device__ __forceinline__ double cmag(double2 z) { return hypot(z.x, z.y); }
 __device__ __forceinline__ uint32_t ilog2_u32(uint32_t v) { return 31u - __clz(v); }
 
 // ------------------------------------------------------------------------------------------------
@@ -439,6 +419,60 @@ __device__ inline void fft_rows_by_passes(float2* a, uint32_t H, uint32_t logB) 
             st += 1;
         }
     }
+}
+
+// the next array of a shared-memory layout: its offset (16-byte aligned)
+__host__ __device__ inline size_t smem_take(size_t* off, size_t bytes) {
+    const size_t o = (*off + 15) & ~size_t(15);
+    *off = o + bytes;
+    return o;
+}
+// warps that count (each with its own counters): 8 up to B = 1024
+__host__ __device__ inline uint32_t split_segments(uint32_t B) { return B <= 1024 ? 8u : 8192u / B; }
+// Stable counting split, in a CTA: per-warp counters, no sort.  place[e] <- the rank of entry e in (bin, index) order, from place[e] = its bin; start[j] <- the first
+// rank of bin j (start[B] = nz).  cnt: split_segments(B) x B counters.
+__device__ __forceinline__ void split_by_bin(uint32_t* place, uint32_t nz, uint32_t B, uint16_t* cnt, uint32_t* start, uint32_t* scan) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nseg = split_segments(B);
+    for (uint32_t i = tid; i < nseg * B / 2; i += kThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0;
+    __syncthreads();
+    const uint32_t per = ((nz + nseg - 1) / nseg + 31u) & ~31u, beg = warp * per, end = min(nz, beg + per);
+    uint16_t* mine = cnt + (size_t)warp * B;
+    if (warp < nseg)
+        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
+            const bool in = e0 + lane < end;
+            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
+            const unsigned same = __match_any_sync(0xffffffffu, b);
+            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(mine[b] + __popc((int)same));
+            __syncwarp();
+        }
+    __syncthreads();
+    for (uint32_t j = tid; j < B; j += kThreads) {
+        uint32_t run = 0;
+        for (uint32_t w = 0; w < nseg; ++w) {
+            const uint32_t c = cnt[w * B + j];
+            cnt[w * B + j] = (uint16_t)run;
+            run += c;
+        }
+        start[j] = run;
+    }
+    __syncthreads();
+    block_exclusive_scan(start, B, scan);  // ends with a barrier
+    if (tid == 0) start[B] = nz;
+    if (warp < nseg)
+        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
+            const bool in = e0 + lane < end;
+            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
+            const unsigned same = __match_any_sync(0xffffffffu, b);
+            uint32_t base = 0;
+            if (in) {
+                base = mine[b];
+                place[e0 + lane] = start[b] + base + (uint32_t)__popc((int)(same & ((1u << lane) - 1u)));
+            }
+            __syncwarp();
+            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(base + __popc((int)same));
+            __syncwarp();
+        }
+    __syncthreads();
 }
 
 // Bucket the nz entries of zhat by bin: bin_start[B+1] (exclusive prefix), bin_list (entry ids of

@@ -54,34 +54,29 @@ struct FinLayout {
     size_t U, ent_idx, ent_bin, ent_val, ent_gain, ent_sub, ent_sub_f, mask, bin_cnt, bin_start, bin_list, cand_idx, cand_val, srt_idx, srt_val, out_idx, out_val, keep, scan;
     size_t total;
 };
-__host__ __device__ inline size_t fin_take(size_t* off, size_t bytes) {
-    const size_t o = (*off + 15) & ~size_t(15);
-    *off = o + bytes;
-    return o;
-}
 // masks: the entries of each bin as bits (the transform's decode), instead of as lists
 __host__ __device__ inline FinLayout fin_layout(uint32_t B, uint32_t H, uint32_t zcap, uint32_t csize, bool masks = false) {
     FinLayout L;
     size_t off = 0;
-    L.U = fin_take(&off, (size_t)H * B * csize);
-    L.ent_idx = fin_take(&off, (size_t)zcap * 4);
-    L.ent_bin = fin_take(&off, (size_t)zcap * 4);
-    L.ent_val = fin_take(&off, (size_t)zcap * 16);
-    L.ent_gain = fin_take(&off, (size_t)zcap * 8);
-    L.ent_sub = fin_take(&off, (size_t)zcap * H * 16);
-    L.ent_sub_f = fin_take(&off, csize == 8 ? (size_t)zcap * H * 8 : 0);  // FP32 data path
-    L.mask = fin_take(&off, masks ? (size_t)B * ((zcap + 31) / 32) * 4 : 0);
-    L.bin_cnt = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
-    L.bin_start = fin_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
-    L.bin_list = fin_take(&off, masks ? 0 : (size_t)zcap * 4);
-    L.cand_idx = fin_take(&off, (size_t)B * 4);
-    L.cand_val = fin_take(&off, (size_t)B * 16);
-    L.srt_idx = fin_take(&off, (size_t)B * 4);
-    L.srt_val = fin_take(&off, (size_t)B * 16);
-    L.out_idx = fin_take(&off, (size_t)(zcap + B) * 4);
-    L.out_val = fin_take(&off, (size_t)(zcap + B) * 16);
-    L.keep = fin_take(&off, (size_t)(zcap + B) * 4);
-    L.scan = fin_take(&off, (size_t)(kThreads + 8) * 4);
+    L.U = smem_take(&off, (size_t)H * B * csize);
+    L.ent_idx = smem_take(&off, (size_t)zcap * 4);
+    L.ent_bin = smem_take(&off, (size_t)zcap * 4);
+    L.ent_val = smem_take(&off, (size_t)zcap * 16);
+    L.ent_gain = smem_take(&off, (size_t)zcap * 8);
+    L.ent_sub = smem_take(&off, (size_t)zcap * H * 16);
+    L.ent_sub_f = smem_take(&off, csize == 8 ? (size_t)zcap * H * 8 : 0);  // FP32 data path
+    L.mask = smem_take(&off, masks ? (size_t)B * ((zcap + 31) / 32) * 4 : 0);
+    L.bin_cnt = smem_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
+    L.bin_start = smem_take(&off, masks ? 0 : (size_t)(B + 1) * 4);
+    L.bin_list = smem_take(&off, masks ? 0 : (size_t)zcap * 4);
+    L.cand_idx = smem_take(&off, (size_t)B * 4);
+    L.cand_val = smem_take(&off, (size_t)B * 16);
+    L.srt_idx = smem_take(&off, (size_t)B * 4);
+    L.srt_val = smem_take(&off, (size_t)B * 16);
+    L.out_idx = smem_take(&off, (size_t)(zcap + B) * 4);
+    L.out_val = smem_take(&off, (size_t)(zcap + B) * 16);
+    L.keep = smem_take(&off, (size_t)(zcap + B) * 4);
+    L.scan = smem_take(&off, (size_t)(kThreads + 8) * 4);
     L.total = off;
     return L;
 }
@@ -279,7 +274,7 @@ __device__ __forceinline__ uint32_t index_at(const DecodeCtx& d, uint32_t j, int
 template <typename Ents>
 __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, const double2* u, const Ents ents, const uint32_t* ent_idx, const double* ent_gain, uint32_t* oi, double* gout,
                                double* ginv, bool* above) {
-    const double mag0 = cmag<double>(u[0]);
+    const double mag0 = cmag(u[0]);
     *ginv = 0.0;  // the FP64 path divides
     const uint32_t L = d.H - 1;
     *above = false;
@@ -288,8 +283,8 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
         if (!ents.any() || !(mag0 > d.ref_lo * d.thr && mag0 <= d.ref_hi * d.thr)) return 0;
         double th[kMaxHash];
         for (uint32_t l = 0; l < L; ++l) {
-            if (fabs(cmag<double>(u[l + 1]) - mag0) > 0.25 * mag0) return 0;
-            th[l] = phase01<double>(mul_conj(u[0], u[l + 1]));
+            if (fabs(cmag(u[l + 1]) - mag0) > 0.25 * mag0) return 0;
+            th[l] = phase01(mul_conj(u[0], u[l + 1]));
         }
         uint32_t matches = 0, who = 0;
         double gw = 1.0;
@@ -319,12 +314,12 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
     // location ladder, coarsest shift first: q = sigma i mod n/B.  Every modulus is a power of two,
     // so mod and division are masks and exact scalings.
     uint32_t logM = d.logNp - d.logR[L - 1];
-    const double th = phase01<double>(mul_conj(u[0], u[L]));
+    const double th = phase01(mul_conj(u[0], u[L]));
     uint64_t c = (uint64_t)(int64_t)floor(th * ldexp(1.0, (int)logM) + 0.5) & ((uint64_t(1) << logM) - 1);
     for (int l = (int)L - 2; l >= 0; --l) {
         const uint32_t logMp = d.logNp - d.logR[l];
         const uint32_t logRatio = logMp - logM;
-        const double thl = phase01<double>(mul_conj(u[0], u[l + 1]));
+        const double thl = phase01(mul_conj(u[0], u[l + 1]));
         const double y = thl * ldexp(1.0, (int)logRatio) - ldexp((double)c, -(int)logM);
         const int64_t h = (int64_t)floor(y + 0.5) & (int64_t)((uint64_t(1) << logRatio) - 1);
         c += (uint64_t(1) << logM) * (uint64_t)h;
@@ -335,7 +330,7 @@ __device__ __noinline__ int decode_bin_fp64(const DecodeCtx& d, uint32_t j, cons
     const int32_t o = (int32_t)dd - (int32_t)(d.Np >> 1);
     const uint32_t i = index_at(d, j, o);
     for (uint32_t l = 0; l < L; ++l)
-        if (fabs(cmag<double>(u[l + 1]) - mag0) > d.iso_tol * mag0) return 0;
+        if (fabs(cmag(u[l + 1]) - mag0) > d.iso_tol * mag0) return 0;
     if (Ents::kDirect) {
         *oi = (uint32_t)o;
         return 1;
@@ -765,7 +760,7 @@ __device__ __forceinline__ bool dropped(double2 v, const ExactArgs& a) {
         const int c = cmp_guarded(f, a.drop_f);
         if (c != 0) return c < 0;
     }
-    return cmag<double>(v) < a.prune * a.thr;
+    return cmag(v) < a.prune * a.thr;
 }
 
 // Step 2 across chunks: U[h][brev(r)] = sum over chunks c, in order, of part[c][h][r].  Each thread
@@ -1218,84 +1213,37 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
 struct LargeLayout {
     size_t e_idx, pre, key, cval, start, slot, s_idx, s_gain, s_t0, s_tf, cnt, out_idx, out_val, keep, scan, total;
 };
-__host__ __device__ inline uint32_t split_segments(uint32_t B) { return B <= 1024 ? 8u : 8192u / B; }
 // nz entries, up to B candidates, tot merged entries; the merge's arrays take the place of the entries'
 __host__ __device__ inline LargeLayout large_layout(uint32_t B, uint32_t H, uint32_t nz, uint32_t tot, bool fp64,
                                                     bool val_on_chip) {
     LargeLayout L;
     size_t off = 0;
     const uint32_t P = B < 1024 ? 1024 : B;  // the sort's keys, padded
-    L.scan = fin_take(&off, (size_t)(kThreads + 8) * 4);
-    L.e_idx = fin_take(&off, (size_t)nz * 4);
+    L.scan = smem_take(&off, (size_t)(kThreads + 8) * 4);
+    L.e_idx = smem_take(&off, (size_t)nz * 4);
     // the decoded bins share their place with the split's counters
     const size_t cnt = nz ? (size_t)split_segments(B) * B * 2 : 0, pre = (size_t)B * 8;
-    L.pre = L.cnt = fin_take(&off, pre > cnt ? pre : cnt);
-    L.key = fin_take(&off, (size_t)P * 8);
-    L.cval = fin_take(&off, val_on_chip ? (size_t)B * 16 : 0);
+    L.pre = L.cnt = smem_take(&off, pre > cnt ? pre : cnt);
+    L.key = smem_take(&off, (size_t)P * 8);
+    L.cval = smem_take(&off, val_on_chip ? (size_t)B * 16 : 0);
     const size_t shared = off;
-    L.start = fin_take(&off, (size_t)(B + 1) * 4);
-    L.slot = fin_take(&off, (size_t)nz * 4);
-    L.s_idx = fin_take(&off, (size_t)nz * 4);
-    L.s_gain = fin_take(&off, (size_t)nz * 8);
-    L.s_t0 = fin_take(&off, (size_t)nz * 16);
-    L.s_tf = fin_take(&off, (size_t)nz * H * (fp64 ? 16 : 8));
+    L.start = smem_take(&off, (size_t)(B + 1) * 4);
+    L.slot = smem_take(&off, (size_t)nz * 4);
+    L.s_idx = smem_take(&off, (size_t)nz * 4);
+    L.s_gain = smem_take(&off, (size_t)nz * 8);
+    L.s_t0 = smem_take(&off, (size_t)nz * 16);
+    L.s_tf = smem_take(&off, (size_t)nz * H * (fp64 ? 16 : 8));
     const size_t end = off;
     off = shared;
-    L.out_idx = fin_take(&off, (size_t)tot * 4);
-    L.out_val = fin_take(&off, (size_t)tot * 16);
-    L.keep = fin_take(&off, (size_t)(tot + 1) * 4);
+    L.out_idx = smem_take(&off, (size_t)tot * 4);
+    L.out_val = smem_take(&off, (size_t)tot * 16);
+    L.keep = smem_take(&off, (size_t)(tot + 1) * 4);
     L.total = off > end ? off : end;
     return L;
 }
 // device-memory slice of a request: the candidates' values, then everything at its largest
 size_t exact_large_bytes(uint32_t B, uint32_t H, uint32_t zcap, bool fp64) {
     return (size_t)B * 16 + large_layout(B, H, zcap, zcap + B, fp64, false).total;
-}
-
-// place[e] <- the rank of entry e in (bin, index) order, from place[e] = its bin; start[j] <- the first
-// rank of bin j (start[B] = nz).  cnt: split_segments(B) x B counters.
-__device__ void split_by_bin(uint32_t* place, uint32_t nz, uint32_t B, uint16_t* cnt, uint32_t* start, uint32_t* scan) {
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nseg = split_segments(B);
-    for (uint32_t i = tid; i < nseg * B / 2; i += kThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0;
-    __syncthreads();
-    const uint32_t per = ((nz + nseg - 1) / nseg + 31u) & ~31u, beg = warp * per, end = min(nz, beg + per);
-    uint16_t* mine = cnt + (size_t)warp * B;
-    if (warp < nseg)
-        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
-            const bool in = e0 + lane < end;
-            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
-            const unsigned same = __match_any_sync(0xffffffffu, b);
-            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(mine[b] + __popc((int)same));
-            __syncwarp();
-        }
-    __syncthreads();
-    for (uint32_t j = tid; j < B; j += kThreads) {
-        uint32_t run = 0;
-        for (uint32_t w = 0; w < nseg; ++w) {
-            const uint32_t c = cnt[w * B + j];
-            cnt[w * B + j] = (uint16_t)run;
-            run += c;
-        }
-        start[j] = run;
-    }
-    __syncthreads();
-    block_exclusive_scan(start, B, scan);  // ends with a barrier
-    if (tid == 0) start[B] = nz;
-    if (warp < nseg)
-        for (uint32_t e0 = beg; e0 < end; e0 += 32) {
-            const bool in = e0 + lane < end;
-            const uint32_t b = in ? place[e0 + lane] : kNoIndex;
-            const unsigned same = __match_any_sync(0xffffffffu, b);
-            uint32_t base = 0;
-            if (in) {
-                base = mine[b];
-                place[e0 + lane] = start[b] + base + (uint32_t)__popc((int)(same & ((1u << lane) - 1u)));
-            }
-            __syncwarp();
-            if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(base + __popc((int)same));
-            __syncwarp();
-        }
-    __syncthreads();
 }
 
 // whether decode_bin goes beyond its first test on a bin whose subtracted u_0 is u
@@ -1310,7 +1258,7 @@ __device__ __forceinline__ bool worth_decoding(const DecodeCtx& d, double2 u, bo
         if (cmp_guarded(f, d.thr_f) < 0 && (!entries || cmp_guarded(f, d.ref_hi_f) > 0 || cmp_guarded(f, d.ref_lo_f) < 0))
             return false;
     }
-    const double m = cmag<double>(u);
+    const double m = cmag(u);
     return m > d.thr || (entries && m > d.ref_lo * d.thr && m <= d.ref_hi * d.thr);
 }
 
@@ -1710,13 +1658,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_round
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t s = a.req_base + blockIdx.y, c = blockIdx.x;
     const ReqView rq = req_view(a.reqs, a.x, a.n * sizeof(typename Cx<R>::T), a.seed, s, a.nmask);
-    uint32_t sigma, b;
-    if (a.bins_only) {
-        sigma = a.e_sigma;
-        b = a.e_b;
-    } else {
-        exact_hash(rq.seed, rq.id, a.round, a.nmask, &sigma, &b);
-    }
+    const uint32_t sigma = a.e_sigma, b = a.e_b;
     gather_fold<R>(a, rq.x, rq.xmask, s, c, sigma, b, smem);
     // arrival: the last CTA of request s finishes the round (nobody waits)
     if (arrive(a.counter + s, a.chunks) == 0) return;

@@ -319,27 +319,18 @@ constexpr uint32_t kFinPer = kFinSlab / kThreads;
 struct GenFinLayout {
     size_t U, term, slot, cnt, start, ub, scan, total;
 };
-__host__ __device__ inline size_t gtake(size_t* off, size_t bytes) {
-    const size_t o = (*off + 15) & ~size_t(15);
-    *off = o + bytes;
-    return o;
-}
-// warps that count a slab (each its own counters): 8 up to B = 1024
-__host__ __device__ inline uint32_t fin_segments(uint32_t B) {
-    return B <= 1024 ? 8u : 8192u / B;
-}
 // nzmax: the most entries zhat can have when the round starts
 __host__ __device__ inline GenFinLayout gen_fin_layout(uint32_t B, uint32_t nzmax) {
     GenFinLayout L;
     const uint32_t ns = nzmax < kFinSlab ? nzmax : kFinSlab;
     size_t off = 0;
-    L.U = gtake(&off, (size_t)2 * B * 8);
-    L.term = gtake(&off, (size_t)ns * 2 * 16);
-    L.slot = gtake(&off, (size_t)ns * 4);
-    L.cnt = gtake(&off, ns ? (size_t)fin_segments(B) * B * 2 : 0);
-    L.start = gtake(&off, ns ? (size_t)(B + 1) * 4 : 0);
-    L.ub = gtake(&off, ns && B < (uint32_t)kThreads ? (size_t)4 * B * 8 : 0);
-    L.scan = gtake(&off, (size_t)(kThreads + 8) * 4);
+    L.U = smem_take(&off, (size_t)2 * B * 8);
+    L.term = smem_take(&off, (size_t)ns * 2 * 16);
+    L.slot = smem_take(&off, (size_t)ns * 4);
+    L.cnt = smem_take(&off, ns ? (size_t)split_segments(B) * B * 2 : 0);
+    L.start = smem_take(&off, ns ? (size_t)(B + 1) * 4 : 0);
+    L.ub = smem_take(&off, ns && B < (uint32_t)kThreads ? (size_t)4 * B * 8 : 0);
+    L.scan = smem_take(&off, (size_t)(kThreads + 8) * 4);
     L.total = off;
     return L;
 }
@@ -421,7 +412,7 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
         }
         return;
     }
-    const uint32_t nseg = fin_segments(B), slab = min(a.nzmax, kFinSlab);
+    const uint32_t slab = min(a.nzmax, kFinSlab);
     for (uint32_t z0 = 0; z0 < nz; z0 += slab) {
         const uint32_t m = min(slab, nz - z0);
         const bool first = z0 == 0, last = z0 + m == nz;
@@ -442,48 +433,7 @@ __global__ void __launch_bounds__(kThreads) k_gen_finish(const GenArgs a) {
                 gz[q] = make_double2(gain * z.x, gain * z.y);
             }
         }
-        for (uint32_t i = tid; i < nseg * B / 2; i += kThreads) reinterpret_cast<uint32_t*>(cnt)[i] = 0;
-        __syncthreads();
-        // places by (bin, entry): warp w < nseg counts its share of the slab per bin, the counts are
-        // summed over bins and warps, and the warp's entries take their places in order
-        const uint32_t per = ((m + nseg - 1) / nseg + 31u) & ~31u, e_beg = warp * per, e_end = min(m, e_beg + per);
-        uint16_t* mine = cnt + (size_t)warp * B;
-        if (warp < nseg)
-            for (uint32_t e0 = e_beg; e0 < e_end; e0 += 32) {
-                const bool in = e0 + lane < e_end;
-                const uint32_t b = in ? slot[e0 + lane] : kNoIndex;
-                const unsigned same = __match_any_sync(0xffffffffu, b);
-                if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(mine[b] + __popc((int)same));
-                __syncwarp();
-            }
-        __syncthreads();
-        for (uint32_t j = tid; j < B; j += kThreads) {
-            uint32_t run = 0;
-            for (uint32_t w = 0; w < nseg; ++w) {
-                const uint32_t c = cnt[w * B + j];
-                cnt[w * B + j] = (uint16_t)run;
-                run += c;
-            }
-            start[j] = run;
-        }
-        __syncthreads();
-        block_exclusive_scan(start, B, scan);  // ends with a barrier
-        if (tid == 0) start[B] = m;
-        if (warp < nseg)
-            for (uint32_t e0 = e_beg; e0 < e_end; e0 += 32) {
-                const bool in = e0 + lane < e_end;
-                const uint32_t b = in ? slot[e0 + lane] : kNoIndex;
-                const unsigned same = __match_any_sync(0xffffffffu, b);
-                uint32_t base = 0;
-                if (in) {
-                    base = mine[b];
-                    slot[e0 + lane] = start[b] + base + (uint32_t)__popc((int)(same & ((1u << lane) - 1u)));
-                }
-                __syncwarp();
-                if (in && lane == (uint32_t)__ffs((int)same) - 1u) mine[b] = (uint16_t)(base + __popc((int)same));
-                __syncwarp();
-            }
-        __syncthreads();
+        split_by_bin(slot, m, B, cnt, start, scan);  // (a barrier before it reads the slots)
 #pragma unroll
         for (uint32_t q = 0; q < kFinPer; ++q) {
             const uint32_t e = tid + q * kThreads;
@@ -768,11 +718,11 @@ struct LocLayout {
 __host__ __device__ inline LocLayout loc_layout(uint32_t npairs, uint32_t nb, uint32_t R_est) {
     LocLayout L;
     size_t off = 0;
-    L.beta = gtake(&off, (size_t)npairs * 8);
-    L.vx = gtake(&off, (size_t)nb * R_est * 8);
-    L.vy = gtake(&off, (size_t)nb * R_est * 8);
-    L.c = gtake(&off, (size_t)npairs * nb * 4);
-    L.ok = gtake(&off, (size_t)nb * R_est * 4);
+    L.beta = smem_take(&off, (size_t)npairs * 8);
+    L.vx = smem_take(&off, (size_t)nb * R_est * 8);
+    L.vy = smem_take(&off, (size_t)nb * R_est * 8);
+    L.c = smem_take(&off, (size_t)npairs * nb * 4);
+    L.ok = smem_take(&off, (size_t)nb * R_est * 4);
     L.total = off;
     return L;
 }
@@ -846,7 +796,7 @@ __global__ void __launch_bounds__(kThreads) k_gen_locate(const GenArgs a) {
                 bool hit = ad < hw;
                 if (ad + kPhaseGuard - hw <= 2u * kPhaseGuard) {
                     const double2* pb = rbins + (size_t)2 * (D * a.R_loc + r) * B;
-                    hit = vote_hit_exact(phase01<double>(mul_conj_rn(pb[j], pb[B + j])), e >> sh, M, a.s);
+                    hit = vote_hit_exact(phase01(mul_conj_rn(pb[j], pb[B + j])), e >> sh, M, a.s);
                 }
                 v += hit ? 1u : 0u;
             }
@@ -947,10 +897,10 @@ __host__ __device__ inline SelLayout sel_layout(uint32_t B, uint32_t kprime, uin
     const uint32_t nJ = kprime < B ? kprime : B;
     L.P = 2;
     while (L.P < nJ) L.P <<= 1;
-    L.table = gtake(&off, (size_t)L.H * 4);
-    L.js = gtake(&off, (size_t)L.P * 8);
-    L.zi = gtake(&off, (size_t)zcap * 4);
-    L.dup = gtake(&off, (size_t)L.P * 4);
+    L.table = smem_take(&off, (size_t)L.H * 4);
+    L.js = smem_take(&off, (size_t)L.P * 8);
+    L.zi = smem_take(&off, (size_t)zcap * 4);
+    L.dup = smem_take(&off, (size_t)L.P * 4);
     L.total = off;
     return L;
 }
@@ -1218,7 +1168,7 @@ __global__ void __launch_bounds__(kThreads) k_locate_votes(const VoteArgs a) {
         uint8_t v = 1;
         locate_bin(a.t, a.nrep, a.beta,
                    [&](uint32_t r) {
-                       return phase01<double>(mul_conj_rn(a.u[(size_t)r * a.B + j], a.up[(size_t)r * a.B + j]));
+                       return phase01(mul_conj_rn(a.u[(size_t)r * a.B + j], a.up[(size_t)r * a.B + j]));
                    },
                    sb_fp, a.w_fp, logM, a.s, hw_fix, l, v, a.votes + (size_t)j * a.t);
         a.l_fp[j] = l;
@@ -1236,11 +1186,11 @@ __host__ __device__ inline EstLayout est_layout(uint32_t m) {
     uint32_t P = 1;
     while (P < m) P <<= 1;
     L.P = P;
-    L.w = gtake(&off, (size_t)m * 16);
-    L.mag = gtake(&off, (size_t)m * 8);
-    L.perm = gtake(&off, (size_t)P * 4);
-    L.keep = gtake(&off, (size_t)m * 4);
-    L.scan = gtake(&off, (size_t)(kThreads + 8) * 4);
+    L.w = smem_take(&off, (size_t)m * 16);
+    L.mag = smem_take(&off, (size_t)m * 8);
+    L.perm = smem_take(&off, (size_t)P * 4);
+    L.keep = smem_take(&off, (size_t)m * 4);
+    L.scan = smem_take(&off, (size_t)(kThreads + 8) * 4);
     L.total = off;
     return L;
 }

@@ -240,7 +240,7 @@ struct GenArgs {
     const float2* x;
     float2* xperm;         // [batch][n] x_{sigma m} under the round's LocateInner sigma, or null
     uint64_t n;
-    uint32_t nmask, logn;
+    uint32_t nmask;
     uint64_t seed;
     uint32_t round;
     uint32_t req_base;     // request index of the launch's first request
