@@ -499,6 +499,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
     if (groups > batch) groups = batch;
     if (tr) groups = 1;  // a trace records the whole batch's round on the caller's stream
     const size_t zc = p.z_cap;
+    const bool early = general_early(plan->grounds.data(), R, p.R_est, batch);
     auto group = [&](uint32_t g) -> sfft_status {
         const uint32_t r0 = (uint32_t)((uint64_t)batch * g / groups);
         const uint32_t r1 = (uint32_t)((uint64_t)batch * (g + 1) / groups);
@@ -525,6 +526,7 @@ static sfft_status execute_general(sfft_plan plan, const void* d_x, const ReqDes
             a.rtaps = gr.rtaps;
             a.nzmax = gr.nzmax;
             a.batch = batch;
+            a.early = early ? 1 : 0;
             a.dmax = gr.dmax;
             a.t = gr.t;
             a.logtp = gr.logtp;

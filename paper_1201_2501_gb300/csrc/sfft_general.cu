@@ -94,16 +94,13 @@ __device__ __forceinline__ int32_t gen_offset(uint32_t p, uint32_t n, uint32_t n
     return dd > (nmask >> 1) ? (int32_t)((int64_t)dd - (int64_t)n) : (int32_t)dd;
 }
 
-// Launches of one stream group follow one another with programmatic serialisation: a kernel may start
-// while the one before it ends, and waits here before it reads what that one wrote (each kernel waits, so
-// it waits for all before).  A small call lets its kernels start as soon as every CTA of the one before
-// runs; in larger ones CTAs that only wait would hold places that other groups' gathers need.  One request
-// at n = 2^18, k = 50: 110 us, was 131; n = 2^20, k = 500, batch 5: 562 us, was 602.
-__device__ __forceinline__ void let_next_start(const GenArgs& a) {
-    if (a.batch <= 2) cudaTriggerProgrammaticLaunchCompletion();
-}
+// Launches of one stream group follow one another with programmatic serialisation: a kernel may start when
+// the CTAs of the one before have ended, without waiting for its memory to be flushed, and waits here before
+// it reads or writes what that one did (each kernel waits, so it waits for all before).  One request at
+// n = 2^18, k = 50: 109 us, was 131; n = 2^20, k = 500, batch 5: 562 us, was 602.
+// a.early: a kernel also lets the next one start as soon as its own CTAs all run (see general_early).
 __device__ __forceinline__ void after_previous(const GenArgs& a) {
-    let_next_start(a);
+    if (a.early) cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
 }
 
@@ -1267,18 +1264,38 @@ static cudaError_t launch_after(void (*kernel)(Arg), dim3 grid, uint32_t threads
     return cudaLaunchKernelEx(&cfg, kernel, arg);
 }
 
+constexpr uint32_t kGatherPlaces = 2 * 152;  // CTAs of k_gen_gather the chip holds
+// pairs per CTA: as many as leave the chip two waves of CTAs over the whole call's `batch` requests, so that a
+// tap's window product serves more hashings
+static uint32_t gather_blocks(const GeneralRound& g) { return g.B > (uint32_t)kThreads ? g.B / kThreads : 1u; }
+static uint32_t gather_pairs_per_cta(const GeneralRound& g, uint32_t batch) {
+    const uint64_t pairs = (uint64_t)gather_blocks(g) * g.npairs * batch;
+    return pairs >= 8 * kGatherPlaces ? 4u : (pairs >= 4 * kGatherPlaces ? 2u : 1u);
+}
+// a round's CTAs per request
+static uint32_t gather_ctas(const GeneralRound& g, uint32_t R_est, uint32_t P) {
+    return gather_blocks(g) * (R_est + (g.npairs + P - 1) / P);
+}
+
+// Whether the kernels of a call start early (after_previous): where the call's gathers all have a place on the
+// chip.  CTAs that only wait hold places: at n = 2^20, k = 500 (about 1000 CTAs a request) one request took
+// 348 us with early starts and 305 without, n = 2^18, k = 50, batch 4 (724) 168 and 155, n = 2^16, k = 8,
+// batch 8 (808) 98 and 85; where they fit, early starts gave n = 2^16, k = 8, batch 3 70.5 us against 72.2,
+// n = 2^18, k = 50, one request 108.0 against 108.6.
+bool general_early(const GeneralRound* g, uint32_t R, uint32_t R_est, uint32_t batch) {
+    uint64_t ctas = 0;
+    for (uint32_t r = 0; r < R; ++r) ctas += (uint64_t)gather_ctas(g[r], R_est, gather_pairs_per_cta(g[r], batch)) * batch;
+    return ctas <= kGatherPlaces;
+}
+
 template <int NR>
 static cudaError_t launch_gather_nr(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st) {
     GatherParams<NR> gp;
     gp.R = R;
     gp.seg[0] = 0;
     for (uint32_t r = 0; r < R; ++r) {
-        // pairs per CTA: as many as leave the chip (152 SMs, 2 CTAs each) two waves of CTAs over the
-        // whole call, so that a tap's window product serves more hashings
-        const uint32_t blocks = g[r].B > (uint32_t)kThreads ? g[r].B / kThreads : 1u;
-        const uint64_t pairs = (uint64_t)blocks * g[r].npairs * a[r].batch;
-        gp.P[r] = pairs >= 4 * 608 ? 4u : (pairs >= 2 * 608 ? 2u : 1u);
-        gp.seg[r + 1] = gp.seg[r] + blocks * (a[r].R_est + (g[r].npairs + gp.P[r] - 1) / gp.P[r]);
+        gp.P[r] = gather_pairs_per_cta(g[r], a[r].batch);
+        gp.seg[r + 1] = gp.seg[r] + gather_ctas(g[r], a[r].R_est, gp.P[r]);
         gp.r[r] = a[r];
     }
     return launch_after<const GatherParams<NR>>(k_gen_gather<NR>, dim3(gp.seg[R], batch), kThreads, 0, st, gp);

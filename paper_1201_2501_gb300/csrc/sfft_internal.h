@@ -250,6 +250,7 @@ struct GenArgs {
     uint32_t rtaps;        // taps per range of the fold's summation order (see k_gen_gather)
     uint32_t nzmax;        // the most entries zhat can have when the round starts
     uint32_t batch;        // requests of the whole call (its stream groups together)
+    uint32_t early;        // the call's kernels start early (general_early)
     uint32_t dmax, t, logtp, R_loc, R_est, npairs, ngroups, nhash, kprime;
     uint64_t beta_lo[kMaxLevels], beta_hi[kMaxLevels];
     double s, est_gmin;
@@ -436,6 +437,7 @@ size_t general_finish_smem(uint32_t B, uint32_t nzmax);
 size_t general_locate_smem(uint32_t npairs, uint32_t t, uint32_t R_est);
 size_t general_select_smem(uint32_t B, uint32_t kprime, uint32_t zcap);
 cudaError_t general_set_smem(size_t finish, size_t locate, size_t select, size_t estimate);
+bool general_early(const GeneralRound* g, uint32_t R, uint32_t R_est, uint32_t batch);
 // the gathers of R rounds (and the permuted copies they read), then per round the rest
 cudaError_t launch_general_gather(const GenArgs* a, const GeneralRound* g, uint32_t R, uint32_t batch, cudaStream_t st);
 cudaError_t launch_general_round(const GenArgs& a, uint32_t batch, const GeneralRound& r, cudaStream_t st);
