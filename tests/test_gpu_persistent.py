@@ -116,3 +116,29 @@ def test_a_wait_that_nothing_ends_gives_up_with_a_status(sf):
     got = _rows(sf.sfft_execute(plan, torch.as_tensor(s.x[None]).cuda(), 5, f["z_cap"]), 1)[0]
     assert np.array_equal(got[0], s.support)
     plan.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_every_kind_of_decode_in_one_batch(sf, prec):
+    """A plan whose decode keeps its entries as bit masks runs by lists beside one that needs lists, and beside
+    one with arrays sized by what is found: the bits of its own execution, k up to the capacity of the masks."""
+    sizes = [(14, 8), (16, 64 if prec == 0 else 40), (18, 66), (16, 200)]
+    fields = [exact_fields(1 << m, k, z_cap=256 if k in (40, 64) else max(4 * k, 64)) for m, k in sizes]
+    plans = [sf.Plan(gpu_params(sf, f, prec), 3) for f in fields]
+    dt = np.complex128 if prec else np.complex64
+    sigs = [(pi, workloads.exact_sparse(1 << m, k, workloads.seed_for(8, 900 + 10 * pi + i), dtype=dt))
+            for i in range(3) for pi, (m, k) in enumerate(sizes)]
+    xs = [torch.as_tensor(s.x).cuda() for _, s in sigs]
+    cap = max(f["z_cap"] for f in fields)
+    for chosen in ([0, 1, 2, 3], [0, 1, 2], [0, 1], [2, 3], [0, 3]):
+        at = [r for r, (pi, _) in enumerate(sigs) if pi in chosen]
+        bp = sf.BatchPlan([plans[pi] for pi in chosen], len(at))
+        got = _rows(bp.execute([chosen.index(sigs[r][0]) for r in at], [xs[r] for r in at], [31 + r for r in at], at, cap),
+                    len(at))
+        for g, r in zip(got, at):
+            one = _rows(sf.sfft_execute_requests(plans[sigs[r][0]], [xs[r]], [31 + r], [r], cap), 1)[0]
+            assert np.array_equal(g[0], one[0]) and np.array_equal(g[1], one[1]) and g[2] == one[2], (chosen, r)
+            assert np.array_equal(g[0], sigs[r][1].support)
+        bp.close()
+    for p in plans:
+        p.close()
