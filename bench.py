@@ -386,7 +386,7 @@ def run_general(args):
                        "l2l2_ratio_mean": float(np.mean(ratios)), "l2l2_ratio_max": float(np.max(ratios))},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": None,
-                         "kernel": "k_gen_gather + k_gen_finish + k_gen_locate + k_gen_estimate (all rounds)",
+                         "kernel": "k_gen_permute + k_gen_gather + k_gen_finish + k_gen_locate + k_gen_select (all rounds)",
                          "bytes_per_transform": samples * 32, "samples_per_transform": samples,
                          "peak_kind": peak_kind},
             "e2e": e2e, "clocks": clk.summary(),
@@ -1140,8 +1140,8 @@ def mixed_batch_measurement(sfft, args):
     """Uneven instances in one batch: n = 2^e and k drawn uniformly from the grids above (log-uniform
     over 2^16..2^24 and 8..512), half exactly k-sparse and half k heavy coefficients (|X| in [1, 10])
     plus complex Gaussian time noise at SNR 20 dB, every signal resident on the device.  The exact half
-    runs as ONE persistent launch over all its plans (sfft_batch_execute); the noisy half as per-round
-    launches of each plan on a second stream, at the same time.  Device-timed with CUDA events."""
+    runs through sfft_batch_execute over all its plans at once (two launches side by side); the noisy half as
+    sfft_execute of each plan on a second stream, at the same time.  Device-timed with CUDA events."""
     import torch
 
     from paper_1201_2501_gb300 import workloads
@@ -1228,13 +1228,13 @@ def mixed_batch_measurement(sfft, args):
                     "(|X| = 1), half k heavy (|X| = 10^U[0,1]) + complex Gaussian time noise at SNR 20 dB; "
                     "library default B and w (bins_per_k 4 / 8, alpha0 1/2, delta 1e-6)",
         "requests": nreq, "exact_requests": len(ex), "general_requests": nreq - len(ex),
-        "exact_plans_in_one_persistent_launch": len(xplans), "general_plans": len(gruns),
+        "exact_plans_in_one_call": len(xplans), "general_plans": len(gruns),
         "ms_total": ms_both, "transforms_per_s": nreq / (ms_both / 1000.0),
         "ms_exact_alone": ms_exact, "ms_general_alone": ms_general,
         "exact_support_fraction": exact_ok / max(1, len(ex)),
         "general_rel_l2_to_heavy_mean": float(np.mean(rel)) if rel else None,
-        "what": "device time of both halves launched together (persistent exact launch on one stream, "
-                "per-round general launches on another)",
+        "what": "device time of both halves launched together (the exact half's mixed batch on one stream, "
+                "the general plans on another)",
     }
 
 
@@ -1418,8 +1418,8 @@ def main():
     ap.add_argument("--mixed", action="store_true", help="also time the uneven mixed batch (1024 requests)")
     ap.add_argument("--mixed-requests", type=int, default=1024)
     ap.add_argument("--path", default="step", choices=["step", "persistent"],
-                    help="one k_exact_step launch per step and stream group (all rounds), or the persistent "
-                         "work-queue launch")
+                    help="one k_exact_step launch per step and stream group (all rounds), or the same batch as "
+                         "requests of a mixed batch (sfft_batch_execute)")
     ap.add_argument("--precision-table", action="store_true", help="print the precision-variant table instead")
     ap.add_argument("--precision-batch", type=int, default=16)
     ap.add_argument("--serve-requests", type=int, default=2000)

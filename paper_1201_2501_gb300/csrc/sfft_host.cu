@@ -220,22 +220,62 @@ void twiddle_tables_host(uint64_t n, uint32_t sh, std::vector<double2>* out) {
     for (uint64_t a = 0; a < hi; ++a) (*out)[lo + a] = root_of_unity(a << sh, n);
 }
 
+namespace {
+// h + l, |l| <= ulp(h) / 2: about 106 bits, of doubles alone, so that every host rounds a table alike (a long
+// double has 64 bits on x86-64 and 113 on Arm)
+struct Wide {
+    double h, l;
+};
+Wide wide(double a, double b) {  // a + b, |a| >= |b| or a == 0
+    const double s = a + b;
+    return {s, b - (s - a)};
+}
+Wide sum(Wide a, Wide b) {
+    const double s = a.h + b.h, t = s - a.h;
+    return wide(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
+}
+Wide product(Wide a, Wide b) {
+    const double p = a.h * b.h;
+    return wide(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+Wide quotient(Wide a, double d) {
+    const double q = a.h / d;
+    return wide(q, (std::fma(-q, d, a.h) + a.l) / d);
+}
+// sin a and cos a - 1 for a = 2 pi m / n, m <= n / 8, from their power series
+void sin_cosm1(uint64_t m, uint64_t n, Wide* sn, Wide* cm1) {
+    const Wide a = product({6.283185307179586232, 2.449293598294706414e-16}, {(double)m / (double)n, 0.0});
+    const Wide minus_a2 = product(a, {-a.h, -a.l});
+    Wide odd = a, even = quotient(minus_a2, 2);
+    *sn = odd;
+    *cm1 = even;
+    for (int k = 3; k <= 29; k += 2) {  // a^29 / 29! < 2^-110
+        odd = quotient(product(odd, minus_a2), (double)k * (k - 1));
+        even = quotient(product(even, minus_a2), (double)k * (k + 1));
+        *sn = sum(*sn, odd);
+        *cm1 = sum(*cm1, even);
+    }
+}
+// exp(-2 pi i m / n), n a power of two of 8 or more, m < n
+double2 root_rounded(uint64_t m, uint64_t n) {
+    const uint64_t quarter = n / 4, q = m / quarter, rem = m % quarter;
+    Wide sn, cm1;
+    sin_cosm1(rem <= n / 8 ? rem : quarter - rem, n, &sn, &cm1);
+    double c = sum({1.0, 0.0}, cm1).h, s = sn.h;
+    if (rem > n / 8) std::swap(c, s);
+    return q == 0 ? make_double2(c, -s) : q == 1 ? make_double2(-s, -c) : q == 2 ? make_double2(-c, s) : make_double2(s, c);
+}
+}  // namespace
+
 void twiddle_tables_exact_host(uint64_t n, uint32_t sh, std::vector<double2>* out) {
     const uint64_t lo = uint64_t(1) << sh, hi = n >> sh;
-    const long double two_pi = 6.283185307179586476925286766559005768L;
-    auto root = [&](uint64_t m) {
-        const long double th = two_pi * (long double)m / (long double)n;
-        return make_double2((double)cosl(th), (double)-sinl(th));
-    };
     out->resize(lo + hi);
-    for (uint64_t b = 0; b < lo; ++b) {  // cos - 1 = -2 sin^2 of the half angle
-        const long double half = sinl(two_pi * (long double)b / (long double)n / 2);
-        (*out)[b] = make_double2((double)(-2 * half * half), root(b).y);
+    for (uint64_t b = 0; b < lo; ++b) {  // (lo <= n / 8)
+        Wide sn, cm1;
+        sin_cosm1(b, n, &sn, &cm1);
+        (*out)[b] = make_double2(cm1.h, -sn.h);
     }
-    for (uint64_t a = 0; a < hi; ++a) (*out)[lo + a] = root(a << sh);
-    // the quarter turns exactly
-    for (int q = 1; q < 4 && hi >= 4; ++q)
-        (*out)[lo + hi / 4 * q] = make_double2(q == 2 ? -1.0 : 0.0, q == 1 ? -1.0 : (q == 3 ? 1.0 : 0.0));
+    for (uint64_t a = 0; a < hi; ++a) (*out)[lo + a] = root_rounded(a << sh, n);
 }
 
 void window_gprime_host(uint64_t n, uint32_t B, double alpha, double delta, uint64_t len, double* W) {

@@ -404,7 +404,7 @@ inline uint32_t ilog2_host(uint64_t v) {  // v a power of two
 // FP64 twiddle factor tables for n = 2^L and split sh: out[b] = exp(-2 pi i b / n), b < 2^sh, then
 // out[2^sh + a] = exp(-2 pi i a 2^sh / n), a < n / 2^sh
 void twiddle_tables_host(uint64_t n, uint32_t sh, std::vector<double2>* out);
-// the same less one in the first part (root_pow_fine), every entry rounded from extended precision
+// the same less one in the first part (root_pow_fine), every entry correctly rounded on any host
 void twiddle_tables_exact_host(uint64_t n, uint32_t sh, std::vector<double2>* out);
 void window_table_host(uint64_t n, const double* g, int64_t T, uint64_t len, double* W);
 int64_t window_halfwidth(uint32_t B, double alpha, double delta);
