@@ -113,7 +113,7 @@ uint32_t exact_owner_ring(uint64_t maxshift, uint32_t B, bool fp64) {
 // g w^e of a tap, w = exp(-2 pi i / n), e = sigma b t (taken mod n): a sincospif in FP32; from the factor
 // tables in FP64, whose sincospi took most of the FP64 gather's time.  With the bins' FFT and the
 // subtraction terms from the tables and the decisions in guarded FP32 (decode_bin_guarded): n = 2^20,
-// k = 64, batch 16: 142 us a call, was 230; n = 2^14, k = 8, one request: 48 us, was 76.
+// k = 64, batch 16: 134 us a call, was 228; n = 2^14, k = 8, one request: 42 us, was 73.
 __device__ __forceinline__ float2 tap_factor(const ExactArgs& a, float g, uint32_t ex, float two_over_n) {
     const uint32_t e = ex & a.nmask;
     const int32_t es = e > (a.nmask >> 1) ? (int32_t)((int64_t)e - (int64_t)a.n) : (int32_t)e;
@@ -1208,7 +1208,7 @@ __device__ bool finish_round(const ExactArgs& a, uint32_t s, uint32_t sigma, uin
 // memory only when they do not fit a.large_smem bytes): the entries' terms lie by bin (stable counting
 // split with per-warp counters), the bins are read straight from the round's area, and the candidates
 // are sorted by a bitonic network.  Bound by latency (about 40 barriers, 80 with a sort).  Measured with
-// gather_owner at n = 2^24, k = 1000, batch 12: 592 us a call, was 1005 (arrays sized by capacity in
+// gather_owner at n = 2^24, k = 1000, batch 12: 543 us a call, was 1026 (arrays sized by capacity in
 // device memory, long bin lists sorted by insertion, one CTA per SM, 140 partial folds per round).
 struct LargeLayout {
     size_t e_idx, pre, key, cval, start, slot, s_idx, s_gain, s_t0, s_tf, cnt, out_idx, out_val, keep, scan, total;
@@ -1863,7 +1863,7 @@ __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_chan_decode
 // request)), the decodes are chained by arrival counters and nothing waits.  A round's argument block
 // comes from device memory, its per-request fields are pointed at the request's own workspace.  Against
 // the device queue it replaces, where a request's next round was gathered only after the last one's
-// decode: 452 us, was 880 (96 requests of six plans, n = 2^16 .. 2^22).
+// decode: 408 us, was 870 (96 requests of six plans, n = 2^16 .. 2^22).
 template <typename R, int KIND>
 __global__ void __launch_bounds__(kThreads, SFFT_ROUND_MIN_BLOCKS) k_exact_batch(const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];

@@ -260,9 +260,10 @@ __device__ __forceinline__ void gather_pairs(const GenArgs& a, const ReqView& rq
 // Every round's hashings in one launch (their samples do not depend on zhat): grid (CTAs of all
 // rounds, requests), request by request so that a signal and its copies stay in L2; a round's CTAs
 // are its EstimateValues hashings, then its blocks of P pairs, residue blocks fastest.  The small
-// rounds' few CTAs run beside the first round's.  Whole calls, against one gather per round: n = 2^22,
-// k = 256, batch 8: 774 us, was 963; n = 2^18, k = 50, one request: 132 us, was 150; n = 2^26, k = 64,
-// batch 4: 603 us, was 670 (26.3 M random sectors of HBM: 44 G/s).
+// rounds' few CTAs run beside the first round's.  Whole calls, against one gather per round (which plans near
+// the memory limit still use): n = 2^22, k = 256, batch 8: 742 us, 922; n = 2^18, k = 50, one request: 109 us,
+// 130; n = 2^20, k = 500, batch 5: 566 us, 601.  n = 2^26, k = 64, batch 4 reads 26.3 M random sectors of HBM
+// at 44 G/s.
 template <int NR>
 struct GatherParams {
     uint32_t R;
